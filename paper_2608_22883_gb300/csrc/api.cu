@@ -312,7 +312,8 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
     void* src_row = nullptr;
     void* fix = nullptr;                     // bf16: count word + listed key elements
     const bool bf = p->dtype == FOVEA_BF16;
-    const long long fix_cap = bf ? (long long)total * d / 8 + 4096 : 0;
+    // the list holds 0.47 % of the keys of well-scaled tokens (gemm_build.cu)
+    const long long fix_cap = bf ? (long long)total * d / 32 + 4096 : 0;
     if ((st = alloc_dev(&m->keys, (size_t)total * d * es, "keys")) != FOVEA_OK ||
         (st = alloc_dev(&m->values, (size_t)total * d * es, "values")) != FOVEA_OK ||
         (st = alloc_dev(reinterpret_cast<void**>(&m->orig_index), total * sizeof(int32_t),
@@ -338,26 +339,33 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
         err = launch_ln_rows(p->dtype, v, (const int32_t*)src_row, total, d, p->ln_v_gamma,
                              p->ln_v_beta, p->ln_eps, nullptr, nullptr, 0, m->err, xv, s); }
       if (err != cudaSuccess) return cuda_fail(err, "ln_v");
-      GemmArgs a;
-      init_args(a);
-      a.k_total = d;
-      a.a_split = d;
-      a.b_split = d;
-      a.A0 = p->W_K; a.A1 = p->W_U; a.lda0 = d; a.lda1 = d;
-      a.B0 = xv; a.B1 = xv; a.ldb0 = d; a.ldb1 = d;
-      a.epi_split = d;
-      a.out0 = m->keys; a.out1 = m->values; a.ldc = d;
-      a.err = m->err;
-      a.fix_list = fix_list; a.fix_count = fix_count; a.fix_cap = (int)fix_cap;
-      a.ngroups = 1;
-      a.groups[0] = GemmGroup{0, 2 * d, 0, total, 0};
-      TmaOperand A0{p->W_K, d, d, d}, A1{p->W_U, d, d, d}, B0{xv, total, d, d}, B1{nullptr, 0, 0, 0};
+      PairGemm pg{};
+      pg.rows = total;
+      pg.ldc = d;
+      pg.err = m->err;
       if (bf) {
+        pg.out[0] = m->keys; pg.out[1] = m->values;
+        pg.fix_list = fix_list; pg.fix_count = fix_count; pg.fix_cap = (int)fix_cap;
         err = cudaMemsetAsync(fix_count, 0, sizeof(int), s);
         if (err != cudaSuccess) return cuda_fail(err, "cudaMemsetAsync");
+        KernelTimer t("memory_proj", s);
+        err = launch_pair_gemm(kPairKeys, pg, TmaOperand{p->W_K, d, d, d},
+                               TmaOperand{p->W_U, d, d, d}, TmaOperand{xv, total, d, d}, s);
+      } else {
+        GemmArgs a;
+        init_args(a);
+        a.k_total = d;
+        a.a_split = d;
+        a.b_split = d;
+        a.A0 = p->W_K; a.A1 = p->W_U; a.lda0 = d; a.lda1 = d;
+        a.B0 = xv; a.B1 = xv; a.ldb0 = d; a.ldb1 = d;
+        a.epi_split = d;
+        a.out0 = m->keys; a.out1 = m->values; a.ldc = d;
+        a.ngroups = 1;
+        a.groups[0] = GemmGroup{0, 2 * d, 0, total, 0};
+        KernelTimer t("memory_proj", s);
+        err = launch_gemm_simt(p->dtype, kEpiStore, a, 2 * d, total, s);
       }
-      { KernelTimer t("memory_proj", s);
-        err = run_gemm(p->dtype, bf ? kEpiStoreKeys : kEpiStore, a, A0, A1, B0, B1, 2 * d, total, s); }
       if (err != cudaSuccess) return cuda_fail(err, "memory projection");
       if (bf) {
         // keys whose fp32 value sat near a bf16 rounding midpoint: exact recompute
@@ -392,21 +400,12 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
           { KernelTimer t("transpose_wq", s);
             err = launch_transpose_bf16(p->W_Q, d, d, wqt, s); }
           if (err != cudaSuccess) return cuda_fail(err, "transpose W_Q");
-          GemmArgs fa;
-          init_args(fa);
-          fa.k_total = d;
-          fa.b_split = d;
-          fa.B0 = m->keys; fa.ldb0 = d;
-          fa.out0 = m->folded;
-          fa.out1 = static_cast<__nv_bfloat16*>(m->folded) + d;
-          fa.ldc = 2 * d;
-          fa.err = m->err;
-          fa.ngroups = 1;
-          fa.groups[0] = GemmGroup{0, d, 0, total, 0};
+          pg.out[0] = m->folded;
+          pg.out_lo = static_cast<__nv_bfloat16*>(m->folded) + d;
+          pg.ldc = 2 * d;
           { KernelTimer t("memory_fold", s);
-            err = launch_gemm_tc(kEpiStoreHiLo, fa, TmaOperand{wqt, d, d, d},
-                                 TmaOperand{nullptr, 0, 0, 0}, TmaOperand{m->keys, total, d, d},
-                                 TmaOperand{nullptr, 0, 0, 0}, d, total, s); }
+            err = launch_pair_gemm(kPairHiLo, pg, TmaOperand{wqt, d, d, d},
+                                   TmaOperand{nullptr, 0, 0, 0}, TmaOperand{m->keys, total, d, d}, s); }
           if (err != cudaSuccess) return cuda_fail(err, "query folding of the keys");
           int fe = 0;
           err = cudaMemcpyAsync(&fe, m->err, sizeof(int), cudaMemcpyDeviceToHost, s);
@@ -431,20 +430,12 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
         if (ps != FOVEA_OK) return ps;
         const __nv_bfloat16* wf1r = static_cast<const __nv_bfloat16*>(p->W_f1) + d;
         const __nv_bfloat16* wg1r = static_cast<const __nv_bfloat16*>(p->W_g1) + d;
-        GemmArgs pa;
-        init_args(pa);
-        pa.k_total = d;
-        pa.a_split = H;
-        pa.b_split = d;
-        pa.B0 = m->values; pa.ldb0 = d;
-        pa.out0 = m->proj; pa.ldc = 2 * H;
-        pa.err = m->err;
-        pa.ngroups = 1;
-        pa.groups[0] = GemmGroup{0, 2 * H, 0, total, 0};
+        pg.out[0] = m->proj;
+        pg.out[1] = static_cast<__nv_bfloat16*>(m->proj) + H;
+        pg.ldc = 2 * H;
         { KernelTimer t("memory_proj_fusion", s);
-          err = launch_gemm_tc(kEpiStore, pa, TmaOperand{wf1r, H, d, 2 * d},
-                               TmaOperand{wg1r, H, d, 2 * d}, TmaOperand{m->values, total, d, d},
-                               TmaOperand{nullptr, 0, 0, 0}, 2 * H, total, s); }
+          err = launch_pair_gemm(kPairStore, pg, TmaOperand{wf1r, H, d, 2 * d},
+                                 TmaOperand{wg1r, H, d, 2 * d}, TmaOperand{m->values, total, d, d}, s); }
         if (err == cudaSuccess) err = cudaStreamSynchronize(s);
         if (err != cudaSuccess) return cuda_fail(err, "fusion projection of the values");
         int m_max = 0;

@@ -135,8 +135,6 @@ enum EpiKind : int {
   kEpiBiasSilu = 2,   // out0[row * ldc + col] = T(silu(acc + bias{0,1}[col]))
   kEpiBiasF32 = 3,    // out0 (fp32)[row * ldc + col] = acc + bias0[col]
   kEpiStoreHiLo = 4,  // out0 = T(acc), out1 = T(acc - out0): acc carried as two stored values
-  kEpiStoreKeys = 5,  // kEpiStore, and columns < epi_split whose acc lies near a bf16
-                      // rounding midpoint are listed for an exact recomputation
   kEpiQueryH = 6,     // columns < epi_split as kEpiStoreHiLo; columns >= epi_split:
                       // out2 (fp32)[row * ldc2 + col - epi_split] = acc
   kEpiScoresFolded = 7,  // kEpiScores with one row operand (x_h) against the folded
@@ -152,10 +150,6 @@ enum EpiKind : int {
                          // key << 32 | ~column) into cand[row * cand_ld + slot * cand_k + r],
                          // slot = feature tile * splits + rank, r = 0, 1, ... in descending
                          // key order (zeros last: fewer columns than cand_k)
-};
-
-struct KeyFix {       // one listed key element: memory row, feature
-  int row, col;
 };
 
 struct GemmArgs {
@@ -178,7 +172,6 @@ struct GemmArgs {
   void* out2; long long ldc2;                      // kEpiQueryH
   const void* bias0; const void* bias1;
   const float* row_scale; float scale;
-  KeyFix* fix_list; int* fix_count; int fix_cap;   // kEpiStoreKeys
   int splits;         // tensor-core path: CTAs of a cluster sharing one output tile (split K)
   int stages;         // tensor-core path: depth of the shared-memory ring
   int tx_bytes;       // tensor-core path: bytes one ring stage receives (row box + feature tile)
@@ -280,9 +273,6 @@ cudaError_t launch_select_gather(int dtype, const float* scores, const SeqTable&
                                  float* r_out, void* r_lo, const void* P, int H, const float* Gh,
                                  const void* b_f1, const void* b_g1, void* act, int* err,
                                  cudaStream_t s, long long p_prefetch_bytes = 0);
-// Exact rounding of listed key elements: k = sum_l x[row, l] W[col, l]
-// evaluated in double-float, rounded once to bf16.  list == nullptr refines
-// every element of the [rows, d] key matrix.
 // out[c * rows + r] = in[r * cols + c] for a bf16 [rows, cols] matrix, rows
 // and cols multiples of 32 (the query folding's W_Q^T, once per memory build).
 cudaError_t launch_transpose_bf16(const void* in, int rows, int cols, void* out, cudaStream_t s);
@@ -307,8 +297,6 @@ cudaError_t launch_merge_candidates(const unsigned long long* cand, int N, int s
 // tiles times its split-K factor).
 int lm_head_slots(int vocab, int d_model, int N);
 
-cudaError_t launch_refine_keys(const void* xv, const void* W, int d, const KeyFix* list,
-                               const int* count, int cap, int rows, void* K, cudaStream_t s);
 // Rows past the depth gate: h_out = h and gate 0.
 cudaError_t launch_finalize(int dtype, const void* h, const float* c, const void* act, int H, int d,
                             const void* w_g2, const void* b_g2, const void* rms_gamma, float eps,
@@ -336,13 +324,42 @@ struct GemmPlan {
   int kps;                    // k-blocks of 64 per ring stage
 };
 GemmPlan plan_gemm_tc(int epi, const GemmArgs& a, int max_m, int max_n);
-// Tensor map of a row-major [rows, cols] bf16 matrix (row stride ld
-// elements), 128-byte swizzle, box = 64 columns x box_rows rows.
-bool encode_bf16_map(CUtensorMap* m, const void* base, long long rows, long long cols,
-                     long long ld, int box_rows);
+// Tensor map (cached per thread) of a row-major [rows, cols] bf16 matrix, cols
+// a multiple of 64, as (64 k, rows, cols / 64 k-blocks) with 128-byte swizzle;
+// box = 64 x box_rows x kps.
+bool encode_kblock_map(CUtensorMap* m, const TmaOperand& op, int box_rows, int kps);
 // A2 (optional): the feature operand of output columns >= a_split2.
 cudaError_t launch_gemm_tc(int epi, const GemmArgs& a, const TmaOperand& A0, const TmaOperand& A1,
                            const TmaOperand& B0, const TmaOperand& B1, int max_m, int max_n,
                            cudaStream_t s, const TmaOperand& A2 = TmaOperand{nullptr, 0, 0, 0});
+
+// The memory build's GEMMs out = R . F^T on CTA pairs (gemm_build.cu): R
+// [rows, K] token rows against one or two feature matrices F0, F1 [cols, K]
+// (bf16), fp32 sums stored as bf16 with row stride ldc.
+enum PairEpi : int {
+  kPairStore = 0,     // part p (F0, F1) to out[p]
+  kPairKeys = 1,      // the same, and part 0's elements near a rounding midpoint are listed
+  kPairHiLo = 2,      // one part: hi = bf16(sum) to out[0], bf16(sum - hi) to out_lo
+};
+struct KeyFix {       // one listed key element: memory row, feature
+  int row, col;
+};
+struct PairGemm {
+  int rows;                                      // token rows
+  void* out[2]; void* out_lo; long long ldc;
+  KeyFix* fix_list; int* fix_count; int fix_cap; // kPairKeys
+  int* err;
+  // filled by the launch
+  int k_blocks, cols[2], tiles0, feat_tiles, row_tiles;
+  unsigned long long wait_ns;
+};
+cudaError_t launch_pair_gemm(PairEpi epi, PairGemm a, const TmaOperand& F0, const TmaOperand& F1,
+                             const TmaOperand& R, cudaStream_t s);
+
+// Exact rounding of listed key elements: k = sum_l x[row, l] W[col, l]
+// evaluated in double-float, rounded once to bf16.  list == nullptr refines
+// every element of the [rows, d] key matrix.
+cudaError_t launch_refine_keys(const void* xv, const void* W, int d, const KeyFix* list,
+                               const int* count, int cap, int rows, void* K, cudaStream_t s);
 
 }  // namespace fovea

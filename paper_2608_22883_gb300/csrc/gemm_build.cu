@@ -1,0 +1,514 @@
+// The memory build's GEMMs C = X . W^T (bf16, fp32 sums) on CTA pairs: the
+// keys and values (W_K ; W_U against LN(v)), the folded keys (W_Q^T against
+// the keys) and the projected values ([W_f1 ; W_g1]_r against the values).
+// Thousands of token rows meet thousands of features, so, unlike the draft
+// step's GEMMs (gemm_tc.cu), these are bound by the tensor pipe and by what
+// feeds it.
+//
+// Tile and split.  A pair of CTAs (one cluster, tcgen05 cta_group::2) owns a
+// tile of 256 tokens x 256 features: each CTA stages its 128 token rows and
+// its half of the features, and the pair's MMA (M = 256, N = 256) reads both
+// halves.  A one-CTA tile of 128 x 256 moves 48 KB through shared memory per
+// k-block twice (TMA write, tensor-core read), 750 cycles at 128 B/cycle
+// against the MMA's 516; the pair moves 32 KB per CTA, which the MMA covers.
+// The grid is persistent, one pair per two SMs, and the accumulator is
+// double-buffered in tensor memory (2 x 256 columns), so the epilogue of one
+// buffer runs under the MMAs of the other.
+//
+// Chunked sums.  The tensor core adds a product sum to its fp32 accumulator
+// with truncation, once per 16 elements of the contraction, so a long
+// contraction drifts by about 2^-17 of the result's scale.  Here every chunk
+// of kChunkSu * KPS * 64 = 256 elements starts a fresh accumulator, and the
+// epilogue threads add the chunks in registers with rounded fp32 additions.
+// A key must be the correctly rounded bf16 of its exact sum; the keys whose
+// sum lies so near a rounding midpoint that the GEMM cannot tell are listed
+// and recomputed exactly (refine_keys_kernel).  The window of that list
+// follows the error of the sum (kKeyWindow below).
+//
+// Roles (320 threads): warp 0 lanes 0 and 1 issue the TMA loads of this CTA's
+// features and tokens, warp 1 allocates the tensor memory and, in the leader
+// CTA (cluster rank 0), its lane 0 issues the MMAs of the pair; warps 2 .. 9
+// run the epilogue: warp w reads accumulator lanes (tokens) 32 (w % 4) .. +31
+// and one half of the columns, 128 fp32 sums per thread.  Stage barriers
+// (`full`) live in the leader and count both CTAs' bytes; commits signal
+// both CTAs (`empty`, `tfull`); the epilogue warps of both release a buffer
+// to the leader (`tempty`).
+//
+// Every wait is bounded.  A role whose wait gives up sets its CTA's abort
+// flag and leaves its loop; the pair meets at a cluster barrier, which both
+// CTAs reach because all waits are bounded, and when either has aborted the
+// leader commits the MMAs it issued, both wait for them and for the copies
+// in flight (bounded), and only then is the tensor memory freed.
+#include "tc_ptx.cuh"
+
+namespace fovea {
+namespace pair {
+
+using namespace tc;
+
+constexpr int BM = 128;                  // token rows per CTA (256 per pair)
+constexpr int BN = 256;                  // features per pair
+constexpr int BNH = BN / 2;              // features each CTA stages
+constexpr int KPS = 2;                   // k-blocks of 64 per stage
+constexpr int kSmemRows = BM * 128;      // bytes of one k-block of tokens
+constexpr int kSmemFeat = BNH * 128;     // bytes of one k-block of this CTA's features
+constexpr int kStageBytes = KPS * (kSmemRows + kSmemFeat);
+constexpr int kStages = 3;
+constexpr int kChunkSu = 2;              // stages per accumulator chunk
+constexpr int kEpiWarps = 8;
+constexpr int kThreads = 64 + 32 * kEpiWarps;
+constexpr int kWarpStage = 32 * 128;     // an epilogue warp's staging: 32 rows x 64 bf16
+constexpr int kSmemBytes = 1024 + kStages * kStageBytes + kEpiWarps * kWarpStage + 256;
+constexpr int kBandRows = 8;             // row tiles a wave of pairs shares
+constexpr uint32_t kTmemCols = 512;
+// kind::f16: D fp32, A and B bf16, both K-major, N = 256, M = 256
+constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
+                            ((uint32_t)(2 * BM >> 4) << 24);
+
+// Key window: an element is listed when its sum lies within
+// kKeyWindow * max(|sum|, scale) of a bf16 rounding midpoint, scale being the
+// RMS of the token's sums over its half of the tile.  With chunked sums the
+// farthest mis-rounded key from its midpoint, over 3.7e8 keys at d = 256 ..
+// 8192 (none refined, compared with float64), lay 2^-20.4 of that magnitude
+// away, with no trend in d (0.017 % of the keys were mis-rounded); 2^-19
+// keeps a margin of 2.6x and lists 0.47 % of the keys.  One accumulator over
+// the whole contraction needs 2^-15 and lists 5 %: at 32768 tokens, d = 4096
+// their recomputation took 11.0 ms of a 17.5 ms build, now 1.0 ms.
+constexpr float kKeyWindow = 1.0f / 524288.0f;   // 2^-19
+
+__device__ __forceinline__ uint32_t cta_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void tma_load_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar,
+                                              int x, int y, int z) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z)
+      : "memory");
+}
+__device__ __forceinline__ void umma_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
+                                          uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
+      "l"(adesc), "l"(bdesc), "r"(kIdesc), "r"(accumulate)
+      : "memory");
+}
+// Completion of the MMAs issued so far, signalled to the barrier at this
+// offset in both CTAs of the pair.
+__device__ __forceinline__ void commit_pair(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
+      " [%0], %1;" ::"r"(smem_u32(bar)), "h"((unsigned short)3)
+      : "memory");
+}
+__device__ __forceinline__ void arrive_cluster(uint32_t caddr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(caddr) : "memory");
+}
+__device__ __forceinline__ uint32_t try_wait_cluster(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok;
+}
+// mbar_wait with cluster-scope acquire: the barrier is signalled by the peer.
+static __device__ __noinline__ bool wait_cluster(uint64_t* bar, uint32_t parity,
+                                                 volatile int* abort_flag, uint64_t limit_ns) {
+  if (try_wait_cluster(bar, parity)) return true;
+  const uint64_t t0 = globaltimer_ns();
+  while (true) {
+    for (int i = 0; i < 64; ++i)
+      if (try_wait_cluster(bar, parity)) return true;
+    if (abort_flag != nullptr && *abort_flag) return false;
+    if (globaltimer_ns() - t0 > limit_ns) return false;
+  }
+}
+// 16 consecutive fp32 accumulator columns of this thread's lane.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ uint32_t ld_dsmem_u32(uint32_t caddr) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(caddr) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+  const __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&p);
+}
+
+// The midpoint of the two bf16 values around a finite fp32 value is its upper
+// 16 bits followed by 0x8000.  An element whose window reaches the spacing of
+// the bf16 values around it (a sum far below the scale) is always listed, as
+// is one that is not finite.
+__device__ __forceinline__ bool near_midpoint(float acc, float scale) {
+  const float mid = __uint_as_float((__float_as_uint(acc) & 0xFFFF0000u) | 0x8000u);
+  const float window = kKeyWindow * fmaxf(fabsf(acc), scale);
+  return !(fabsf(acc - mid) > window && fabsf(acc) * 0.001953125f >= window);
+}
+
+// One tile of the output: where it lies.
+struct Tile {
+  int part, m0, n_cols, row0;
+};
+__device__ __forceinline__ Tile tile_at(const PairGemm& a, int t) {
+  // bands of kBandRows row tiles; within a band consecutive tiles walk the
+  // rows, so that the pairs of a wave share both operands through L2
+  const int per_band = kBandRows * a.feat_tiles;
+  const int band = t / per_band;
+  const int rows_here = min(kBandRows, a.row_tiles - band * kBandRows);
+  const int local = t - band * per_band;
+  const int ft = local / rows_here;
+  Tile r;
+  r.row0 = (band * kBandRows + local % rows_here) * 2 * BM;
+  r.part = ft < a.tiles0 ? 0 : 1;
+  r.m0 = (r.part ? ft - a.tiles0 : ft) * BN;
+  r.n_cols = min(BN, a.cols[r.part] - r.m0);
+  return r;
+}
+
+// KEYS: part 0 is the keys (rounded, near-midpoint elements listed); HILO:
+// hi = bf16(sum) to out[0] and bf16(sum - hi) to out_lo.
+template <bool KEYS, bool HILO>
+__global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
+    pair_gemm_kernel(const __grid_constant__ CUtensorMap tmF0,
+                     const __grid_constant__ CUtensorMap tmF1,
+                     const __grid_constant__ CUtensorMap tmR, const __grid_constant__ PairGemm a) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  uint8_t* staging = smem + kStages * kStageBytes;
+  uint64_t* full = reinterpret_cast<uint64_t*>(staging + kEpiWarps * kWarpStage);
+  uint64_t* empty = full + kStages;
+  uint64_t* tfull = empty + kStages;
+  uint64_t* tempty = tfull + 2;
+  uint64_t* drain = tempty + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cta_rank();
+  const int pairs = (int)gridDim.x >> 1, pid = (int)blockIdx.x >> 1;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kStages; ++i) {
+      mbar_init(&full[i], 1);
+      mbar_init(&empty[i], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&tfull[i], 1);
+      mbar_init(&tempty[i], 2 * kEpiWarps);
+    }
+    mbar_init(drain, 1);
+    *abort_flag = 0;
+    fence_mbar_init();
+    prefetch_tmap(&tmF0);
+    prefetch_tmap(&tmR);
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)), "r"(kTmemCols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();                        // the peer's barriers are initialised
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  pdl_wait();
+  pdl_trigger();
+  const int tiles = a.feat_tiles * a.row_tiles;
+  const int su_total = (a.k_blocks + KPS - 1) / KPS;   // past the last k-block the maps fill zeros
+
+  if (warp == 0 && lane < 2) {
+    // ---- TMA producers: lane 0 features, lane 1 tokens.  The leader's lane 0
+    // posts the bytes of both CTAs on its full barrier.
+    int i = 0;
+    bool go = true;
+    for (int t = pid; go && t < tiles; t += pairs) {
+      const Tile ti = tile_at(a, t);
+      const CUtensorMap* map = lane == 1 ? &tmR : ti.part ? &tmF1 : &tmF0;
+      const int y = lane == 1 ? ti.row0 + (int)rank * BM : ti.m0 + (int)rank * BNH;
+      for (int su = 0; su < su_total; ++su, ++i) {
+        const int st = i % kStages;
+        if (i >= kStages &&
+            !wait_cluster(&empty[st], ((uint32_t)(i / kStages) & 1u) ^ 1u, abort_flag, a.wait_ns)) {
+          *abort_flag = 1;
+          go = false;
+          break;
+        }
+        if (lane == 0 && rank == 0) mbar_expect_tx(&full[st], 2u * kStageBytes);
+        const uint32_t dst = smem_u32(smem + st * kStageBytes) + (lane == 1 ? 0u : (uint32_t)(KPS * kSmemRows));
+        tma_load_pair(dst, map, map_dsmem(smem_u32(&full[st]), 0), 0, y, su * KPS);
+      }
+    }
+    // the last stages' releases have arrived here before the CTA may leave
+    if (go && lane == 0)
+      for (int j = i > kStages ? i - kStages : 0; j < i; ++j)
+        if (!wait_cluster(&empty[j % kStages], (uint32_t)(j / kStages) & 1u, abort_flag, a.wait_ns)) {
+          *abort_flag = 1;
+          break;
+        }
+  } else if (warp == 1 && lane == 0 && rank == 0) {
+    // ---- MMA issuer of the pair ----
+    int i = 0, c = 0;
+    bool go = true;
+    for (int t = pid; go && t < tiles; t += pairs) {
+      for (int su0 = 0; go && su0 < su_total; su0 += kChunkSu, ++c) {
+        const int buf = c & 1;
+        const uint32_t d = tmem_base + (uint32_t)(buf * BN);
+        if (c >= 2 &&
+            !wait_cluster(&tempty[buf], ((uint32_t)(c >> 1) & 1u) ^ 1u, abort_flag, a.wait_ns)) {
+          *abort_flag = 1;
+          go = false;
+          break;
+        }
+        tc_fence_after();
+        const int su1 = min(su0 + kChunkSu, su_total);
+        for (int su = su0; su < su1; ++su, ++i) {
+          const int st = i % kStages;
+          if (!wait_cluster(&full[st], (uint32_t)(i / kStages) & 1u, abort_flag, a.wait_ns)) {
+            *abort_flag = 1;
+            go = false;
+            break;
+          }
+          const uint32_t stg = smem_u32(smem + st * kStageBytes);
+#pragma unroll
+          for (int j = 0; j < KPS; ++j) {
+            const uint64_t ad = sw128_desc(stg + (uint32_t)(j * kSmemRows));
+            const uint64_t bd = sw128_desc(stg + (uint32_t)(KPS * kSmemRows + j * kSmemFeat));
+#pragma unroll
+            for (int k = 0; k < 4; ++k)          // 32 bytes (16 elements) per MMA
+              umma_pair(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k),
+                        (su > su0 || j > 0 || k > 0) ? 1u : 0u);
+          }
+          commit_pair(&empty[st]);
+        }
+        if (go) commit_pair(&tfull[buf]);
+      }
+    }
+  } else if (warp >= 2) {
+    // ---- epilogue ----
+    const int quarter = warp & 3, half = (warp - 2) >> 2;
+    uint8_t* stg = staging + (warp - 2) * kWarpStage;
+    const uint32_t lanes = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * BNH);
+    int c = 0;
+    bool go = true;
+    for (int t = pid; go && t < tiles; t += pairs) {
+      const Tile ti = tile_at(a, t);
+      float acc[BNH];
+#pragma unroll
+      for (int j = 0; j < BNH; ++j) acc[j] = 0.0f;
+      for (int su0 = 0; su0 < su_total; su0 += kChunkSu, ++c) {
+        const int buf = c & 1;
+        const bool ok = wait_cluster(&tfull[buf], (uint32_t)(c >> 1) & 1u, abort_flag, a.wait_ns);
+        if (!__all_sync(0xffffffffu, ok)) {      // tcgen05.ld below is a .sync.aligned instruction
+          *abort_flag = 1;
+          go = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t src = lanes + (uint32_t)(buf * BN);
+#pragma unroll
+        for (int q = 0; q < BNH / 16; ++q) {
+          float v[16];
+          tmem_ld16(src + (uint32_t)(16 * q), v);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) acc[16 * q + j] += v[j];
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) arrive_cluster(map_dsmem(smem_u32(&tempty[buf]), 0));
+      }
+      if (!go) break;
+      const int row = ti.row0 + (int)rank * BM + quarter * 32;   // first token of this warp
+      const int cols = min(BNH, ti.n_cols - half * BNH);         // valid columns of this half
+      if (cols <= 0) continue;                                   // uniform in the warp
+      const int col0 = ti.m0 + half * BNH;
+      uint32_t need[BNH / 32];
+      if (KEYS && ti.part == 0) {
+        float ss = 0.0f;                       // columns past the matrix are zeros
+#pragma unroll
+        for (int j = 0; j < BNH; ++j) ss = fmaf(acc[j], acc[j], ss);
+        const float scale = sqrtf(ss / (float)cols);
+        int cnt = 0;
+#pragma unroll
+        for (int q = 0; q < BNH / 32; ++q) {
+          uint32_t bits = 0u;
+          if (row + lane < a.rows && 32 * q < cols) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if (near_midpoint(acc[32 * q + j], scale)) bits |= 1u << j;
+          }
+          need[q] = bits;
+          cnt += __popc(bits);
+        }
+        // the warp's listed elements take consecutive slots of the list
+        int incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int u = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += u;
+        }
+        int base = 0;
+        if (lane == 31 && incl > 0) base = atomicAdd(a.fix_count, incl);
+        int slot = __shfl_sync(0xffffffffu, base, 31) + incl - cnt;
+#pragma unroll
+        for (int q = 0; q < BNH / 32; ++q) {
+          uint32_t bits = need[q];
+          while (bits != 0u) {
+            const int j = __ffs(bits) - 1;
+            bits &= bits - 1u;
+            if (slot < a.fix_cap) a.fix_list[slot] = KeyFix{row + lane, col0 + 32 * q + j};
+            ++slot;
+          }
+        }
+      }
+      // 32 rows x 64 columns at a time through the warp's staging (16-byte
+      // chunks swizzled by row: conflict-free both ways), written out 128
+      // bytes of a row per eight lanes
+      __nv_bfloat16* outs[2] = {static_cast<__nv_bfloat16*>(a.out[ti.part]),
+                                HILO ? static_cast<__nv_bfloat16*>(a.out_lo) : nullptr};
+#pragma unroll
+      for (int g = 0; g < BNH / 64; ++g) {
+        if (64 * g >= cols) break;
+#pragma unroll
+        for (int w = 0; w < (HILO ? 2 : 1); ++w) {
+#pragma unroll
+          for (int ch = 0; ch < 8; ++ch) {
+            uint32_t p[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              float& x = acc[64 * g + 8 * ch + 2 * e];
+              float& y = acc[64 * g + 8 * ch + 2 * e + 1];
+              p[e] = pack_bf16(x, y);
+              if (HILO && w == 0) {              // what hi leaves, for the second pass
+                x -= __uint_as_float(p[e] << 16);
+                y -= __uint_as_float(p[e] & 0xFFFF0000u);
+              }
+            }
+            *reinterpret_cast<uint4*>(stg + lane * 128 + ((ch ^ (lane & 7)) << 4)) =
+                make_uint4(p[0], p[1], p[2], p[3]);
+          }
+          __syncwarp();
+#pragma unroll
+          for (int it = 0; it < 8; ++it) {
+            const int r = it * 4 + (lane >> 3), ch = lane & 7;
+            const uint4 u = *reinterpret_cast<const uint4*>(stg + r * 128 + ((ch ^ (r & 7)) << 4));
+            if (row + r < a.rows)
+              *reinterpret_cast<uint4*>(outs[w] + (long long)(row + r) * a.ldc + col0 + 64 * g + 8 * ch) = u;
+          }
+          __syncwarp();
+        }
+      }
+    }
+  }
+  __syncwarp();
+  // ---- both CTAs' roles have ended ----
+  tc_fence_before();
+  cluster_sync();
+  tc_fence_after();
+  const uint32_t mine = smem_u32(const_cast<int*>(abort_flag));
+  const bool aborted = *abort_flag != 0 || ld_dsmem_u32(map_dsmem(mine, rank ^ 1u)) != 0u;
+  if (aborted) {
+    if (threadIdx.x == 0) atomicOr(a.err, kErrTimeout);
+    if (rank == 0 && warp == 1 && lane == 0) commit_pair(drain);   // the issuing thread's MMAs
+    if (lane == 0) {
+      wait_cluster(drain, 0, nullptr, kDefaultWaitLimitNs);
+      const uint64_t t0 = globaltimer_ns();          // copies in flight land
+      while (globaltimer_ns() - t0 < 2000000ull) {}
+    }
+    __syncwarp();
+  }
+  tc_fence_before();
+  cluster_sync();                        // no CTA leaves while the peer may still signal it
+  tc_fence_after();
+  if (warp == 1)
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
+                 "r"(kTmemCols) : "memory");
+}
+
+// Pairs of this kernel resident on the GPU at once (per device).
+template <bool KEYS, bool HILO>
+static cudaError_t launch(PairGemm& a, const CUtensorMap* maps, cudaStream_t s) {
+  auto kern = pair_gemm_kernel<KEYS, HILO>;
+  static int resident[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.stream = s;
+  int n = dev < 64 ? resident[dev] : 0;
+  if (n == 0) {
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute cl[1];
+    cl[0].id = cudaLaunchAttributeClusterDimension;
+    cl[0].val.clusterDim.x = 2;
+    cl[0].val.clusterDim.y = 1;
+    cl[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(2);
+    cfg.attrs = cl;
+    cfg.numAttrs = 1;
+    e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+    if (e != cudaSuccess) return e;
+    if (n <= 0) return cudaErrorInvalidConfiguration;
+    if (dev < 64) resident[dev] = n;
+  }
+  const int tiles = a.feat_tiles * a.row_tiles;
+  // equal rounds: as many pairs as the tiles of a round need
+  const int rounds = (tiles + n - 1) / n;
+  cfg.gridDim = dim3(2 * ((tiles + rounds - 1) / rounds));
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, maps[0], maps[1], maps[2], a);
+}
+
+}  // namespace pair
+
+cudaError_t launch_pair_gemm(PairEpi epi, PairGemm a, const TmaOperand& F0, const TmaOperand& F1,
+                             const TmaOperand& R, cudaStream_t s) {
+  if (a.rows <= 0) return cudaSuccess;
+  a.k_blocks = (int)(R.cols / 64);
+  a.cols[0] = (int)F0.rows;
+  a.cols[1] = F1.base != nullptr ? (int)F1.rows : 0;
+  a.tiles0 = (a.cols[0] + pair::BN - 1) / pair::BN;
+  a.feat_tiles = a.tiles0 + (a.cols[1] + pair::BN - 1) / pair::BN;
+  a.row_tiles = (a.rows + 2 * pair::BM - 1) / (2 * pair::BM);
+  a.wait_ns = wait_limit_ns();
+  CUtensorMap maps[3];
+  const TmaOperand& f1 = F1.base != nullptr ? F1 : F0;
+  if (!encode_kblock_map(&maps[0], F0, pair::BNH, pair::KPS) ||
+      !encode_kblock_map(&maps[1], f1, pair::BNH, pair::KPS) ||
+      !encode_kblock_map(&maps[2], R, pair::BM, pair::KPS))
+    return cudaErrorInvalidValue;
+  switch (epi) {
+    case kPairKeys: return pair::launch<true, false>(a, maps, s);
+    case kPairHiLo: return pair::launch<false, true>(a, maps, s);
+    default: return pair::launch<false, false>(a, maps, s);
+  }
+}
+
+}  // namespace fovea

@@ -1,14 +1,14 @@
-// tcgen05 GEMM C = A . B^T for the bf16 path (sm_103a): the memory
-// projections k = W_K LN(v), u = W_U LN(v), the folded keys W_Q^T k, the
-// query projection W_Q, the scores per sequence, and the two fusion layers.
+// tcgen05 GEMM C = A . B^T of the bf16 draft step (sm_103a): the query
+// projection W_Q, the scores per sequence, the two fusion layers, and the LM
+// head (the memory build's GEMMs are in gemm_build.cu).
 // Neither score form rounds the query map to bf16: the unfolded scores carry
 // q = W_Q x as a bf16 hi/lo pair (q ~= q_hi + q_lo, about 16 significant
 // bits) and each key tile meets both parts; the folded scores carry the
 // folded keys kappa = W_Q^T k as a hi/lo pair and each x tile meets both.
 //
 // Operand roles.  In the GemmArgs vocabulary A holds the output columns
-// (weights, keys: the "feature" operand) and B the output rows (draft states,
-// tokens: the "row" operand).  On the tensor core the row operand is the MMA
+// (weights, keys: the "feature" operand) and B the output rows (draft states:
+// the "row" operand).  On the tensor core the row operand is the MMA
 // A operand (M = 128 rows; a 64-row batch is zero-filled by TMA) and the
 // feature operand is the MMA B operand (N = BN <= 256 features).  A tcgen05
 // MMA costs about the same time for any N up to 256, so a wide feature tile
@@ -95,25 +95,6 @@ struct Cfg {
   static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) |
                                     ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 };
-
-// Key epilogue: a key element is listed for exact recomputation when its
-// fp32 accumulator lies within w * max(|acc|, scale) of a bf16 rounding
-// midpoint, scale being the RMS of the token's values in this tile (the
-// magnitude of the partial sums) and w = 2^-15 * max(1, K / 4096) for a
-// contraction of length K.  The largest distance of a mis-rounded element
-// from its midpoint, measured over 4.1e7 keys at K = 3584 .. 5120, was
-// 2^-16.2 of that magnitude, so the window keeps a margin above 2x and an
-// element outside it rounds as the exact value would.
-__device__ __forceinline__ bool near_midpoint(float acc, __nv_bfloat16 r, float scale, int k_total) {
-  const unsigned short bits = __bfloat16_as_ushort(r);
-  const float rf = __bfloat162float(r);
-  const float up = __bfloat162float(__ushort_as_bfloat16((unsigned short)(bits + 1)));
-  const float dn = __bfloat162float(__ushort_as_bfloat16((unsigned short)(bits - 1)));
-  const float dist = fminf(fabsf(acc - 0.5f * (rf + up)), fabsf(acc - 0.5f * (rf + dn)));
-  const float window =
-      ldexpf(fmaxf(fabsf(acc), scale), -15) * fmaxf(1.0f, (float)k_total * (1.0f / 4096.0f));
-  return !(dist > window);
-}
 
 // kEpiAct: the fp32 term added before the activation (G_h), for the column
 // quads [qlo, qlo + qn) of the tile's rows, staged in shared memory as
@@ -635,99 +616,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const int quarter = warp & 3, half = warp >> 2;
   const int row_in_tile = quarter * 32 + lane;
-  const int n = n0 + row_in_tile;
-  const bool row_ok = n < g.n;
   const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16);
   const int n_cols = min(BN, m_end - m0);
 
-  if constexpr (EPI == kEpiStoreKeys) {
-    // keys and values (never split).  Each thread owns one token's row: warps
-    // 0-3 the first half of the tile's columns, warps 4-7 the second (both
-    // take the row's scale over all columns).  The bf16 values go row-major
-    // into shared memory over the idle stage ring (pitch BN + 8 elements: a
-    // quarter warp's 16-byte stores hit distinct banks), the listed key
-    // elements into the fix list with one atomic per warp, and the CTA then
-    // writes the tile with 16-byte stores along the rows.
-    constexpr int kPitch = BN * 2 + 16;
-    constexpr int kChunks = BN / 64;                 // 32-column chunks per half
-    const int rows_real = min(BM, g.n - n0);
-    if (ok) {
-      float ss = 0.0f;
-#pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 32) {
-        float v[32];
-        tmem_ld32(taddr + (uint32_t)c0, v);
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (c0 + j < n_cols) ss = fmaf(v[j], v[j], ss);
-      }
-      const float key_scale = sqrtf(ss / (float)max(n_cols, 1));
-      uint32_t need[kChunks];
-      int cnt = 0;
-#pragma unroll
-      for (int ci = 0; ci < kChunks; ++ci) {
-        need[ci] = 0u;
-        const int c0 = half * (BN / 2) + ci * 32;
-        if (c0 >= n_cols) continue;                  // uniform across the warp
-        float v[32];
-        tmem_ld32(taddr + (uint32_t)c0, v);
-        uint32_t pk[16];
-#pragma unroll
-        for (int j = 0; j < 32; j += 2) {
-          const __nv_bfloat16 r0 = __float2bfloat16_rn(v[j]), r1 = __float2bfloat16_rn(v[j + 1]);
-          pk[j / 2] = (uint32_t)__bfloat16_as_ushort(r0) | ((uint32_t)__bfloat16_as_ushort(r1) << 16);
-          const int m = m0 + c0 + j;
-          if (row_ok && m < args.epi_split && c0 + j < n_cols &&
-              near_midpoint(v[j], r0, key_scale, args.k_total))
-            need[ci] |= 1u << j;
-          if (row_ok && m + 1 < args.epi_split && c0 + j + 1 < n_cols &&
-              near_midpoint(v[j + 1], r1, key_scale, args.k_total))
-            need[ci] |= 2u << j;
-        }
-        uint4* dst = reinterpret_cast<uint4*>(smem + row_in_tile * kPitch + c0 * 2);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          dst[q] = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
-        cnt += __popc(need[ci]);
-      }
-      // the warp's listed elements take consecutive slots of the fix list
-      int incl = cnt;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-      }
-      const int wtotal = __shfl_sync(0xffffffffu, incl, 31);
-      int base = 0;
-      if (lane == 31 && wtotal > 0) base = atomicAdd(args.fix_count, wtotal);
-      int slot = __shfl_sync(0xffffffffu, base, 31) + incl - cnt;
-      const long long row = (long long)g.b_row0 + n;
-#pragma unroll
-      for (int ci = 0; ci < kChunks; ++ci) {
-        uint32_t bits = need[ci];
-        while (bits != 0u) {
-          const int j = __ffs(bits) - 1;
-          bits &= bits - 1u;
-          if (slot < args.fix_cap)
-            args.fix_list[slot] = KeyFix{(int)row, m0 + half * (BN / 2) + ci * 32 + j};
-          ++slot;
-        }
-      }
-    }
-    __syncthreads();
-    typedef __nv_bfloat16 Tb;
-    constexpr int kRowChunks = BN / 8;                // 16-byte chunks of a row
-    for (int it = threadIdx.x; it < rows_real * kRowChunks; it += kThreads) {
-      const int r = it / kRowChunks, c8 = (it % kRowChunks) * 8;
-      if (c8 >= n_cols) continue;
-      const int m = m0 + c8;                         // epi_split % 8 == 0
-      const long long row = (long long)g.b_row0 + n0 + r;
-      Tb* dst = m < args.epi_split
-                    ? static_cast<Tb*>(args.out0) + row * args.ldc + m
-                    : static_cast<Tb*>(args.out1) + row * args.ldc + (m - args.epi_split);
-      *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(smem + r * kPitch + c8 * 2);
-    }
-  } else {
+  {
     // The accumulator tile goes row-major [rows_real][BN + 4] fp32 into shared
     // memory over the stage ring (idle: every MMA has completed, every copy
     // has landed); the pitch of BN + 4 floats spreads a warp's 16-byte stores
@@ -934,19 +826,6 @@ static EncodeTiledFn encoder() {
   return fn;
 }
 
-// [rows, cols] bf16, row stride ld elements; box = 64 columns x box_rows rows.
-static bool make_map(CUtensorMap* m, const TmaOperand& op, int box_rows) {
-  EncodeTiledFn enc = encoder();
-  if (enc == nullptr || op.base == nullptr || op.rows <= 0 || op.cols <= 0) return false;
-  cuuint64_t dims[2] = {(cuuint64_t)op.cols, (cuuint64_t)op.rows};
-  cuuint64_t strides[1] = {(cuuint64_t)op.ld * 2};
-  cuuint32_t box[2] = {(cuuint32_t)tc::BK, (cuuint32_t)box_rows};
-  cuuint32_t es[2] = {1, 1};
-  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(op.base), dims, strides, box,
-             es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // [rows, cols] bf16 (row stride ld elements, cols a multiple of 64) viewed as
 // (64 k, rows, cols / 64 k-blocks); box = 64 x box_rows x kps: kps
 // consecutive k-blocks of box_rows rows per copy, one 128-byte-swizzled
@@ -998,9 +877,8 @@ static bool cached_map3(CUtensorMap* m, const TmaOperand& op, int box_rows, int 
   return true;
 }
 
-bool encode_bf16_map(CUtensorMap* m, const void* base, long long rows, long long cols,
-                     long long ld, int box_rows) {
-  return make_map(m, TmaOperand{base, rows, cols, ld}, box_rows);
+bool encode_kblock_map(CUtensorMap* m, const TmaOperand& op, int box_rows, int kps) {
+  return cached_map3(m, op, box_rows, kps);
 }
 
 static std::atomic<unsigned long long> g_wait_limit_ns{kDefaultWaitLimitNs};
@@ -1201,7 +1079,7 @@ static void plan_for(const GemmArgs& a, int max_m, int max_n, long long row_tile
         (double)kps * 4.0 * mma_cycles(BN) * ((DUAL || DF) ? 2 : 1) / 2070.0;
     const int sb = C::stage_bytes(kps, rbox, DF);
     for (int S = 1; S <= 8; ++S) {
-      if (S > 1 && (EPI == kEpiStoreKeys || S > su_total)) break;
+      if (S > 1 && S > su_total) break;
       // the weighted-sum GEMM over <= 1024 entries: when its narrowest tiles
       // already fill half the GPU, the split-K reduction and activation
       // epilogue (measured ~4 us per round) outweigh the shorter main loop,
@@ -1211,8 +1089,8 @@ static void plan_for(const GemmArgs& a, int max_m, int max_n, long long row_tile
       const long long ctas = active * S;
       // the accumulator tile [rows][BN + 4] fp32 (and after it, for kEpiAct
       // the added term, for split kEpiLogits the reduced logits, [rows][BN])
-      const int staging = EPI == kEpiStoreKeys ? rows * (BN * 2 + 16)
-                          : rows * (BN + 4 + ((EPI == kEpiAct || (EPI == kEpiLogits && S > 1)) ? BN : 0)) * 4;
+      const int staging =
+          rows * (BN + 4 + ((EPI == kEpiAct || (EPI == kEpiLogits && S > 1)) ? BN : 0)) * 4;
       for (int budget : {tc::kSmemBudget, tc::kSmemBudgetPair}) {
         if (sb > budget) continue;
         const int stages = stages_for(nst, budget, sb);
@@ -1253,11 +1131,9 @@ static GemmPlan plan_epi(const GemmArgs& a, int max_m, int max_n) {
 
 static GemmPlan plan_gemm_tc_uncached(int epi, const GemmArgs& a, int max_m, int max_n) {
   switch (epi) {
-    case kEpiStore: return plan_epi<kEpiStore>(a, max_m, max_n);
     case kEpiScores: return plan_epi<kEpiScores>(a, max_m, max_n);
     case kEpiBiasSilu: return plan_epi<kEpiBiasSilu>(a, max_m, max_n);
     case kEpiStoreHiLo: return plan_epi<kEpiStoreHiLo>(a, max_m, max_n);
-    case kEpiStoreKeys: return plan_epi<kEpiStoreKeys>(a, max_m, max_n);
     case kEpiQueryH: return plan_epi<kEpiQueryH>(a, max_m, max_n);
     case kEpiScoresFolded: return plan_epi<kEpiScoresFolded>(a, max_m, max_n);
     case kEpiAct: return plan_epi<kEpiAct>(a, max_m, max_n);
@@ -1330,11 +1206,9 @@ cudaError_t launch_gemm_tc(int epi, const GemmArgs& args, const TmaOperand& A0, 
     return cudaErrorInvalidValue;
   const int tiles_x = feature_tiles(a, max_m, plan.bn);
   switch (epi) {
-    case kEpiStore: return launch_tc_epi<kEpiStore>(a, maps, plan, tiles_x, max_n, s);
     case kEpiScores: return launch_tc_epi<kEpiScores>(a, maps, plan, tiles_x, max_n, s);
     case kEpiBiasSilu: return launch_tc_epi<kEpiBiasSilu>(a, maps, plan, tiles_x, max_n, s);
     case kEpiStoreHiLo: return launch_tc_epi<kEpiStoreHiLo>(a, maps, plan, tiles_x, max_n, s);
-    case kEpiStoreKeys: return launch_tc_epi<kEpiStoreKeys>(a, maps, plan, tiles_x, max_n, s);
     case kEpiQueryH: return launch_tc_epi<kEpiQueryH>(a, maps, plan, tiles_x, max_n, s);
     case kEpiScoresFolded: return launch_tc_epi<kEpiScoresFolded>(a, maps, plan, tiles_x, max_n, s);
     case kEpiAct: return launch_tc_epi<kEpiAct>(a, maps, plan, tiles_x, max_n, s);

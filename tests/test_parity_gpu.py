@@ -144,6 +144,39 @@ def test_memory_build_matches_oracle(fovea, name):
     mem.destroy()
 
 
+# tiles of 256 tokens x 256 features on CTA pairs, k-blocks of 64 in stages of
+# two and chunks of four: token counts at the edges of a CTA's and a pair's
+# rows and past a band of 8 row tiles; d with partial feature tiles, an odd
+# number of k-blocks, fewer k-blocks than a stage, a chunk, the ring
+@pytest.mark.parametrize("d,m_sizes", [(64, [1]), (192, [128]), (256, [129, 3]), (320, [255]),
+                                       (448, [257]), (576, [385, 0, 130]), (128, [2100])])
+def test_memory_build_tile_edges(fovea, d, m_sizes):
+    """Keys are the correctly rounded W_K LN(v); a value is one bf16 rounding
+    (2^-9 of its magnitude) of a sum whose fp32 error is far below that; the
+    folded pair holds W_Q^T k to 2^-16 plus d fp32 additions."""
+    w = workloads.generate_custom("edges", d, m_sizes, [1] * len(m_sizes), seed=d, H=128)
+    s = store(w)
+    params = params_for(s, fovea)
+    mem = fovea.build_memory(params, s.dev["v"], s.dev.get("mask"))
+    K, U, _, offs = mem.views()
+    kappa = mem.folded_keys(params).double().cpu().numpy()
+    kappa = kappa[:, :d] + kappa[:, d:]
+    p64 = {n: s.f64[n] for n in workloads.PARAM_NAMES}
+    orc = oracle.build_memory(p64, s.f64["v"], s.f64.get("mask"), mirror=True, ln_eps=LN_EPS)
+    exact_u = oracle.fold_keys(p64, orc, mirror=False)
+    for b in range(w.B):
+        lo, hi = offs[b], offs[b + 1]
+        if hi == lo:
+            continue
+        assert np.mean(K[lo:hi].double().cpu().numpy() != orc.keys[b]) <= 1e-5
+        u = U[lo:hi].double().cpu().numpy()
+        assert np.all(np.abs(u - orc.values[b]) <= 2.0 ** -7 * np.abs(orc.values[b]) + 1e-5)
+        bound = 2.0 ** -16 * np.abs(exact_u.folded[b]) + \
+            d * 2.0 ** -24 * (np.abs(orc.keys[b]) @ np.abs(p64["W_Q"]))
+        assert np.all(np.abs(kappa[lo:hi] - exact_u.folded[b]) <= bound)
+    mem.destroy()
+
+
 def test_plain_fusion_when_weights_differ(fovea):
     """The memory keeps the values projected through the r-half of the first
     fusion layer for the W_f1 / W_g1 it was built with.  A bf16 call given
