@@ -337,7 +337,7 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
       if (err != cudaSuccess) return cuda_fail(err, "compact");
       { KernelTimer t("ln_v", s);
         err = launch_ln_rows(p->dtype, v, (const int32_t*)src_row, total, d, p->ln_v_gamma,
-                             p->ln_v_beta, p->ln_eps, nullptr, nullptr, 0, m->err, xv, s); }
+                             p->ln_v_beta, p->ln_eps, xv, s); }
       if (err != cudaSuccess) return cuda_fail(err, "ln_v");
       PairGemm pg{};
       pg.rows = total;

@@ -235,9 +235,9 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t sme
 // Sets the message fovea_last_error() returns on this thread (api.cu).
 fovea_status report_error(fovea_status st, const char* msg);
 
+// LN of the gathered token rows (rowops.cu): out[r] = LN(x[src_row[r]]).
 cudaError_t launch_ln_rows(int dtype, const void* x, const int32_t* src_row, int rows, int d,
-                           const void* gamma, const void* beta, float eps, const void* E,
-                           const int32_t* depth, int max_depth, int* err, void* out,
+                           const void* gamma, const void* beta, float eps, void* out,
                            cudaStream_t s);
 // LN of the draft hidden states plus the depth embedding (rowops.cu), fp32.
 cudaError_t launch_ln_query(int dtype, const void* h, int rows, int d, const void* gamma,

@@ -6,20 +6,17 @@
 namespace fovea {
 
 // ---------------------------------------------------------------------------
-// LN over rows of d elements (memory equation: LN(v_i); query equation:
-// LN(h_n) + E_dep[l_n]).  One CTA per row.  A single pass accumulates sum(x)
-// and sum(x^2) in double-float (the square of a stored value is formed
-// exactly with an FMA), one block reduction gives mean and variance
-// (var = E[x^2] - mean^2, free of cancellation at double-float precision),
-// and the affine map is evaluated in double-float, so the single rounding to
-// the stored type is taken on an almost exact value (the value a float64
-// evaluation rounds).  16-byte vector loads; the row, gamma, beta and the
-// depth embedding are all requested before any arithmetic.  When the depth
-// embedding table fits (<= 64 KB), each thread copies its columns of every
-// row of it into shared memory before griddepcontrol.wait (weights: not
-// written by the previous kernel), so the depth lookup adds no dependent
-// global load.  Optional gather of source rows; an invalid depth sets
-// kErrDepth and uses depth 0.
+// LN over rows of d elements (memory equation: LN(v_i)), an optional gather of
+// source rows.  sum(x) and sum(x^2) are taken in double-float (var = E[x^2] -
+// mean^2, free of cancellation at that precision) and the affine map is
+// evaluated in double-float, so the single rounding to the stored type is
+// taken on an almost exact value (the value a float64 evaluation rounds).
+//
+// fp32 (ln_rows_kernel): one CTA per row, every element in double-float.
+// bf16 (ln_tokens_kernel): the same stored values at the cost of fp32
+// arithmetic.  In bf16, fp32 rounds an element as the exact value would
+// unless it lies within the fp32 error bound of a rounding midpoint (about
+// one element in 2000); only those take the double-float map.
 // ---------------------------------------------------------------------------
 constexpr int kLnThreads = 512;
 
@@ -34,49 +31,31 @@ template <> struct LnVec<float> {
 template <class T>
 __global__ void __launch_bounds__(kLnThreads) ln_rows_kernel(
     const T* __restrict__ x, const int32_t* __restrict__ src_row, int d,
-    const T* __restrict__ gamma, const T* __restrict__ beta, float eps,
-    const T* __restrict__ E, const int32_t* __restrict__ depth, int max_depth, int e_smem,
-    int* err, T* __restrict__ out) {
+    const T* __restrict__ gamma, const T* __restrict__ beta, float eps, T* __restrict__ out) {
   constexpr int V = LnVec<T>::N;
   constexpr int kLnMaxVec = LnVec<T>::MAX;
   __shared__ dfloat red[2][kLnThreads / 32];
-  extern __shared__ __align__(16) uint8_t ln_dyn[];
-  T* e_s = reinterpret_cast<T*>(ln_dyn);            // [max_depth + 1, d] when e_smem
   const int row = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nvec = d / V;
-  float xv[kLnMaxVec][V], gv[kLnMaxVec][V], bv[kLnMaxVec][V], ev[kLnMaxVec][V];
+  float xv[kLnMaxVec][V], gv[kLnMaxVec][V], bv[kLnMaxVec][V];
 #pragma unroll
   for (int j = 0; j < kLnMaxVec; ++j) {      // weights: independent of the predecessor
     const int vi = tid + j * kLnThreads;
     if (vi < nvec) {
       ln_load<T>(gamma + vi * V, gv[j]);
       ln_load<T>(beta + vi * V, bv[j]);
-      if (E != nullptr && e_smem)
-        for (int r = 0; r <= max_depth; ++r)
-          cp_async16(e_s + (long long)r * d + vi * V, E + (long long)r * d + vi * V);
     }
   }
   pdl_wait();
   pdl_trigger();
   const long long src = src_row ? (long long)src_row[row] : (long long)row;
-  int dep = 0;
-  if (E != nullptr) {
-    dep = depth[row];
-    if (dep < 0 || dep > max_depth) {
-      if (tid == 0) atomicOr(err, kErrDepth);
-      dep = 0;
-    }
-  }
   const T* xr = x + src * d;
-  const T* er = E != nullptr ? (e_smem ? e_s : E) + (long long)dep * d : nullptr;
-  if (er != nullptr && e_smem) cp_async_wait_all();   // this thread's own copies
 #pragma unroll
   for (int j = 0; j < kLnMaxVec; ++j) {
     const int vi = tid + j * kLnThreads;
     if (vi < nvec) {
       ln_load<T>(xr + vi * V, xv[j]);
-      if (er != nullptr) ln_load<T>(er + vi * V, ev[j]);
     }
   }
   dfloat s1 = {0.0f, 0.0f}, s2 = {0.0f, 0.0f};
@@ -124,10 +103,161 @@ __global__ void __launch_bounds__(kLnThreads) ln_rows_kernel(
       for (int i = 0; i < V; ++i) {
         dfloat y = df_mul(df_add_f(neg_mean, xv[j][i]), rstd);
         y = df_add_f(df_mul_f(y, gv[j][i]), bv[j][i]);
-        if (er != nullptr) y = df_add_f(y, ev[j][i]);
         res[i] = df_store<T>(y);
       }
       *reinterpret_cast<uint4*>(o + vi * V) = *reinterpret_cast<const uint4*>(res);
+    }
+  }
+}
+
+// Packed pairs of fp32 values (one instruction per pair on sm_100 and later).
+struct f32x2 {
+  unsigned long long v;
+};
+__device__ __forceinline__ f32x2 x2_pack(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 x2_unpack(f32x2 a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+  return r;
+}
+__device__ __forceinline__ f32x2 x2_add(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ f32x2 x2_sub(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ f32x2 x2_mul(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+// The running sum s and the sum c of its rounding errors (Ogita, Rump and
+// Oishi, Sum2), two independent sums at once.
+__device__ __forceinline__ void x2_sum2(f32x2& s, f32x2& c, f32x2 x) {
+  const f32x2 t = x2_add(s, x);
+  const f32x2 bb = x2_sub(t, s);
+  c = x2_add(c, x2_add(x2_sub(s, x2_sub(t, bb)), x2_sub(x, bb)));
+  s = t;
+}
+__device__ __forceinline__ void sum2_join(float& s, float& c, float s2, float c2) {
+  const dfloat t = df_two_sum(s, s2);
+  s = t.hi;
+  c = __fadd_rn(__fadd_rn(c, c2), t.lo);
+}
+
+// One warp per row, the row, gamma and beta in shared memory; CTAs of four
+// warps loop over the rows.  Bound by its instructions and by HBM alike: per
+// element 8 packed operations of the two compensated sums (the squares are
+// exact: a bf16 value has 8 significant bits) and about 15 of the map and its
+// midpoint test.  No CTA barrier and one reduction per row, where a CTA per
+// row took two barriers and double-float arithmetic on every element: 32768
+// rows of 4096 took 932 us, now 219 us (2.4 TB/s).
+constexpr int kLnTokWarps = 4;
+constexpr int kLnTokLoads = 8;          // 16-byte loads in flight per lane
+
+__global__ void __launch_bounds__(32 * kLnTokWarps) ln_tokens_kernel(
+    const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ src_row, int rows, int d,
+    const __nv_bfloat16* __restrict__ gamma, const __nv_bfloat16* __restrict__ beta, float eps,
+    __nv_bfloat16* __restrict__ out) {
+  extern __shared__ __align__(16) uint4 ln_sm[];     // gamma [d], beta [d], a row per warp
+  const int nvec = d / 8, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint4* g_s = ln_sm;
+  uint4* b_s = ln_sm + nvec;
+  uint4* x_s = ln_sm + (2 + warp) * nvec;
+  for (int i = threadIdx.x; i < nvec; i += 32 * kLnTokWarps) {
+    g_s[i] = reinterpret_cast<const uint4*>(gamma)[i];
+    b_s[i] = reinterpret_cast<const uint4*>(beta)[i];
+  }
+  pdl_wait();
+  pdl_trigger();
+  __syncthreads();
+  for (int row = blockIdx.x * kLnTokWarps + warp; row < rows; row += gridDim.x * kLnTokWarps) {
+    const uint4* xr = reinterpret_cast<const uint4*>(x + (long long)src_row[row] * d);
+    f32x2 s1 = x2_pack(0.0f, 0.0f), c1 = s1, s2 = s1, c2 = s1;
+#pragma unroll 1
+    for (int j0 = lane; j0 < nvec; j0 += 32 * kLnTokLoads) {
+      uint4 raw[kLnTokLoads];
+#pragma unroll
+      for (int j = 0; j < kLnTokLoads; ++j) {
+        const int vi = j0 + 32 * j;
+        raw[j] = vi < nvec ? __ldg(xr + vi) : make_uint4(0u, 0u, 0u, 0u);   // zeros add nothing
+      }
+#pragma unroll
+      for (int j = 0; j < kLnTokLoads; ++j) {
+        const int vi = j0 + 32 * j;
+        if (vi < nvec) x_s[vi] = raw[j];
+        const uint32_t w[4] = {raw[j].x, raw[j].y, raw[j].z, raw[j].w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const f32x2 v = x2_pack(__uint_as_float(w[q] << 16), __uint_as_float(w[q] & 0xFFFF0000u));
+          x2_sum2(s1, c1, v);
+          x2_sum2(s2, c2, x2_mul(v, v));
+        }
+      }
+    }
+    float a = x2_unpack(s1).x, ac = x2_unpack(c1).x, b = x2_unpack(s2).x, bc = x2_unpack(c2).x;
+    sum2_join(a, ac, x2_unpack(s1).y, x2_unpack(c1).y);
+    sum2_join(b, bc, x2_unpack(s2).y, x2_unpack(c2).y);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      sum2_join(a, ac, __shfl_xor_sync(0xffffffffu, a, o), __shfl_xor_sync(0xffffffffu, ac, o));
+      sum2_join(b, bc, __shfl_xor_sync(0xffffffffu, b, o), __shfl_xor_sync(0xffffffffu, bc, o));
+    }
+    const dfloat mean = df_div_f(df_two_sum(a, ac), (float)d);
+    const dfloat ex2 = df_div_f(df_two_sum(b, bc), (float)d);
+    const dfloat neg_mean = {-mean.hi, -mean.lo};
+    const dfloat rstd = df_rsqrt(df_add_f(df_add(ex2, df_mul(neg_mean, mean)), eps));
+    // fp32 error of y = (x - mean) rstd gamma + beta: at most three times 2^-24
+    // of the product (x - mean_hi, rstd_hi for rstd, their product), 2^-24 of
+    // the result, and mean_lo <= 2^-24 |mean|: inside the window
+    // 2^-22 (|product| + |y|) + 2^-23 |mean| rstd |gamma|
+    const float mr = fabsf(mean.hi) * rstd.hi * 1.1920929e-7f;
+    __nv_bfloat16* o = out + (long long)row * d;
+#pragma unroll 1                                       // a lane reads the vectors it stored above
+    for (int vi = lane; vi < nvec; vi += 32) {
+      const uint4 xv = x_s[vi], gr = g_s[vi], br = b_s[vi];
+      const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w};
+      const uint32_t gw[4] = {gr.x, gr.y, gr.z, gr.w}, bw[4] = {br.x, br.y, br.z, br.w};
+      uint32_t ow[4], slow = 0u;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float y[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float xf = __uint_as_float(h ? xw[q] & 0xFFFF0000u : xw[q] << 16);
+          const float gf = __uint_as_float(h ? gw[q] & 0xFFFF0000u : gw[q] << 16);
+          const float bf = __uint_as_float(h ? bw[q] & 0xFFFF0000u : bw[q] << 16);
+          const float u = (xf - mean.hi) * rstd.hi;
+          y[h] = fmaf(u, gf, bf);
+          const float window =
+              fmaf(fmaf(fabsf(u), fabsf(gf), fabsf(y[h])), 2.3841858e-7f, mr * fabsf(gf));
+          // midpoint of the two bf16 values around y; a window that reaches
+          // their spacing, or a value that is not finite, is recomputed too
+          const float mid = __uint_as_float((__float_as_uint(y[h]) & 0xFFFF0000u) | 0x8000u);
+          if (!(fabsf(y[h] - mid) > window && fabsf(y[h]) * 0.001953125f > window))
+            slow |= 1u << (2 * q + h);
+        }
+        const __nv_bfloat162 p = __floats2bfloat162_rn(y[0], y[1]);
+        ow[q] = *reinterpret_cast<const uint32_t*>(&p);
+      }
+      reinterpret_cast<uint4*>(o)[vi] = make_uint4(ow[0], ow[1], ow[2], ow[3]);
+      while (slow != 0u) {                             // the exact value, after the vector store
+        const int e = 8 * vi + __ffs(slow) - 1;
+        slow &= slow - 1u;
+        const float xf = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(x_s)[e]);
+        const float gf = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(g_s)[e]);
+        const float bf = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(b_s)[e]);
+        const dfloat t = df_mul(df_add_f(neg_mean, xf), rstd);
+        o[e] = df_to_bf16(df_add_f(df_mul_f(t, gf), bf));
+      }
     }
   }
 }
@@ -139,8 +269,12 @@ __global__ void __launch_bounds__(kLnThreads) ln_rows_kernel(
 // stored type.  Against the float64 evaluation the stored value differs by
 // one unit in the last place only where the exact value lies within fp32
 // rounding of a midpoint of the stored type (for bf16 about one element in
-// 10^4; the query it feeds moves by ~1e-6 of its scale).  Same loads, depth
-// check and shared-memory depth table as ln_rows_kernel; one CTA per row.
+// 10^4; the query it feeds moves by ~1e-6 of its scale).  One CTA per row;
+// 16-byte loads, all requested before any arithmetic.  When the depth
+// embedding table fits (<= 64 KB) and the rows are few, each thread copies its
+// columns of every row of it into shared memory before griddepcontrol.wait
+// (weights: not written by the previous kernel), so the depth lookup adds no
+// dependent global load.  An invalid depth sets kErrDepth and uses depth 0.
 template <class T>
 __global__ void __launch_bounds__(kLnThreads, 2) ln_query_kernel(
     const T* __restrict__ x, int d, const T* __restrict__ gamma, const T* __restrict__ beta,
@@ -287,38 +421,28 @@ cudaError_t launch_ln_query(int dtype, const void* h, int rows, int d, const voi
 }
 
 cudaError_t launch_ln_rows(int dtype, const void* x, const int32_t* src_row, int rows, int d,
-                           const void* gamma, const void* beta, float eps, const void* E,
-                           const int32_t* depth, int max_depth, int* err, void* out,
+                           const void* gamma, const void* beta, float eps, void* out,
                            cudaStream_t s) {
   if (rows == 0) return cudaSuccess;
-  constexpr int kESmemMax = 64 * 1024;
-  const size_t es = dtype == FOVEA_BF16 ? 2 : 4;
-  const size_t e_bytes = E != nullptr ? (size_t)(max_depth + 1) * d * es : 0;
-  const int e_smem = E != nullptr && e_bytes <= (size_t)kESmemMax ? 1 : 0;
-  const size_t smem = e_smem ? e_bytes : 0;
-  if (dtype == FOVEA_BF16) {
-    using T = __nv_bfloat16;
-    static bool configured = false;
-    if (!configured) {
-      cudaError_t e = cudaFuncSetAttribute(ln_rows_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           kESmemMax);
-      if (e != cudaSuccess) return e;
-      configured = true;
-    }
-    return launch_pdl(ln_rows_kernel<T>, dim3(rows), dim3(kLnThreads), smem, s, (const T*)x,
-                      src_row, d, (const T*)gamma, (const T*)beta, eps, (const T*)E, depth,
-                      max_depth, e_smem, err, (T*)out);
-  }
-  static bool configured_f = false;
-  if (!configured_f) {
-    cudaError_t e = cudaFuncSetAttribute(ln_rows_kernel<float>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kESmemMax);
-    if (e != cudaSuccess) return e;
-    configured_f = true;
-  }
-  return launch_pdl(ln_rows_kernel<float>, dim3(rows), dim3(kLnThreads), smem, s, (const float*)x,
-                    src_row, d, (const float*)gamma, (const float*)beta, eps, (const float*)E,
-                    depth, max_depth, e_smem, err, (float*)out);
+  if (dtype != FOVEA_BF16)
+    return launch_pdl(ln_rows_kernel<float>, dim3(rows), dim3(kLnThreads), 0, s, (const float*)x,
+                      src_row, d, (const float*)gamma, (const float*)beta, eps, (float*)out);
+  int dev = 0, sms = 0, per_sm = 0;
+  const size_t smem = (size_t)d * 2 * (2 + kLnTokWarps);       // at most 96 KB
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(ln_tokens_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             FOVEA_MAX_D * 2 * (2 + kLnTokWarps));
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ln_tokens_kernel, 32 * kLnTokWarps,
+                                                      smem);
+  if (e != cudaSuccess) return e;
+  const int ctas = (rows + kLnTokWarps - 1) / kLnTokWarps;
+  const int most = sms * (per_sm > 0 ? per_sm : 1);
+  return launch_pdl(ln_tokens_kernel, dim3(ctas < most ? ctas : most), dim3(32 * kLnTokWarps),
+                    smem, s, (const __nv_bfloat16*)x, src_row, rows, d, (const __nv_bfloat16*)gamma,
+                    (const __nv_bfloat16*)beta, eps, (__nv_bfloat16*)out);
 }
 
 // ---------------------------------------------------------------------------

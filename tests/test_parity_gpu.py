@@ -177,6 +177,32 @@ def test_memory_build_tile_edges(fovea, d, m_sizes):
     mem.destroy()
 
 
+# row lengths below, at and past a warp's pass of 256 elements and its batch of
+# eight vectors per lane; means up to 1000 standard deviations away, where the
+# fp32 map is seldom sure of its rounding
+@pytest.mark.parametrize("d,mean,std", [(64, 0.0, 1.0), (320, 5.0, 1.0), (2048, 0.0, 1.0),
+                                        (2112, 5.0, 1.0), (2112, 64.0, 0.0625), (8192, 0.0, 1.0)])
+def test_token_layer_norm_is_correctly_rounded(fovea, d, mean, std):
+    """With W_K = I a key is LN(v) itself: the bf16 rounding of the float64
+    value.  The variance E[x^2] - mean^2 keeps 2^-46 of E[x^2] in
+    double-float, so the product (x - mean) rstd gamma errs by at most 2^-44
+    (1 + E[x^2] / (var + eps)) of itself: the key lies between the roundings of
+    the exact value less and plus that bound."""
+    w = workloads.generate_custom("ln", d, [37, 4], [1, 1], seed=d, H=128)
+    w.params["W_K"] = np.eye(d, dtype=np.float32)
+    w.v = (mean + std * w.v).astype(np.float32)
+    s = store(w)
+    mem = fovea.build_memory(params_for(s, fovea), s.dev["v"], s.dev.get("mask"))
+    K = mem.views()[0].double().cpu().numpy()
+    p64 = {n: s.f64[n] for n in workloads.PARAM_NAMES}
+    x = np.concatenate([s.f64["v"][b, :m] for b, m in enumerate(w.m_sizes)])
+    y = oracle.layer_norm(x, p64["ln_v_gamma"], p64["ln_v_beta"], LN_EPS)
+    bound = 2.0 ** -44 * np.abs(y - p64["ln_v_beta"]) * \
+        (1 + (x ** 2).mean(1, keepdims=True) / (x.var(axis=1, keepdims=True) + LN_EPS))
+    assert np.all((K >= oracle.round_bf16(y - bound)) & (K <= oracle.round_bf16(y + bound)))
+    mem.destroy()
+
+
 def test_plain_fusion_when_weights_differ(fovea):
     """The memory keeps the values projected through the r-half of the first
     fusion layer for the W_f1 / W_g1 it was built with.  A bf16 call given
