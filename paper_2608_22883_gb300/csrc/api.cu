@@ -398,7 +398,11 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
         if ((fs = alloc_dev(&wqt, (size_t)d * d * 2, "transposed W_Q")) != FOVEA_OK) return fs;
         auto fold = [&]() -> fovea_status {
           { KernelTimer t("transpose_wq", s);
-            err = launch_transpose_bf16(p->W_Q, d, d, wqt, s); }
+            static thread_local ImageTable one;
+            one.B = 1;
+            one.off[0] = 0;
+            one.m[0] = d;
+            err = launch_transpose_images(p->W_Q, d, d, one, wqt, s); }
           if (err != cudaSuccess) return cuda_fail(err, "transpose W_Q");
           pg.out[0] = m->folded;
           pg.out_lo = static_cast<__nv_bfloat16*>(m->folded) + d;

@@ -273,10 +273,6 @@ cudaError_t launch_select_gather(int dtype, const float* scores, const SeqTable&
                                  float* r_out, void* r_lo, const void* P, int H, const float* Gh,
                                  const void* b_f1, const void* b_g1, void* act, int* err,
                                  cudaStream_t s, long long p_prefetch_bytes = 0);
-// out[c * rows + r] = in[r * cols + c] for a bf16 [rows, cols] matrix, rows
-// and cols multiples of 32 (the query folding's W_Q^T, once per memory build).
-cudaError_t launch_transpose_bf16(const void* in, int rows, int cols, void* out, cudaStream_t s);
-
 // Images of a memory: first entry and valid count of each (kernel parameter).
 struct ImageTable {
   int B;
@@ -284,7 +280,7 @@ struct ImageTable {
   int m[FOVEA_MAX_SEQ];
 };
 // out [B, C, ld]: image b's [m_b, C] rows of `in` (from row off_b) transposed,
-// zero-padded to ld entries (C and ld multiples of 32).
+// zero-padded to ld entries (C and ld multiples of 64).
 cudaError_t launch_transpose_images(const void* in, int C, int ld, const ImageTable& tab,
                                     void* out, cudaStream_t s);
 
