@@ -118,8 +118,6 @@ struct fovea_memory {
   void* keys = nullptr;              // [total, d]
   void* values = nullptr;            // [total, d]
   int32_t* orig_index = nullptr;     // [total]
-  int* err = nullptr;                // device error word
-  int refined = 0;                   // key elements re-rounded exactly at build
   // bf16: the values projected through the r-half of the first fusion layer,
   // p_i = [W_f1 ; W_g1][:, d:2d] u_i  ([total, 2H]), and the weights they
   // were built with (a call with other W_f1 / W_g1 pointers or H does not
@@ -190,32 +188,101 @@ static fovea_status check_step_params(const fovea_params* p) {
   return FOVEA_OK;
 }
 
-static fovea_status alloc_dev(void** ptr, size_t bytes, const char* what) {
+// ---------------------------------------------------------------------------
+// Device memory of the handles and of a build's temporaries: one stream-ordered
+// pool per device.  cudaMalloc and cudaFree cost 30 - 180 us each, ten to
+// twelve of them 0.8 ms of a one-image build whose kernels take 0.3 ms; an
+// allocation from the pool costs about 1 us (mapping it anew, 0.3 ms for a
+// one-image build's buffers).  After every build and every freed handle the
+// pool keeps at most kPoolKeep bytes that nothing uses (under 1 % of the
+// device), and it gives everything back when the device's last handle goes.
+// (Its own release threshold counts the bytes in use too, so it is off.)  The
+// driver orders the pool's reuse between streams and threads.
+// ---------------------------------------------------------------------------
+namespace {
+constexpr unsigned long long kPoolKeep = 2ull << 30;
+constexpr int kMaxDevices = 64;
+struct DevicePool {
+  cudaMemPool_t pool = nullptr;
+  int users = 0;                     // live handles and builds under way
+};
+std::mutex g_pool_mu;
+DevicePool g_pools[kMaxDevices];
+
+// The pool of device `dev`, created at its first use; one more user of it.
+cudaError_t pool_enter(int dev, cudaMemPool_t* out) {
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  DevicePool& p = g_pools[dev];
+  if (p.pool == nullptr) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    cudaError_t e = cudaMemPoolCreate(&pool, &props);
+    if (e != cudaSuccess) return e;
+    unsigned long long never = ~0ull;
+    e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &never);
+    if (e != cudaSuccess) {
+      cudaMemPoolDestroy(pool);
+      return e;
+    }
+    p.pool = pool;
+  }
+  ++p.users;
+  *out = p.pool;
+  return cudaSuccess;
+}
+// Gives back what the pool holds beyond kPoolKeep unused bytes.
+void pool_trim(cudaMemPool_t pool) {
+  unsigned long long used = 0, held = 0;
+  if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess &&
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+      held > used + kPoolKeep)
+    cudaMemPoolTrimTo(pool, used + kPoolKeep);
+}
+// One user less; the last one returns all unused memory.
+void pool_leave(int dev) {
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  DevicePool& p = g_pools[dev];
+  if (--p.users == 0) cudaMemPoolTrimTo(p.pool, 0);
+  else pool_trim(p.pool);
+}
+}  // namespace
+
+static fovea_status alloc_dev(void** ptr, size_t bytes, const char* what, cudaMemPool_t pool,
+                              cudaStream_t s) {
   *ptr = nullptr;
   if (bytes == 0) return FOVEA_OK;
   const char* fault = getenv("FOVEA_FAULT_ALLOC");
   if (fault != nullptr && fault[0] == '1')
     return fail(FOVEA_ERR_OOM, "allocation of %s (%zu bytes) failed (FOVEA_FAULT_ALLOC=1)", what,
                 bytes);
-  cudaError_t e = cudaMalloc(ptr, bytes);
+  cudaError_t e = cudaMallocFromPoolAsync(ptr, bytes, pool, s);
   if (e != cudaSuccess) {
     cudaGetLastError();
     *ptr = nullptr;
-    return fail(FOVEA_ERR_OOM, "cudaMalloc of %s (%zu bytes): %s", what, bytes,
+    return fail(FOVEA_ERR_OOM, "allocation of %s (%zu bytes): %s", what, bytes,
                 cudaGetErrorString(e));
   }
   return FOVEA_OK;
 }
 
+// Frees a handle.  Like cudaFree, it waits for the device first, so work still
+// enqueued when the caller lets go of the handle finishes on its memory.
 static void free_memory(fovea_memory* m) {
   if (m == nullptr) return;
-  cudaFree(m->keys);
-  cudaFree(m->values);
-  cudaFree(m->proj);
-  cudaFree(m->projT);
-  cudaFree(m->folded);
-  cudaFree(m->orig_index);
-  cudaFree(m->err);
+  int cur = -1;
+  cudaGetDevice(&cur);
+  if (cur != m->device) cudaSetDevice(m->device);
+  cudaDeviceSynchronize();
+  for (void* p : {m->keys, m->values, m->proj, m->projT, m->folded,
+                  static_cast<void*>(m->orig_index)})
+    if (p != nullptr) cudaFreeAsync(p, nullptr);
+  cudaStreamSynchronize(nullptr);
+  pool_leave(m->device);
+  if (cur >= 0 && cur != m->device) cudaSetDevice(cur);
   delete m;
 }
 
@@ -265,173 +332,149 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
   const int d = p->d_model;
   const size_t es = esize(p->dtype);
 
+  if (capturing(s))
+    return fail(FOVEA_ERR_CUDA, "fovea_build_memory synchronises: the stream is being captured");
+  const char* fault = getenv("FOVEA_FAULT_ALLOC");
+  if (fault != nullptr && fault[0] == '1')
+    return fail(FOVEA_ERR_OOM, "allocation of build scratch failed (FOVEA_FAULT_ALLOC=1)");
+  int dev = 0;
+  cudaMemPool_t pool = nullptr;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = pool_enter(dev, &pool);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return fail(FOVEA_ERR_OOM, "device memory pool: %s", cudaGetErrorString(e));
+  }
+
   fovea_memory* m = new fovea_memory();
+  m->device = dev;
   m->B = B;
   m->M_max = M_max;
   m->d = d;
   m->dtype = p->dtype;
-  cudaGetDevice(&m->device);
-  st = alloc_dev(reinterpret_cast<void**>(&m->err), 256, "error word");
-  if (st != FOVEA_OK) { free_memory(m); return st; }
-  void* scratch = nullptr;           // counts [B] | key_off [B] (int32)
-  st = alloc_dev(&scratch, align_up(2 * B * sizeof(int32_t), 256), "build scratch");
-  if (st != FOVEA_OK) { free_memory(m); return st; }
-  int32_t* d_counts = static_cast<int32_t*>(scratch);
-  int32_t* d_keyoff = d_counts + B;
-
-  auto cleanup = [&](fovea_status code) {
-    cudaStreamSynchronize(s);
-    cudaFree(scratch);
-    free_memory(m);
-    return code;
-  };
-  cudaError_t e = cudaMemsetAsync(m->err, 0, 256, s);
-  if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaMemsetAsync"));
-
-  m->counts.assign(B, M_max);
-  if (mask != nullptr && M_max > 0) {
-    { KernelTimer t("count_valid", s); e = launch_count_valid(mask, B, M_max, d_counts, s); }
-    if (e != cudaSuccess) return cleanup(cuda_fail(e, "count_valid"));
-    e = cudaMemcpyAsync(m->counts.data(), d_counts, B * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cleanup(cuda_fail(e, "reading valid counts"));
-  }
-  m->offsets.assign(B + 1, 0);
-  for (int b = 0; b < B; ++b) {
-    if (m->counts[b] > FOVEA_MAX_ENTRIES)
-      return cleanup(fail(FOVEA_ERR_UNSUPPORTED, "image %d has %d valid entries (limit %d)", b,
-                          m->counts[b], FOVEA_MAX_ENTRIES));
-    m->offsets[b + 1] = m->offsets[b] + m->counts[b];
-  }
-  m->total = (int)m->offsets[B];
-  const int total = m->total;
-  if (total > 0) {
-    std::vector<int32_t> keyoff(B);
-    for (int b = 0; b < B; ++b) keyoff[b] = (int32_t)m->offsets[b];
-    void* xv = nullptr;
-    void* src_row = nullptr;
-    void* fix = nullptr;                     // bf16: count word + listed key elements
+  // temporaries: error word and list count, valid counts | source rows | LN(v) |
+  // listed key elements | W_Q^T
+  void* scratch = nullptr;
+  void* src_row = nullptr;
+  void* xv = nullptr;
+  void* fix = nullptr;
+  void* wqt = nullptr;
+  auto run = [&]() -> fovea_status {
+    fovea_status rs = alloc_dev(&scratch, 256 + align_up(B * sizeof(int32_t), 256), "build scratch", pool, s);
+    if (rs != FOVEA_OK) return rs;
+    int* errw = static_cast<int*>(scratch);           // error word, then the list's count
+    int32_t* d_counts = reinterpret_cast<int32_t*>(static_cast<uint8_t*>(scratch) + 256);
+    FOVEA_CUDA(cudaMemsetAsync(scratch, 0, 256, s), "cudaMemsetAsync");
+    m->counts.assign(B, M_max);
+    cudaError_t err = cudaSuccess;
+    if (mask != nullptr && M_max > 0) {
+      { KernelTimer t("count_valid", s); err = launch_count_valid(mask, B, M_max, d_counts, s); }
+      if (err != cudaSuccess) return cuda_fail(err, "count_valid");
+      err = cudaMemcpyAsync(m->counts.data(), d_counts, B * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+      if (err == cudaSuccess) err = cudaStreamSynchronize(s);
+      if (err != cudaSuccess) return cuda_fail(err, "reading valid counts");
+    }
+    m->offsets.assign(B + 1, 0);
+    int m_max = 0;
+    static thread_local ImageTable itab;
+    itab.B = B;
+    for (int b = 0; b < B; ++b) {
+      if (m->counts[b] > FOVEA_MAX_ENTRIES)
+        return fail(FOVEA_ERR_UNSUPPORTED, "image %d has %d valid entries (limit %d)", b,
+                    m->counts[b], FOVEA_MAX_ENTRIES);
+      itab.off[b] = (int)m->offsets[b];
+      itab.m[b] = m->counts[b];
+      m_max = std::max(m_max, m->counts[b]);
+      m->offsets[b + 1] = m->offsets[b] + m->counts[b];
+    }
+    m->total = (int)m->offsets[B];
+    const int total = m->total;
+    if (total == 0) return FOVEA_OK;
     const bool bf = p->dtype == FOVEA_BF16;
+    const int H = p->mlp_hidden;
+    // bf16 with W_Q given: the folded keys; with the fusion weights given: the
+    // projected values and their transpose per image
+    const bool fold = bf && p->W_Q != nullptr && aligned16(p->W_Q);
+    const bool proj = bf && p->W_f1 != nullptr && p->W_g1 != nullptr && H > 0 && H % 128 == 0 &&
+                      H <= FOVEA_MAX_H && aligned16(p->W_f1) && aligned16(p->W_g1);
+    const int ld = (m_max + 63) / 64 * 64;
     // the list holds 0.47 % of the keys of well-scaled tokens (gemm_build.cu)
     const long long fix_cap = bf ? (long long)total * d / 32 + 4096 : 0;
-    if ((st = alloc_dev(&m->keys, (size_t)total * d * es, "keys")) != FOVEA_OK ||
-        (st = alloc_dev(&m->values, (size_t)total * d * es, "values")) != FOVEA_OK ||
-        (st = alloc_dev(reinterpret_cast<void**>(&m->orig_index), total * sizeof(int32_t),
-                        "index")) != FOVEA_OK ||
-        (st = alloc_dev(&src_row, total * sizeof(int32_t), "source rows")) != FOVEA_OK ||
-        (st = alloc_dev(&xv, (size_t)total * d * es, "LN(v)")) != FOVEA_OK ||
-        (bf && (st = alloc_dev(&fix, 256 + (size_t)fix_cap * sizeof(KeyFix), "key fix list")) != FOVEA_OK)) {
-      cudaFree(xv);
-      cudaFree(src_row);
-      cudaFree(fix);
-      return cleanup(st);
-    }
-    int* fix_count = static_cast<int*>(fix);
-    KeyFix* fix_list = bf ? reinterpret_cast<KeyFix*>(static_cast<uint8_t*>(fix) + 256) : nullptr;
-    auto run = [&]() -> fovea_status {
-      cudaError_t err = cudaMemcpyAsync(d_keyoff, keyoff.data(), B * sizeof(int32_t),
-                                        cudaMemcpyHostToDevice, s);
-      if (err != cudaSuccess) return cuda_fail(err, "cudaMemcpyAsync");
-      { KernelTimer t("compact", s);
-        err = launch_compact(mask, B, M_max, d_keyoff, m->orig_index, (int32_t*)src_row, s); }
-      if (err != cudaSuccess) return cuda_fail(err, "compact");
-      { KernelTimer t("ln_v", s);
-        err = launch_ln_rows(p->dtype, v, (const int32_t*)src_row, total, d, p->ln_v_gamma,
-                             p->ln_v_beta, p->ln_eps, xv, s); }
-      if (err != cudaSuccess) return cuda_fail(err, "ln_v");
+    if ((rs = alloc_dev(&m->keys, (size_t)total * d * es, "keys", pool, s)) != FOVEA_OK ||
+        (rs = alloc_dev(&m->values, (size_t)total * d * es, "values", pool, s)) != FOVEA_OK ||
+        (rs = alloc_dev(reinterpret_cast<void**>(&m->orig_index), total * sizeof(int32_t), "index",
+                        pool, s)) != FOVEA_OK ||
+        (rs = alloc_dev(&src_row, total * sizeof(int32_t), "source rows", pool, s)) != FOVEA_OK ||
+        (rs = alloc_dev(&xv, (size_t)total * d * es, "LN(v)", pool, s)) != FOVEA_OK ||
+        (bf && (rs = alloc_dev(&fix, (size_t)fix_cap * sizeof(KeyFix), "key fix list", pool, s)) != FOVEA_OK) ||
+        (fold && (rs = alloc_dev(&m->folded, (size_t)total * 2 * d * 2, "folded keys", pool, s)) != FOVEA_OK) ||
+        (fold && (rs = alloc_dev(&wqt, (size_t)d * d * 2, "transposed W_Q", pool, s)) != FOVEA_OK) ||
+        (proj && (rs = alloc_dev(&m->proj, (size_t)total * 2 * H * 2, "projected values", pool, s)) != FOVEA_OK) ||
+        (proj && (rs = alloc_dev(&m->projT, (size_t)B * 2 * H * ld * 2, "transposed projected values",
+                                 pool, s)) != FOVEA_OK))
+      return rs;
+    { KernelTimer t("compact", s);
+      err = launch_compact(mask, B, M_max, itab, m->orig_index, (int32_t*)src_row, s); }
+    if (err != cudaSuccess) return cuda_fail(err, "compact");
+    { KernelTimer t("ln_v", s);
+      err = launch_ln_rows(p->dtype, v, (const int32_t*)src_row, total, d, p->ln_v_gamma,
+                           p->ln_v_beta, p->ln_eps, xv, s); }
+    if (err != cudaSuccess) return cuda_fail(err, "ln_v");
+    if (!bf) {
+      static thread_local GemmArgs a;
+      init_args(a);
+      a.k_total = d;
+      a.a_split = d;
+      a.b_split = d;
+      a.A0 = p->W_K; a.A1 = p->W_U; a.lda0 = d; a.lda1 = d;
+      a.B0 = xv; a.B1 = xv; a.ldb0 = d; a.ldb1 = d;
+      a.epi_split = d;
+      a.out0 = m->keys; a.out1 = m->values; a.ldc = d;
+      a.ngroups = 1;
+      a.groups[0] = GemmGroup{0, 2 * d, 0, total, 0};
+      { KernelTimer t("memory_proj", s);
+        err = launch_gemm_simt(p->dtype, kEpiStore, a, 2 * d, total, s); }
+      if (err != cudaSuccess) return cuda_fail(err, "memory projection");
+    } else {
       PairGemm pg{};
       pg.rows = total;
       pg.ldc = d;
-      pg.err = m->err;
-      if (bf) {
-        pg.out[0] = m->keys; pg.out[1] = m->values;
-        pg.fix_list = fix_list; pg.fix_count = fix_count; pg.fix_cap = (int)fix_cap;
-        err = cudaMemsetAsync(fix_count, 0, sizeof(int), s);
-        if (err != cudaSuccess) return cuda_fail(err, "cudaMemsetAsync");
-        KernelTimer t("memory_proj", s);
+      pg.err = errw;
+      pg.out[0] = m->keys; pg.out[1] = m->values;
+      pg.fix_list = static_cast<KeyFix*>(fix); pg.fix_count = errw + 1; pg.fix_cap = (int)fix_cap;
+      const TmaOperand none{nullptr, 0, 0, 0};
+      { KernelTimer t("memory_proj", s);
         err = launch_pair_gemm(kPairKeys, pg, TmaOperand{p->W_K, d, d, d},
-                               TmaOperand{p->W_U, d, d, d}, TmaOperand{xv, total, d, d}, s);
-      } else {
-        GemmArgs a;
-        init_args(a);
-        a.k_total = d;
-        a.a_split = d;
-        a.b_split = d;
-        a.A0 = p->W_K; a.A1 = p->W_U; a.lda0 = d; a.lda1 = d;
-        a.B0 = xv; a.B1 = xv; a.ldb0 = d; a.ldb1 = d;
-        a.epi_split = d;
-        a.out0 = m->keys; a.out1 = m->values; a.ldc = d;
-        a.ngroups = 1;
-        a.groups[0] = GemmGroup{0, 2 * d, 0, total, 0};
-        KernelTimer t("memory_proj", s);
-        err = launch_gemm_simt(p->dtype, kEpiStore, a, 2 * d, total, s);
-      }
+                               TmaOperand{p->W_U, d, d, d}, TmaOperand{xv, total, d, d}, s); }
       if (err != cudaSuccess) return cuda_fail(err, "memory projection");
-      if (bf) {
-        // keys whose fp32 value sat near a bf16 rounding midpoint: exact recompute
-        { KernelTimer t("refine_keys", s);
-          err = launch_refine_keys(xv, p->W_K, d, fix_list, fix_count, (int)fix_cap, total, m->keys, s); }
-        if (err != cudaSuccess) return cuda_fail(err, "refine_keys");
-      }
-      int herr[2] = {0, 0};
-      err = cudaMemcpyAsync(&herr[0], m->err, sizeof(int), cudaMemcpyDeviceToHost, s);
-      if (err == cudaSuccess && bf)
-        err = cudaMemcpyAsync(&herr[1], fix_count, sizeof(int), cudaMemcpyDeviceToHost, s);
-      if (err == cudaSuccess) err = cudaStreamSynchronize(s);
-      if (err != cudaSuccess) return cuda_fail(err, "memory build");
-      if (herr[0] & kErrTimeout)
-        return fail(FOVEA_ERR_TIMEOUT, "a bounded device wait gave up during the memory build");
-      m->refined = herr[1];
-      if (bf && herr[1] > fix_cap) {      // list overflowed: refine every key element
-        { KernelTimer t("refine_keys", s);
-          err = launch_refine_keys(xv, p->W_K, d, nullptr, nullptr, 0, total, m->keys, s); }
-        if (err == cudaSuccess) err = cudaStreamSynchronize(s);
-        if (err != cudaSuccess) return cuda_fail(err, "refine_keys");
-      }
-      // bf16 with W_Q given: the folded keys kappa_i = W_Q^T k_i, a GEMM of
-      // W_Q^T (transposed once here) with the stored keys, kept as the hi / lo
-      // pair of its fp32 accumulator (no bf16 rounding of the query map)
-      if (bf && p->W_Q != nullptr && aligned16(p->W_Q)) {
-        fovea_status fs = alloc_dev(&m->folded, (size_t)total * 2 * d * 2, "folded keys");
-        if (fs != FOVEA_OK) return fs;
-        void* wqt = nullptr;
-        if ((fs = alloc_dev(&wqt, (size_t)d * d * 2, "transposed W_Q")) != FOVEA_OK) return fs;
-        auto fold = [&]() -> fovea_status {
-          { KernelTimer t("transpose_wq", s);
-            static thread_local ImageTable one;
-            one.B = 1;
-            one.off[0] = 0;
-            one.m[0] = d;
-            err = launch_transpose_images(p->W_Q, d, d, one, wqt, s); }
-          if (err != cudaSuccess) return cuda_fail(err, "transpose W_Q");
-          pg.out[0] = m->folded;
-          pg.out_lo = static_cast<__nv_bfloat16*>(m->folded) + d;
-          pg.ldc = 2 * d;
-          { KernelTimer t("memory_fold", s);
-            err = launch_pair_gemm(kPairHiLo, pg, TmaOperand{wqt, d, d, d},
-                                   TmaOperand{nullptr, 0, 0, 0}, TmaOperand{m->keys, total, d, d}, s); }
-          if (err != cudaSuccess) return cuda_fail(err, "query folding of the keys");
-          int fe = 0;
-          err = cudaMemcpyAsync(&fe, m->err, sizeof(int), cudaMemcpyDeviceToHost, s);
-          if (err == cudaSuccess) err = cudaStreamSynchronize(s);
-          if (err != cudaSuccess) return cuda_fail(err, "query folding");
-          if (fe & kErrTimeout)
-            return fail(FOVEA_ERR_TIMEOUT, "a bounded device wait gave up while folding the keys");
-          return FOVEA_OK;
-        };
-        fs = fold();
-        cudaStreamSynchronize(s);
-        cudaFree(wqt);
-        if (fs != FOVEA_OK) return fs;
+      // keys whose fp32 value sat near a bf16 rounding midpoint: exact recompute
+      { KernelTimer t("refine_keys", s);
+        err = launch_refine_keys(xv, p->W_K, d, pg.fix_list, pg.fix_count, (int)fix_cap, total,
+                                 m->keys, s); }
+      if (err != cudaSuccess) return cuda_fail(err, "refine_keys");
+      if (fold) {
+        // kappa_i = W_Q^T k_i, a GEMM of W_Q^T (transposed once here) with the
+        // stored keys, kept as the hi / lo pair of its fp32 accumulator (no
+        // bf16 rounding of the query map)
+        static thread_local ImageTable one;
+        one.B = 1;
+        one.off[0] = 0;
+        one.m[0] = d;
+        { KernelTimer t("transpose_wq", s);
+          err = launch_transpose_images(p->W_Q, d, d, one, wqt, s); }
+        if (err != cudaSuccess) return cuda_fail(err, "transpose W_Q");
+        pg.out[0] = m->folded;
+        pg.out_lo = static_cast<__nv_bfloat16*>(m->folded) + d;
+        pg.ldc = 2 * d;
+        { KernelTimer t("memory_fold", s);
+          err = launch_pair_gemm(kPairHiLo, pg, TmaOperand{wqt, d, d, d}, none,
+                                 TmaOperand{m->keys, total, d, d}, s); }
+        if (err != cudaSuccess) return cuda_fail(err, "query folding of the keys");
         m->fold_wq = p->W_Q;
       }
-      // bf16 with the fusion weights given: p_i = [W_f1 ; W_g1]_r u_i, the
-      // first fusion layer's r-half applied to every value once per image
-      const int H = p->mlp_hidden;
-      if (bf && p->W_f1 != nullptr && p->W_g1 != nullptr && H > 0 && H % 128 == 0 &&
-          H <= FOVEA_MAX_H && aligned16(p->W_f1) && aligned16(p->W_g1)) {
-        fovea_status ps = alloc_dev(&m->proj, (size_t)total * 2 * H * 2, "projected values");
-        if (ps != FOVEA_OK) return ps;
+      if (proj) {
+        // p_i = [W_f1 ; W_g1]_r u_i, the first fusion layer's r-half applied to
+        // every value once per image
         const __nv_bfloat16* wf1r = static_cast<const __nv_bfloat16*>(p->W_f1) + d;
         const __nv_bfloat16* wg1r = static_cast<const __nv_bfloat16*>(p->W_g1) + d;
         pg.out[0] = m->proj;
@@ -440,39 +483,33 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
         { KernelTimer t("memory_proj_fusion", s);
           err = launch_pair_gemm(kPairStore, pg, TmaOperand{wf1r, H, d, 2 * d},
                                  TmaOperand{wg1r, H, d, 2 * d}, TmaOperand{m->values, total, d, d}, s); }
-        if (err == cudaSuccess) err = cudaStreamSynchronize(s);
         if (err != cudaSuccess) return cuda_fail(err, "fusion projection of the values");
-        int m_max = 0;
-        for (int b = 0; b < B; ++b) m_max = std::max(m_max, m->counts[b]);
-        const int ld = (m_max + 63) / 64 * 64;
-        if ((ps = alloc_dev(&m->projT, (size_t)B * 2 * H * ld * 2, "transposed projected values")) != FOVEA_OK)
-          return ps;
-        static thread_local ImageTable itab;
-        itab.B = B;
-        for (int b = 0; b < B; ++b) {
-          itab.off[b] = (int)m->offsets[b];
-          itab.m[b] = m->counts[b];
-        }
         { KernelTimer t("memory_proj_transpose", s);
           err = launch_transpose_images(m->proj, 2 * H, ld, itab, m->projT, s); }
-        if (err == cudaSuccess) err = cudaStreamSynchronize(s);
         if (err != cudaSuccess) return cuda_fail(err, "transposing the projected values");
         m->proj_ld = ld;
         m->proj_wf1 = p->W_f1;
         m->proj_wg1 = p->W_g1;
         m->proj_h = H;
       }
-      return FOVEA_OK;
-    };
-    st = run();
-    cudaStreamSynchronize(s);
-    cudaFree(xv);
-    cudaFree(src_row);
-    cudaFree(fix);
-    if (st != FOVEA_OK) return cleanup(st);
-  }
+    }
+    int herr = 0;
+    err = cudaMemcpyAsync(&herr, errw, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (err == cudaSuccess) err = cudaStreamSynchronize(s);
+    if (err != cudaSuccess) return cuda_fail(err, "memory build");
+    if (herr & kErrTimeout)
+      return fail(FOVEA_ERR_TIMEOUT, "a bounded device wait gave up during the memory build");
+    return FOVEA_OK;
+  };
+  st = run();
+  for (void* t : {scratch, src_row, xv, fix, wqt})
+    if (t != nullptr) cudaFreeAsync(t, s);
   cudaStreamSynchronize(s);
-  cudaFree(scratch);
+  pool_trim(pool);
+  if (st != FOVEA_OK) {
+    free_memory(m);
+    return st;
+  }
   *out = m;
   return FOVEA_OK;
 }

@@ -245,7 +245,13 @@ cudaError_t launch_ln_query(int dtype, const void* h, int rows, int d, const voi
                             int max_depth, int* err, void* out, cudaStream_t s);
 cudaError_t launch_count_valid(const uint8_t* mask, int B, int M_max, int32_t* counts,
                                cudaStream_t s);
-cudaError_t launch_compact(const uint8_t* mask, int B, int M_max, const int32_t* key_off,
+// Images of a memory: first entry and valid count of each (kernel parameter).
+struct ImageTable {
+  int B;
+  int off[FOVEA_MAX_SEQ];
+  int m[FOVEA_MAX_SEQ];
+};
+cudaError_t launch_compact(const uint8_t* mask, int B, int M_max, const ImageTable& tab,
                            int32_t* orig_index, int32_t* src_row, cudaStream_t s);
 // Selection alone (select.cu): counts, indices, and per row the selected
 // compacted memory rows and weights (sel_pos, sel_w, sel_cnt; any may be
@@ -273,12 +279,6 @@ cudaError_t launch_select_gather(int dtype, const float* scores, const SeqTable&
                                  float* r_out, void* r_lo, const void* P, int H, const float* Gh,
                                  const void* b_f1, const void* b_g1, void* act, int* err,
                                  cudaStream_t s, long long p_prefetch_bytes = 0);
-// Images of a memory: first entry and valid count of each (kernel parameter).
-struct ImageTable {
-  int B;
-  int off[FOVEA_MAX_SEQ];
-  int m[FOVEA_MAX_SEQ];
-};
 // out [B, C, ld]: image b's [m_b, C] rows of `in` (from row off_b) transposed,
 // zero-padded to ld entries (C and ld multiples of 64).
 cudaError_t launch_transpose_images(const void* in, int C, int ld, const ImageTable& tab,
@@ -353,8 +353,8 @@ cudaError_t launch_pair_gemm(PairEpi epi, PairGemm a, const TmaOperand& F0, cons
                              const TmaOperand& R, cudaStream_t s);
 
 // Exact rounding of listed key elements: k = sum_l x[row, l] W[col, l]
-// evaluated in double-float, rounded once to bf16.  list == nullptr refines
-// every element of the [rows, d] key matrix.
+// evaluated in double-float, rounded once to bf16.  A list whose device count
+// exceeds its capacity refines every element of the [rows, d] key matrix.
 cudaError_t launch_refine_keys(const void* xv, const void* W, int d, const KeyFix* list,
                                const int* count, int cap, int rows, void* K, cudaStream_t s);
 

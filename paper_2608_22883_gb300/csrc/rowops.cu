@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(kScanThreads) count_valid_kernel(const uint8_t
 
 __global__ void __launch_bounds__(kScanThreads) compact_kernel(const uint8_t* __restrict__ mask,
                                                               int M_max,
-                                                              const int32_t* __restrict__ key_off,
+                                                              const __grid_constant__ ImageTable tab,
                                                               int32_t* __restrict__ orig_index,
                                                               int32_t* __restrict__ src_row) {
   __shared__ int warp_tot[kScanThreads / 32];
@@ -488,7 +488,7 @@ __global__ void __launch_bounds__(kScanThreads) compact_kernel(const uint8_t* __
   int base = 0;
   for (int w = 0; w < warp; ++w) base += warp_tot[w];
   int rank = base + incl - c;
-  const int off = key_off[b];
+  const int off = tab.off[b];
   for (int i = beg; i < end; ++i) {
     if (mb == nullptr || mb[i] != 0) {
       orig_index[off + rank] = i;
@@ -504,9 +504,9 @@ cudaError_t launch_count_valid(const uint8_t* mask, int B, int M_max, int32_t* c
   return cudaGetLastError();
 }
 
-cudaError_t launch_compact(const uint8_t* mask, int B, int M_max, const int32_t* key_off,
+cudaError_t launch_compact(const uint8_t* mask, int B, int M_max, const ImageTable& tab,
                            int32_t* orig_index, int32_t* src_row, cudaStream_t s) {
-  compact_kernel<<<B, kScanThreads, 0, s>>>(mask, M_max, key_off, orig_index, src_row);
+  compact_kernel<<<B, kScanThreads, 0, s>>>(mask, M_max, tab, orig_index, src_row);
   return cudaGetLastError();
 }
 
@@ -654,7 +654,8 @@ __global__ void __launch_bounds__(kRefineThreads) refine_keys_kernel(
     __nv_bfloat16* __restrict__ K) {
   const int lane = threadIdx.x & 31;
   const long long warps = (long long)gridDim.x * (kRefineThreads / 32);
-  const long long n_items = list ? (long long)min(*count, cap) : total;
+  if (list != nullptr && *count > cap) list = nullptr;           // overflowed: every element
+  const long long n_items = list ? (long long)*count : total;
   const int nv = d / 8;                                          // d % 64 == 0
   for (long long it = blockIdx.x * (kRefineThreads / 32) + (threadIdx.x >> 5); it < n_items;
        it += warps) {
