@@ -291,7 +291,7 @@ static cudaError_t run_gemm(int dtype, int epi, const GemmArgs& a, const TmaOper
                             const TmaOperand& A1, const TmaOperand& B0, const TmaOperand& B1,
                             int max_m, int max_n, cudaStream_t s) {
   if (dtype == FOVEA_BF16) return launch_gemm_tc(epi, a, A0, A1, B0, B1, max_m, max_n, s);
-  return launch_gemm_simt(dtype, epi, a, max_m, max_n, s);
+  return launch_gemm_simt(epi, a, max_m, max_n, s);
 }
 
 static void init_args(GemmArgs& a) {
@@ -433,7 +433,7 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
       a.ngroups = 1;
       a.groups[0] = GemmGroup{0, 2 * d, 0, total, 0};
       { KernelTimer t("memory_proj", s);
-        err = launch_gemm_simt(p->dtype, kEpiStore, a, 2 * d, total, s); }
+        err = launch_gemm_simt(kEpiStore, a, 2 * d, total, s); }
       if (err != cudaSuccess) return cuda_fail(err, "memory projection");
     } else {
       PairGemm pg{};

@@ -172,7 +172,7 @@ struct GemmArgs {
   void* out2; long long ldc2;                      // kEpiQueryH
   const void* bias0; const void* bias1;
   const float* row_scale; float scale;
-  int splits;         // tensor-core path: CTAs of a cluster sharing one output tile (split K)
+  int splits;         // CTAs of a cluster sharing one output tile (split K)
   int stages;         // tensor-core path: depth of the shared-memory ring
   int tx_bytes;       // tensor-core path: bytes one ring stage receives (row box + feature tile)
   int kps;            // tensor-core path: k-blocks of 64 per ring stage
@@ -299,11 +299,9 @@ cudaError_t launch_finalize(int dtype, const void* h, const float* c, const void
                             int N, const DepthGate& gate, void* h_out, float* gate_out,
                             cudaStream_t s);
 
-// GEMM C = A . B^T with a chosen epilogue.  `tc` selects the tcgen05 path
-// (bf16 only); otherwise the SIMT path (fp32 and bf16).
+// GEMM C = A . B^T of fp32 operands with a chosen epilogue (SIMT).
 // max_m / max_n bound the per-group extents (grid size).
-cudaError_t launch_gemm_simt(int dtype, int epi, const GemmArgs& a, int max_m, int max_n,
-                             cudaStream_t s);
+cudaError_t launch_gemm_simt(int epi, const GemmArgs& a, int max_m, int max_n, cudaStream_t s);
 
 struct TmaOperand {     // a row-major [rows, cols] bf16 matrix with a row stride
   const void* base;

@@ -203,6 +203,21 @@ def test_token_layer_norm_is_correctly_rounded(fovea, d, mean, std):
     mem.destroy()
 
 
+# 64 x 64 tiles, k-tiles of 32 in a ring of four, split over up to 8 CTAs: row
+# and entry counts at the edges of a tile, contractions of two k-tiles (no
+# split) up to a full split, more tiles than the GPU holds
+@pytest.mark.parametrize("d,m_sizes,rows", [(64, [1, 65], [1, 63]), (64, [64], [65]),
+                                            (192, [127, 0, 3], [2, 5, 64]), (1024, [130], [64]),
+                                            (512, [700] * 6, [100] * 6)])
+def test_fp32_tile_edges(fovea, d, m_sizes, rows):
+    w = workloads.generate_custom("fp32-edges", d, m_sizes, rows, dtype="fp32", k_max=16, seed=d,
+                                  H=128)
+    s = store(w)
+    gpu = run_gpu(s, fovea)
+    orc, mem = run_oracle(s, mirror=False)
+    compare(gpu, orc, s, mem=mem, mirror=False)
+
+
 def test_plain_fusion_when_weights_differ(fovea):
     """The memory keeps the values projected through the r-half of the first
     fusion layer for the W_f1 / W_g1 it was built with.  A bf16 call given
