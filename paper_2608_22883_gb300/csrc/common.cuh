@@ -122,7 +122,8 @@ __device__ __forceinline__ float block_max(float v, float* scratch) {
 // One independent sub-problem of a GEMM C = A . B^T: output rows are B rows
 // (draft states / tokens), output columns are A rows (features / keys).
 struct GemmGroup {
-  int a_row0;        // first A row of this group
+  int a_row0;        // first A row of this group; kEpiScoresFolded: -1 marks a group of G_h
+                     // (its columns are those of A1, then A2, gh_cols of each, against B1)
   int m;             // A rows (output columns) in this group
   int b_row0;        // first B row of this group
   int n;             // B rows (output rows) in this group
@@ -157,6 +158,7 @@ struct GemmArgs {
   int a_split;        // A rows >= a_split come from A1 (row - a_split)
   int a_split2;       // tensor-core path: A rows >= a_split2 come from A2 (row - a_split2)
   int r_by_part;      // tensor-core path: output columns from A1 / A2 read B1 at every k
+  int gh_cols;        // kEpiScoresFolded with G_h groups: columns of A1 (and of A2)
   int b_split;        // contraction index >= b_split comes from B1 (k - b_split)
   int dual_b;         // tensor-core scores: B0 and B1 are the hi / lo parts of one
                       // operand, both multiplied by the same A tile
@@ -176,7 +178,7 @@ struct GemmArgs {
   int stages;         // tensor-core path: depth of the shared-memory ring
   int tx_bytes;       // tensor-core path: bytes one ring stage receives (row box + feature tile)
   int kps;            // tensor-core path: k-blocks of 64 per ring stage
-  int rbox;           // tensor-core path: rows of a row-operand tile (64 or 128)
+  int rbox, rbox1;    // tensor-core path: rows of a row-operand tile of B0 and of B1 (64 .. 128)
   int region;         // tensor-core path: bytes of the ring / partial-tile staging region
   const float* add_in;          // kEpiAct: fp32 term added before the activation
   unsigned long long* cand;     // kEpiLogits: per-row candidate keys
@@ -313,7 +315,7 @@ struct GemmPlan {
   int bn, splits, stages;
   long long partial_floats;   // global fp32 scratch the launch needs (0: none)
   long long tiles;            // output tiles
-  int rbox;                   // rows of a row-operand load (64 or 128)
+  int rbox, rbox1;            // rows of a row-operand load of B0 and of B1 (64 .. 128)
   int region;                 // bytes of the ring / partial-tile staging region
   int kps;                    // k-blocks of 64 per ring stage
 };

@@ -15,11 +15,12 @@ __device__ __forceinline__ void gemm_epilogue(const GemmArgs& a, const GemmGroup
     else
       static_cast<T*>(a.out1)[row * a.ldc + (m - a.epi_split)] = from_f32<T>(acc);
   } else if constexpr (EPI == kEpiScores || EPI == kEpiScoresFolded) {
-    if (EPI == kEpiScoresFolded && m >= a.epi_split) {
-      static_cast<float*>(a.out2)[((long long)g.b_row0 + n) * a.ldc2 + (m - a.epi_split)] = acc;
+    const int split = g.a_row0 < 0 ? 0 : a.epi_split;          // a group of G_h alone
+    if (EPI == kEpiScoresFolded && m >= split) {
+      static_cast<float*>(a.out2)[((long long)g.b_row0 + n) * a.ldc2 + (m - split)] = acc;
       return;
     }
-    const int stride = EPI == kEpiScoresFolded ? min(g.m, a.epi_split) : g.m;
+    const int stride = EPI == kEpiScoresFolded ? min(g.m, split) : g.m;
     const float rs = a.row_scale ? a.row_scale[g.b_row0 + n] : 1.0f;
     static_cast<float*>(a.out0)[g.c_off + (long long)n * stride + m] = acc * a.scale * rs;
   } else if constexpr (EPI == kEpiBiasSilu || EPI == kEpiAct) {
@@ -57,16 +58,17 @@ __device__ __forceinline__ void gemm_epilogue4(const GemmArgs& a, const GemmGrou
   if constexpr (EPI == kEpiStore || EPI == kEpiBiasSilu || EPI == kEpiAct)
     vec = vec && (m + 3 < a.epi_split || m >= a.epi_split);
   if constexpr (EPI == kEpiScores || EPI == kEpiScoresFolded) {
-    if (EPI == kEpiScoresFolded && m >= a.epi_split) {
-      const long long o2 = row * a.ldc2 + (m - a.epi_split);
+    const int split = g.a_row0 < 0 ? 0 : a.epi_split;          // a group of G_h alone
+    if (EPI == kEpiScoresFolded && m >= split) {
+      const long long o2 = row * a.ldc2 + (m - split);
       if (vec && (o2 & 3) == 0) {
         *reinterpret_cast<float4*>(static_cast<float*>(a.out2) + o2) = make_float4(v[0], v[1], v[2], v[3]);
         return;
       }
     }
-    const int stride = EPI == kEpiScoresFolded ? min(g.m, a.epi_split) : g.m;
+    const int stride = EPI == kEpiScoresFolded ? min(g.m, split) : g.m;
     const long long o = g.c_off + (long long)n * stride + m;
-    if (vec && (o & 3) == 0 && (EPI != kEpiScoresFolded || m + 3 < a.epi_split)) {
+    if (vec && (o & 3) == 0 && (EPI != kEpiScoresFolded || m + 3 < split)) {
       const float rs = a.row_scale ? a.row_scale[g.b_row0 + n] : 1.0f;
       *reinterpret_cast<float4*>(static_cast<float*>(a.out0) + o) =
           make_float4(v[0] * a.scale * rs, v[1] * a.scale * rs, v[2] * a.scale * rs,

@@ -393,8 +393,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   // tile straddles two operands.  A group smaller than the grid leaves its
   // extra tiles idle.  The S CTAs of a tile share these decisions, so a
   // tile's CTAs exit together.
-  const int s1 = min(args.a_split, g.m);
-  const int s2 = max(s1, min(args.a_split2, g.m));
+  const bool gh = EPI == kEpiScoresFolded && g.a_row0 < 0;   // a group of G_h: no F0 part
+  const int s1 = gh ? 0 : min(args.a_split, g.m);
+  const int s2 = gh ? min(args.gh_cols, g.m) : max(s1, min(args.a_split2, g.m));
   const int t0 = (s1 + BN - 1) / BN, t1 = (s2 - s1 + BN - 1) / BN, t2 = (g.m - s2 + BN - 1) / BN;
   // Tile order: with one group and no split, consecutive CTAs walk
   // kRasterRows row tiles per feature tile, so that a wave of resident CTAs
@@ -423,12 +424,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   // the lo part f_lo_kb k-blocks after the hi part in the same rows
   const bool dual_f = EPI == kEpiScoresFolded && args.f_lo_kb > 0 && part == 0;
   const int kProducers = (DUAL || dual_f) ? 3 : 2;   // TMA-issuing lanes of warp 0
-  const int KPS = args.kps, rbox = args.rbox;
+  const int KPS = args.kps, rbox = args.r_by_part && part != 0 ? args.rbox1 : args.rbox;
   const int r_tile = rbox * 128;                       // one k-block of the row operand
   const int r_bytes = KPS * r_tile * (DUAL ? 2 : 1);
   const int f_tile = BN * 128;                         // one k-block of the feature operand
   const int stage_bytes = C::stage_bytes(KPS, rbox, dual_f);
-  const int stages = dual_f ? max(1, min(args.stages, args.region / stage_bytes)) : args.stages;
+  const int stages = EPI == kEpiScoresFolded ? max(1, min(args.stages, args.region / stage_bytes))
+                                             : args.stages;
   extern __shared__ uint8_t smem_raw[];
   // the 1024-byte aligned base, derived from smem_raw by pointer arithmetic
   // so that the compiler keeps every access through it in the shared space
@@ -969,6 +971,7 @@ static cudaError_t launch_tc_inst(GemmArgs& a, const CUtensorMap* maps, int tile
   a.region = p.region;
   a.kps = p.kps;
   a.rbox = p.rbox;
+  a.rbox1 = p.rbox1;
   a.tx_bytes = tc::Cfg<BN, DUAL>::stage_bytes(p.kps, p.rbox,
                                               EPI == kEpiScoresFolded && a.f_lo_kb > 0);
   cudaLaunchConfig_t cfg = {};
@@ -1003,6 +1006,12 @@ static cudaError_t launch_tc_epi(GemmArgs& a, const CUtensorMap* maps, const Gem
 }
 
 // Feature tiles of the widest group: each operand part is tiled on its own.
+static int feature_tiles(const GemmArgs& a, int max_m, int bn);
+static int group_tiles(const GemmArgs& a, const GemmGroup& g, int bn) {
+  if (g.a_row0 < 0)                                          // G_h alone
+    return (a.gh_cols + bn - 1) / bn + (g.m - a.gh_cols + bn - 1) / bn;
+  return feature_tiles(a, g.m, bn);
+}
 static int feature_tiles(const GemmArgs& a, int max_m, int bn) {
   const int s1 = std::min(a.a_split, max_m);
   const int s2 = std::max(s1, std::min(a.a_split2, max_m));
@@ -1052,23 +1061,35 @@ static void plan_for(const GemmArgs& a, int max_m, int max_n, long long row_tile
   const bool DF = EPI == kEpiScoresFolded && a.f_lo_kb > 0;
   const int kb_total = a.k_total / tc::BK;
   const int r_split_kb = a.b_split / tc::BK;
-  const long long ftiles = feature_tiles(a, max_m, BN);
+  long long ftiles = feature_tiles(a, max_m, BN);
+  for (int gi = 0; gi < a.ngroups; ++gi)
+    if (a.groups[gi].a_row0 < 0) ftiles = std::max<long long>(ftiles, group_tiles(a, a.groups[gi], BN));
   const long long tiles = ftiles * row_tiles;          // the grid (every group sized to the largest)
   // tiles with work: groups of ragged sizes leave the rest of their grid
   // slots empty (those CTAs exit at once), so the cost counts these
   long long active = 0;
   for (int gi = 0; gi < a.ngroups; ++gi)
-    active += (long long)feature_tiles(a, a.groups[gi].m, BN) *
+    active += (long long)group_tiles(a, a.groups[gi], BN) *
               ((a.groups[gi].n + tc::BM - 1) / tc::BM);
   if (active <= 0 || active > tiles) active = tiles;
   // the same at the narrowest feature tile: the parallelism the GEMM has
   long long active64 = 0;
   for (int gi = 0; gi < a.ngroups; ++gi)
-    active64 += (long long)feature_tiles(a, a.groups[gi].m, 64) *
+    active64 += (long long)group_tiles(a, a.groups[gi], 64) *
                 ((a.groups[gi].n + tc::BM - 1) / tc::BM);
   const int rows = max_n < tc::BM ? max_n : tc::BM;
   // rows of a row tile: >= 64 so that the MMA's 128-row read stays inside its stage
-  const int rbox = std::max(64, std::min(tc::BM, (max_n + 7) / 8 * 8));
+  // (with G_h groups, B0 serves the score groups alone and B1 the G_h groups)
+  int n0 = max_n, n1 = max_n;
+  if (a.gh_cols > 0) {
+    n0 = n1 = 1;
+    for (int gi = 0; gi < a.ngroups; ++gi) {
+      int& n = a.groups[gi].a_row0 < 0 ? n1 : n0;
+      n = std::max(n, a.groups[gi].n);
+    }
+  }
+  auto box_rows = [](int n) { return std::max(64, std::min(tc::BM, (n + 7) / 8 * 8)); };
+  const int rbox = box_rows(n0), rbox1 = box_rows(n1);
   const int sms = num_sms();
   const bool streaming = max_n <= tc::BM;             // one row tile per group
   for (int kps = 4; kps >= 1; kps >>= 1) {
@@ -1077,7 +1098,8 @@ static void plan_for(const GemmArgs& a, int max_m, int max_n, long long row_tile
     const double stage_f = (double)kps * BN * 128 * (DF ? 2 : 1);
     const double stage_mma_us =
         (double)kps * 4.0 * mma_cycles(BN) * ((DUAL || DF) ? 2 : 1) / 2070.0;
-    const int sb = C::stage_bytes(kps, rbox, DF);
+    const int sb = std::max(C::stage_bytes(kps, rbox, DF),
+                            a.gh_cols > 0 ? C::stage_bytes(kps, rbox1, false) : 0);
     for (int S = 1; S <= 8; ++S) {
       if (S > 1 && S > su_total) break;
       // the weighted-sum GEMM over <= 1024 entries: when its narrowest tiles
@@ -1111,7 +1133,7 @@ static void plan_for(const GemmArgs& a, int max_m, int max_n, long long row_tile
                                       waves, S);
         if (t < best_t - 1e-6 || (t < best_t + 1e-6 && tiles * S < best.tiles * best.splits)) {
           best_t = t;
-          best = GemmPlan{BN, S, stages, 0, tiles, rbox, region, kps};
+          best = GemmPlan{BN, S, stages, 0, tiles, rbox, rbox1, region, kps};
         }
       }
     }
@@ -1121,7 +1143,7 @@ static void plan_for(const GemmArgs& a, int max_m, int max_n, long long row_tile
 template <int EPI>
 static GemmPlan plan_epi(const GemmArgs& a, int max_m, int max_n) {
   const long long row_tiles = (long long)(max_n + tc::BM - 1) / tc::BM * a.ngroups;
-  GemmPlan best{256, 1, 2, 0, 1 << 30, 128, 0, 1};
+  GemmPlan best{256, 1, 2, 0, 1 << 30, 128, 128, 0, 1};
   double best_t = 1e30;
   plan_for<256, EPI>(a, max_m, max_n, row_tiles, best, best_t);
   plan_for<128, EPI>(a, max_m, max_n, row_tiles, best, best_t);
@@ -1149,11 +1171,12 @@ GemmPlan plan_gemm_tc(int epi, const GemmArgs& a, int max_m, int max_n) {
   std::string key;
   key.reserve(64 + 16 * a.ngroups);
   char buf[160];
-  snprintf(buf, sizeof buf, "%d|%d|%d|%d|%d|%d|%d|%d|%d|", epi, max_m, max_n, a.k_total, a.b_split,
-           a.a_split, a.a_split2, a.f_lo_kb, a.ngroups);
+  snprintf(buf, sizeof buf, "%d|%d|%d|%d|%d|%d|%d|%d|%d|%d|", epi, max_m, max_n, a.k_total,
+           a.b_split, a.a_split, a.a_split2, a.f_lo_kb, a.gh_cols, a.ngroups);
   key += buf;
   for (int g = 0; g < a.ngroups; ++g) {
-    snprintf(buf, sizeof buf, "%d,%d;", a.groups[g].m, a.groups[g].n);
+    snprintf(buf, sizeof buf, "%s%d,%d;", a.groups[g].a_row0 < 0 ? "h" : "", a.groups[g].m,
+             a.groups[g].n);
     key += buf;
   }
   auto it = cache.find(key);
@@ -1202,9 +1225,11 @@ cudaError_t launch_gemm_tc(int epi, const GemmArgs& args, const TmaOperand& A0, 
   const TmaOperand& b1 = B1.base ? B1 : B0;
   if (!cached_map3(&maps[0], A0, plan.bn, plan.kps) || !cached_map3(&maps[1], a1, plan.bn, plan.kps) ||
       !cached_map3(&maps[2], a2, plan.bn, plan.kps) || !cached_map3(&maps[3], B0, plan.rbox, plan.kps) ||
-      !cached_map3(&maps[4], b1, plan.rbox, plan.kps))
+      !cached_map3(&maps[4], b1, plan.rbox1, plan.kps))
     return cudaErrorInvalidValue;
-  const int tiles_x = feature_tiles(a, max_m, plan.bn);
+  int tiles_x = feature_tiles(a, max_m, plan.bn);
+  for (int g = 0; g < a.ngroups; ++g)
+    if (a.groups[g].a_row0 < 0) tiles_x = std::max(tiles_x, group_tiles(a, a.groups[g], plan.bn));
   switch (epi) {
     case kEpiScores: return launch_tc_epi<kEpiScores>(a, maps, plan, tiles_x, max_n, s);
     case kEpiBiasSilu: return launch_tc_epi<kEpiBiasSilu>(a, maps, plan, tiles_x, max_n, s);

@@ -218,6 +218,24 @@ def test_fp32_tile_edges(fovea, d, m_sizes, rows):
     compare(gpu, orc, s, mem=mem, mirror=False)
 
 
+# G_h as groups of the score launch: one row past a block of 128, row blocks
+# that straddle sequences, sequences without rows or without entries, score
+# tiles of more than 128 rows, feature parts narrower than a tile (H = 128)
+@pytest.mark.parametrize("d,m_sizes,rows,H", [(320, [70, 0, 200, 33], [100, 5, 0, 24], 128),
+                                              (256, [64, 300, 5], [1, 140, 260], 512),
+                                              (192, [40] * 9, [31] * 9, 128)])
+def test_fusion_h_groups_in_the_score_launch(fovea, d, m_sizes, rows, H):
+    w = workloads.generate_custom("gh", d, m_sizes, rows, k_max=16, seed=d, H=H)
+    s = store(w)
+    fovea.timing_enable(True)
+    gpu = run_gpu(s, fovea)
+    names = set(fovea.timing_read())
+    fovea.timing_enable(False)
+    assert "score_fusion_h" in names and "fusion_h" not in names
+    orc, mem = run_oracle(s, mirror=True)
+    compare(gpu, orc, s, mem=mem)
+
+
 def test_plain_fusion_when_weights_differ(fovea):
     """The memory keeps the values projected through the r-half of the first
     fusion layer for the W_f1 / W_g1 it was built with.  A bf16 call given
