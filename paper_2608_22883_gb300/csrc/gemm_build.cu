@@ -17,9 +17,11 @@
 //
 // Chunked sums.  The tensor core adds a product sum to its fp32 accumulator
 // with truncation, once per 16 elements of the contraction, so a long
-// contraction drifts by about 2^-17 of the result's scale.  Here every chunk
-// of kChunkSu * KPS * 64 = 256 elements starts a fresh accumulator, and the
-// epilogue threads add the chunks in registers with rounded fp32 additions.
+// contraction drifts by about 2^-17 of the result's scale.  For the keys every
+// chunk of kChunkSu * KPS * 64 = 256 elements starts a fresh accumulator, and
+// the epilogue threads add the chunks in registers with rounded fp32 additions.
+// The other outputs keep one accumulator: draining one every 256 elements costs
+// a tile a sixth of its rate (folded keys 820 us instead of 628).
 // A key must be the correctly rounded bf16 of its exact sum; the keys whose
 // sum lies so near a rounding midpoint that the GEMM cannot tell are listed
 // and recomputed exactly (refine_keys_kernel).  The window of that list
@@ -54,7 +56,7 @@ constexpr int kSmemRows = BM * 128;      // bytes of one k-block of tokens
 constexpr int kSmemFeat = BNH * 128;     // bytes of one k-block of this CTA's features
 constexpr int kStageBytes = KPS * (kSmemRows + kSmemFeat);
 constexpr int kStages = 3;
-constexpr int kChunkSu = 2;              // stages per accumulator chunk
+constexpr int kChunkSu = 2;              // stages per accumulator chunk of the keys
 constexpr int kEpiWarps = 8;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kWarpStage = 32 * 128;     // an epilogue warp's staging: 32 rows x 64 bf16
@@ -271,7 +273,8 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
     int i = 0, c = 0;
     bool go = true;
     for (int t = pid; go && t < tiles; t += pairs) {
-      for (int su0 = 0; go && su0 < su_total; su0 += kChunkSu, ++c) {
+      const int chunk = KEYS && tile_at(a, t).part == 0 ? kChunkSu : su_total;
+      for (int su0 = 0; go && su0 < su_total; su0 += chunk, ++c) {
         const int buf = c & 1;
         const uint32_t d = tmem_base + (uint32_t)(buf * BN);
         if (c >= 2 &&
@@ -281,7 +284,7 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
           break;
         }
         tc_fence_after();
-        const int su1 = min(su0 + kChunkSu, su_total);
+        const int su1 = min(su0 + chunk, su_total);
         for (int su = su0; su < su1; ++su, ++i) {
           const int st = i % kStages;
           if (!wait_cluster(&full[st], (uint32_t)(i / kStages) & 1u, abort_flag, a.wait_ns)) {
@@ -316,7 +319,8 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
       float acc[BNH];
 #pragma unroll
       for (int j = 0; j < BNH; ++j) acc[j] = 0.0f;
-      for (int su0 = 0; su0 < su_total; su0 += kChunkSu, ++c) {
+      const int chunk = KEYS && ti.part == 0 ? kChunkSu : su_total;
+      for (int su0 = 0; su0 < su_total; su0 += chunk, ++c) {
         const int buf = c & 1;
         const bool ok = wait_cluster(&tfull[buf], (uint32_t)(c >> 1) & 1u, abort_flag, a.wait_ns);
         if (!__all_sync(0xffffffffu, ok)) {      // tcgen05.ld below is a .sync.aligned instruction
