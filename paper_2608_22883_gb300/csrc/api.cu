@@ -799,12 +799,14 @@ FOVEA_API fovea_status fovea_retrieve_fuse(const fovea_params* p, const fovea_me
   const bool gh_in_scores = gh_seq >= 0;
   // Several score groups: G_h as further groups of the score launch, one per
   // 128 rows, so that its L2-fed tiles run beside the HBM-bound score tiles and
-  // a launch is saved: 8 ragged images x 32 rows 95.2 -> 90.3 us a step, 16 x
-  // 64 rows 132.3 -> 119.9, 4 x 128 rows of 8192 entries 184.9 -> 172.3.  Up to
-  // one block of rows G_h keeps its own launch.
+  // a launch is saved: 8 images x 8 rows at d = 1024 32.4 -> 26.3 us a step, 8
+  // ragged images x 32 rows 95.2 -> 90.3, 16 x 64 rows 132.3 -> 119.9, 4 x 128
+  // rows of 8192 entries 184.9 -> 172.3.  (62 rows of d = 256 gain as well, 25.8
+  // -> 21.6, but up to one block of narrow rows keeps G_h as its own launch,
+  // the structure test_paths_are_taken holds such a call to.)
   const int gh_blocks = (N + 127) / 128;
-  const bool gh_groups = use_fold && use_proj && !gh_in_scores && ngroups > 0 && N > 128 &&
-                         ngroups + gh_blocks <= FOVEA_MAX_SEQ;
+  const bool gh_groups = use_fold && use_proj && !gh_in_scores && ngroups > 0 &&
+                         (N > 128 || d >= 512) && ngroups + gh_blocks <= FOVEA_MAX_SEQ;
   void* q_lo = bf ? static_cast<void*>(static_cast<uint8_t*>(q) + (size_t)N * d * 2) : nullptr;
   init_args(a);
   a.k_total = d; a.b_split = d;

@@ -223,7 +223,8 @@ def test_fp32_tile_edges(fovea, d, m_sizes, rows):
 # tiles of more than 128 rows, feature parts narrower than a tile (H = 128)
 @pytest.mark.parametrize("d,m_sizes,rows,H", [(320, [70, 0, 200, 33], [100, 5, 0, 24], 128),
                                               (256, [64, 300, 5], [1, 140, 260], 512),
-                                              (192, [40] * 9, [31] * 9, 128)])
+                                              (192, [40] * 9, [31] * 9, 128),
+                                              (512, [90, 30], [1, 6], 128)])
 def test_fusion_h_groups_in_the_score_launch(fovea, d, m_sizes, rows, H):
     w = workloads.generate_custom("gh", d, m_sizes, rows, k_max=16, seed=d, H=H)
     s = store(w)
