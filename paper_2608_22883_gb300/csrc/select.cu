@@ -1,8 +1,7 @@
 // Cumulative-mass selection kernels (the algorithm is in select_core.cuh):
 // the selection alone (one CTA of 256 threads per draft state), and the
 // selection fused with the readout r_n = sum_{t < K} alpha_t u_{pi(t)} (the
-// alpha / r_n equation of the retrieval section).  The row's scores are
-// staged in shared memory first.
+// alpha / r_n equation of the retrieval section).
 #include <algorithm>
 
 #include "select_core.cuh"
@@ -20,10 +19,17 @@ struct BlockSyncT {
 };
 using BlockSync = BlockSyncT<false>;
 
-template <bool kLargeCaps>
-__global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_constant__ SelectArgs a,
+// PT: scores per thread in registers (rows of up to 256 PT entries), 0: rows
+// of any length, staged in shared memory.  Bound by the latency of its phases:
+// 512 rows of 8192 clustered entries, four CTAs per SM in one wave, take 19 us
+// (26 us with the scores staged in shared memory, every entry in the histogram
+// and candidates ranked by counting), 2048 rows of 576 entries 16 us (20).
+// Registers by row length: at 32 scores per thread rows of 2880 entries cost
+// 3 us more than at 16.
+template <bool kLargeCaps, int PT>
+__global__ void __launch_bounds__(kSelThreads, 4) select_kernel(const __grid_constant__ SelectArgs a,
                                                              const __grid_constant__ SeqTable tab) {
-  extern __shared__ float s_sc[];                            // [M] scores of this row
+  extern __shared__ float s_sc[];                            // PT = 0: [M] scores of this row
   __shared__ SelectSmem sm;
   const int n = blockIdx.x;
   const int tid = threadIdx.x;
@@ -37,13 +43,33 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_consta
     return;
   }
   const float* src = a.scores + tab.score_off[b] + (long long)(n - tab.row_start[b]) * M;
-  for (int i = tid; i < M; i += kSelThreads) {
-    float v = src[i];
-    if (v == 0.0f) v = 0.0f;              // -0 -> +0 so equal scores get equal keys
-    s_sc[i] = v;
+  const int key_off = tab.key_off[b];
+  BlockSyncT<kLargeCaps> sync;
+  if constexpr (PT > 0) {
+    select_row<PT>(a, n, M, key_off, src, sm, tid, sync);
+  } else {
+    for (int i = tid; i < M; i += kSelThreads) s_sc[i] = norm_score(src[i]);
+    __syncthreads();
+    if (!select_wide(a, n, M, key_off, s_sc, sm, tid, sync))
+      select_radix(a, n, M, key_off, s_sc, sm, tid, sync);
   }
-  __syncthreads();
-  select_row(a, n, M, tab.key_off[b], s_sc, sm, tid, BlockSyncT<kLargeCaps>{});
+}
+
+template <bool kLargeCaps>
+static cudaError_t launch_select_caps(const SelectArgs& a, const SeqTable& tab, int N, int max_m,
+                                      cudaStream_t s) {
+  if (max_m <= kFastMaxM)
+    return launch_pdl(select_kernel<kLargeCaps, 8>, dim3(N), dim3(kSelThreads), 0, s, a, tab);
+  if (max_m <= 16 * kSelThreads)
+    return launch_pdl(select_kernel<kLargeCaps, 16>, dim3(N), dim3(kSelThreads), 0, s, a, tab);
+  if (max_m <= kLongMaxM)
+    return launch_pdl(select_kernel<kLargeCaps, 32>, dim3(N), dim3(kSelThreads), 0, s, a, tab);
+  const cudaError_t e = cudaFuncSetAttribute(select_kernel<kLargeCaps, 0>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             FOVEA_MAX_ENTRIES * (int)sizeof(float));
+  if (e != cudaSuccess) return e;
+  return launch_pdl(select_kernel<kLargeCaps, 0>, dim3(N), dim3(kSelThreads),
+                    (size_t)max_m * sizeof(float), s, a, tab);
 }
 
 cudaError_t launch_select(const float* scores, const SeqTable& tab, int N, const int32_t* orig_index,
@@ -52,23 +78,12 @@ cudaError_t launch_select(const float* scores, const SeqTable& tab, int N, const
                           int32_t* sel_cnt, cudaStream_t s, void* alpha_hi, void* alpha_lo,
                           int alpha_ld) {
   if (N == 0) return cudaSuccess;
-  const size_t smem = (size_t)max(max_m, 1) * sizeof(float);
-  static bool configured = false;
-  if (!configured) {
-    for (auto k : {(const void*)select_kernel<false>, (const void*)select_kernel<true>}) {
-      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           FOVEA_MAX_ENTRIES * (int)sizeof(float));
-      if (e != cudaSuccess) return e;
-    }
-    configured = true;
-  }
   SelectArgs a{scores, orig_index, rho, k_min, k_max, counts, indices, sel_pos, sel_w, sel_cnt,
                nullptr, nullptr, nullptr, gate,
                static_cast<__nv_bfloat16*>(alpha_hi), static_cast<__nv_bfloat16*>(alpha_lo),
                alpha_ld};
-  if (k_max > kRankMax)
-    return launch_pdl(select_kernel<true>, dim3(N), dim3(kSelThreads), smem, s, a, tab);
-  return launch_pdl(select_kernel<false>, dim3(N), dim3(kSelThreads), smem, s, a, tab);
+  return k_max > kRankMax ? launch_select_caps<true>(a, tab, N, max_m, s)
+                          : launch_select_caps<false>(a, tab, N, max_m, s);
 }
 
 // Selection and the gathers that consume it, in one kernel: one
@@ -128,7 +143,6 @@ struct GatherArgs {
   const void* b_g1;                 // [H]: bias of columns >= H
   void* act;                        // [N, HP]
   long long p_prefetch;             // bytes of P prefetched into L2 before the wait
-  int red_floats;                   // dynamic shared memory: the row's scores
   // > 0: the selected rows of P are staged in shared memory by bulk copies,
   // this many per round, at dyn + stage_off, with the group sums at dyn + red_off
   int stage_rows, stage_off, red_off;
@@ -270,8 +284,8 @@ __global__ void __launch_bounds__(NT) select_gather_kernel(
     const __grid_constant__ SelectArgs args, const __grid_constant__ SeqTable tab,
     const __grid_constant__ GatherArgs ga) {
   constexpr int V = 16 / (int)sizeof(T);                     // elements per 16-byte vector
-  // dynamic: [red_floats] scores | [chunk_p] G_h | [chunk_p] bias | [red_floats] original
-  // positions of the row's sequence (int32)
+  // dynamic: [chunk_p] G_h | [chunk_p] bias | original positions of the row's
+  // sequence (int32)
   extern __shared__ __align__(16) float dyn[];
   __shared__ SelectSmem sm;
   __shared__ __align__(16) int32_t loc_pos[kRankMax];
@@ -285,8 +299,7 @@ __global__ void __launch_bounds__(NT) select_gather_kernel(
     tc::mbar_init(&stage_bar, 1);
     tc::fence_mbar_init();
   }
-  float* s_sc = dyn;
-  float* gh_s = dyn + ga.red_floats;
+  float* gh_s = dyn;
   T* bias_s = reinterpret_cast<T*>(gh_s + ga.chunk_p);
   if (ga.p_prefetch > 0 && tid == 0) {
     // the projected values (memory: not written by the previous kernel),
@@ -347,34 +360,10 @@ __global__ void __launch_bounds__(NT) select_gather_kernel(
       select_empty(a, n, tid);              // K = 0, r_n = 0
     } else {
       const float* src = a.scores + tab.score_off[b] + (long long)(n - tab.row_start[b]) * M;
-      if (M <= kFastMaxM) {
-        // every load of the thread in flight at once (8 per thread at most)
-        constexpr int PT = kFastMaxM / kSelThreads;
-        float v[PT];
-#pragma unroll
-        for (int j = 0; j < PT; ++j) {
-          const int i = tid + j * kSelThreads;
-          v[j] = i < M ? src[i] : 0.0f;
-        }
-#pragma unroll
-        for (int j = 0; j < PT; ++j) {
-          const int i = tid + j * kSelThreads;
-          if (i < M) s_sc[i] = v[j] == 0.0f ? 0.0f : v[j];   // -0 -> +0: equal keys
-        }
-      } else {
-        for (int i = tid; i < M; i += kSelThreads) {
-          float v = src[i];
-          if (v == 0.0f) v = 0.0f;        // -0 -> +0 so equal scores get equal keys
-          s_sc[i] = v;
-        }
-      }
-      if constexpr (NT == kSelThreads) {
-        __syncthreads();
-        select_row(a, n, M, tab.key_off[b], s_sc, sm, tid, BlockSync{});
-      } else {
-        SelGroupSync{}();
-        select_row(a, n, M, tab.key_off[b], s_sc, sm, tid, SelGroupSync{});
-      }
+      if constexpr (NT == kSelThreads)
+        select_row<kFastMaxM / kSelThreads>(a, n, M, tab.key_off[b], src, sm, tid, BlockSync{});
+      else
+        select_row<kFastMaxM / kSelThreads>(a, n, M, tab.key_off[b], src, sm, tid, SelGroupSync{});
     }
   }
   // rank 0's selection visible to the cluster (one CTA: a CTA barrier, which
@@ -484,11 +473,10 @@ cudaError_t launch_select_gather(int dtype, const float* scores, const SeqTable&
   ga.b_g1 = b_g1;
   ga.act = act;
   ga.p_prefetch = P != nullptr ? p_prefetch_bytes : 0;
-  ga.red_floats = (int)align_up_sz((size_t)std::max(max_m, 1), 4);
   const size_t es = dtype == FOVEA_BF16 ? 2 : 4;
-  // dynamic: scores | G_h | biases | original positions
-  size_t smem = (size_t)ga.red_floats * 4 + (size_t)ga.chunk_p * 4 +
-                align_up_sz((size_t)ga.chunk_p * es, 16) + (size_t)ga.red_floats * 4;
+  // dynamic: G_h | biases | original positions
+  size_t smem = (size_t)ga.chunk_p * 4 + align_up_sz((size_t)ga.chunk_p * es, 16) +
+                align_up_sz((size_t)std::max(max_m, 1), 4) * 4;
   if (smem > 64 * 1024) return cudaErrorInvalidValue;
   ga.err = err;
   if (wide && dtype == FOVEA_BF16 && ga.chunk_p % 8 == 0 && 1024 % (ga.chunk_p / 8) == 0) {

@@ -5,12 +5,11 @@
 // K = min(|V|, K_max, max(K_min, K_raw)), and the renormalised weights over
 // I_n = pi_n(1..K)).
 //
-// The caller stages the row's scores in shared memory (-0 mapped to +0) and
-// calls select_row.  A histogram of the distance to the maximum finds the
-// bin holding the K_eff-th largest score (K_eff = min(K_max, |V|)) without
-// sorting the row: in registers for rows of up to 2048 entries (select_fast),
-// in strided passes over shared memory above that (select_wide).  The entries
-// of the bins up to it are the candidates; only they are put in order, by
+// A histogram of the distance to the maximum finds the bin holding the
+// K_eff-th largest score (K_eff = min(K_max, |V|)) without sorting the row:
+// with the scores in registers for rows of up to 8192 entries (select_fast), in
+// strided passes over shared memory above that (select_wide).  The entries of
+// the bins up to it are the candidates; only they are put in order, by
 // (score desc, position asc): each candidate's rank is its count of larger
 // candidates for up to 256 candidates, a bucket order above that.  An fp32
 // inclusive scan of exp(s - s_max) over the first K_eff gives the cumulative
@@ -87,6 +86,7 @@ struct SelectSmem {
   unsigned long long sorted[FOVEA_MAX_K];     // ordered keys; scratch of bucket_order
   float cum[FOVEA_MAX_K];                    // inclusive scan of exp(s - s_max)
   unsigned int hist[256];
+  unsigned int bin_off[256];                 // the fast path's bins
   float red_m[kSelWarps], red_s[kSelWarps], red_lo[kSelWarps];
   float warp_tot_f[kSelWarps];
   int warp_tot[kSelWarps];
@@ -225,12 +225,16 @@ __device__ void bucket_order(SelectSmem& sm, int C, int tid, Sync sync) {
 }
 
 template <class Sync>
-__device__ __forceinline__ void select_tail(const SelectArgs& a, int n, int key_off,
-                                            const float* s_sc, int K_eff, int C, float smax,
-                                            float sumexp, SelectSmem& sm, int tid, Sync sync);
+__device__ __forceinline__ void select_tail(const SelectArgs& a, int n, int key_off, int K_eff,
+                                            int C, float smax, float sumexp, SelectSmem& sm,
+                                            int tid, Sync sync);
+
+// A score as the selection takes it: -0 as +0, so that equal scores have equal
+// keys.
+__device__ __forceinline__ float norm_score(float v) { return v == 0.0f ? 0.0f : v; }
 
 // Radix select, candidate ordering, mass scan and the outputs of draft state
-// n, whose M (>= 1) scores are staged in s_sc.  key_off is the compacted row
+// n, whose M (>= 1) scores are s_sc (global or shared memory).  key_off is the compacted row
 // of the sequence's first memory entry.
 template <class Sync>
 __device__ void select_finish(const SelectArgs& a, int n, int M, int key_off, const float* s_sc,
@@ -252,7 +256,7 @@ __device__ void select_finish(const SelectArgs& a, int n, int M, int key_off, co
       const int i = base + tid;
       uint32_t bin = 0xFFFFFFFFu;
       if (i < M) {
-        const uint32_t k = ord_key(s_sc[i]);
+        const uint32_t k = ord_key(norm_score(s_sc[i]));
         if ((k & pmask) == prefix) bin = (k >> shift) & 255u;
       }
       const unsigned int peers = __match_any_sync(0xffffffffu, bin);
@@ -304,7 +308,7 @@ __device__ void select_finish(const SelectArgs& a, int n, int M, int key_off, co
   for (int base = 0; base < M; base += kSelThreads) {
     const int i = base + tid;
     uint32_t k = 0;
-    const bool take = i < M && (k = ord_key(s_sc[i])) > T;
+    const bool take = i < M && (k = ord_key(norm_score(s_sc[i]))) > T;
     const unsigned int bal = __ballot_sync(0xffffffffu, take);
     int slot0 = 0;
     if (lane == 0 && bal) slot0 = atomicAdd(&sm.sh_cnt_gt, __popc(bal));
@@ -320,7 +324,7 @@ __device__ void select_finish(const SelectArgs& a, int n, int M, int key_off, co
     const int chunk = (M + kSelThreads - 1) / kSelThreads;
     const int beg = min(M, tid * chunk), end = min(M, beg + chunk);
     int c = 0;
-    for (int i = beg; i < end; ++i) c += ord_key(s_sc[i]) == T;
+    for (int i = beg; i < end; ++i) c += ord_key(norm_score(s_sc[i])) == T;
     int incl = c;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -332,7 +336,7 @@ __device__ void select_finish(const SelectArgs& a, int n, int M, int key_off, co
     int rank = incl - c;
     for (int w = 0; w < warp; ++w) rank += sm.warp_tot[w];
     for (int i = beg; i < end && rank < krem; ++i) {
-      if (ord_key(s_sc[i]) == T) {
+      if (ord_key(norm_score(s_sc[i])) == T) {
         sm.cand[c_gt + rank] = ((unsigned long long)T << 32) | (0xFFFFFFFFu - (uint32_t)i);
         ++rank;
       }
@@ -340,22 +344,21 @@ __device__ void select_finish(const SelectArgs& a, int n, int M, int key_off, co
   }
   sync();
 
-  select_tail(a, n, key_off, s_sc, K_eff, K_eff, smax, sumexp, sm, tid, sync);
+  select_tail(a, n, key_off, K_eff, K_eff, smax, sumexp, sm, tid, sync);
 }
 
-// select_tail for K_eff > kRankMax: the C (K_eff <= C <= FOVEA_MAX_K)
-// candidates bucket-ordered, the cumulative mass over the first K_eff four
-// contiguous entries per thread, and the outputs, the original indices of a
-// thread's outputs requested together before any is written.
+// K_eff > kRankMax, the ordered entries in `ordered`: the cumulative mass over
+// the first K_eff four contiguous entries per thread, and the outputs, the
+// original indices of a thread's outputs requested together before any is
+// written.
 template <class Sync>
-__device__ __forceinline__ void select_tail_large(const SelectArgs& a, int n, int key_off,
-                                                   const float* s_sc, int K_eff, int C, float smax,
-                                                   float sumexp, SelectSmem& sm, int tid, Sync sync) {
+__device__ __forceinline__ void select_mass_large(const SelectArgs& a, int n, int key_off,
+                                                  int K_eff, float smax, float sumexp,
+                                                  const unsigned long long* ordered,
+                                                  SelectSmem& sm, int tid, Sync sync) {
   static_assert(FOVEA_MAX_K <= 4 * kSelThreads, "four ordered entries per thread");
   const int lane = tid & 31, warp = tid >> 5;
   const int k_max = a.k_max;
-  bucket_order(sm, C, tid, sync);           // ends with a barrier
-  const unsigned long long* ordered = sm.cand;
   // ---- cumulative mass: thread tid holds ordered entries 4 tid .. 4 tid + 3
   constexpr int per = 4;
   float e[4];
@@ -363,9 +366,7 @@ __device__ __forceinline__ void select_tail_large(const SelectArgs& a, int n, in
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int t = per * tid + q;
-    e[q] = q < per && t < K_eff
-               ? expf(s_sc[0xFFFFFFFFu - (uint32_t)(ordered[t] & 0xFFFFFFFFull)] - smax)
-               : 0.0f;
+    e[q] = q < per && t < K_eff ? expf(key_score(ordered[t]) - smax) : 0.0f;
     run += e[q];
   }
   float incl = run;
@@ -406,7 +407,7 @@ __device__ __forceinline__ void select_tail_large(const SelectArgs& a, int n, in
     wu[j] = 0.0f;
     if (u < K) {
       pu[j] = (int)(0xFFFFFFFFu - (uint32_t)(ordered[u] & 0xFFFFFFFFull));
-      wu[j] = expf(s_sc[pu[j]] - smax) / denom;
+      wu[j] = expf(key_score(ordered[u]) - smax) / denom;
       if (a.indices) oi[j] = a.orig_index[key_off + pu[j]];
     }
   }
@@ -434,45 +435,28 @@ __device__ __forceinline__ void select_tail_large(const SelectArgs& a, int n, in
   }
 }
 
-// K_eff <= kRankMax: ranking of the C (>= K_eff) candidates in sm.cand by (score desc,
-// position asc), which puts the top K_eff in order in sm.sorted; then the
-// cumulative mass, one ordered entry per thread (K_eff <= kRankMax), the
-// count K and the outputs of draft state n.
-template <class Sync>
-__device__ __forceinline__ void select_tail(const SelectArgs& a, int n, int key_off,
-                                            const float* s_sc, int K_eff, int C, float smax,
-                                            float sumexp, SelectSmem& sm, int tid, Sync sync) {
-  if constexpr (Sync::kLarge) {               // otherwise the launcher keeps K_max <= kRankMax
+// The cumulative mass of the K_eff ordered entries in sm.sorted, the count K
+// and the outputs of draft state n: one ordered entry per thread for K_eff <=
+// kRankMax, four above (kLarge; otherwise the launcher keeps K_max <= kRankMax).
+template <bool kLarge, class Sync>
+__device__ __forceinline__ void select_mass(const SelectArgs& a, int n, int key_off, int K_eff,
+                                            float smax, float sumexp, SelectSmem& sm, int tid,
+                                            Sync sync) {
+  if constexpr (kLarge) {
     if (K_eff > kRankMax) {
-      select_tail_large(a, n, key_off, s_sc, K_eff, C, smax, sumexp, sm, tid, sync);
+      select_mass_large(a, n, key_off, K_eff, smax, sumexp, sm.sorted, sm, tid, sync);
       return;
     }
   }
   const int lane = tid & 31, warp = tid >> 5;
   const int k_max = a.k_max;
-  // ---- rank the candidates: rank = #larger (keys are distinct) -------------
-  for (int c = tid; c < C; c += kSelThreads) {
-    const unsigned long long me = sm.cand[c];
-    int r0 = 0, r1 = 0, r2 = 0, r3 = 0;
-    int j = 0;
-    for (; j + 3 < C; j += 4) {
-      r0 += sm.cand[j] > me;
-      r1 += sm.cand[j + 1] > me;
-      r2 += sm.cand[j + 2] > me;
-      r3 += sm.cand[j + 3] > me;
-    }
-    for (; j < C; ++j) r0 += sm.cand[j] > me;
-    const int r = (r0 + r1) + (r2 + r3);
-    if (r < K_eff) sm.sorted[r] = me;
-  }
-  sync();                                                     // (4)
   // ---- cumulative mass, one ordered entry per thread -----------------------
   const int t = tid;
   float e = 0.0f;
   int pos = 0;
   if (t < K_eff) {
     pos = (int)(0xFFFFFFFFu - (uint32_t)(sm.sorted[t] & 0xFFFFFFFFull));
-    e = expf(s_sc[pos] - smax);
+    e = expf(key_score(sm.sorted[t]) - smax);
   }
   float incl = e;
 #pragma unroll
@@ -499,7 +483,7 @@ __device__ __forceinline__ void select_tail(const SelectArgs& a, int n, int key_
   for (int u = tid; u < k_max; u += kSelThreads) {
     if (u < K) {
       const int pu = u == t ? pos : (int)(0xFFFFFFFFu - (uint32_t)(sm.sorted[u] & 0xFFFFFFFFull));
-      const float eu = u == t ? e : expf(s_sc[pu] - smax);
+      const float eu = u == t ? e : expf(key_score(sm.sorted[u]) - smax);
       const int row = key_off + pu;
       if (a.sel_pos) a.sel_pos[out_row + u] = row;
       if (a.sel_w) a.sel_w[out_row + u] = eu / denom;
@@ -520,39 +504,87 @@ __device__ __forceinline__ void select_tail(const SelectArgs& a, int n, int key_
   }
 }
 
-// Fast path for rows of at most kFastMaxM entries (any K_eff <= FOVEA_MAX_K),
-// with six group barriers and short dependency chains between them: the
-// threads keep their scores in registers; (1) the maximum and the minimum
-// score; (2) the softmax denominator (independent exponentials, summed in a
-// fixed tree) and a 256-bin histogram of s_max - s over [0, s_max - s_min],
-// which gives the bin b* holding the K_eff-th largest score (the bin index is
-// monotone in the score, so the top K_eff entries all lie in bins <= b*);
-// (3) the entries of bins <= b* are gathered (one shared-memory atomic per
-// warp) and ordered among themselves by (score desc, position asc), which
-// puts the top K_eff in order; the mass scan follows (select_tail).  Returns false, having written nothing, when the candidates
-// exceed kFastMaxCand; the caller then runs the radix path.
+// Puts the C (K_eff <= C <= FOVEA_MAX_K) candidates in sm.cand in order by
+// (score desc, position asc), then the mass scan: direct ranks (the count of
+// larger candidates) for K_eff <= kRankMax, a bucket order above.
+template <class Sync>
+__device__ __forceinline__ void select_tail(const SelectArgs& a, int n, int key_off, int K_eff,
+                                            int C, float smax, float sumexp, SelectSmem& sm,
+                                            int tid, Sync sync) {
+  if constexpr (Sync::kLarge) {
+    if (K_eff > kRankMax) {
+      bucket_order(sm, C, tid, sync);         // ends with a barrier; in place in sm.cand
+      select_mass_large(a, n, key_off, K_eff, smax, sumexp, sm.cand, sm, tid, sync);
+      return;
+    }
+  }
+  for (int c = tid; c < C; c += kSelThreads) {
+    const unsigned long long me = sm.cand[c];
+    int r0 = 0, r1 = 0, r2 = 0, r3 = 0;
+    int j = 0;
+    for (; j + 3 < C; j += 4) {
+      r0 += sm.cand[j] > me;
+      r1 += sm.cand[j + 1] > me;
+      r2 += sm.cand[j + 2] > me;
+      r3 += sm.cand[j + 3] > me;
+    }
+    for (; j < C; ++j) r0 += sm.cand[j] > me;
+    const int r = (r0 + r1) + (r2 + r3);
+    if (r < K_eff) sm.sorted[r] = me;
+  }
+  sync();
+  select_mass<false>(a, n, key_off, K_eff, smax, sumexp, sm, tid, sync);
+}
+
+// Fast path for rows of at most 256 PT entries, PT = 8 or 32 scores per thread
+// (any K_eff <= FOVEA_MAX_K), with short dependency chains between its group
+// barriers.  The scores live in the threads' registers, v[j] the entry tid +
+// 256 j (every load of a row in flight at once, nothing staged in shared
+// memory).  (1) The maximum, and a floor T no larger than the K_eff-th largest
+// score: the smallest of the 256 threads' maxima when K_eff <= 256 and every
+// thread has an entry (256 entries are >= T), else the minimum.  (2) The
+// softmax denominator (independent exponentials, summed in a fixed tree) and a
+// 256-bin histogram of s_max - s over [0, s_max - T] of the entries >= T (of
+// 8192 entries about a sixth: the histogram's shared-memory atomics were the
+// longest phase, and the bins get finer); the bin is monotone in the score, so
+// with b* the bin holding the K_eff-th largest, the top K_eff entries all lie
+// in bins <= b*.  (3) The bins' offsets.  (4) The entries of bins <= b*, the
+// candidates, are scattered into bin order, and (5) each takes its rank among
+// its own bin's by (score desc, position asc), which puts the top K_eff in
+// order; the mass scan follows (select_mass).  Returns false, having written
+// nothing, when the candidates exceed kFastMaxCand; the caller then runs the
+// radix path.
 constexpr int kFastMaxM = 2048;                   // 8 scores per thread
+constexpr int kLongMaxM = 8192;                   // 32 scores per thread
 constexpr int kFastMaxCand = FOVEA_MAX_K;         // candidates ranked directly
 
-template <class Sync>
-__device__ bool select_fast(const SelectArgs& a, int n, int M, int key_off, const float* s_sc,
-                            SelectSmem& sm, int tid, Sync sync) {
-  constexpr int PT = kFastMaxM / kSelThreads;
-  static_assert(PT == 8, "the denominator tree below sums eight terms per thread");
-  const int lane = tid & 31, warp = tid >> 5;
-  const int k_max = a.k_max;
-  const int K_eff = min(k_max, M);
-  float v[PT];
-  float lmax = -INFINITY, lmin = INFINITY;
+// The row's scores in registers, -infinity past its end.
+template <int PT>
+__device__ __forceinline__ void load_scores(const float* src, int M, int tid, float (&v)[PT]) {
 #pragma unroll
   for (int j = 0; j < PT; ++j) {
     const int i = tid + j * kSelThreads;
-    v[j] = i < M ? s_sc[i] : -INFINITY;
-    if (i < M) {
+    v[j] = i < M ? src[i] : -INFINITY;
+  }
+#pragma unroll
+  for (int j = 0; j < PT; ++j) v[j] = norm_score(v[j]);
+}
+
+template <int PT, class Sync>
+__device__ bool select_fast(const SelectArgs& a, int n, int M, int key_off, const float (&v)[PT],
+                            SelectSmem& sm, int tid, Sync sync) {
+  static_assert(PT % 8 == 0, "the denominator tree below sums eight terms at a time");
+  const int lane = tid & 31, warp = tid >> 5;
+  const int K_eff = min(a.k_max, M);
+  float lmax = -INFINITY, lmin = INFINITY;
+#pragma unroll
+  for (int j = 0; j < PT; ++j) {
+    if (tid + j * kSelThreads < M) {
       lmax = fmaxf(lmax, v[j]);
       lmin = fminf(lmin, v[j]);
     }
   }
+  if (K_eff <= kSelThreads && M >= kSelThreads) lmin = lmax;   // the floor from the maxima
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     lmax = fmaxf(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
@@ -563,31 +595,34 @@ __device__ bool select_fast(const SelectArgs& a, int n, int M, int key_off, cons
     sm.red_m[warp] = lmax;
     sm.red_lo[warp] = lmin;
   }
-  if (tid == 0) sm.sh_cnt_gt = 0;
   sync();                                                     // (1)
-  float smax = sm.red_m[0], smin = sm.red_lo[0];
+  float smax = sm.red_m[0], floor_s = sm.red_lo[0];
 #pragma unroll
   for (int w = 1; w < kSelWarps; ++w) {
     smax = fmaxf(smax, sm.red_m[w]);
-    smin = fminf(smin, sm.red_lo[w]);
+    floor_s = fminf(floor_s, sm.red_lo[w]);
   }
   // ---- softmax denominator and histogram of the distance to the maximum ----
-  const float range = smax - smin;
+  const float range = smax - floor_s;
   const float inv_w = range > 0.0f ? 255.0f / range : 0.0f;
-  float ex[PT];
-  int bin[PT];
+  auto bin_of = [&](float x) {
+    const int b = (int)((smax - x) * inv_w);
+    return b < 0 ? 0 : (b > 255 ? 255 : b);
+  };
+  float lsum = 0.0f;
 #pragma unroll
-  for (int j = 0; j < PT; ++j) {
-    const int i = tid + j * kSelThreads;
-    ex[j] = i < M ? expf(v[j] - smax) : 0.0f;
-    bin[j] = 256;
-    if (i < M) {
-      const int b = (int)((smax - v[j]) * inv_w);
-      bin[j] = b < 0 ? 0 : (b > 255 ? 255 : b);
-      atomicAdd(&sm.hist[bin[j]], 1u);
+  for (int j0 = 0; j0 < PT; j0 += 8) {
+    float ex[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const bool real = tid + (j0 + j) * kSelThreads < M;
+      ex[j] = real ? expf(v[j0 + j] - smax) : 0.0f;
+      // (not below the floor: a NaN score is binned too, and counts as a candidate)
+      if (real && !(v[j0 + j] < floor_s)) atomicAdd(&sm.hist[bin_of(v[j0 + j])], 1u);
     }
+    const float g = ((ex[0] + ex[1]) + (ex[2] + ex[3])) + ((ex[4] + ex[5]) + (ex[6] + ex[7]));
+    lsum = j0 == 0 ? g : lsum + g;
   }
-  float lsum = ((ex[0] + ex[1]) + (ex[2] + ex[3])) + ((ex[4] + ex[5]) + (ex[6] + ex[7]));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
   if (lane == 0) sm.red_s[warp] = lsum;
@@ -595,8 +630,9 @@ __device__ bool select_fast(const SelectArgs& a, int n, int M, int key_off, cons
   float sumexp = sm.red_s[0];
 #pragma unroll
   for (int w = 1; w < kSelWarps; ++w) sumexp += sm.red_s[w];
-  // every warp finds b* itself: lane l owns bins 8l .. 8l + 7
-  int bstar;
+  // every warp finds b* and the candidate count itself: lane l owns bins 8l ..
+  // 8l + 7; warp 0 leaves the bins' offsets in sm.bin_off
+  int bstar, C;
   {
     unsigned int cnt[8], tot = 0;
 #pragma unroll
@@ -611,50 +647,50 @@ __device__ bool select_fast(const SelectArgs& a, int n, int M, int key_off, cons
       if (lane >= o) incl += t;
     }
     const unsigned int ballot = __ballot_sync(0xffffffffu, incl >= (unsigned)K_eff);
-    const int L = __ffs(ballot) - 1;      // exists: the bins hold M >= K_eff entries
-    int bl = 0;
-    if (lane == L) {
-      unsigned int run = incl - tot;
+    const int L = __ffs(ballot) - 1;      // exists: at least K_eff entries are binned
+    int bl = 0, cl = 0;
+    unsigned int run = incl - tot;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if (bl == 0 && run + cnt[j] >= (unsigned)K_eff) bl = 8 * lane + j + 1;
-        run += cnt[j];
+    for (int j = 0; j < 8; ++j) {
+      if (warp == 0) sm.bin_off[8 * lane + j] = run;
+      run += cnt[j];
+      if (bl == 0 && run >= (unsigned)K_eff) {
+        bl = 8 * lane + j + 1;
+        cl = (int)run;
       }
     }
     bstar = __shfl_sync(0xffffffffu, bl, L) - 1;
+    C = __shfl_sync(0xffffffffu, cl, L);
   }
-  // ---- candidates: the entries of bins <= b*, one atomic per warp ----------
-  {
-    unsigned int bal[PT];
-    int wtot = 0;
-#pragma unroll
-    for (int j = 0; j < PT; ++j) {
-      bal[j] = __ballot_sync(0xffffffffu, bin[j] <= bstar);
-      wtot += __popc(bal[j]);
-    }
-    int slot = 0;
-    if (lane == 0 && wtot > 0) slot = atomicAdd(&sm.sh_cnt_gt, wtot);
-    slot = __shfl_sync(0xffffffffu, slot, 0);
-    const unsigned int below = (1u << lane) - 1u;
-#pragma unroll
-    for (int j = 0; j < PT; ++j) {
-      if (bin[j] <= bstar) {
-        const int sj = slot + __popc(bal[j] & below);
-        if (sj < kFastMaxCand)
-          sm.cand[sj] = ((unsigned long long)ord_key(v[j]) << 32) |
-                        (0xFFFFFFFFu - (uint32_t)(tid + j * kSelThreads));
-      }
-      slot += __popc(bal[j]);
-    }
-  }
-  sync();                                                     // (3)
-  const int C = sm.sh_cnt_gt;
   if (C > kFastMaxCand) return false;                         // uniform
-  select_tail(a, n, key_off, s_sc, K_eff, C, smax, sumexp, sm, tid, sync);
+  sync();                                                     // (3)
+  // ---- candidates into bin order -------------------------------------------
+#pragma unroll
+  for (int j = 0; j < PT; ++j) {
+    if (tid + j * kSelThreads < M && !(v[j] < floor_s)) {
+      const int b = bin_of(v[j]);
+      if (b <= bstar)
+        sm.cand[atomicAdd(&sm.bin_off[b], 1u)] = ((unsigned long long)ord_key(v[j]) << 32) |
+                                                 (0xFFFFFFFFu - (uint32_t)(tid + j * kSelThreads));
+    }
+  }
+  sync();                                                     // (4)
+  // bin_off[b] is now the end of bin b, and the start of bin b + 1
+  for (int c = tid; c < C; c += kSelThreads) {
+    const unsigned long long me = sm.cand[c];
+    const int b = bin_of(key_score(me));
+    const int beg = b ? (int)sm.bin_off[b - 1] : 0, end = (int)sm.bin_off[b];
+    int r = beg;
+    for (int i = beg; i < end; ++i) r += sm.cand[i] > me;
+    if (r < K_eff) sm.sorted[r] = me;
+  }
+  sync();                                                     // (5)
+  select_mass<Sync::kLarge>(a, n, key_off, K_eff, smax, sumexp, sm, tid, sync);
   return true;
 }
 
-// Wide path: the fast path's steps for rows of more than kFastMaxM entries, the scores read from shared memory in strided passes
+// Wide path: the fast path's steps for rows of more than kLongMaxM entries, the
+// scores read from shared memory (s_sc, staged and visible) in strided passes
 // instead of registers and the distance to the maximum binned into kWideBins
 // bins (the histogram occupies sm.cum, which the mass scan only writes after
 // it is dead): (1) maximum and minimum; (2) softmax denominator (each
@@ -755,24 +791,29 @@ __device__ bool select_wide(const SelectArgs& a, int n, int M, int key_off, cons
   sync();                                                     // (5)
   const int C = sm.sh_cnt_gt;
   if (C > kFastMaxCand) return false;                         // uniform
-  select_tail(a, n, key_off, s_sc, K_eff, C, smax, sumexp, sm, tid, sync);
+  select_tail(a, n, key_off, K_eff, C, smax, sumexp, sm, tid, sync);
   return true;
 }
 
-// Selection of draft state n from its staged scores (s_sc, M >= 1 entries,
-// staged and visible to the group): the fast or wide path where it applies,
-// else the radix path.
+// The radix path, from the row's scores in global or shared memory.
 template <class Sync>
-__device__ __forceinline__ void select_row(const SelectArgs& a, int n, int M, int key_off,
-                                           const float* s_sc, SelectSmem& sm, int tid, Sync sync) {
-  if (M <= kFastMaxM ? select_fast(a, n, M, key_off, s_sc, sm, tid, sync)
-                     : select_wide(a, n, M, key_off, s_sc, sm, tid, sync))
-    return;
+__device__ __forceinline__ void select_radix(const SelectArgs& a, int n, int M, int key_off,
+                                             const float* s_sc, SelectSmem& sm, int tid, Sync sync) {
   float lmax = -INFINITY, lsum = 0.0f;
-  for (int i = tid; i < M; i += kSelThreads) combine_ms(lmax, lsum, s_sc[i], 1.0f);
+  for (int i = tid; i < M; i += kSelThreads) combine_ms(lmax, lsum, norm_score(s_sc[i]), 1.0f);
   float smax, sumexp;
   select_stats(lmax, lsum, sm, tid, sync, smax, sumexp);
   select_finish(a, n, M, key_off, s_sc, smax, sumexp, sm, tid, sync);
+}
+
+// Selection of draft state n from its M (1 .. 256 PT) scores in global memory:
+// the fast path, else the radix path.
+template <int PT, class Sync>
+__device__ __forceinline__ void select_row(const SelectArgs& a, int n, int M, int key_off,
+                                           const float* src, SelectSmem& sm, int tid, Sync sync) {
+  float v[PT];
+  load_scores(src, M, tid, v);
+  if (!select_fast(a, n, M, key_off, v, sm, tid, sync)) select_radix(a, n, M, key_off, src, sm, tid, sync);
 }
 
 // Outputs of a draft state whose sequence has no valid entry: K = 0.

@@ -237,6 +237,30 @@ def test_fusion_h_groups_in_the_score_launch(fovea, d, m_sizes, rows, H):
     compare(gpu, orc, s, mem=mem)
 
 
+# rows at the edges of 8, 16 and 32 scores per thread in registers and of the
+# staged path beyond, one below and at 256 entries (the floor from the threads'
+# maxima); with three distinct tokens more than 1024 candidates tie, and the
+# radix path takes them
+@pytest.mark.parametrize("M", [255, 256, 2048, 2049, 4096, 4097, 8191, 8192, 8193])
+@pytest.mark.parametrize("k", [40, 300])
+@pytest.mark.parametrize("ties", [False, True])
+def test_selection_row_lengths(fovea, M, k, ties):
+    """K fixed (k_min = k_max): the selected lists are the oracle's.  Equal
+    tokens have equal keys and scores, so ties go by position, exactly."""
+    k = min(k, M)
+    w = workloads.generate_custom("rows", 64, [M, 5], [3, 2], k_max=k, k_min=k, seed=M + k, H=128)
+    if ties:
+        w.v[0] = w.v[0, np.random.default_rng(M).integers(0, 3, M)]
+    s = store(w)
+    gpu = run_gpu(s, fovea)
+    orc, mem = run_oracle(s, mirror=True)
+    if ties:
+        np.testing.assert_array_equal(gpu["indices"][:, :k], orc["indices"][:, :k])
+        np.testing.assert_array_equal(gpu["counts"], orc["counts"])
+    else:
+        compare(gpu, orc, s, mem=mem)
+
+
 def test_plain_fusion_when_weights_differ(fovea):
     """The memory keeps the values projected through the r-half of the first
     fusion layer for the W_f1 / W_g1 it was built with.  A bf16 call given
