@@ -127,9 +127,8 @@ static __device__ __noinline__ bool wait_cluster(uint64_t* bar, uint32_t parity,
                                                  volatile int* abort_flag, uint64_t limit_ns) {
   if (try_wait_cluster(bar, parity)) return true;
   const uint64_t t0 = globaltimer_ns();
-  while (true) {
-    for (int i = 0; i < 64; ++i)
-      if (try_wait_cluster(bar, parity)) return true;
+  while (true) {                            // (a try suspends the thread for a while by itself)
+    if (try_wait_cluster(bar, parity)) return true;
     if (abort_flag != nullptr && *abort_flag) return false;
     if (globaltimer_ns() - t0 > limit_ns) return false;
   }
@@ -268,9 +267,12 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
           *abort_flag = 1;
           break;
         }
-  } else if (warp == 1 && lane == 0 && rank == 0) {
-    // ---- MMA issuer of the pair ----
-    int i = 0, c = 0;
+  } else if (warp == 1 && rank == 0) {
+    // ---- MMA issuer of the pair: the warp runs the loop converged (stage
+    // addresses and descriptors in uniform registers), one elected lane issues
+    const uint64_t desc0 = sw128_desc(smem_u32(smem));
+    uint32_t st = 0, ph = 0;
+    int c = 0;
     bool go = true;
     for (int t = pid; go && t < tiles; t += pairs) {
       const int chunk = KEYS && tile_at(a, t).part == 0 ? kChunkSu : su_total;
@@ -278,33 +280,41 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
         const int buf = c & 1;
         const uint32_t d = tmem_base + (uint32_t)(buf * BN);
         if (c >= 2 &&
-            !wait_cluster(&tempty[buf], ((uint32_t)(c >> 1) & 1u) ^ 1u, abort_flag, a.wait_ns)) {
+            !__all_sync(0xffffffffu, wait_cluster(&tempty[buf], ((uint32_t)(c >> 1) & 1u) ^ 1u,
+                                                  abort_flag, a.wait_ns))) {
           *abort_flag = 1;
           go = false;
           break;
         }
         tc_fence_after();
         const int su1 = min(su0 + chunk, su_total);
-        for (int su = su0; su < su1; ++su, ++i) {
-          const int st = i % kStages;
-          if (!wait_cluster(&full[st], (uint32_t)(i / kStages) & 1u, abort_flag, a.wait_ns)) {
+        for (int su = su0; su < su1; ++su) {
+          if (!__all_sync(0xffffffffu, wait_cluster(&full[st], ph, abort_flag, a.wait_ns))) {
             *abort_flag = 1;
             go = false;
             break;
           }
-          const uint32_t stg = smem_u32(smem + st * kStageBytes);
+          if (elect_one()) {
+            // descriptor start addresses are in units of 16 bytes
+            const uint64_t ad = desc0 + (uint64_t)(st * (uint32_t)(kStageBytes >> 4));
+            const uint64_t bd = ad + (uint64_t)((KPS * kSmemRows) >> 4);
 #pragma unroll
-          for (int j = 0; j < KPS; ++j) {
-            const uint64_t ad = sw128_desc(stg + (uint32_t)(j * kSmemRows));
-            const uint64_t bd = sw128_desc(stg + (uint32_t)(KPS * kSmemRows + j * kSmemFeat));
+            for (int j = 0; j < KPS; ++j)
 #pragma unroll
-            for (int k = 0; k < 4; ++k)          // 32 bytes (16 elements) per MMA
-              umma_pair(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k),
-                        (su > su0 || j > 0 || k > 0) ? 1u : 0u);
+              for (int k = 0; k < 4; ++k)          // 32 bytes (16 elements) per MMA
+                umma_pair(d, ad + (uint64_t)((j * kSmemRows >> 4) + 2 * k),
+                          bd + (uint64_t)((j * kSmemFeat >> 4) + 2 * k),
+                          (su > su0 || j > 0 || k > 0) ? 1u : 0u);
+            commit_pair(&empty[st]);
           }
-          commit_pair(&empty[st]);
+          __syncwarp();
+          if (++st == (uint32_t)kStages) {
+            st = 0;
+            ph ^= 1u;
+          }
         }
-        if (go) commit_pair(&tfull[buf]);
+        if (go && elect_one()) commit_pair(&tfull[buf]);
+        __syncwarp();
       }
     }
   } else if (warp >= 2) {
@@ -433,7 +443,7 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
   const bool aborted = *abort_flag != 0 || ld_dsmem_u32(map_dsmem(mine, rank ^ 1u)) != 0u;
   if (aborted) {
     if (threadIdx.x == 0) atomicOr(a.err, kErrTimeout);
-    if (rank == 0 && warp == 1 && lane == 0) commit_pair(drain);   // the issuing thread's MMAs
+    if (rank == 0 && warp == 1 && elect_one()) commit_pair(drain);   // the issuing lane's MMAs
     if (lane == 0) {
       wait_cluster(drain, 0, nullptr, kDefaultWaitLimitNs);
       const uint64_t t0 = globaltimer_ns();          // copies in flight land
