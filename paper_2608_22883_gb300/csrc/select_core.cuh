@@ -70,14 +70,15 @@ __device__ __forceinline__ void put_alpha(const SelectArgs& a, int n, int pos, f
   a.alpha_lo[o] = __float2bfloat16_rn(w - __bfloat162float(hi));
 }
 
-// Zero-fills row n of the dense weights (group of `nthreads`, index tid).
+// Zero-fills row n of the dense weights (group of `nthreads`, index tid; alpha_ld
+// is a multiple of 64), 16 bytes per store: a long row is 32 KB.
 __device__ __forceinline__ void clear_alpha(const SelectArgs& a, int n, int tid, int nthreads) {
   if (a.alpha_hi == nullptr) return;
-  const long long o = (long long)n * a.alpha_ld;
-  const __nv_bfloat16 z = __float2bfloat16_rn(0.0f);
-  for (int j = tid; j < a.alpha_ld; j += nthreads) {
-    a.alpha_hi[o + j] = z;
-    a.alpha_lo[o + j] = z;
+  uint4* hi = reinterpret_cast<uint4*>(a.alpha_hi + (long long)n * a.alpha_ld);
+  uint4* lo = reinterpret_cast<uint4*>(a.alpha_lo + (long long)n * a.alpha_ld);
+  for (int j = tid; j < a.alpha_ld / 8; j += nthreads) {
+    hi[j] = make_uint4(0u, 0u, 0u, 0u);
+    lo[j] = make_uint4(0u, 0u, 0u, 0u);
   }
 }
 

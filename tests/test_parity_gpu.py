@@ -261,6 +261,26 @@ def test_selection_row_lengths(fovea, M, k, ties):
         compare(gpu, orc, s, mem=mem)
 
 
+# the weighted-sum GEMM over each image's own k-blocks (caps above 256 take the
+# dense weights): one entry, the edges of a k-block of 64 and of a stage of
+# four, no entry, a row tile that reaches into the next sequence's weights
+@pytest.mark.parametrize("m_sizes,rows,H", [([1, 64, 65, 0, 257], [3, 1, 5, 2, 9], 128),
+                                            ([256, 320, 63], [130, 7, 64], 512),
+                                            ([700], [2], 128)])
+def test_dense_weights_entry_edges(fovea, m_sizes, rows, H):
+    w = workloads.generate_custom("act", 128, m_sizes, rows, k_max=300, rho=0.97, seed=len(rows), H=H)
+    s = store(w)
+    fovea.timing_enable(True)
+    gpu = run_gpu(s, fovea)
+    names = set(fovea.timing_read())
+    fovea.timing_enable(False)
+    assert "act_gemm" in names
+    orc, mem = run_oracle(s, mirror=True)
+    # flat rows with K in the hundreds: one entry moves the mass by ~1e-3, so
+    # the 1e-4 band catches up to a quarter of them
+    compare(gpu, orc, s, mem=mem, max_exempt=0.35)
+
+
 def test_plain_fusion_when_weights_differ(fovea):
     """The memory keeps the values projected through the r-half of the first
     fusion layer for the W_f1 / W_g1 it was built with.  A bf16 call given
