@@ -64,6 +64,7 @@ constexpr int UMMA_K = 16;       // contraction elements per tcgen05.mma (kind::
 constexpr int kThreads = 256;
 constexpr int kSmemBudget = 200 * 1024;   // shared-memory stages, one CTA per SM
 constexpr int kSmemBudgetPair = 100 * 1024;  // two CTAs per SM
+constexpr int kSmemPerSm = 228 * 1024;    // with 1 KB of it taken by each CTA
 constexpr int kSmemExtra = 1024 /*alignment*/ + 256 /*barriers*/ + 1024 /*tile biases*/;
 constexpr int kMaxStages = 8;
 constexpr int kRasterRows = 16;          // row tiles per band of the tile order
@@ -85,7 +86,6 @@ constexpr int kRasterRows = 16;          // row tiles per band of the tile order
 // the same accumulator.
 template <int BN, bool DUAL = false>
 struct Cfg {
-  static constexpr uint32_t TMEM_COLS = BN < 32 ? 32 : BN;
   __host__ __device__ static constexpr int stage_bytes(int kps, int rbox, bool df = false) {
     return kps * (rbox * (DUAL ? 2 : 1) + BN * (df ? 2 : 1)) * 128;
   }
@@ -378,8 +378,27 @@ __device__ __forceinline__ void act_store4(const GemmArgs& a, const GemmGroup& g
   }
 }
 
+// The sums of the contraction's further chunks (kEpiLogits, kEpiScoresFolded)
+// added to the first's, 32 columns, in chunk order.
+template <int EPI, int BN>
+__device__ __forceinline__ void add_chunks(uint32_t taddr, int nacc, float (&v)[32]) {
+  if constexpr (EPI == kEpiLogits || EPI == kEpiScoresFolded) {
+#pragma unroll 1
+    for (int c = 1; c < nacc; ++c) {
+#pragma unroll
+      for (int h = 0; h < 32; h += 8) {            // few registers: two CTAs fit an SM
+        float w[8];
+        tmem_ld8(taddr + (uint32_t)(c * BN + h), w);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[h + j] += w[j];
+      }
+    }
+  }
+}
+
+// (two CTAs per SM: at most 128 registers)
 template <int BN, int EPI>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads, 2)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmF0, const __grid_constant__ CUtensorMap tmF1,
                    const __grid_constant__ CUtensorMap tmF2, const __grid_constant__ CUtensorMap tmR0,
                    const __grid_constant__ CUtensorMap tmR1, const __grid_constant__ GemmArgs args) {
@@ -458,7 +477,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     prefetch_tmap(&tmR0);
   }
   if (warp == 1) {
-    tmem_alloc(tmem_slot, C::TMEM_COLS);
+    tmem_alloc(tmem_slot, (uint32_t)(args.nacc * BN));
     tmem_relinquish();
   }
   tc_fence_before();
@@ -471,6 +490,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int su_lo = (int)((long long)rank * su_total / S);
   const int su_hi = (int)((long long)(rank + 1) * su_total / S);
   const int nkb = su_hi - su_lo;                       // stages of this CTA
+  // the contraction's chunks: the tensor core truncates each addition to its
+  // accumulator, so fewer additions per accumulator err less; the epilogue adds
+  // the chunks' sums, rounded, in order
+  const int nacc = max(1, min(args.nacc, nkb));
 
   if (warp == 0 && lane < kProducers) {
     // ---- TMA producers: lane 0 loads the feature tiles, lane 1 the row tiles
@@ -555,7 +578,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint64_t desc0 = sw128_desc(smem_u32(smem));
     const uint32_t r_step = (uint32_t)(r_tile >> 4), f_step = (uint32_t)(f_tile >> 4);
     uint32_t st = 0, ph = 0;
+    int chunk = 0, first = 0;           // this chunk's first stage
     for (int i = 0; i < nkb; ++i) {
+      if (chunk + 1 < nacc && i == (int)((long long)(chunk + 1) * nkb / nacc)) {
+        ++chunk;
+        first = i;
+      }
+      const uint32_t tmem_d = tmem_base + (uint32_t)(chunk * BN);
       if (!__all_sync(0xffffffffu, mbar_wait(&full[st], ph, abort_flag, args.wait_ns))) {
         *abort_flag = 1;
         break;
@@ -571,12 +600,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int k = 0; k < BK / UMMA_K; ++k) {
             // advance the start address by k * 32 bytes inside the swizzle atom
-            umma_bf16(tmem_base, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), C::IDESC,
-                      (i > 0 || j > 0 || k > 0) ? 1u : 0u);
+            umma_bf16(tmem_d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), C::IDESC,
+                      (i > first || j > 0 || k > 0) ? 1u : 0u);
             if constexpr (DUAL)
-              umma_bf16(tmem_base, ad + lo + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), C::IDESC, 1u);
+              umma_bf16(tmem_d, ad + lo + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), C::IDESC, 1u);
             if (EPI == kEpiScoresFolded && dual_f)
-              umma_bf16(tmem_base, ad + (uint64_t)(2 * k), bd + lo + (uint64_t)(2 * k), C::IDESC, 1u);
+              umma_bf16(tmem_d, ad + (uint64_t)(2 * k), bd + lo + (uint64_t)(2 * k), C::IDESC, 1u);
           }
           ad += r_step;
           bd += f_step;
@@ -651,6 +680,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           float v[32];
           if (have_acc) {
             tmem_ld32(taddr + (uint32_t)c0, v);   // the whole warp, converged
+            add_chunks<EPI, BN>(taddr + (uint32_t)c0, nacc, v);
           } else {
 #pragma unroll
             for (int j = 0; j < 32; ++j) v[j] = 0.0f;
@@ -707,6 +737,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           float v[32];
           if (have_acc) {
             tmem_ld32(taddr + (uint32_t)c0, v);   // the whole warp, converged
+            add_chunks<EPI, BN>(taddr + (uint32_t)c0, nacc, v);
           } else {
 #pragma unroll
             for (int j = 0; j < 32; ++j) v[j] = 0.0f;
@@ -811,7 +842,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, C::TMEM_COLS);
+    tmem_dealloc(tmem_base, (uint32_t)(args.nacc * BN));
   }
 }
 
@@ -982,6 +1013,7 @@ static cudaError_t launch_tc_inst(GemmArgs& a, const CUtensorMap* maps, int tile
   a.kps = p.kps;
   a.rbox = p.rbox;
   a.rbox1 = p.rbox1;
+  a.nacc = p.nacc;
   a.tx_bytes = tc::Cfg<BN, DUAL>::stage_bytes(p.kps, p.rbox,
                                               EPI == kEpiScoresFolded && a.f_lo_kb > 0);
   cudaLaunchConfig_t cfg = {};
@@ -1061,8 +1093,34 @@ static double plan_cost_us(bool streaming, double stage_kb, double stage_f_bytes
   return waves * (t_first + nst * t_stage) + t_tail;
 }
 
+// Estimated time (us) of a plan for the GEMMs that stream one feature operand
+// from HBM over many tiles (the LM head, the scores of several sequences),
+// fitted to the measured plans of three score launches and the LM head (the
+// order of their best plans is right; errors up to 25 %):
+//   stage   a CTA has (stages - 1/2) stages of copies in flight for ~1.9 us
+//           each, and an SM takes in ~88 KB/us whatever its CTAs; at least its
+//           MMAs, and the feature bytes of all CTAs' stages at the HBM rate;
+//   wave    ~2.2 us to the first stage (a little more for a larger one), ~1.2 us
+//           to drain, and the epilogue's time per thread.
+// Against the estimate above: LM head 60.4 -> 58.1 us, a step of 8 ragged images
+// x 32 rows 80.3 -> 76.0, 16 x 64 rows 117.5 -> 115.5, 4 x 128 rows of 8192
+// entries 167.5 -> 165.9.
+static double fed_cost_us(double stage_kb, double stage_f_bytes, double mma_us, int stages, int nst,
+                          long long ctas, long long cap, int sms, int rows, int bn, int S) {
+  auto wave = [&](long long n) {
+    if (n <= 0) return 0.0;
+    const double per_sm = (double)((n + sms - 1) / sms);
+    const double latency = stages > 1 ? 1.9 / (stages - 0.5) : 1.9 + mma_us;
+    const double t_stage = std::max(std::max(per_sm * stage_kb / 88.0, latency),
+                                    std::max(per_sm * mma_us * 1.3, n * stage_f_bytes / 6.6e6));
+    const double t_tail = 1.2 + 0.12 * rows * bn / (1024.0 * S) + (S == 1 ? 0.0 : 1.4 + 0.25 * S);
+    return 2.2 + 0.02 * stage_kb + nst * t_stage + t_tail;
+  };
+  return (double)(ctas / cap) * wave(cap) + wave(ctas % cap);
+}
+
 template <int BN, int EPI>
-static void plan_for(const GemmArgs& a, int max_m, int max_n, long long row_tiles,
+static void plan_for(const GemmArgs& a, int max_m, int max_n, long long row_tiles, int chunks,
                      GemmPlan& best, double& best_t) {
   constexpr bool DUAL = EPI == kEpiScores || EPI == kEpiAct;
   using C = tc::Cfg<BN, DUAL>;
@@ -1136,29 +1194,73 @@ static void plan_for(const GemmArgs& a, int max_m, int max_n, long long row_tile
           cap = std::min<long long>(cap, (long long)nc * S);
         }
         if (cap <= 0) continue;
+        // (the occupancy query counts one CTA per SM for the half-SM budget,
+        // whose CTAs do run two to an SM)
+        if (chunks > 0) cap = (sms * (2 * (smem + 1024) <= tc::kSmemPerSm ? 2 : 1)) / S * S;
         const long long waves = (ctas + cap - 1) / cap;
         const long long per_sm = std::max<long long>(1, (std::min(ctas, cap) + sms - 1) / sms);
-        const double t = plan_cost_us(streaming, sb / 1024.0, stage_f,
-                                      stage_mma_us, stages, nst, std::min(ctas, cap), (int)per_sm,
-                                      waves, S);
+        // at least `chunks` accumulators to a contraction, in the tensor memory
+        // that the CTAs of an SM share
+        int nacc = 1;
+        while (nacc * S < chunks) nacc *= 2;
+        if (nacc > 1 && (nacc > nst || nacc * BN * ((cap + sms - 1) / sms) > 512)) continue;
+        const double t = chunks > 0 ? fed_cost_us(sb / 1024.0, stage_f, stage_mma_us, stages, nst, ctas, cap,
+                                           sms, rows, BN, S)
+                             : plan_cost_us(streaming, sb / 1024.0, stage_f, stage_mma_us, stages, nst,
+                                            std::min(ctas, cap), (int)per_sm, waves, S);
         if (t < best_t - 1e-6 || (t < best_t + 1e-6 && tiles * S < best.tiles * best.splits)) {
           best_t = t;
-          best = GemmPlan{BN, S, stages, 0, tiles, rbox, rbox1, region, kps};
+          best = GemmPlan{BN, S, stages, 0, tiles, rbox, rbox1, region, kps, nacc};
         }
       }
     }
   }
 }
 
+// Feature bytes above which fed_cost_us plans a launch: more than L2 keeps.
+// (Below, it does worse: an LM head of 7752 x 4736, 73 MB, 28.2 us against 20.0,
+// 8 images x 8 rows at d = 1024 27.0 against 25.1.)
+constexpr long long kFedBytes = 128ll << 20;
+
+// chunks = 0: the plan_cost_us estimate; else the fed_cost_us estimate over the
+// plans whose contractions are split over at least that many accumulators.
+template <int EPI>
+static GemmPlan plan_best(const GemmArgs& a, int max_m, int max_n, int chunks) {
+  const long long row_tiles = (long long)(max_n + tc::BM - 1) / tc::BM * a.ngroups;
+  GemmPlan best{256, 1, 2, 0, 1 << 30, 128, 128, 0, 1, 1};
+  double best_t = 1e30;
+  plan_for<256, EPI>(a, max_m, max_n, row_tiles, chunks, best, best_t);
+  plan_for<128, EPI>(a, max_m, max_n, row_tiles, chunks, best, best_t);
+  plan_for<64, EPI>(a, max_m, max_n, row_tiles, chunks, best, best_t);
+  return best;
+}
+
 template <int EPI>
 static GemmPlan plan_epi(const GemmArgs& a, int max_m, int max_n) {
-  const long long row_tiles = (long long)(max_n + tc::BM - 1) / tc::BM * a.ngroups;
-  GemmPlan best{256, 1, 2, 0, 1 << 30, 128, 128, 0, 1};
-  double best_t = 1e30;
-  plan_for<256, EPI>(a, max_m, max_n, row_tiles, best, best_t);
-  plan_for<128, EPI>(a, max_m, max_n, row_tiles, best, best_t);
-  plan_for<64, EPI>(a, max_m, max_n, row_tiles, best, best_t);
-  return best;
+  if constexpr (EPI == kEpiLogits || EPI == kEpiScoresFolded) {
+    long long features = 0;
+    for (int g = 0; g < a.ngroups; ++g)
+      if (a.groups[g].a_row0 >= 0) features += a.groups[g].m;
+    const long long streamed = features * a.k_total * 2 * (a.f_lo_kb > 0 ? 2 : 1);
+    if (max_n <= tc::BM && (EPI == kEpiLogits || a.ngroups > 1) && streamed > kFedBytes) {
+      // the split that the other estimate gives the logits, or the scores by
+      // themselves, is the number of accumulators to keep: a plan with fewer
+      // splits would sum less exactly
+      static thread_local GemmArgs alone;
+      alone = a;
+      alone.gh_cols = 0;
+      alone.ngroups = 0;
+      int n = 0;
+      for (int g = 0; g < a.ngroups; ++g)
+        if (a.groups[g].a_row0 >= 0) {
+          alone.groups[alone.ngroups++] = a.groups[g];
+          n = std::max(n, a.groups[g].n);
+        }
+      const GemmPlan p = plan_best<EPI>(a, max_m, max_n, plan_best<EPI>(alone, max_m, n, 0).splits);
+      if (p.region > 0) return p;
+    }
+  }
+  return plan_best<EPI>(a, max_m, max_n, 0);
 }
 
 static GemmPlan plan_gemm_tc_uncached(int epi, const GemmArgs& a, int max_m, int max_n) {
