@@ -122,6 +122,8 @@ def kernel_bytes(name: str, w: workloads.Workload, uniq_values: int, projected: 
         return uniq_values * d * es + N * d * (4 + es)
     if name == "select_fuse":     # scores in; projected rows, G_h, biases in; activations out
         return scores + uniq_values * 2 * H * es + 4 * N * 2 * H + es * (2 * H + N * 2 * H) + N * 4 + N * w.k_max * 4
+    if name == "gather_fuse":     # the selection, projected rows, G_h, biases in; activations out
+        return uniq_values * 2 * H * es + 4 * N * 2 * H + es * (2 * H + N * 2 * H) + N * 4 + 2 * N * w.k_max * 4
     if name == "select_readout":
         return scores + uniq_values * d * es + N * d * (4 + es) + N * 4 + N * w.k_max * 4
     if name == "select":
@@ -538,7 +540,7 @@ def main():
     # ---- roofline ----
     c_np, i_np = counts.cpu().numpy(), indices.cpu().numpy()
     dense = "act_gemm" in per_kernel
-    projected = "select_fuse" in per_kernel or dense
+    projected = "select_fuse" in per_kernel or "gather_fuse" in per_kernel or dense
     folded = "score_folded" in per_kernel or "score_fusion_h" in per_kernel
     # the method's algorithmic bytes (full fusion weights, value rows), and
     # what this path's step moves (projected values: the h-half weights and

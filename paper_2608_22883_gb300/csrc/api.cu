@@ -140,6 +140,15 @@ struct fovea_memory {
   const void* fold_wq = nullptr;
 };
 
+// Caps up to this select and gather in one kernel (two CTAs a row at most);
+// above it the gathers have a kernel of their own over the whole GPU.  Step of
+// 64 rows, d = 4096, one kernel against two: K = 128 27.6 / 25.9 us, K = 256
+// 31.3 / 28.5, with the readout 42.5 / 38.3; the paper's setting behind its
+// depth gate 43.9 / 30.9.  At K = 64 two kernels are 0.7 us faster on the GPU
+// (25.6 / 24.9), less than the host pays for a launch, so that line holds up to
+// a row per SM; 300 rows without a readout gain 46.0 / 40.7.
+constexpr int kFuseSelectMaxK = 64;
+
 static size_t esize(int dtype) { return dtype == FOVEA_BF16 ? 2 : 4; }
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -774,9 +783,9 @@ FOVEA_API fovea_status fovea_retrieve_fuse(const fovea_params* p, const fovea_me
   // G_h alone (or is skipped without the projected values).
   const bool bf = dt == FOVEA_BF16;
   // The r-half of the first fusion layer from the projected values: either
-  // gathered row by row in the selection kernel (rows of <= 2048 entries,
-  // k_max <= 256, a batch that fills the GPU in about a wave), or, with the
-  // selection weights written as dense rows, one GEMM against the memory's
+  // gathered row by row, in the selection kernel or in a kernel after it (rows
+  // of <= 2048 entries, k_max <= 256, a batch that fills the GPU in about a
+  // wave), or, with the selection weights written as dense rows, one GEMM against the memory's
   // transposed projected values (long rows, large caps, large batches).
   const bool have_proj = bf && mem->proj != nullptr && mem->proj_wf1 == p->W_f1 &&
                          mem->proj_wg1 == p->W_g1 && mem->proj_h == H;
@@ -965,7 +974,8 @@ FOVEA_API fovea_status fovea_retrieve_fuse(const fovea_params* p, const fovea_me
     if (e != cudaSuccess) return cuda_fail(e, "select");
     if (readout != nullptr) {
       { KernelTimer t("readout", s);
-        e = launch_readout(dt, mem->values, sel_cnt, sel_pos, sel_w, N, k_max, d, readout, r_lo, s); }
+        e = launch_readout(dt, RowGather{sel_cnt, sel_pos, sel_w, k_max, mem->values, d, readout, nullptr},
+                           N, s); }
       if (e != cudaSuccess) return cuda_fail(e, "readout");
     }
     // [a_f | a_g] = SiLU(G_h + alpha P + [b_f1 | b_g1]): per image, the
@@ -993,6 +1003,16 @@ FOVEA_API fovea_status fovea_retrieve_fuse(const fovea_params* p, const fovea_me
                          TmaOperand{nullptr, 0, 0, 0}, TmaOperand{alpha_hi, N, mem->proj_ld, mem->proj_ld},
                          TmaOperand{alpha_lo, N, mem->proj_ld, mem->proj_ld}, 2 * H, max_rows, s); }
     if (e != cudaSuccess) return cuda_fail(e, "act_gemm");
+  } else if (use_proj && (k_max > kFuseSelectMaxK || (N > device_sms() && readout == nullptr))) {
+    { KernelTimer t("select", s);
+      e = launch_select(scores, tab, N, mem->orig_index, rho, k_min, k_max, max_m, gate_rows,
+                        counts, indices, sel_pos, sel_w, sel_cnt, s); }
+    if (e != cudaSuccess) return cuda_fail(e, "select");
+    { KernelTimer t("gather_fuse", s);
+      e = launch_readout(dt, RowGather{sel_cnt, sel_pos, sel_w, k_max,
+                                       readout != nullptr ? mem->values : nullptr, d, readout,
+                                       nullptr, mem->proj, H, gh, p->b_f1, p->b_g1, act}, N, s); }
+    if (e != cudaSuccess) return cuda_fail(e, "gather_fuse");
   } else if (use_proj) {
     { KernelTimer t("select_fuse", s);
       e = launch_select_gather(dt, scores, tab, N, mem->orig_index, rho, k_min, k_max, max_m,
@@ -1013,7 +1033,8 @@ FOVEA_API fovea_status fovea_retrieve_fuse(const fovea_params* p, const fovea_me
                           counts, indices, sel_pos, sel_w, sel_cnt, s); }
       if (e != cudaSuccess) return cuda_fail(e, "select");
       { KernelTimer t("readout", s);
-        e = launch_readout(dt, mem->values, sel_cnt, sel_pos, sel_w, N, k_max, d, readout, r_lo, s); }
+        e = launch_readout(dt, RowGather{sel_cnt, sel_pos, sel_w, k_max, mem->values, d, readout, r_lo},
+                           N, s); }
       if (e != cudaSuccess) return cuda_fail(e, "readout");
     }
 

@@ -265,9 +265,22 @@ cudaError_t launch_select(const float* scores, const SeqTable& tab, int N, const
                           int32_t* counts, int32_t* indices, int32_t* sel_pos, float* sel_w,
                           int32_t* sel_cnt, cudaStream_t s, void* alpha_hi = nullptr,
                           void* alpha_lo = nullptr, int alpha_ld = 0);
-cudaError_t launch_readout(int dtype, const void* U, const int32_t* sel_cnt, const int32_t* sel_pos,
-                           const float* sel_w, int N, int k_max, int d, float* r_out, void* r_lo,
-                           cudaStream_t s);
+// The gathers of a selection (rowops.cu): the readout of U (null: none) to
+// r_out (fp32) and / or r_lo, and, when P is given, act = SiLU(Gh + sum_t
+// alpha_t P[pi(t)] + [b_f1 ; b_g1]) over 2H columns.
+struct RowGather {
+  const int32_t* sel_cnt;          // [N]
+  const int32_t* sel_pos;          // [N, k_max]
+  const float* sel_w;              // [N, k_max]
+  int k_max;
+  const void* U; int d;            // [rows, d]
+  float* r_out; void* r_lo;        // [N, d], either may be null
+  const void* P; int H;            // [rows, 2H]
+  const float* Gh;                 // [N, 2H]
+  const void* b_f1; const void* b_g1;
+  void* act;                       // [N, 2H]
+};
+cudaError_t launch_readout(int dtype, const RowGather& a, int N, cudaStream_t s);
 // Selection fused with the gathers that consume it (select.cu), for rows of
 // at most 2048 valid entries and k_max <= 256 (select_readout_fits): the
 // readout r (r_out fp32 and / or r_lo, either may be null; U unused when

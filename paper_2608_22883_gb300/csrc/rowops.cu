@@ -511,16 +511,20 @@ cudaError_t launch_compact(const uint8_t* mask, int B, int M_max, const ImageTab
 }
 
 // ---------------------------------------------------------------------------
-// Readout r_n = sum_{t < K} alpha_t u_{pi(t)} (the alpha / r_n equation).
-// Grid (N rows, column chunks of 64 x vector width); 8 warps per CTA split the
-// selected entries (warp w takes t = w, w + 8, ...), each lane owns one
-// 16-byte vector of columns and keeps several gathers in flight; the warps'
-// partial sums are combined in warp order (fixed order, fp32).  The weights
-// were renormalised over I_n by the select kernel.
+// The gathers of a selection made by select_kernel (sel_cnt, sel_pos, sel_w):
+// the readout r_n = sum_{t < K} alpha_t u_{pi(t)} (the alpha / r_n equation)
+// and, in bf16 with the projected values, the first fusion layer
+// SiLU(G_h + sum alpha_t p_{pi(t)} + [b_f1 ; b_g1]).
+// Grid (N rows, chunks of 32 x vector width columns: those of P first, then
+// those of U); 8 warps per CTA split the selected entries (warp w takes t = w,
+// w + 8, ...), each lane owns one 16-byte vector of columns and keeps eight
+// gathers in flight; the warps' partial sums are combined in warp order (fixed
+// order, fp32).  Bound by the latency of its gathers out of L2: a row's work
+// spreads over up to 20 CTAs, where the selection + gather kernel has two.
 // ---------------------------------------------------------------------------
 constexpr int kReadoutWarps = 8;
 constexpr int kReadoutThreads = 32 * kReadoutWarps;
-constexpr int kReadoutUnroll = 4;
+constexpr int kReadoutUnroll = 8;
 
 template <class T>
 struct Vec16;
@@ -528,64 +532,46 @@ template <> struct Vec16<__nv_bfloat16> { static constexpr int N = 8; };
 template <> struct Vec16<float> { static constexpr int N = 4; };
 
 template <class T>
-__device__ __forceinline__ void load_vec(const T* p, float (&v)[Vec16<T>::N]);
-template <>
-__device__ __forceinline__ void load_vec<__nv_bfloat16>(const __nv_bfloat16* p, float (&v)[8]) {
-  const uint4 raw = __ldg(reinterpret_cast<const uint4*>(p));
-  const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&raw);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float2 f = __bfloat1622float2(h2[i]);
-    v[2 * i] = f.x;
-    v[2 * i + 1] = f.y;
-  }
-}
-template <>
-__device__ __forceinline__ void load_vec<float>(const float* p, float (&v)[4]) {
-  const float4 raw = __ldg(reinterpret_cast<const float4*>(p));
-  v[0] = raw.x; v[1] = raw.y; v[2] = raw.z; v[3] = raw.w;
-}
-
-template <class T>
-__global__ void __launch_bounds__(kReadoutThreads) readout_kernel(
-    const T* __restrict__ U, const int32_t* __restrict__ sel_cnt,
-    const int32_t* __restrict__ sel_pos, const float* __restrict__ sel_w, int k_max, int d,
-    float* __restrict__ r_out, T* __restrict__ r_lo) {
+__global__ void __launch_bounds__(kReadoutThreads, 4) readout_kernel(const __grid_constant__ RowGather a) {
   constexpr int V = Vec16<T>::N;
   __shared__ float part[kReadoutWarps][32 * V];
   const int n = blockIdx.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int col = (blockIdx.y * 32 + lane) * V;
+  const int p_chunks = a.P != nullptr ? (2 * a.H + 32 * V - 1) / (32 * V) : 0;
+  const bool proj = (int)blockIdx.y < p_chunks;
+  const int chunk = proj ? blockIdx.y : (int)blockIdx.y - p_chunks;
+  const int width = proj ? 2 * a.H : a.d;              // columns, and the row stride
+  const T* X = static_cast<const T*>(proj ? a.P : a.U);
+  const int col = (chunk * 32 + lane) * V;
   pdl_wait();
   pdl_trigger();
-  const int K = sel_cnt[n];
-  const int32_t* pos = sel_pos + (long long)n * k_max;
-  const float* w = sel_w + (long long)n * k_max;
+  const int K = a.sel_cnt[n];
+  const int32_t* pos = a.sel_pos + (long long)n * a.k_max;
+  const float* w = a.sel_w + (long long)n * a.k_max;
   float acc[V];
 #pragma unroll
   for (int i = 0; i < V; ++i) acc[i] = 0.0f;
-  if (col < d) {
-    int t = warp;
-    for (; t + (kReadoutUnroll - 1) * kReadoutWarps < K; t += kReadoutUnroll * kReadoutWarps) {
-      float u[kReadoutUnroll][V];
+  if (col < width) {
+    for (int t = warp; t < K; t += kReadoutUnroll * kReadoutWarps) {
+      uint4 raw[kReadoutUnroll];               // as loaded: few registers, more CTAs per SM
       float wt[kReadoutUnroll];
 #pragma unroll
       for (int j = 0; j < kReadoutUnroll; ++j) {
         const int tj = t + j * kReadoutWarps;
-        wt[j] = w[tj];
-        load_vec<T>(U + (long long)pos[tj] * d + col, u[j]);
+        wt[j] = 0.0f;
+        raw[j] = make_uint4(0u, 0u, 0u, 0u);
+        if (tj < K) {
+          wt[j] = w[tj];
+          raw[j] = __ldg(reinterpret_cast<const uint4*>(X + (long long)pos[tj] * width + col));
+        }
       }
 #pragma unroll
-      for (int j = 0; j < kReadoutUnroll; ++j)
+      for (int j = 0; j < kReadoutUnroll; ++j) {
+        float u[V];
+        ln_unpack<T>(raw[j], u);
 #pragma unroll
-        for (int i = 0; i < V; ++i) acc[i] = fmaf(wt[j], u[j][i], acc[i]);
-    }
-    for (; t < K; t += kReadoutWarps) {
-      float u[V];
-      load_vec<T>(U + (long long)pos[t] * d + col, u);
-      const float wt = w[t];
-#pragma unroll
-      for (int i = 0; i < V; ++i) acc[i] = fmaf(wt, u[i], acc[i]);
+        for (int i = 0; i < V; ++i) acc[i] = fmaf(wt[j], u[i], acc[i]);
+      }
     }
   }
 #pragma unroll
@@ -594,29 +580,33 @@ __global__ void __launch_bounds__(kReadoutThreads) readout_kernel(
   // combine the warps' partial sums in warp order; thread i of the CTA owns
   // element i of the chunk
   for (int e = threadIdx.x; e < 32 * V; e += kReadoutThreads) {
-    const int c = blockIdx.y * 32 * V + e;
-    if (c >= d) continue;
+    const int c = chunk * 32 * V + e;
+    if (c >= width) continue;
     float sum = 0.0f;
 #pragma unroll
     for (int wi = 0; wi < kReadoutWarps; ++wi) sum += part[wi][e];
-    if (r_out != nullptr) r_out[(long long)n * d + c] = sum;
-    r_lo[(long long)n * d + c] = from_f32<T>(sum);
+    const long long o = (long long)n * width + c;
+    if (proj) {
+      const float bias = to_f32(c < a.H ? static_cast<const T*>(a.b_f1)[c]
+                                        : static_cast<const T*>(a.b_g1)[c - a.H]);
+      const float z = sum + a.Gh[o] + bias;
+      static_cast<T*>(a.act)[o] = from_f32<T>(z * sigmoidf_(z));
+    } else {
+      if (a.r_out != nullptr) a.r_out[o] = sum;
+      if (a.r_lo != nullptr) static_cast<T*>(a.r_lo)[o] = from_f32<T>(sum);
+    }
   }
 }
 
-cudaError_t launch_readout(int dtype, const void* U, const int32_t* sel_cnt, const int32_t* sel_pos,
-                           const float* sel_w, int N, int k_max, int d, float* r_out, void* r_lo,
-                           cudaStream_t s) {
+cudaError_t launch_readout(int dtype, const RowGather& a, int N, cudaStream_t s) {
   if (N == 0) return cudaSuccess;
-  if (dtype == FOVEA_BF16) {
-    using T = __nv_bfloat16;
-    dim3 grid(N, (d / 8 + 31) / 32);
-    return launch_pdl(readout_kernel<T>, grid, dim3(kReadoutThreads), 0, s, (const T*)U, sel_cnt,
-                      sel_pos, sel_w, k_max, d, r_out, (T*)r_lo);
-  }
-  dim3 grid(N, (d / 4 + 31) / 32);
-  return launch_pdl(readout_kernel<float>, grid, dim3(kReadoutThreads), 0, s, (const float*)U,
-                    sel_cnt, sel_pos, sel_w, k_max, d, r_out, (float*)r_lo);
+  const int cols = 32 * (dtype == FOVEA_BF16 ? 8 : 4);
+  const int chunks = (a.P != nullptr ? (2 * a.H + cols - 1) / cols : 0) +
+                     (a.U != nullptr ? (a.d + cols - 1) / cols : 0);
+  const dim3 grid(N, chunks);
+  if (dtype == FOVEA_BF16)
+    return launch_pdl(readout_kernel<__nv_bfloat16>, grid, dim3(kReadoutThreads), 0, s, a);
+  return launch_pdl(readout_kernel<float>, grid, dim3(kReadoutThreads), 0, s, a);
 }
 
 // ---------------------------------------------------------------------------

@@ -281,6 +281,24 @@ def test_dense_weights_entry_edges(fovea, m_sizes, rows, H):
     compare(gpu, orc, s, mem=mem, max_exempt=0.35)
 
 
+# caps above 64, or more rows than SMs without a readout, gather in a kernel of
+# their own: fewer and more entries than its 8 warps x 8 loads, a partial
+# column chunk (2H = 256, d = 320), gated rows, empty images, K = 0
+@pytest.mark.parametrize("d,m_sizes,rows,k,H", [(320, [300, 0, 70], [9, 2, 3], 65, 128),
+                                                (256, [600], [7], 256, 512),
+                                                (256, [5, 130], [1, 8], 128, 256)])
+def test_gather_after_the_selection(fovea, d, m_sizes, rows, k, H):
+    w = workloads.generate_custom("gather", d, m_sizes, rows, k_max=k, k_min=min(k, 40), seed=k, H=H)
+    s = store(w)
+    fovea.timing_enable(True)
+    gpu = run_gpu(s, fovea, l_max=3)
+    names = set(fovea.timing_read())
+    fovea.timing_enable(False)
+    assert {"select", "gather_fuse"} <= names and "act_gemm" not in names
+    orc, mem = run_oracle(s, mirror=True, l_max=3)
+    compare(gpu, orc, s, mem=mem, max_exempt=0.2)
+
+
 def test_plain_fusion_when_weights_differ(fovea):
     """The memory keeps the values projected through the r-half of the first
     fusion layer for the W_f1 / W_g1 it was built with.  A bf16 call given
