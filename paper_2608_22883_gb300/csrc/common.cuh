@@ -52,13 +52,28 @@ template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(flo
   return __float2bfloat16_rn(x);
 }
 
-// Logistic sigmoid with the hardware exponential and a correctly rounded
-// reciprocal (a few fp32 ulps from the exact value, far below the bf16
-// rounding of the activations and the gate's tolerance; exp(-z) = inf for
-// z < -88 gives exactly 0, as the zero-gate reading needs).  The activation
-// epilogues evaluate it per element, where the full-precision expf and
-// division dominated their time.
+// Logistic sigmoid of the gate with the hardware exponential and a correctly
+// rounded reciprocal (exp(-z) = inf for z < -88 gives exactly 0, as the
+// zero-gate reading needs).
 __device__ __forceinline__ float sigmoidf_(float z) { return __frcp_rn(1.0f + __expf(-z)); }
+
+// SiLU z / (1 + exp(-z)) of the first fusion layer, evaluated per element in
+// the activation epilogues (z * sigmoidf_(z) took half of the weighted-sum
+// GEMM's epilogue: 2.2 of 4.6 us for a 64 x 128 tile).  exp(-z) = 2^t with t =
+// -z log2 e, its rounding error put back to first order, and one approximate
+// division.  Measured against float64 for z in [-86, 30]: mean error 0.73 x
+// 2^-24, largest 5.2 (z * sigmoidf_(z): 12.0 and 65; for |z| < 4 0.73 and 0.81).
+// The exponential's argument is held to [-88, 87]: below z = -87 SiLU is below
+// 1e-35 in size and stays there.
+__device__ __forceinline__ float siluf_(float z) {
+  constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
+  constexpr float kLog2eLo = (float)(1.4426950408889634 - (double)kLog2e);
+  const float zc = fminf(fmaxf(z, -87.0f), 88.0f);
+  const float t = -zc * kLog2e;
+  const float lo = fmaf(-zc, kLog2eLo, fmaf(-zc, kLog2e, -t));
+  const float e = exp2f(t);
+  return __fdividef(z, 1.0f + fmaf(e, lo * kLn2, e));
+}
 
 // Programmatic dependent launch: kernels of the step are launched so that a
 // kernel may start while its predecessor finishes.  pdl_wait() blocks until

@@ -29,7 +29,7 @@ __device__ __forceinline__ void gemm_epilogue(const GemmArgs& a, const GemmGroup
                                        : to_f32(static_cast<const T*>(a.bias1)[m - a.epi_split]);
     float z = acc + bias;
     if constexpr (EPI == kEpiAct) z += a.add_in[row * a.ldc2 + m];
-    static_cast<T*>(a.out0)[row * a.ldc + m] = from_f32<T>(z * sigmoidf_(z));
+    static_cast<T*>(a.out0)[row * a.ldc + m] = from_f32<T>(siluf_(z));
   } else if constexpr (EPI == kEpiStoreHiLo || EPI == kEpiQueryH) {
     const long long row = (long long)g.b_row0 + n;
     if (EPI == kEpiQueryH && m >= a.epi_split) {
@@ -114,7 +114,7 @@ __device__ __forceinline__ void gemm_epilogue4(const GemmArgs& a, const GemmGrou
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const float z = v[j] + bias4[j] + add[j];
-        r[j] = from_f32<T>(z * sigmoidf_(z));
+        r[j] = from_f32<T>(siluf_(z));
       }
       *reinterpret_cast<uint2*>(static_cast<T*>(a.out0) + o) = *reinterpret_cast<const uint2*>(r);
       return;

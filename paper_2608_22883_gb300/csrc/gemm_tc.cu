@@ -364,7 +364,7 @@ __device__ __forceinline__ void act_store4(const GemmArgs& a, const GemmGroup& g
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const float z = v[j] + add4[j] + bias4[j];
-    y[j] = z * sigmoidf_(z);
+    y[j] = siluf_(z);
   }
   if (nv == 4 && (reinterpret_cast<uintptr_t>(out) & 7) == 0) {
     const __nv_bfloat162 lo = __floats2bfloat162_rn(y[0], y[1]);

@@ -590,7 +590,7 @@ __global__ void __launch_bounds__(kReadoutThreads, 4) readout_kernel(const __gri
       const float bias = to_f32(c < a.H ? static_cast<const T*>(a.b_f1)[c]
                                         : static_cast<const T*>(a.b_g1)[c - a.H]);
       const float z = sum + a.Gh[o] + bias;
-      static_cast<T*>(a.act)[o] = from_f32<T>(z * sigmoidf_(z));
+      static_cast<T*>(a.act)[o] = from_f32<T>(siluf_(z));
     } else {
       if (a.r_out != nullptr) a.r_out[o] = sum;
       if (a.r_lo != nullptr) static_cast<T*>(a.r_lo)[o] = from_f32<T>(sum);

@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(NT) select_gather_kernel(
     auto fin = [&](int vc, int i, float sum) {
       const int c = vc * V + i;
       const float z = sum + gh_s[c] + to_f32(bias_s[c]);
-      act[c] = from_f32<T>(z * sigmoidf_(z));
+      act[c] = from_f32<T>(siluf_(z));
     };
     if (ga.stage_rows > 0) {
       T* buf = reinterpret_cast<T*>(reinterpret_cast<uint8_t*>(dyn) + ga.stage_off);
