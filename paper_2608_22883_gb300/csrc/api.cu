@@ -371,7 +371,7 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
   auto run = [&]() -> fovea_status {
     fovea_status rs = alloc_dev(&scratch, 256 + align_up(B * sizeof(int32_t), 256), "build scratch", pool, s);
     if (rs != FOVEA_OK) return rs;
-    int* errw = static_cast<int*>(scratch);           // error word, then the list's count
+    int* errw = static_cast<int*>(scratch);           // error word
     int32_t* d_counts = reinterpret_cast<int32_t*>(static_cast<uint8_t*>(scratch) + 256);
     FOVEA_CUDA(cudaMemsetAsync(scratch, 0, 256, s), "cudaMemsetAsync");
     m->counts.assign(B, M_max);
@@ -407,15 +407,13 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
     const bool proj = bf && p->W_f1 != nullptr && p->W_g1 != nullptr && H > 0 && H % 128 == 0 &&
                       H <= FOVEA_MAX_H && aligned16(p->W_f1) && aligned16(p->W_g1);
     const int ld = (m_max + 63) / 64 * 64;
-    // the list holds 0.47 % of the keys of well-scaled tokens (gemm_build.cu)
-    const long long fix_cap = bf ? (long long)total * d / 32 + 4096 : 0;
     if ((rs = alloc_dev(&m->keys, (size_t)total * d * es, "keys", pool, s)) != FOVEA_OK ||
         (rs = alloc_dev(&m->values, (size_t)total * d * es, "values", pool, s)) != FOVEA_OK ||
         (rs = alloc_dev(reinterpret_cast<void**>(&m->orig_index), total * sizeof(int32_t), "index",
                         pool, s)) != FOVEA_OK ||
         (rs = alloc_dev(&src_row, total * sizeof(int32_t), "source rows", pool, s)) != FOVEA_OK ||
         (rs = alloc_dev(&xv, (size_t)total * d * es, "LN(v)", pool, s)) != FOVEA_OK ||
-        (bf && (rs = alloc_dev(&fix, (size_t)fix_cap * sizeof(KeyFix), "key fix list", pool, s)) != FOVEA_OK) ||
+        (bf && (rs = alloc_dev(&fix, (size_t)total * d / 8, "key marks", pool, s)) != FOVEA_OK) ||
         (fold && (rs = alloc_dev(&m->folded, (size_t)total * 2 * d * 2, "folded keys", pool, s)) != FOVEA_OK) ||
         (fold && (rs = alloc_dev(&wqt, (size_t)d * d * 2, "transposed W_Q", pool, s)) != FOVEA_OK) ||
         (proj && (rs = alloc_dev(&m->proj, (size_t)total * 2 * H * 2, "projected values", pool, s)) != FOVEA_OK) ||
@@ -450,7 +448,7 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
       pg.ldc = d;
       pg.err = errw;
       pg.out[0] = m->keys; pg.out[1] = m->values;
-      pg.fix_list = static_cast<KeyFix*>(fix); pg.fix_count = errw + 1; pg.fix_cap = (int)fix_cap;
+      pg.fix_bits = static_cast<uint32_t*>(fix);
       const TmaOperand none{nullptr, 0, 0, 0};
       { KernelTimer t("memory_proj", s);
         err = launch_pair_gemm(kPairKeys, pg, TmaOperand{p->W_K, d, d, d},
@@ -458,8 +456,7 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
       if (err != cudaSuccess) return cuda_fail(err, "memory projection");
       // keys whose fp32 value sat near a bf16 rounding midpoint: exact recompute
       { KernelTimer t("refine_keys", s);
-        err = launch_refine_keys(xv, p->W_K, d, pg.fix_list, pg.fix_count, (int)fix_cap, total,
-                                 m->keys, s); }
+        err = launch_refine_keys(xv, p->W_K, d, pg.fix_bits, total, m->keys, s); }
       if (err != cudaSuccess) return cuda_fail(err, "refine_keys");
       if (fold) {
         // kappa_i = W_Q^T k_i, a GEMM of W_Q^T (transposed once here) with the

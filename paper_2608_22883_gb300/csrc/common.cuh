@@ -364,16 +364,13 @@ cudaError_t launch_gemm_tc(int epi, const GemmArgs& a, const TmaOperand& A0, con
 // (bf16), fp32 sums stored as bf16 with row stride ldc.
 enum PairEpi : int {
   kPairStore = 0,     // part p (F0, F1) to out[p]
-  kPairKeys = 1,      // the same, and part 0's elements near a rounding midpoint are listed
+  kPairKeys = 1,      // the same, and part 0's elements near a rounding midpoint are marked
   kPairHiLo = 2,      // one part: hi = bf16(sum) to out[0], bf16(sum - hi) to out_lo
-};
-struct KeyFix {       // one listed key element: memory row, feature
-  int row, col;
 };
 struct PairGemm {
   int rows;                                      // token rows
   void* out[2]; void* out_lo; long long ldc;
-  KeyFix* fix_list; int* fix_count; int fix_cap; // kPairKeys
+  uint32_t* fix_bits;                            // kPairKeys: bit c % 32 of [row * ldc / 32 + c / 32]
   int* err;
   // filled by the launch
   int k_blocks, cols[2], tiles0, feat_tiles, row_tiles;
@@ -382,10 +379,9 @@ struct PairGemm {
 cudaError_t launch_pair_gemm(PairEpi epi, PairGemm a, const TmaOperand& F0, const TmaOperand& F1,
                              const TmaOperand& R, cudaStream_t s);
 
-// Exact rounding of listed key elements: k = sum_l x[row, l] W[col, l]
-// evaluated in double-float, rounded once to bf16.  A list whose device count
-// exceeds its capacity refines every element of the [rows, d] key matrix.
-cudaError_t launch_refine_keys(const void* xv, const void* W, int d, const KeyFix* list,
-                               const int* count, int cap, int rows, void* K, cudaStream_t s);
+// Exact rounding of the marked key elements (bits [rows, d / 32]): k = sum_l
+// x[row, l] W[col, l] evaluated in double-float, rounded once to bf16.
+cudaError_t launch_refine_keys(const void* xv, const void* W, int d, const uint32_t* bits, int rows,
+                               void* K, cudaStream_t s);
 
 }  // namespace fovea

@@ -23,8 +23,8 @@
 // The other outputs keep one accumulator: draining one every 256 elements costs
 // a tile a sixth of its rate (folded keys 820 us instead of 628).
 // A key must be the correctly rounded bf16 of its exact sum; the keys whose
-// sum lies so near a rounding midpoint that the GEMM cannot tell are listed
-// and recomputed exactly (refine_keys_kernel).  The window of that list
+// sum lies so near a rounding midpoint that the GEMM cannot tell are marked
+// and recomputed exactly (refine_keys_kernel).  The window of the marks
 // follows the error of the sum (kKeyWindow below).
 //
 // Roles (320 threads): warp 0 lanes 0 and 1 issue the TMA loads of this CTA's
@@ -67,15 +67,15 @@ constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
                             ((uint32_t)(2 * BM >> 4) << 24);
 
-// Key window: an element is listed when its sum lies within
+// Key window: an element is marked when its sum lies within
 // kKeyWindow * max(|sum|, scale) of a bf16 rounding midpoint, scale being the
 // RMS of the token's sums over its half of the tile.  With chunked sums the
 // farthest mis-rounded key from its midpoint, over 3.7e8 keys at d = 256 ..
 // 8192 (none refined, compared with float64), lay 2^-20.4 of that magnitude
 // away, with no trend in d (0.017 % of the keys were mis-rounded); 2^-19
-// keeps a margin of 2.6x and lists 0.47 % of the keys.  One accumulator over
-// the whole contraction needs 2^-15 and lists 5 %: at 32768 tokens, d = 4096
-// their recomputation took 11.0 ms of a 17.5 ms build, now 1.0 ms.
+// keeps a margin of 2.6x and marks 0.47 % of the keys.  One accumulator over
+// the whole contraction needs 2^-15 and marks 5 %: at 32768 tokens, d = 4096
+// their recomputation took 11.0 ms of a 17.5 ms build, now 0.85 ms.
 constexpr float kKeyWindow = 1.0f / 524288.0f;   // 2^-19
 
 __device__ __forceinline__ uint32_t cta_rank() {
@@ -159,7 +159,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 
 // The midpoint of the two bf16 values around a finite fp32 value is its upper
 // 16 bits followed by 0x8000.  An element whose window reaches the spacing of
-// the bf16 values around it (a sum far below the scale) is always listed, as
+// the bf16 values around it (a sum far below the scale) is always marked, as
 // is one that is not finite.
 __device__ __forceinline__ bool near_midpoint(float acc, float scale) {
   const float mid = __uint_as_float((__float_as_uint(acc) & 0xFFFF0000u) | 0x8000u);
@@ -187,7 +187,7 @@ __device__ __forceinline__ Tile tile_at(const PairGemm& a, int t) {
   return r;
 }
 
-// KEYS: part 0 is the keys (rounded, near-midpoint elements listed); HILO:
+// KEYS: part 0 is the keys (rounded, near-midpoint elements marked); HILO:
 // hi = bf16(sum) to out[0] and bf16(sum - hi) to out_lo.
 template <bool KEYS, bool HILO>
 __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
@@ -362,7 +362,6 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
 #pragma unroll
         for (int j = 0; j < BNH; ++j) ss = fmaf(acc[j], acc[j], ss);
         const float scale = sqrtf(ss / (float)cols);
-        int cnt = 0;
 #pragma unroll
         for (int q = 0; q < BNH / 32; ++q) {
           uint32_t bits = 0u;
@@ -372,27 +371,14 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
               if (near_midpoint(acc[32 * q + j], scale)) bits |= 1u << j;
           }
           need[q] = bits;
-          cnt += __popc(bits);
         }
-        // the warp's listed elements take consecutive slots of the list
-        int incl = cnt;
+        // every word of the token's row is written, 8 bytes at a time (columns
+        // come in multiples of 64)
+        if (row + lane < a.rows) {
+          uint32_t* m = a.fix_bits + (long long)(row + lane) * (a.ldc >> 5) + (col0 >> 5);
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int u = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += u;
-        }
-        int base = 0;
-        if (lane == 31 && incl > 0) base = atomicAdd(a.fix_count, incl);
-        int slot = __shfl_sync(0xffffffffu, base, 31) + incl - cnt;
-#pragma unroll
-        for (int q = 0; q < BNH / 32; ++q) {
-          uint32_t bits = need[q];
-          while (bits != 0u) {
-            const int j = __ffs(bits) - 1;
-            bits &= bits - 1u;
-            if (slot < a.fix_cap) a.fix_list[slot] = KeyFix{row + lane, col0 + 32 * q + j};
-            ++slot;
-          }
+          for (int q = 0; q < BNH / 32; q += 2)
+            if (32 * q < cols) *reinterpret_cast<uint2*>(m + q) = make_uint2(need[q], need[q + 1]);
         }
       }
       // 32 rows x 64 columns at a time through the warp's staging (16-byte

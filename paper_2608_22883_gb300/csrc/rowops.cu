@@ -610,68 +610,84 @@ cudaError_t launch_readout(int dtype, const RowGather& a, int N, cudaStream_t s)
 }
 
 // ---------------------------------------------------------------------------
-// Exact rounding of listed key elements (memory equation k_i = W_K LN(v_i)):
-// one warp per element, 16-byte loads of both rows.  Products of two bf16
+// Exact rounding of the marked key elements (memory equation k_i = W_K
+// LN(v_i)): a CTA per token, one warp per marked element, the token's row in
+// shared memory and the element's weight row by 16-byte loads.  Products of two bf16
 // values are exact in fp32; each lane sums its products with the cascaded
 // (compensated) summation of Ogita, Rump and Oishi ("Accurate sum and dot
 // product", 2005, Algorithm Sum2: TwoSum of the running sum and the product,
 // the rounding errors added separately), whose error is below
 // eps |S| + (n eps)^2 sum |p| -- about 2^-27 of the key for d <= 8192, far
-// inside the distance of any listed element from a bf16 midpoint that matters
+// inside the distance of any marked element from a bf16 midpoint that matters
 // -- and the lanes' (sum, error) pairs are combined in double-float before
 // the single rounding to bf16.
+//
+// Bound by the L2 reads of the weight rows (19 marked elements per token of d
+// = 4096, 8 KB each) and by the summation's instructions, two products side by
+// side in packed fp32 arithmetic.  A warp per element of a list in no order
+// read both rows from L2 and summed one product at a time: 1025 us at 32768
+// tokens of d = 4096, now 846, and 291 us at 10368 tokens of d = 3584, now 227.
 // ---------------------------------------------------------------------------
 constexpr int kRefineThreads = 256;
+// Tokens per SM up to which two CTAs share a token: five CTAs fit an SM, so
+// few tokens leave each warp three elements in a row.  A build of 576 tokens
+// at d = 4096 takes 287 us with two CTAs per token, 291 with one (10368
+// tokens: 1066 and 1070).
+constexpr int kRefineSplitRows = 8;
+static_assert(FOVEA_MAX_D <= 32 * kRefineThreads, "one word of marks per thread");
 
-__device__ __forceinline__ void sum2_bf16x8(const uint4& xa, const uint4& wa, float& s, float& c) {
+// Eight products of two bf16 vectors into the running sums s and error sums c,
+// two independent sums side by side (packed fp32 arithmetic).
+__device__ __forceinline__ void sum2_bf16x8(const uint4& xa, const uint4& wa, f32x2& s, f32x2& c) {
   const uint32_t xs[4] = {xa.x, xa.y, xa.z, xa.w}, ws[4] = {wa.x, wa.y, wa.z, wa.w};
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const float xf = __uint_as_float(h ? (xs[q] & 0xFFFF0000u) : (xs[q] << 16));
-      const float wf = __uint_as_float(h ? (ws[q] & 0xFFFF0000u) : (ws[q] << 16));
-      const dfloat t = df_two_sum(s, __fmul_rn(xf, wf));       // the product is exact
-      s = t.hi;
-      c = __fadd_rn(c, t.lo);
-    }
+    const f32x2 x = x2_pack(__uint_as_float(xs[q] << 16), __uint_as_float(xs[q] & 0xFFFF0000u));
+    const f32x2 w = x2_pack(__uint_as_float(ws[q] << 16), __uint_as_float(ws[q] & 0xFFFF0000u));
+    x2_sum2(s, c, x2_mul(x, w));                                // the products are exact
   }
 }
 
 __global__ void __launch_bounds__(kRefineThreads) refine_keys_kernel(
     const __nv_bfloat16* __restrict__ xv, const __nv_bfloat16* __restrict__ W, int d,
-    const KeyFix* __restrict__ list, const int* __restrict__ count, int cap, long long total,
-    __nv_bfloat16* __restrict__ K) {
-  const int lane = threadIdx.x & 31;
-  const long long warps = (long long)gridDim.x * (kRefineThreads / 32);
-  if (list != nullptr && *count > cap) list = nullptr;           // overflowed: every element
-  const long long n_items = list ? (long long)*count : total;
+    const uint32_t* __restrict__ bits, __nv_bfloat16* __restrict__ K) {
+  extern __shared__ uint4 refine_sm[];                           // [d / 8] the token's row, [d] columns
+  __shared__ int n_cols;
   const int nv = d / 8;                                          // d % 64 == 0
-  for (long long it = blockIdx.x * (kRefineThreads / 32) + (threadIdx.x >> 5); it < n_items;
-       it += warps) {
-    long long row;
-    int col;
-    if (list) {
-      row = list[it].row;
-      col = list[it].col;
-    } else {
-      row = it / d;
-      col = (int)(it % d);
-    }
-    const uint4* x = reinterpret_cast<const uint4*>(xv + row * d);
+  uint16_t* cols = reinterpret_cast<uint16_t*>(refine_sm + nv);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const long long row = blockIdx.x;
+  const uint4* x = reinterpret_cast<const uint4*>(xv + row * d);
+  // d <= 32 kRefineThreads; of several CTAs of a token each takes every
+  // gridDim.y-th word of marks
+  uint32_t m = tid < d / 32 && tid % (int)gridDim.y == (int)blockIdx.y ? bits[row * (d / 32) + tid] : 0u;
+  if (tid == 0) n_cols = 0;
+  for (int l = tid; l < nv; l += kRefineThreads) refine_sm[l] = x[l];
+  __syncthreads();
+  if (m != 0u) {
+    int at = atomicAdd(&n_cols, __popc(m));
+    for (; m != 0u; m &= m - 1u) cols[at++] = (uint16_t)(32 * tid + __ffs(m) - 1);
+  }
+  __syncthreads();
+  const int n = n_cols;
+  for (int it = tid >> 5; it < n; it += kRefineThreads / 32) {
+    const int col = cols[it];
     const uint4* w = reinterpret_cast<const uint4*>(W + (long long)col * d);
-    float s0 = 0.0f, c0 = 0.0f, s1 = 0.0f, c1 = 0.0f;
-    for (int l = lane; l < nv; l += 64) {
-      const uint4 xa = x[l], wa = w[l];
-      uint4 xb = make_uint4(0u, 0u, 0u, 0u), wb = xb;
-      if (l + 32 < nv) {
-        xb = x[l + 32];
-        wb = w[l + 32];
-      }
-      sum2_bf16x8(xa, wa, s0, c0);
-      sum2_bf16x8(xb, wb, s1, c1);
+    f32x2 s0 = x2_pack(0.0f, 0.0f), c0 = s0, s1 = s0, c1 = s0;
+    int l = lane;
+    for (; l + 96 < nv; l += 128) {
+      uint4 wv[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) wv[j] = __ldg(w + l + 32 * j);
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        sum2_bf16x8(refine_sm[l + 32 * j], wv[j], j & 1 ? s1 : s0, j & 1 ? c1 : c0);
     }
-    dfloat acc = df_add(df_two_sum(s0, c0), df_two_sum(s1, c1));
+#pragma unroll 1
+    for (; l < nv; l += 32) sum2_bf16x8(refine_sm[l], __ldg(w + l), s0, c0);
+    const float2 sa = x2_unpack(s0), ca = x2_unpack(c0), sb = x2_unpack(s1), cb = x2_unpack(c1);
+    dfloat acc = df_add(df_add(df_two_sum(sa.x, ca.x), df_two_sum(sa.y, ca.y)),
+                        df_add(df_two_sum(sb.x, cb.x), df_two_sum(sb.y, cb.y)));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       const dfloat t = {__shfl_xor_sync(0xffffffffu, acc.hi, o), __shfl_xor_sync(0xffffffffu, acc.lo, o)};
@@ -733,16 +749,16 @@ cudaError_t launch_transpose_images(const void* in, int C, int ld, const ImageTa
   return cudaGetLastError();
 }
 
-cudaError_t launch_refine_keys(const void* xv, const void* W, int d, const KeyFix* list,
-                               const int* count, int cap, int rows, void* K, cudaStream_t s) {
-  const long long total = (long long)rows * d;
-  if (total == 0) return cudaSuccess;
+cudaError_t launch_refine_keys(const void* xv, const void* W, int d, const uint32_t* bits, int rows,
+                               void* K, cudaStream_t s) {
+  if (rows == 0 || d == 0) return cudaSuccess;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  refine_keys_kernel<<<sms * 8, kRefineThreads, 0, s>>>(
-      (const __nv_bfloat16*)xv, (const __nv_bfloat16*)W, d, list, count, cap, total,
-      (__nv_bfloat16*)K);
+  const int parts = rows <= kRefineSplitRows * sms ? 2 : 1;
+  refine_keys_kernel<<<dim3(rows, parts), kRefineThreads, 4 * d, s>>>((const __nv_bfloat16*)xv,
+                                                         (const __nv_bfloat16*)W, d, bits,
+                                                         (__nv_bfloat16*)K);
   return cudaGetLastError();
 }
 

@@ -177,6 +177,30 @@ def test_memory_build_tile_edges(fovea, d, m_sizes):
     mem.destroy()
 
 
+# one and two CTAs per token; a token's row below, at and past a warp's batch of
+# four vectors per lane, and the longest row
+@pytest.mark.parametrize("d,m", [(64, 3), (1024, 5), (1088, 1300), (8192, 2)])
+def test_keys_beside_a_rounding_midpoint(fovea, d, m):
+    """LN(v) = beta = (1, 2^-8, 2^-30, 0, ...): every key is 1 + 2^-8, the
+    midpoint between 1 and 1 + 2^-7, plus or minus 2^-30, which an fp32 sum
+    drops.  All elements are marked, and each must land on its side."""
+    w = workloads.generate_custom("midpoints", d, [m], [1], seed=d, H=128)
+    w.params["ln_v_gamma"] = np.zeros(d, dtype=np.float32)
+    beta = np.zeros(d, dtype=np.float32)
+    beta[:3] = 1.0, 2.0 ** -8, 2.0 ** -30
+    w.params["ln_v_beta"] = beta
+    up = np.arange(d) % 3 == 0
+    W = np.zeros((d, d), dtype=np.float32)
+    W[:, :2] = 1.0
+    W[:, 2] = np.where(up, 1.0, -1.0)
+    w.params["W_K"] = W
+    s = store(w)
+    mem = fovea.build_memory(params_for(s, fovea), s.dev["v"], s.dev.get("mask"))
+    K = mem.views()[0].double().cpu().numpy()
+    assert np.array_equal(K, np.broadcast_to(np.where(up, 1.0 + 2.0 ** -7, 1.0), K.shape))
+    mem.destroy()
+
+
 # row lengths below, at and past a warp's pass of 256 elements and its batch of
 # eight vectors per lane; means up to 1000 standard deviations away, where the
 # fp32 map is seldom sure of its rounding
