@@ -445,19 +445,20 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
     } else {
       PairGemm pg{};
       pg.rows = total;
-      pg.ldc = d;
       pg.err = errw;
       pg.out[0] = m->keys; pg.out[1] = m->values;
+      pg.ldc[0] = pg.ldc[1] = d;
       pg.fix_bits = static_cast<uint32_t*>(fix);
-      const TmaOperand none{nullptr, 0, 0, 0};
+      const TmaOperand none{nullptr, 0, 0, 0}, tokens{xv, total, d, d};
+      const TmaOperand kv[3] = {TmaOperand{p->W_K, d, d, d}, TmaOperand{p->W_U, d, d, d}, none};
       { KernelTimer t("memory_proj", s);
-        err = launch_pair_gemm(kPairKeys, pg, TmaOperand{p->W_K, d, d, d},
-                               TmaOperand{p->W_U, d, d, d}, TmaOperand{xv, total, d, d}, s); }
+        err = launch_pair_gemm(true, pg, kv, tokens, tokens, s); }
       if (err != cudaSuccess) return cuda_fail(err, "memory projection");
       // keys whose fp32 value sat near a bf16 rounding midpoint: exact recompute
       { KernelTimer t("refine_keys", s);
         err = launch_refine_keys(xv, p->W_K, d, pg.fix_bits, total, m->keys, s); }
       if (err != cudaSuccess) return cuda_fail(err, "refine_keys");
+      TmaOperand F[3] = {none, none, none};
       if (fold) {
         // kappa_i = W_Q^T k_i, a GEMM of W_Q^T (transposed once here) with the
         // stored keys, kept as the hi / lo pair of its fp32 accumulator (no
@@ -469,27 +470,28 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
         { KernelTimer t("transpose_wq", s);
           err = launch_transpose_images(p->W_Q, d, d, one, wqt, s); }
         if (err != cudaSuccess) return cuda_fail(err, "transpose W_Q");
+        F[0] = TmaOperand{wqt, d, d, d};
         pg.out[0] = m->folded;
         pg.out_lo = static_cast<__nv_bfloat16*>(m->folded) + d;
-        pg.ldc = 2 * d;
-        { KernelTimer t("memory_fold", s);
-          err = launch_pair_gemm(kPairHiLo, pg, TmaOperand{wqt, d, d, d}, none,
-                                 TmaOperand{m->keys, total, d, d}, s); }
-        if (err != cudaSuccess) return cuda_fail(err, "query folding of the keys");
-        m->fold_wq = p->W_Q;
+        pg.ldc[0] = 2 * d;
       }
       if (proj) {
         // p_i = [W_f1 ; W_g1]_r u_i, the first fusion layer's r-half applied to
         // every value once per image
-        const __nv_bfloat16* wf1r = static_cast<const __nv_bfloat16*>(p->W_f1) + d;
-        const __nv_bfloat16* wg1r = static_cast<const __nv_bfloat16*>(p->W_g1) + d;
-        pg.out[0] = m->proj;
-        pg.out[1] = static_cast<__nv_bfloat16*>(m->proj) + H;
-        pg.ldc = 2 * H;
-        { KernelTimer t("memory_proj_fusion", s);
-          err = launch_pair_gemm(kPairStore, pg, TmaOperand{wf1r, H, d, 2 * d},
-                                 TmaOperand{wg1r, H, d, 2 * d}, TmaOperand{m->values, total, d, d}, s); }
-        if (err != cudaSuccess) return cuda_fail(err, "fusion projection of the values");
+        F[1] = TmaOperand{static_cast<const __nv_bfloat16*>(p->W_f1) + d, H, d, 2 * d};
+        F[2] = TmaOperand{static_cast<const __nv_bfloat16*>(p->W_g1) + d, H, d, 2 * d};
+        pg.out[1] = m->proj;
+        pg.out[2] = static_cast<__nv_bfloat16*>(m->proj) + H;
+        pg.ldc[1] = pg.ldc[2] = 2 * H;
+      }
+      if (fold || proj) {
+        KernelTimer t("memory_fold", s);
+        err = launch_pair_gemm(false, pg, F, TmaOperand{m->keys, total, d, d},
+                               TmaOperand{m->values, total, d, d}, s);
+      }
+      if (err != cudaSuccess) return cuda_fail(err, "folding the keys and projecting the values");
+      if (fold) m->fold_wq = p->W_Q;
+      if (proj) {
         { KernelTimer t("memory_proj_transpose", s);
           err = launch_transpose_images(m->proj, 2 * H, ld, itab, m->projT, s); }
         if (err != cudaSuccess) return cuda_fail(err, "transposing the projected values");

@@ -359,25 +359,23 @@ cudaError_t launch_gemm_tc(int epi, const GemmArgs& a, const TmaOperand& A0, con
                            const TmaOperand& B0, const TmaOperand& B1, int max_m, int max_n,
                            cudaStream_t s, const TmaOperand& A2 = TmaOperand{nullptr, 0, 0, 0});
 
-// The memory build's GEMMs out = R . F^T on CTA pairs (gemm_build.cu): R
-// [rows, K] token rows against one or two feature matrices F0, F1 [cols, K]
-// (bf16), fp32 sums stored as bf16 with row stride ldc.
-enum PairEpi : int {
-  kPairStore = 0,     // part p (F0, F1) to out[p]
-  kPairKeys = 1,      // the same, and part 0's elements near a rounding midpoint are marked
-  kPairHiLo = 2,      // one part: hi = bf16(sum) to out[0], bf16(sum - hi) to out_lo
-};
+// The memory build's GEMMs out[i] = R . F[i]^T on CTA pairs (gemm_build.cu):
+// token rows R [rows, K] (R0 for part 0, R1 for the others) against up to
+// three feature matrices F[i] [cols, K] (bf16; a null base: no such part),
+// fp32 sums stored as bf16 with row stride ldc[i].  keys: part 0's elements
+// near a rounding midpoint are marked; else part 0 is stored as a pair, hi =
+// bf16(sum) to out[0] and bf16(sum - hi) to out_lo.
 struct PairGemm {
   int rows;                                      // token rows
-  void* out[2]; void* out_lo; long long ldc;
-  uint32_t* fix_bits;                            // kPairKeys: bit c % 32 of [row * ldc / 32 + c / 32]
+  void* out[3]; long long ldc[3]; void* out_lo;
+  uint32_t* fix_bits;                            // keys: bit c % 32 of [row * ldc[0] / 32 + c / 32]
   int* err;
   // filled by the launch
-  int k_blocks, cols[2], tiles0, feat_tiles, row_tiles;
+  int k_blocks, cols[3], tile_end[3], feat_tiles, row_tiles;
   unsigned long long wait_ns;
 };
-cudaError_t launch_pair_gemm(PairEpi epi, PairGemm a, const TmaOperand& F0, const TmaOperand& F1,
-                             const TmaOperand& R, cudaStream_t s);
+cudaError_t launch_pair_gemm(bool keys, PairGemm a, const TmaOperand (&F)[3], const TmaOperand& R0,
+                             const TmaOperand& R1, cudaStream_t s);
 
 // Exact rounding of the marked key elements (bits [rows, d / 32]): k = sum_l
 // x[row, l] W[col, l] evaluated in double-float, rounded once to bf16.

@@ -1,6 +1,8 @@
 // The memory build's GEMMs C = X . W^T (bf16, fp32 sums) on CTA pairs: the
-// keys and values (W_K ; W_U against LN(v)), the folded keys (W_Q^T against
-// the keys) and the projected values ([W_f1 ; W_g1]_r against the values).
+// keys and values (W_K ; W_U against LN(v)), then, in one launch, the folded
+// keys (W_Q^T against the keys) and the projected values ([W_f1 ; W_g1]_r
+// against the values): a one-image build's 48 and 12 tiles fill one wave of
+// pairs together (build 266 us, 291 with two launches; 32768 tokens: the same).
 // Thousands of token rows meet thousands of features, so, unlike the draft
 // step's GEMMs (gemm_tc.cu), these are bound by the tensor pipe and by what
 // feeds it.
@@ -181,19 +183,23 @@ __device__ __forceinline__ Tile tile_at(const PairGemm& a, int t) {
   const int ft = local / rows_here;
   Tile r;
   r.row0 = (band * kBandRows + local % rows_here) * 2 * BM;
-  r.part = ft < a.tiles0 ? 0 : 1;
-  r.m0 = (r.part ? ft - a.tiles0 : ft) * BN;
+  r.part = ft < a.tile_end[0] ? 0 : ft < a.tile_end[1] ? 1 : 2;
+  r.m0 = (r.part ? ft - a.tile_end[r.part - 1] : ft) * BN;
   r.n_cols = min(BN, a.cols[r.part] - r.m0);
   return r;
 }
 
-// KEYS: part 0 is the keys (rounded, near-midpoint elements marked); HILO:
-// hi = bf16(sum) to out[0] and bf16(sum - hi) to out_lo.
+// KEYS: part 0 is the keys (rounded, near-midpoint elements marked); HILO: part
+// 0 is stored as hi = bf16(sum) to out[0] and bf16(sum - hi) to out_lo.  The
+// other parts are rounded sums.  Part 0 reads the tokens of tmR0, the others
+// those of tmR1.
 template <bool KEYS, bool HILO>
 __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
     pair_gemm_kernel(const __grid_constant__ CUtensorMap tmF0,
                      const __grid_constant__ CUtensorMap tmF1,
-                     const __grid_constant__ CUtensorMap tmR, const __grid_constant__ PairGemm a) {
+                     const __grid_constant__ CUtensorMap tmF2,
+                     const __grid_constant__ CUtensorMap tmR0,
+                     const __grid_constant__ CUtensorMap tmR1, const __grid_constant__ PairGemm a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   uint8_t* staging = smem + kStages * kStageBytes;
@@ -221,7 +227,7 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
     *abort_flag = 0;
     fence_mbar_init();
     prefetch_tmap(&tmF0);
-    prefetch_tmap(&tmR);
+    prefetch_tmap(&tmR0);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -245,7 +251,8 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
     bool go = true;
     for (int t = pid; go && t < tiles; t += pairs) {
       const Tile ti = tile_at(a, t);
-      const CUtensorMap* map = lane == 1 ? &tmR : ti.part ? &tmF1 : &tmF0;
+      const CUtensorMap* map = lane == 1 ? (ti.part ? &tmR1 : &tmR0)
+                                         : ti.part == 0 ? &tmF0 : ti.part == 1 ? &tmF1 : &tmF2;
       const int y = lane == 1 ? ti.row0 + (int)rank * BM : ti.m0 + (int)rank * BNH;
       for (int su = 0; su < su_total; ++su, ++i) {
         const int st = i % kStages;
@@ -375,7 +382,7 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
         // every word of the token's row is written, 8 bytes at a time (columns
         // come in multiples of 64)
         if (row + lane < a.rows) {
-          uint32_t* m = a.fix_bits + (long long)(row + lane) * (a.ldc >> 5) + (col0 >> 5);
+          uint32_t* m = a.fix_bits + (long long)(row + lane) * (a.ldc[0] >> 5) + (col0 >> 5);
 #pragma unroll
           for (int q = 0; q < BNH / 32; q += 2)
             if (32 * q < cols) *reinterpret_cast<uint2*>(m + q) = make_uint2(need[q], need[q + 1]);
@@ -384,13 +391,16 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
       // 32 rows x 64 columns at a time through the warp's staging (16-byte
       // chunks swizzled by row: conflict-free both ways), written out 128
       // bytes of a row per eight lanes
-      __nv_bfloat16* outs[2] = {static_cast<__nv_bfloat16*>(a.out[ti.part]),
-                                HILO ? static_cast<__nv_bfloat16*>(a.out_lo) : nullptr};
+      const bool hilo = HILO && ti.part == 0;
+      const long long ldc = a.ldc[ti.part];
 #pragma unroll
       for (int g = 0; g < BNH / 64; ++g) {
         if (64 * g >= cols) break;
 #pragma unroll
         for (int w = 0; w < (HILO ? 2 : 1); ++w) {
+          if (w == 1 && !hilo) break;
+          __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(w == 0 ? a.out[ti.part] : a.out_lo) +
+                               col0 + 64 * g;
 #pragma unroll
           for (int ch = 0; ch < 8; ++ch) {
             uint32_t p[4];
@@ -399,7 +409,7 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
               float& x = acc[64 * g + 8 * ch + 2 * e];
               float& y = acc[64 * g + 8 * ch + 2 * e + 1];
               p[e] = pack_bf16(x, y);
-              if (HILO && w == 0) {              // what hi leaves, for the second pass
+              if (HILO && w == 0 && hilo) {      // what hi leaves, for the second pass
                 x -= __uint_as_float(p[e] << 16);
                 y -= __uint_as_float(p[e] & 0xFFFF0000u);
               }
@@ -413,7 +423,7 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
             const int r = it * 4 + (lane >> 3), ch = lane & 7;
             const uint4 u = *reinterpret_cast<const uint4*>(stg + r * 128 + ((ch ^ (r & 7)) << 4));
             if (row + r < a.rows)
-              *reinterpret_cast<uint4*>(outs[w] + (long long)(row + r) * a.ldc + col0 + 64 * g + 8 * ch) = u;
+              *reinterpret_cast<uint4*>(dst + (long long)(row + r) * ldc + 8 * ch) = u;
           }
           __syncwarp();
         }
@@ -483,32 +493,35 @@ static cudaError_t launch(PairGemm& a, const CUtensorMap* maps, cudaStream_t s) 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, maps[0], maps[1], maps[2], a);
+  return cudaLaunchKernelEx(&cfg, kern, maps[0], maps[1], maps[2], maps[3], maps[4], a);
 }
 
 }  // namespace pair
 
-cudaError_t launch_pair_gemm(PairEpi epi, PairGemm a, const TmaOperand& F0, const TmaOperand& F1,
-                             const TmaOperand& R, cudaStream_t s) {
-  if (a.rows <= 0) return cudaSuccess;
-  a.k_blocks = (int)(R.cols / 64);
-  a.cols[0] = (int)F0.rows;
-  a.cols[1] = F1.base != nullptr ? (int)F1.rows : 0;
-  a.tiles0 = (a.cols[0] + pair::BN - 1) / pair::BN;
-  a.feat_tiles = a.tiles0 + (a.cols[1] + pair::BN - 1) / pair::BN;
+cudaError_t launch_pair_gemm(bool keys, PairGemm a, const TmaOperand (&F)[3], const TmaOperand& R0,
+                             const TmaOperand& R1, cudaStream_t s) {
+  a.feat_tiles = 0;
+  CUtensorMap maps[5];                 // F0, F1, F2, R0, R1; absent parts repeat a present one
+  const TmaOperand* some = &F[0];
+  for (const TmaOperand& f : F)
+    if (f.base != nullptr) some = &f;
+  for (int i = 0; i < 3; ++i) {
+    a.cols[i] = F[i].base != nullptr ? (int)F[i].rows : 0;
+    a.feat_tiles += (a.cols[i] + pair::BN - 1) / pair::BN;
+    a.tile_end[i] = a.feat_tiles;
+    if (!encode_kblock_map(&maps[i], F[i].base != nullptr ? F[i] : *some, pair::BNH, pair::KPS))
+      return cudaErrorInvalidValue;
+  }
+  if (a.rows <= 0 || a.feat_tiles == 0) return cudaSuccess;
+  a.k_blocks = (int)(some->cols / 64);
   a.row_tiles = (a.rows + 2 * pair::BM - 1) / (2 * pair::BM);
   a.wait_ns = wait_limit_ns();
-  CUtensorMap maps[3];
-  const TmaOperand& f1 = F1.base != nullptr ? F1 : F0;
-  if (!encode_kblock_map(&maps[0], F0, pair::BNH, pair::KPS) ||
-      !encode_kblock_map(&maps[1], f1, pair::BNH, pair::KPS) ||
-      !encode_kblock_map(&maps[2], R, pair::BM, pair::KPS))
+  const TmaOperand& r0 = R0.base != nullptr ? R0 : R1;
+  const TmaOperand& r1 = R1.base != nullptr ? R1 : R0;
+  if (!encode_kblock_map(&maps[3], r0, pair::BM, pair::KPS) ||
+      !encode_kblock_map(&maps[4], r1, pair::BM, pair::KPS))
     return cudaErrorInvalidValue;
-  switch (epi) {
-    case kPairKeys: return pair::launch<true, false>(a, maps, s);
-    case kPairHiLo: return pair::launch<false, true>(a, maps, s);
-    default: return pair::launch<false, false>(a, maps, s);
-  }
+  return keys ? pair::launch<true, false>(a, maps, s) : pair::launch<false, true>(a, maps, s);
 }
 
 }  // namespace fovea
