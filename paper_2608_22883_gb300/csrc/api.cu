@@ -210,6 +210,14 @@ static fovea_status check_step_params(const fovea_params* p) {
 // ---------------------------------------------------------------------------
 namespace {
 constexpr unsigned long long kPoolKeep = 2ull << 30;
+// Tokens up to which the folding GEMM reads W_Q along its rows (an MN-major
+// operand) instead of a transposed copy.  The GEMM takes the same time either
+// way (787 us at 32768 tokens of d = 4096); the copy costs its 13 us and the
+// temporary.  Builds one at a time, without and with the copy: 303 and 384 us
+// (576 tokens, d = 4096), 1476 and 1533 (9216), 2412 and 2474 (16384), 4560
+// and 4621 (32768); back to back at 32768, where the copy is 0.4 % of the
+// build, 3495 and 3374, so the copy stays there.
+constexpr int kFoldByRowTokens = 16384;
 constexpr int kMaxDevices = 64;
 struct DevicePool {
   cudaMemPool_t pool = nullptr;
@@ -361,8 +369,8 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
   m->M_max = M_max;
   m->d = d;
   m->dtype = p->dtype;
-  // temporaries: error word and list count, valid counts | source rows | LN(v) |
-  // listed key elements | W_Q^T
+  // temporaries: error word, valid counts | source rows | LN(v) | marks of the
+  // key elements | W_Q^T
   void* scratch = nullptr;
   void* src_row = nullptr;
   void* xv = nullptr;
@@ -415,7 +423,8 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
         (rs = alloc_dev(&xv, (size_t)total * d * es, "LN(v)", pool, s)) != FOVEA_OK ||
         (bf && (rs = alloc_dev(&fix, (size_t)total * d / 8, "key marks", pool, s)) != FOVEA_OK) ||
         (fold && (rs = alloc_dev(&m->folded, (size_t)total * 2 * d * 2, "folded keys", pool, s)) != FOVEA_OK) ||
-        (fold && (rs = alloc_dev(&wqt, (size_t)d * d * 2, "transposed W_Q", pool, s)) != FOVEA_OK) ||
+        (fold && total > kFoldByRowTokens &&
+         (rs = alloc_dev(&wqt, (size_t)d * d * 2, "transposed W_Q", pool, s)) != FOVEA_OK) ||
         (proj && (rs = alloc_dev(&m->proj, (size_t)total * 2 * H * 2, "projected values", pool, s)) != FOVEA_OK) ||
         (proj && (rs = alloc_dev(&m->projT, (size_t)B * 2 * H * ld * 2, "transposed projected values",
                                  pool, s)) != FOVEA_OK))
@@ -460,17 +469,20 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
       if (err != cudaSuccess) return cuda_fail(err, "refine_keys");
       TmaOperand F[3] = {none, none, none};
       if (fold) {
-        // kappa_i = W_Q^T k_i, a GEMM of W_Q^T (transposed once here) with the
-        // stored keys, kept as the hi / lo pair of its fp32 accumulator (no
+        // kappa_i = W_Q^T k_i, a GEMM of W_Q^T (read along W_Q's rows, or
+        // transposed once here) with the stored keys, kept as the hi / lo pair of its fp32 accumulator (no
         // bf16 rounding of the query map)
-        static thread_local ImageTable one;
-        one.B = 1;
-        one.off[0] = 0;
-        one.m[0] = d;
-        { KernelTimer t("transpose_wq", s);
-          err = launch_transpose_images(p->W_Q, d, d, one, wqt, s); }
-        if (err != cudaSuccess) return cuda_fail(err, "transpose W_Q");
-        F[0] = TmaOperand{wqt, d, d, d};
+        if (wqt != nullptr) {
+          static thread_local ImageTable one;
+          one.B = 1;
+          one.off[0] = 0;
+          one.m[0] = d;
+          { KernelTimer t("transpose_wq", s);
+            err = launch_transpose_images(p->W_Q, d, d, one, wqt, s); }
+          if (err != cudaSuccess) return cuda_fail(err, "transpose W_Q");
+        }
+        pg.f0_by_row = wqt == nullptr;
+        F[0] = TmaOperand{wqt != nullptr ? wqt : p->W_Q, d, d, d};
         pg.out[0] = m->folded;
         pg.out_lo = static_cast<__nv_bfloat16*>(m->folded) + d;
         pg.ldc[0] = 2 * d;

@@ -68,6 +68,13 @@ constexpr uint32_t kTmemCols = 512;
 // kind::f16: D fp32, A and B bf16, both K-major, N = 256, M = 256
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
                             ((uint32_t)(2 * BM >> 4) << 24);
+// f0_by_row: the folded part's features are W_Q read as it lies, the contraction
+// along its rows: B MN-major (bit 16).  A stage holds two blocks of 64 features, each
+// KPS * 64 contraction rows of 128 bytes (128-byte swizzle): 16 KB from one
+// block of features to the next, 1 KB from 8 contraction rows to the next.
+constexpr uint32_t kIdescMn = kIdesc | (1u << 16);
+constexpr uint64_t kMnBlock = (uint64_t)(KPS * 64 * 128 >> 4);
+static_assert(BNH == KPS * 64, "one box for both orders of the features");
 
 // Key window: an element is marked when its sum lies within
 // kKeyWindow * max(|sum|, scale) of a bf16 rounding midpoint, scale being the
@@ -94,12 +101,12 @@ __device__ __forceinline__ void tma_load_pair(uint32_t dst, const CUtensorMap* m
       : "memory");
 }
 __device__ __forceinline__ void umma_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
-                                          uint32_t accumulate) {
+                                          uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(kIdesc), "r"(accumulate)
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 // Completion of the MMAs issued so far, signalled to the barrier at this
@@ -190,7 +197,8 @@ __device__ __forceinline__ Tile tile_at(const PairGemm& a, int t) {
 }
 
 // KEYS: part 0 is the keys (rounded, near-midpoint elements marked); HILO: part
-// 0 is stored as hi = bf16(sum) to out[0] and bf16(sum - hi) to out_lo.  The
+// 0's sums are stored as hi = bf16(sum) to out[0] and bf16(sum - hi) to out_lo,
+// and its feature matrix may lie as [K, cols] (f0_by_row).  The
 // other parts are rounded sums.  Part 0 reads the tokens of tmR0, the others
 // those of tmR1.
 template <bool KEYS, bool HILO>
@@ -264,7 +272,10 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
         }
         if (lane == 0 && rank == 0) mbar_expect_tx(&full[st], 2u * kStageBytes);
         const uint32_t dst = smem_u32(smem + st * kStageBytes) + (lane == 1 ? 0u : (uint32_t)(KPS * kSmemRows));
-        tma_load_pair(dst, map, map_dsmem(smem_u32(&full[st]), 0), 0, y, su * KPS);
+        if (HILO && lane == 0 && ti.part == 0 && a.f0_by_row)
+          tma_load_pair(dst, map, map_dsmem(smem_u32(&full[st]), 0), 0, su * KPS * 64, y / 64);
+        else
+          tma_load_pair(dst, map, map_dsmem(smem_u32(&full[st]), 0), 0, y, su * KPS);
       }
     }
     // the last stages' releases have arrived here before the CTA may leave
@@ -282,7 +293,9 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
     int c = 0;
     bool go = true;
     for (int t = pid; go && t < tiles; t += pairs) {
-      const int chunk = KEYS && tile_at(a, t).part == 0 ? kChunkSu : su_total;
+      const bool first = tile_at(a, t).part == 0;
+      const int chunk = KEYS && first ? kChunkSu : su_total;
+      const bool mn = HILO && first && a.f0_by_row;
       for (int su0 = 0; go && su0 < su_total; su0 += chunk, ++c) {
         const int buf = c & 1;
         const uint32_t d = tmem_base + (uint32_t)(buf * BN);
@@ -304,14 +317,19 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
           if (elect_one()) {
             // descriptor start addresses are in units of 16 bytes
             const uint64_t ad = desc0 + (uint64_t)(st * (uint32_t)(kStageBytes >> 4));
-            const uint64_t bd = ad + (uint64_t)((KPS * kSmemRows) >> 4);
+            const uint64_t bd = ad + (uint64_t)((KPS * kSmemRows) >> 4) +
+                                (mn ? (kMnBlock - 1) << 16 : 0);   // its leading-dimension offset
+            const uint32_t idesc = mn ? kIdescMn : kIdesc;
+            // per 16 elements of the contraction: 32 bytes of a K-major row,
+            // 16 rows of an MN-major block
 #pragma unroll
             for (int j = 0; j < KPS; ++j)
 #pragma unroll
-              for (int k = 0; k < 4; ++k)          // 32 bytes (16 elements) per MMA
+              for (int k = 0; k < 4; ++k)
                 umma_pair(d, ad + (uint64_t)((j * kSmemRows >> 4) + 2 * k),
-                          bd + (uint64_t)((j * kSmemFeat >> 4) + 2 * k),
-                          (su > su0 || j > 0 || k > 0) ? 1u : 0u);
+                          bd + (uint64_t)(mn ? (4 * j + k) * (16 * 128 >> 4)
+                                             : (j * kSmemFeat >> 4) + 2 * k),
+                          idesc, (su > su0 || j > 0 || k > 0) ? 1u : 0u);
             commit_pair(&empty[st]);
           }
           __syncwarp();

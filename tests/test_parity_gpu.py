@@ -147,9 +147,11 @@ def test_memory_build_matches_oracle(fovea, name):
 # tiles of 256 tokens x 256 features on CTA pairs, k-blocks of 64 in stages of
 # two and chunks of four: token counts at the edges of a CTA's and a pair's
 # rows and past a band of 8 row tiles; d with partial feature tiles, an odd
-# number of k-blocks, fewer k-blocks than a stage, a chunk, the ring
+# number of k-blocks, fewer k-blocks than a stage, a chunk, the ring; and more
+# tokens than the folding GEMM reads W_Q along its rows for
 @pytest.mark.parametrize("d,m_sizes", [(64, [1]), (192, [128]), (256, [129, 3]), (320, [255]),
-                                       (448, [257]), (576, [385, 0, 130]), (128, [2100])])
+                                       (448, [257]), (576, [385, 0, 130]), (128, [2100]),
+                                       (64, [8192, 8193])])
 def test_memory_build_tile_edges(fovea, d, m_sizes):
     """Keys are the correctly rounded W_K LN(v); a value is one bf16 rounding
     (2^-9 of its magnitude) of a sum whose fp32 error is far below that; the
