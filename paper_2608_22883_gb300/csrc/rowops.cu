@@ -153,25 +153,36 @@ __device__ __forceinline__ void sum2_join(float& s, float& c, float s2, float c2
   c = __fadd_rn(__fadd_rn(c, c2), t.lo);
 }
 
-// One warp per row, the row, gamma and beta in shared memory; CTAs of four
-// warps loop over the rows.  Bound by its instructions and by HBM alike: per
-// element 8 packed operations of the two compensated sums (the squares are
-// exact: a bf16 value has 8 significant bits) and about 15 of the map and its
-// midpoint test.  No CTA barrier and one reduction per row, where a CTA per
-// row took two barriers and double-float arithmetic on every element: 32768
-// rows of 4096 took 932 us, now 219 us (2.4 TB/s).
+// One warp per row (kRowWarps = 1; for few rows the CTA's four), the row, gamma
+// and beta in shared memory; CTAs of four warps loop over the rows.  Bound by
+// its instructions and by HBM alike: per element 8 packed operations of the two
+// compensated sums (the squares are exact: a bf16 value has 8 significant bits)
+// and about 15 of the map and its midpoint test.  A row per warp needs no CTA
+// barrier and one reduction, where a CTA per row took two barriers and
+// double-float arithmetic on every element: 32768 rows of 4096 took 932 us, now
+// 219 us (2.4 TB/s).
 constexpr int kLnTokWarps = 4;
 constexpr int kLnTokLoads = 8;          // 16-byte loads in flight per lane
+// Rows per SM up to which the four warps of a CTA share a row: with a row per
+// warp 576 rows leave an SM four warps, each with 128 elements per lane in
+// series.  A build of 576 tokens at d = 4096 takes 242 us with shared rows, 252
+// with a row per warp; 2304 tokens 558 and 581, 4608 tokens 862 and 882.
+constexpr int kLnTokSplitRows = 16;
 
+template <int kRowWarps>
 __global__ void __launch_bounds__(32 * kLnTokWarps) ln_tokens_kernel(
     const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ src_row, int rows, int d,
     const __nv_bfloat16* __restrict__ gamma, const __nv_bfloat16* __restrict__ beta, float eps,
     __nv_bfloat16* __restrict__ out) {
-  extern __shared__ __align__(16) uint4 ln_sm[];     // gamma [d], beta [d], a row per warp
-  const int nvec = d / 8, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  extern __shared__ __align__(16) uint4 ln_sm[];     // gamma [d], beta [d], the rows in work
+  __shared__ float4 parts[kLnTokWarps];
+  constexpr int kRows = kLnTokWarps / kRowWarps;     // rows a CTA works on at a time
+  constexpr int kLanes = 32 * kRowWarps;             // threads of a row
+  constexpr int kLoads = kLnTokLoads / (kRowWarps > 1 ? 2 : 1);
+  const int nvec = d / 8, lane = threadIdx.x % kLanes, mine = threadIdx.x / kLanes;
   uint4* g_s = ln_sm;
   uint4* b_s = ln_sm + nvec;
-  uint4* x_s = ln_sm + (2 + warp) * nvec;
+  uint4* x_s = ln_sm + (2 + mine) * nvec;
   for (int i = threadIdx.x; i < nvec; i += 32 * kLnTokWarps) {
     g_s[i] = reinterpret_cast<const uint4*>(gamma)[i];
     b_s[i] = reinterpret_cast<const uint4*>(beta)[i];
@@ -179,20 +190,20 @@ __global__ void __launch_bounds__(32 * kLnTokWarps) ln_tokens_kernel(
   pdl_wait();
   pdl_trigger();
   __syncthreads();
-  for (int row = blockIdx.x * kLnTokWarps + warp; row < rows; row += gridDim.x * kLnTokWarps) {
+  for (int row = blockIdx.x * kRows + mine; row < rows; row += gridDim.x * kRows) {
     const uint4* xr = reinterpret_cast<const uint4*>(x + (long long)src_row[row] * d);
     f32x2 s1 = x2_pack(0.0f, 0.0f), c1 = s1, s2 = s1, c2 = s1;
 #pragma unroll 1
-    for (int j0 = lane; j0 < nvec; j0 += 32 * kLnTokLoads) {
-      uint4 raw[kLnTokLoads];
+    for (int j0 = lane; j0 < nvec; j0 += kLanes * kLoads) {
+      uint4 raw[kLoads];
 #pragma unroll
-      for (int j = 0; j < kLnTokLoads; ++j) {
-        const int vi = j0 + 32 * j;
+      for (int j = 0; j < kLoads; ++j) {
+        const int vi = j0 + kLanes * j;
         raw[j] = vi < nvec ? __ldg(xr + vi) : make_uint4(0u, 0u, 0u, 0u);   // zeros add nothing
       }
 #pragma unroll
-      for (int j = 0; j < kLnTokLoads; ++j) {
-        const int vi = j0 + 32 * j;
+      for (int j = 0; j < kLoads; ++j) {
+        const int vi = j0 + kLanes * j;
         if (vi < nvec) x_s[vi] = raw[j];
         const uint32_t w[4] = {raw[j].x, raw[j].y, raw[j].z, raw[j].w};
 #pragma unroll
@@ -211,6 +222,17 @@ __global__ void __launch_bounds__(32 * kLnTokWarps) ln_tokens_kernel(
       sum2_join(a, ac, __shfl_xor_sync(0xffffffffu, a, o), __shfl_xor_sync(0xffffffffu, ac, o));
       sum2_join(b, bc, __shfl_xor_sync(0xffffffffu, b, o), __shfl_xor_sync(0xffffffffu, bc, o));
     }
+    if constexpr (kRowWarps > 1) {                   // the CTA's one row: its warps' sums in order
+      if ((threadIdx.x & 31) == 0) parts[threadIdx.x >> 5] = make_float4(a, ac, b, bc);
+      __syncthreads();
+      a = parts[0].x; ac = parts[0].y; b = parts[0].z; bc = parts[0].w;
+#pragma unroll
+      for (int w = 1; w < kRowWarps; ++w) {
+        sum2_join(a, ac, parts[w].x, parts[w].y);
+        sum2_join(b, bc, parts[w].z, parts[w].w);
+      }
+      __syncthreads();                               // before the next row's parts
+    }
     const dfloat mean = df_div_f(df_two_sum(a, ac), (float)d);
     const dfloat ex2 = df_div_f(df_two_sum(b, bc), (float)d);
     const dfloat neg_mean = {-mean.hi, -mean.lo};
@@ -222,7 +244,7 @@ __global__ void __launch_bounds__(32 * kLnTokWarps) ln_tokens_kernel(
     const float mr = fabsf(mean.hi) * rstd.hi * 1.1920929e-7f;
     __nv_bfloat16* o = out + (long long)row * d;
 #pragma unroll 1                                       // a lane reads the vectors it stored above
-    for (int vi = lane; vi < nvec; vi += 32) {
+    for (int vi = lane; vi < nvec; vi += kLanes) {
       const uint4 xv = x_s[vi], gr = g_s[vi], br = b_s[vi];
       const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w};
       const uint32_t gw[4] = {gr.x, gr.y, gr.z, gr.w}, bw[4] = {br.x, br.y, br.z, br.w};
@@ -428,19 +450,21 @@ cudaError_t launch_ln_rows(int dtype, const void* x, const int32_t* src_row, int
     return launch_pdl(ln_rows_kernel<float>, dim3(rows), dim3(kLnThreads), 0, s, (const float*)x,
                       src_row, d, (const float*)gamma, (const float*)beta, eps, (float*)out);
   int dev = 0, sms = 0, per_sm = 0;
-  const size_t smem = (size_t)d * 2 * (2 + kLnTokWarps);       // at most 96 KB
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(ln_tokens_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             FOVEA_MAX_D * 2 * (2 + kLnTokWarps));
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ln_tokens_kernel, 32 * kLnTokWarps,
-                                                      smem);
   if (e != cudaSuccess) return e;
-  const int ctas = (rows + kLnTokWarps - 1) / kLnTokWarps;
+  const bool split = rows <= kLnTokSplitRows * sms;
+  const int at_once = split ? 1 : kLnTokWarps;
+  const auto kern = split ? ln_tokens_kernel<kLnTokWarps> : ln_tokens_kernel<1>;
+  const size_t smem = (size_t)d * 2 * (2 + at_once);           // at most 96 KB
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           FOVEA_MAX_D * 2 * (2 + at_once));
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kLnTokWarps, smem);
+  if (e != cudaSuccess) return e;
+  const int ctas = (rows + at_once - 1) / at_once;
   const int most = sms * (per_sm > 0 ? per_sm : 1);
-  return launch_pdl(ln_tokens_kernel, dim3(ctas < most ? ctas : most), dim3(32 * kLnTokWarps),
+  return launch_pdl(kern, dim3(ctas < most ? ctas : most), dim3(32 * kLnTokWarps),
                     smem, s, (const __nv_bfloat16*)x, src_row, rows, d, (const __nv_bfloat16*)gamma,
                     (const __nv_bfloat16*)beta, eps, (__nv_bfloat16*)out);
 }

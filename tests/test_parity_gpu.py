@@ -204,17 +204,18 @@ def test_keys_beside_a_rounding_midpoint(fovea, d, m):
 
 
 # row lengths below, at and past a warp's pass of 256 elements and its batch of
-# eight vectors per lane; means up to 1000 standard deviations away, where the
-# fp32 map is seldom sure of its rounding
+# eight vectors per lane, four warps per row (few rows) and one; means up to 1000
+# standard deviations away, where the fp32 map is seldom sure of its rounding
+@pytest.mark.parametrize("m", [37, 2500])
 @pytest.mark.parametrize("d,mean,std", [(64, 0.0, 1.0), (320, 5.0, 1.0), (2048, 0.0, 1.0),
                                         (2112, 5.0, 1.0), (2112, 64.0, 0.0625), (8192, 0.0, 1.0)])
-def test_token_layer_norm_is_correctly_rounded(fovea, d, mean, std):
+def test_token_layer_norm_is_correctly_rounded(fovea, d, mean, std, m):
     """With W_K = I a key is LN(v) itself: the bf16 rounding of the float64
     value.  The variance E[x^2] - mean^2 keeps 2^-46 of E[x^2] in
     double-float, so the product (x - mean) rstd gamma errs by at most 2^-44
     (1 + E[x^2] / (var + eps)) of itself: the key lies between the roundings of
     the exact value less and plus that bound."""
-    w = workloads.generate_custom("ln", d, [37, 4], [1, 1], seed=d, H=128)
+    w = workloads.generate_custom("ln", d, [m, 4], [1, 1], seed=d, H=128)
     w.params["W_K"] = np.eye(d, dtype=np.float32)
     w.v = (mean + std * w.v).astype(np.float32)
     s = store(w)
