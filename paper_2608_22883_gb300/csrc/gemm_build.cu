@@ -31,7 +31,7 @@
 //
 // Roles (320 threads): warp 0 lanes 0 and 1 issue the TMA loads of this CTA's
 // features and tokens, warp 1 allocates the tensor memory and, in the leader
-// CTA (cluster rank 0), its lane 0 issues the MMAs of the pair; warps 2 .. 9
+// CTA (cluster rank 0), an elected lane issues the MMAs of the pair; warps 2 .. 9
 // run the epilogue: warp w reads accumulator lanes (tokens) 32 (w % 4) .. +31
 // and one half of the columns, 128 fp32 sums per thread.  Stage barriers
 // (`full`) live in the leader and count both CTAs' bytes; commits signal
