@@ -1200,10 +1200,16 @@ static void plan_for(const GemmArgs& a, int max_m, int max_n, long long row_tile
         const long long waves = (ctas + cap - 1) / cap;
         const long long per_sm = std::max<long long>(1, (std::min(ctas, cap) + sms - 1) / sms);
         // at least `chunks` accumulators to a contraction, in the tensor memory
-        // that the CTAs of an SM share
+        // that the CTAs of an SM share.  The CTAs of a cluster wait for one
+        // another, so no such CTA may wait in tcgen05.alloc for a CTA of another
+        // stream's launch, which may wait for its own cluster in turn: they take
+        // half of the tensor memory at most (by their registers, more than 85 a
+        // thread, two CTAs of this kernel fit an SM at most).  A CTA without a
+        // cluster waits for nobody once it has its columns.
         int nacc = 1;
         while (nacc * S < chunks) nacc *= 2;
-        if (nacc > 1 && (nacc > nst || nacc * BN * ((cap + sms - 1) / sms) > 512)) continue;
+        const long long sharers = S > 1 ? 2 : (cap + sms - 1) / sms;
+        if (nacc > 1 && (nacc > nst || nacc * BN * sharers > 512)) continue;
         const double t = chunks > 0 ? fed_cost_us(sb / 1024.0, stage_f, stage_mma_us, stages, nst, ctas, cap,
                                            sms, rows, BN, S)
                              : plan_cost_us(streaming, sb / 1024.0, stage_f, stage_mma_us, stages, nst,

@@ -493,6 +493,69 @@ def test_repeat_calls_are_deterministic(fovea):
     fovea.sync_errors(ws)
 
 
+# launches of several sequences that stream more than L2 holds (their plans keep
+# several accumulators per CTA), with and without split K; and the LM head
+@pytest.mark.parametrize("B,m,rows", [(8, 1100, 5), (2, 4300, 40)])
+def test_two_streams_at_once(fovea, B, m, rows):
+    """Two threads, each on a stream of its own, run steps and LM heads at the
+    same time: tensor memory is shared by the launches of both, and each gets
+    what a run by itself gives, bit for bit."""
+    import threading
+    d, N = 4096, B * rows
+    g = torch.Generator(device="cuda")
+    g.manual_seed(B)
+
+    def normal(*shape, scale=1.0):
+        return (torch.randn(shape, generator=g, device="cuda") * scale).to(torch.bfloat16)
+
+    weights = {n: normal(d, scale=0.1) for n in ("ln_v_beta", "ln_h_beta", "b_f2")}
+    weights.update({n: normal(d, scale=0.1) + 1 for n in ("ln_v_gamma", "ln_h_gamma", "rms_gamma")})
+    weights.update({n: normal(d, d, scale=d ** -0.5) for n in ("W_K", "W_U", "W_Q")})
+    weights.update({n: normal(512, 2 * d, scale=(2 * d) ** -0.5) for n in ("W_f1", "W_g1")})
+    weights.update({n: normal(512, scale=0.05) for n in ("b_f1", "b_g1", "w_g2")})
+    weights.update(E_dep=normal(7, d, scale=0.1), W_f2=normal(d, 512, scale=512 ** -0.5), b_g2=normal(1))
+    params = fovea.Params(weights, d_model=d)
+    mem = fovea.build_memory(params, normal(B, m, d))
+    W_LM = normal(20000, d, scale=d ** -0.5)
+    h = [normal(N, d) for _ in range(2)]
+    depth = torch.zeros(N, dtype=torch.int32, device="cuda")
+    offsets = [rows * b for b in range(B + 1)]
+    ws = [fovea.new_workspace(params, mem, offsets, 32) for _ in range(2)]
+    lm_ws = [fovea.lm_head_workspace(W_LM.shape[0], d, N, 6) for _ in range(2)]
+
+    def call(i):
+        out = fovea.step(params, mem, h[i], depth, offsets, None, 0.9, 1, 32, workspace=ws[i])
+        idx, val, z = fovea.lm_head_topk(W_LM, out["h_out"], 6, lm_ws[i])
+        return [out[k] for k in ("h_out", "counts", "indices", "readout", "gate")] + [idx, val, z]
+
+    alone = [call(i) for i in range(2)]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    got, errors = [None, None], []
+
+    def loop(i):
+        try:
+            with torch.cuda.stream(streams[i]):
+                for _ in range(20):
+                    got[i] = call(i)
+        except Exception as e:              # reported by the main thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=loop, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors, errors
+    for i in range(2):
+        fovea.sync_errors(ws[i])
+        fovea.sync_errors(lm_ws[i])
+        for a, b in zip(alone[i], got[i]):
+            assert torch.equal(a, b)
+    mem.destroy()
+
+
 def test_invalid_depth_sets_error_word(fovea):
     w = small_workload("bf16-ragged")
     w.depth = w.depth.copy()
