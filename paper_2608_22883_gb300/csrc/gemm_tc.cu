@@ -1121,7 +1121,7 @@ static double fed_cost_us(double stage_kb, double stage_f_bytes, double mma_us, 
 
 template <int BN, int EPI>
 static void plan_for(const GemmArgs& a, int max_m, int max_n, long long row_tiles, int chunks,
-                     GemmPlan& best, double& best_t) {
+                     bool fed, GemmPlan& best, double& best_t) {
   constexpr bool DUAL = EPI == kEpiScores || EPI == kEpiAct;
   using C = tc::Cfg<BN, DUAL>;
   // folded scores with hi / lo folded keys: the key part's stages hold two
@@ -1196,7 +1196,8 @@ static void plan_for(const GemmArgs& a, int max_m, int max_n, long long row_tile
         if (cap <= 0) continue;
         // (the occupancy query counts one CTA per SM for the half-SM budget,
         // whose CTAs do run two to an SM)
-        if (chunks > 0) cap = (sms * (2 * (smem + 1024) <= tc::kSmemPerSm ? 2 : 1)) / S * S;
+        const int per_sm_smem = 2 * (smem + 1024) <= tc::kSmemPerSm ? 2 : 1;
+        if (fed) cap = sms * per_sm_smem / S * S;
         const long long waves = (ctas + cap - 1) / cap;
         const long long per_sm = std::max<long long>(1, (std::min(ctas, cap) + sms - 1) / sms);
         // at least `chunks` accumulators to a contraction, in the tensor memory
@@ -1208,9 +1209,8 @@ static void plan_for(const GemmArgs& a, int max_m, int max_n, long long row_tile
         // cluster waits for nobody once it has its columns.
         int nacc = 1;
         while (nacc * S < chunks) nacc *= 2;
-        const long long sharers = S > 1 ? 2 : (cap + sms - 1) / sms;
-        if (nacc > 1 && (nacc > nst || nacc * BN * sharers > 512)) continue;
-        const double t = chunks > 0 ? fed_cost_us(sb / 1024.0, stage_f, stage_mma_us, stages, nst, ctas, cap,
+        if (nacc > 1 && (nacc > nst || nacc * BN * (S > 1 ? 2 : per_sm_smem) > 512)) continue;
+        const double t = fed ? fed_cost_us(sb / 1024.0, stage_f, stage_mma_us, stages, nst, ctas, cap,
                                            sms, rows, BN, S)
                              : plan_cost_us(streaming, sb / 1024.0, stage_f, stage_mma_us, stages, nst,
                                             std::min(ctas, cap), (int)per_sm, waves, S);
@@ -1228,16 +1228,16 @@ static void plan_for(const GemmArgs& a, int max_m, int max_n, long long row_tile
 // 8 images x 8 rows at d = 1024 27.0 against 25.1.)
 constexpr long long kFedBytes = 128ll << 20;
 
-// chunks = 0: the plan_cost_us estimate; else the fed_cost_us estimate over the
-// plans whose contractions are split over at least that many accumulators.
+// The fed_cost_us or the plan_cost_us estimate over the plans whose contractions
+// are split over at least `chunks` accumulators.
 template <int EPI>
-static GemmPlan plan_best(const GemmArgs& a, int max_m, int max_n, int chunks) {
+static GemmPlan plan_best(const GemmArgs& a, int max_m, int max_n, int chunks, bool fed) {
   const long long row_tiles = (long long)(max_n + tc::BM - 1) / tc::BM * a.ngroups;
   GemmPlan best{256, 1, 2, 0, 1 << 30, 128, 128, 0, 1, 1};
   double best_t = 1e30;
-  plan_for<256, EPI>(a, max_m, max_n, row_tiles, chunks, best, best_t);
-  plan_for<128, EPI>(a, max_m, max_n, row_tiles, chunks, best, best_t);
-  plan_for<64, EPI>(a, max_m, max_n, row_tiles, chunks, best, best_t);
+  plan_for<256, EPI>(a, max_m, max_n, row_tiles, chunks, fed, best, best_t);
+  plan_for<128, EPI>(a, max_m, max_n, row_tiles, chunks, fed, best, best_t);
+  plan_for<64, EPI>(a, max_m, max_n, row_tiles, chunks, fed, best, best_t);
   return best;
 }
 
@@ -1248,25 +1248,39 @@ static GemmPlan plan_epi(const GemmArgs& a, int max_m, int max_n) {
     for (int g = 0; g < a.ngroups; ++g)
       if (a.groups[g].a_row0 >= 0) features += a.groups[g].m;
     const long long streamed = features * a.k_total * 2 * (a.f_lo_kb > 0 ? 2 : 1);
-    if (max_n <= tc::BM && (EPI == kEpiLogits || a.ngroups > 1) && streamed > kFedBytes) {
-      // the split that the other estimate gives the logits, or the scores by
-      // themselves, is the number of accumulators to keep: a plan with fewer
-      // splits would sum less exactly
+    const bool fed = max_n <= tc::BM && (EPI == kEpiLogits || a.ngroups > 1) && streamed > kFedBytes;
+    if (fed || a.gh_cols > 0) {
+      // the splits that the plan_cost_us estimate gives the logits, or the
+      // scores and G_h each in a launch of its own, are the accumulators to
+      // keep: a plan with fewer sums less exactly.  (G_h of 1024 rows at d =
+      // 5120 and of 512 at 4096: four by itself, one as the scores' plan has it.)
       static thread_local GemmArgs alone;
       alone = a;
       alone.gh_cols = 0;
       alone.ngroups = 0;
-      int n = 0;
-      for (int g = 0; g < a.ngroups; ++g)
+      int n = 0, n_gh = 0;
+      for (int g = 0; g < a.ngroups; ++g) {
         if (a.groups[g].a_row0 >= 0) {
           alone.groups[alone.ngroups++] = a.groups[g];
           n = std::max(n, a.groups[g].n);
+        } else {
+          n_gh += a.groups[g].n;
         }
-      const GemmPlan p = plan_best<EPI>(a, max_m, max_n, plan_best<EPI>(alone, max_m, n, 0).splits);
+      }
+      int chunks = plan_best<EPI>(alone, max_m, n, 1, false).splits;
+      if (a.gh_cols > 0) {
+        alone.a_split = a.gh_cols;
+        alone.r_by_part = 0;
+        alone.f_lo_kb = 0;
+        alone.ngroups = 1;
+        alone.groups[0] = GemmGroup{0, 2 * a.gh_cols, 0, n_gh, 0};
+        chunks = std::max(chunks, plan_best<kEpiQueryH>(alone, 2 * a.gh_cols, n_gh, 1, false).splits);
+      }
+      const GemmPlan p = plan_best<EPI>(a, max_m, max_n, chunks, fed);
       if (p.region > 0) return p;
     }
   }
-  return plan_best<EPI>(a, max_m, max_n, 0);
+  return plan_best<EPI>(a, max_m, max_n, 1, false);
 }
 
 static GemmPlan plan_gemm_tc_uncached(int epi, const GemmArgs& a, int max_m, int max_n) {

@@ -493,6 +493,77 @@ def test_repeat_calls_are_deterministic(fovea):
     fovea.sync_errors(ws)
 
 
+def device_weights(g, d, H=512):
+    """Weights and a generator of bf16 normals on the device (wide models)."""
+    def normal(*shape, scale=1.0):
+        return (torch.randn(shape, generator=g, device="cuda") * scale).to(torch.bfloat16)
+
+    weights = {n: normal(d, scale=0.1) for n in ("ln_v_beta", "ln_h_beta", "b_f2")}
+    weights.update({n: normal(d, scale=0.1) + 1 for n in ("ln_v_gamma", "ln_h_gamma", "rms_gamma")})
+    weights.update({n: normal(d, d, scale=d ** -0.5) for n in ("W_K", "W_U", "W_Q")})
+    weights.update({n: normal(H, 2 * d, scale=(2 * d) ** -0.5) for n in ("W_f1", "W_g1")})
+    weights.update({n: normal(H, scale=0.05) for n in ("b_f1", "b_g1", "w_g2")})
+    weights.update(E_dep=normal(7, d, scale=0.1), W_f2=normal(d, H, scale=H ** -0.5), b_g2=normal(1))
+    return weights, normal
+
+
+def workspace_regions(ws, N, d, k_max, score_elems, H=512):
+    """The scores, the activations and G_h that a bf16 step leaves in its
+    workspace (regions of 256-byte multiples behind a header of 4 KB)."""
+    off, out = 4096, {}
+    for name, shape, dt in (("xh", (N, d), torch.bfloat16), ("q", (N, 2 * d), torch.bfloat16),
+                            ("scores", (score_elems,), torch.float32), ("pos", (N, k_max), torch.int32),
+                            ("w", (N, k_max), torch.float32), ("cnt", (N,), torch.int32),
+                            ("r_lo", (N, d), torch.bfloat16), ("act", (N, 2 * H), torch.bfloat16),
+                            ("c", (N, d), torch.float32), ("gh", (N, 2 * H), torch.float32)):
+        n = int(np.prod(shape)) * torch.empty(0, dtype=dt).element_size()
+        out[name] = ws[off:off + n].view(dt).view(shape)
+        off = (off + n + 255) // 256 * 256
+    return out
+
+
+def truncation_bias(got, ref):
+    """The mean shortfall of sums, over their mean size.  The tensor core drops
+    what an addition to its accumulator shifts out, half a unit in the last
+    place on average, 2^-24 of an accumulator that grows to the sum's size (as
+    the square root of the additions, and unevenly over a binade): about 0.25 x
+    2^-24 of the sum per addition of 16 products."""
+    return float(((ref - got) * torch.sign(ref)).mean() / ref.abs().mean())
+
+
+# the h-half of the first fusion layer (G_h) in the score launch of several
+# sequences: launches of their own split its contraction over gh_accs
+# accumulators and the scores' over score_accs
+@pytest.mark.parametrize("d,m,B,rows,gh_accs,score_accs", [(4096, 300, 8, 8, 6, 3), (4096, 300, 2, 8, 6, 8),
+                                                           (1024, 300, 8, 100, 1, 3),
+                                                           (5120, 576, 16, 64, 4, 1)])
+def test_sums_of_the_score_launch_keep_their_accumulators(fovea, d, m, B, rows, gh_accs, score_accs):
+    """The shortfall of either sum is that of as many accumulators as its own
+    launch would take (0.3 for 0.25: the scatter between shapes)."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d + B)
+    weights, normal = device_weights(g, d)
+    params = fovea.Params(weights, d_model=d)
+    mem = fovea.build_memory(params, normal(B, m, d))
+    N = B * rows
+    h, depth = normal(N, d), torch.zeros(N, dtype=torch.int32, device="cuda")
+    fovea.timing_enable(True)
+    out = fovea.step(params, mem, h, depth, [rows * b for b in range(B + 1)], None, 0.9, 1, 16)
+    fovea.sync_errors(out["workspace"])
+    names = set(fovea.timing_read())
+    fovea.timing_enable(False)
+    assert "score_fusion_h" in names
+    r = workspace_regions(out["workspace"], N, d, 16, N * m)
+    w = torch.cat([weights["W_f1"][:, :d], weights["W_g1"][:, :d]]).double()
+    assert truncation_bias(r["gh"].double(), h.double() @ w.T) <= 0.3 * d / 16 / gh_accs * 2.0 ** -24
+    kappa = mem.folded_keys(params).double()
+    kappa = (kappa[:, :d] + kappa[:, d:]).view(B, m, d)
+    z = torch.einsum("brd,bmd->brm", r["xh"].double().view(B, rows, d), kappa) / d ** 0.5
+    got = r["scores"].double().view(B, rows, m)
+    assert truncation_bias(got, z) <= 0.3 * 2 * d / 16 / score_accs * 2.0 ** -24       # hi and lo
+    mem.destroy()
+
+
 # launches of several sequences that stream more than L2 holds (their plans keep
 # several accumulators per CTA), with and without split K; and the LM head
 @pytest.mark.parametrize("B,m,rows", [(8, 1100, 5), (2, 4300, 40)])
@@ -505,15 +576,7 @@ def test_two_streams_at_once(fovea, B, m, rows):
     g = torch.Generator(device="cuda")
     g.manual_seed(B)
 
-    def normal(*shape, scale=1.0):
-        return (torch.randn(shape, generator=g, device="cuda") * scale).to(torch.bfloat16)
-
-    weights = {n: normal(d, scale=0.1) for n in ("ln_v_beta", "ln_h_beta", "b_f2")}
-    weights.update({n: normal(d, scale=0.1) + 1 for n in ("ln_v_gamma", "ln_h_gamma", "rms_gamma")})
-    weights.update({n: normal(d, d, scale=d ** -0.5) for n in ("W_K", "W_U", "W_Q")})
-    weights.update({n: normal(512, 2 * d, scale=(2 * d) ** -0.5) for n in ("W_f1", "W_g1")})
-    weights.update({n: normal(512, scale=0.05) for n in ("b_f1", "b_g1", "w_g2")})
-    weights.update(E_dep=normal(7, d, scale=0.1), W_f2=normal(d, 512, scale=512 ** -0.5), b_g2=normal(1))
+    weights, normal = device_weights(g, d)
     params = fovea.Params(weights, d_model=d)
     mem = fovea.build_memory(params, normal(B, m, d))
     W_LM = normal(20000, d, scale=d ** -0.5)
