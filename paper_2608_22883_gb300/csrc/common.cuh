@@ -374,6 +374,7 @@ struct PairGemm {
   int* err;
   // filled by the launch
   int k_blocks, cols[3], tile_end[3], feat_tiles, row_tiles;
+  int chunk0[3], chunk[3];                       // stages of a part's first accumulator, of others
   unsigned long long wait_ns;
 };
 cudaError_t launch_pair_gemm(bool keys, PairGemm a, const TmaOperand (&F)[3], const TmaOperand& R0,

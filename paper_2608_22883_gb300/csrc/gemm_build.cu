@@ -19,11 +19,18 @@
 //
 // Chunked sums.  The tensor core adds a product sum to its fp32 accumulator
 // with truncation, once per 16 elements of the contraction, so a long
-// contraction drifts by about 2^-17 of the result's scale.  For the keys every
-// chunk of kChunkSu * KPS * 64 = 256 elements starts a fresh accumulator, and
-// the epilogue threads add the chunks in registers with rounded fp32 additions.
-// The other outputs keep one accumulator: draining one every 256 elements costs
-// a tile a sixth of its rate (folded keys 820 us instead of 628).
+// contraction falls short by about 2^-26 of the result per addition.  For the
+// keys every chunk of kChunkSu * KPS * 64 = 256 elements starts a fresh
+// accumulator, and the epilogue threads add the chunks in registers with rounded
+// fp32 additions.  The projected values, and the folded keys of up to
+// kChunkFoldRows tokens, take about eight chunks (of at least 256 elements): the
+// accumulators that a split contraction of one-CTA tiles gave them.  The first
+// is twice as long, so that its MMAs cover the epilogue's stores of the tile
+// before: a build of 10368 tokens of d = 3584 takes 1039 us (1034 with one
+// accumulator, 1066 with equal chunks), one image 242 (241), 32768 tokens 3400
+// (3402).  The values and the folded keys of more tokens keep one
+// accumulator: draining one every 256 elements costs a tile a sixth of its rate
+// (folded keys of 32768 tokens 820 us instead of 628).
 // A key must be the correctly rounded bf16 of its exact sum; the keys whose
 // sum lies so near a rounding midpoint that the GEMM cannot tell are marked
 // and recomputed exactly (refine_keys_kernel).  The window of the marks
@@ -43,6 +50,8 @@
 // CTAs reach because all waits are bounded, and when either has aborted the
 // leader commits the MMAs it issued, both wait for them and for the copies
 // in flight (bounded), and only then is the tensor memory freed.
+#include <algorithm>
+
 #include "tc_ptx.cuh"
 
 namespace fovea {
@@ -59,6 +68,8 @@ constexpr int kSmemFeat = BNH * 128;     // bytes of one k-block of this CTA's f
 constexpr int kStageBytes = KPS * (kSmemRows + kSmemFeat);
 constexpr int kStages = 3;
 constexpr int kChunkSu = 2;              // stages per accumulator chunk of the keys
+constexpr int kChunks = 8;               // accumulator chunks of the projected values ...
+constexpr int kChunkFoldRows = 8192;     // ... and of the folded keys of up to this many tokens
 constexpr int kEpiWarps = 8;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kWarpStage = 32 * 128;     // an epilogue warp's staging: 32 rows x 64 bf16
@@ -293,10 +304,11 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
     int c = 0;
     bool go = true;
     for (int t = pid; go && t < tiles; t += pairs) {
-      const bool first = tile_at(a, t).part == 0;
-      const int chunk = KEYS && first ? kChunkSu : su_total;
-      const bool mn = HILO && first && a.f0_by_row;
-      for (int su0 = 0; go && su0 < su_total; su0 += chunk, ++c) {
+      const int part = tile_at(a, t).part;
+      const int chunk = a.chunk[part];
+      const bool mn = HILO && part == 0 && a.f0_by_row;
+      int su0 = 0;
+      for (int len = a.chunk0[part]; go && su0 < su_total; su0 += len, len = chunk, ++c) {
         const int buf = c & 1;
         const uint32_t d = tmem_base + (uint32_t)(buf * BN);
         if (c >= 2 &&
@@ -307,7 +319,7 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
           break;
         }
         tc_fence_after();
-        const int su1 = min(su0 + chunk, su_total);
+        const int su1 = min(su0 + len, su_total);
         for (int su = su0; su < su1; ++su) {
           if (!__all_sync(0xffffffffu, wait_cluster(&full[st], ph, abort_flag, a.wait_ns))) {
             *abort_flag = 1;
@@ -354,8 +366,9 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
       float acc[BNH];
 #pragma unroll
       for (int j = 0; j < BNH; ++j) acc[j] = 0.0f;
-      const int chunk = KEYS && ti.part == 0 ? kChunkSu : su_total;
-      for (int su0 = 0; su0 < su_total; su0 += chunk, ++c) {
+      const int chunk = a.chunk[ti.part];
+      int su0 = 0;
+      for (int len = a.chunk0[ti.part]; su0 < su_total; su0 += len, len = chunk, ++c) {
         const int buf = c & 1;
         const bool ok = wait_cluster(&tfull[buf], (uint32_t)(c >> 1) & 1u, abort_flag, a.wait_ns);
         if (!__all_sync(0xffffffffu, ok)) {      // tcgen05.ld below is a .sync.aligned instruction
@@ -532,6 +545,13 @@ cudaError_t launch_pair_gemm(bool keys, PairGemm a, const TmaOperand (&F)[3], co
   }
   if (a.rows <= 0 || a.feat_tiles == 0) return cudaSuccess;
   a.k_blocks = (int)(some->cols / 64);
+  const int su_total = (a.k_blocks + pair::KPS - 1) / pair::KPS;
+  for (int i = 0; i < 3; ++i) {
+    const bool chunked = i > 0 || a.rows <= pair::kChunkFoldRows;
+    a.chunk[i] = keys ? (i == 0 ? pair::kChunkSu : su_total)
+                      : chunked ? std::max(pair::kChunkSu, su_total / pair::kChunks) : su_total;
+    a.chunk0[i] = keys ? a.chunk[i] : 2 * a.chunk[i];
+  }
   a.row_tiles = (a.rows + 2 * pair::BM - 1) / (2 * pair::BM);
   a.wait_ns = wait_limit_ns();
   const TmaOperand& r0 = R0.base != nullptr ? R0 : R1;

@@ -564,6 +564,48 @@ def test_sums_of_the_score_launch_keep_their_accumulators(fovea, d, m, B, rows, 
     mem.destroy()
 
 
+# builds whose folded keys and projected values were split over at least this
+# many accumulators as GEMMs of one-CTA tiles
+@pytest.mark.parametrize("d,tokens,accs", [(4096, 64, 4), (3584, 128, 7), (2048, 600, 3), (1024, 70, 2),
+                                           (4096, 3000, 4)])
+def test_folded_keys_keep_their_accumulators(fovea, d, tokens, accs):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d + tokens)
+    weights, normal = device_weights(g, d)
+    params = fovea.Params(weights, d_model=d)
+    mem = fovea.build_memory(params, normal(1, tokens, d))
+    kappa = mem.folded_keys(params).double()
+    ref = mem.views()[0].double() @ weights["W_Q"].double()
+    assert truncation_bias(kappa[:, :d] + kappa[:, d:], ref) <= 0.3 * d / 16 / accs * 2.0 ** -24
+    mem.destroy()
+
+
+@pytest.mark.parametrize("d,accs", [(4096, 4), (8192, 4), (2048, 4)])
+def test_projected_values_keep_their_accumulators(fovea, d, accs):
+    """512 images of one token, h = 0 and no bias: the activations left in the
+    workspace are SiLU(p), p the stored projected values.  Rounding p to bf16
+    keeps the mean shortfall of its sum (a shortfall of e moves one value in
+    ulp / e by an ulp), and so does SiLU, whose slope is about that of the
+    line from 0."""
+    B = 512
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d)
+    weights, normal = device_weights(g, d)
+    for n in ("b_f1", "b_g1"):
+        weights[n].zero_()
+    params = fovea.Params(weights, d_model=d)
+    mem = fovea.build_memory(params, normal(B, 1, d))
+    out = fovea.step(params, mem, torch.zeros((B, d), dtype=torch.bfloat16, device="cuda"),
+                     torch.zeros(B, dtype=torch.int32, device="cuda"), list(range(B + 1)), None, 0.9, 1, 1)
+    fovea.sync_errors(out["workspace"])
+    act = workspace_regions(out["workspace"], B, d, 1, B)["act"].double()
+    w = torch.cat([weights["W_f1"][:, d:], weights["W_g1"][:, d:]]).double()
+    p = (mem.views()[1].double() @ w.T).to(torch.bfloat16).double()
+    ref = torch.nn.functional.silu(p).to(torch.bfloat16).double()
+    assert truncation_bias(act, ref) <= 0.45 * d / 16 / accs * 2.0 ** -24
+    mem.destroy()
+
+
 # launches of several sequences that stream more than L2 holds (their plans keep
 # several accumulators per CTA), with and without split K; and the LM head
 @pytest.mark.parametrize("B,m,rows", [(8, 1100, 5), (2, 4300, 40)])
