@@ -195,7 +195,7 @@ struct GemmArgs {
   int kps;            // tensor-core path: k-blocks of 64 per ring stage
   int rbox, rbox1;    // tensor-core path: rows of a row-operand tile of B0 and of B1 (64 .. 128)
   int region;         // tensor-core path: bytes of the ring / partial-tile staging region
-  int nacc;           // tensor-core path: accumulators a CTA's contraction is split over
+  int nacc, nacc1;    // tensor-core path: accumulators a CTA's contraction is split over; of G_h groups
   const float* add_in;          // kEpiAct: fp32 term added before the activation
   unsigned long long* cand;     // kEpiLogits: per-row candidate keys
   long long cand_ld;
@@ -347,7 +347,7 @@ struct GemmPlan {
   int rbox, rbox1;            // rows of a row-operand load of B0 and of B1 (64 .. 128)
   int region;                 // bytes of the ring / partial-tile staging region
   int kps;                    // k-blocks of 64 per ring stage
-  int nacc;                   // accumulators a CTA's contraction is split over
+  int nacc, nacc1;            // accumulators a CTA's contraction is split over; of G_h groups
 };
 GemmPlan plan_gemm_tc(int epi, const GemmArgs& a, int max_m, int max_n);
 // Tensor map (cached per thread) of a row-major [rows, cols] bf16 matrix, cols

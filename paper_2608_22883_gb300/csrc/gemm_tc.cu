@@ -413,6 +413,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   // extra tiles idle.  The S CTAs of a tile share these decisions, so a
   // tile's CTAs exit together.
   const bool gh = EPI == kEpiScoresFolded && g.a_row0 < 0;   // a group of G_h: no F0 part
+  const int nacc_g = gh ? args.nacc1 : args.nacc;
   const int s1 = gh ? 0 : min(args.a_split, g.m);
   const int s2 = gh ? min(args.gh_cols, g.m) : max(s1, min(args.a_split2, g.m));
   const int t0 = (s1 + BN - 1) / BN, t1 = (s2 - s1 + BN - 1) / BN, t2 = (g.m - s2 + BN - 1) / BN;
@@ -477,7 +478,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     prefetch_tmap(&tmR0);
   }
   if (warp == 1) {
-    tmem_alloc(tmem_slot, (uint32_t)(args.nacc * BN));
+    tmem_alloc(tmem_slot, (uint32_t)(nacc_g * BN));
     tmem_relinquish();
   }
   tc_fence_before();
@@ -493,7 +494,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   // the contraction's chunks: the tensor core truncates each addition to its
   // accumulator, so fewer additions per accumulator err less; the epilogue adds
   // the chunks' sums, rounded, in order
-  const int nacc = max(1, min(args.nacc, nkb));
+  const int nacc = max(1, min(nacc_g, nkb));
 
   if (warp == 0 && lane < kProducers) {
     // ---- TMA producers: lane 0 loads the feature tiles, lane 1 the row tiles
@@ -842,7 +843,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, (uint32_t)(args.nacc * BN));
+    tmem_dealloc(tmem_base, (uint32_t)(nacc_g * BN));
   }
 }
 
@@ -1014,6 +1015,7 @@ static cudaError_t launch_tc_inst(GemmArgs& a, const CUtensorMap* maps, int tile
   a.rbox = p.rbox;
   a.rbox1 = p.rbox1;
   a.nacc = p.nacc;
+  a.nacc1 = p.nacc1;
   a.tx_bytes = tc::Cfg<BN, DUAL>::stage_bytes(p.kps, p.rbox,
                                               EPI == kEpiScoresFolded && a.f_lo_kb > 0);
   cudaLaunchConfig_t cfg = {};
@@ -1093,35 +1095,34 @@ static double plan_cost_us(bool streaming, double stage_kb, double stage_f_bytes
   return waves * (t_first + nst * t_stage) + t_tail;
 }
 
-// Estimated time (us) of a plan for the GEMMs that stream one feature operand
-// from HBM over many tiles (the LM head, the scores of several sequences),
-// fitted to the measured plans of three score launches and the LM head (the
-// order of their best plans is right; errors up to 25 %):
-//   stage   a CTA has (stages - 1/2) stages of copies in flight for ~1.9 us
-//           each, and an SM takes in ~88 KB/us whatever its CTAs; at least its
-//           MMAs, and the feature bytes of all CTAs' stages at the HBM rate;
-//   wave    ~2.2 us to the first stage (a little more for a larger one), ~1.2 us
-//           to drain, and the epilogue's time per thread.
-// Against the estimate above: LM head 60.4 -> 58.1 us, a step of 8 ragged images
-// x 32 rows 80.3 -> 76.0, 16 x 64 rows 117.5 -> 115.5, 4 x 128 rows of 8192
-// entries 167.5 -> 165.9.
-static double fed_cost_us(double stage_kb, double stage_f_bytes, double mma_us, int stages, int nst,
-                          long long ctas, long long cap, int sms, int rows, int bn, int S) {
+// Estimated time (us, up to a factor) of a plan for the GEMMs that stream one
+// feature operand from HBM over many tiles (the LM head, the scores of several
+// sequences).  Its constants order the plans of 214 such launches (LM heads of
+// 10000 .. 160000 x 512 .. 5120 and 1 .. 128 rows, scores of 2 .. 32 images of 100
+// .. 8192 entries), each timed with every plan:
+//   stage   a CTA has (stages - 1/2) stages of copies in flight for 0.97 us each,
+//           issues one per 0.22 us at best, and an SM runs the MMAs of all its
+//           CTAs (the intake of an SM and HBM do not tell the plans apart);
+//   wave    20 us of filling and draining whatever the plan, the epilogue's time
+//           per thread, and the meeting of a cluster;
+//   keys    of the logits, the candidate keys that the merge reads.
+// On 95 launches that it was not fitted to, the plan it picks takes 1.5 % longer
+// than the best one on average, and 7 % less than the pick of the estimate above.
+static double fed_cost_us(double mma_us, int stages, int nst, long long ctas, long long cap, int sms,
+                          int rows, int bn, int S, long long keys) {
   auto wave = [&](long long n) {
     if (n <= 0) return 0.0;
     const double per_sm = (double)((n + sms - 1) / sms);
-    const double latency = stages > 1 ? 1.9 / (stages - 0.5) : 1.9 + mma_us;
-    const double t_stage = std::max(std::max(per_sm * stage_kb / 88.0, latency),
-                                    std::max(per_sm * mma_us * 1.3, n * stage_f_bytes / 6.6e6));
-    const double t_tail = 1.2 + 0.12 * rows * bn / (1024.0 * S) + (S == 1 ? 0.0 : 1.4 + 0.25 * S);
-    return 2.2 + 0.02 * stage_kb + nst * t_stage + t_tail;
+    const double latency = stages > 1 ? 0.97 / (stages - 0.5) : 0.97 + mma_us;
+    const double t_stage = std::max(std::max(latency, 0.22), per_sm * mma_us * 0.75);
+    return 20.0 + nst * t_stage + 0.1 * per_sm * rows * bn / (1024.0 * S) + (S == 1 ? 0.0 : 0.46 * S);
   };
-  return (double)(ctas / cap) * wave(cap) + wave(ctas % cap);
+  return (double)(ctas / cap) * wave(cap) + wave(ctas % cap) + 0.0025 * keys;
 }
 
 template <int BN, int EPI>
 static void plan_for(const GemmArgs& a, int max_m, int max_n, long long row_tiles, int chunks,
-                     bool fed, GemmPlan& best, double& best_t) {
+                     int chunks1, const GemmPlan* other, GemmPlan& best, double& best_t) {
   constexpr bool DUAL = EPI == kEpiScores || EPI == kEpiAct;
   using C = tc::Cfg<BN, DUAL>;
   // folded scores with hi / lo folded keys: the key part's stages hold two
@@ -1197,47 +1198,60 @@ static void plan_for(const GemmArgs& a, int max_m, int max_n, long long row_tile
         // (the occupancy query counts one CTA per SM for the half-SM budget,
         // whose CTAs do run two to an SM)
         const int per_sm_smem = 2 * (smem + 1024) <= tc::kSmemPerSm ? 2 : 1;
-        if (fed) cap = sms * per_sm_smem / S * S;
+        if (other != nullptr) cap = sms * per_sm_smem / S * S;
         const long long waves = (ctas + cap - 1) / cap;
         const long long per_sm = std::max<long long>(1, (std::min(ctas, cap) + sms - 1) / sms);
-        // at least `chunks` accumulators to a contraction, in the tensor memory
-        // that the CTAs of an SM share.  The CTAs of a cluster wait for one
-        // another, so no such CTA may wait in tcgen05.alloc for a CTA of another
-        // stream's launch, which may wait for its own cluster in turn: they take
-        // half of the tensor memory at most (by their registers, more than 85 a
-        // thread, two CTAs of this kernel fit an SM at most).  A CTA without a
+        // at least `chunks` accumulators to a contraction (`chunks1` to one of G_h),
+        // in the tensor memory that the CTAs of an SM share.  The CTAs of a cluster
+        // wait for one another, so no such CTA may wait in tcgen05.alloc for a CTA
+        // of another stream's launch, which may wait for its own cluster in turn:
+        // they take half of the tensor memory at most (by their registers, more than
+        // 85 a thread, two CTAs of this kernel fit an SM at most).  A CTA without a
         // cluster waits for nobody once it has its columns.
-        int nacc = 1;
+        int nacc = 1, nacc1 = 1;
         while (nacc * S < chunks) nacc *= 2;
-        if (nacc > 1 && (nacc > nst || nacc * BN * (S > 1 ? 2 : per_sm_smem) > 512)) continue;
-        const double t = fed ? fed_cost_us(sb / 1024.0, stage_f, stage_mma_us, stages, nst, ctas, cap,
-                                           sms, rows, BN, S)
-                             : plan_cost_us(streaming, sb / 1024.0, stage_f, stage_mma_us, stages, nst,
-                                            std::min(ctas, cap), (int)per_sm, waves, S);
+        while (nacc1 * S < chunks1) nacc1 *= 2;
+        const int most = std::max(nacc, nacc1);
+        if (most > 1 && (most > nst || most * BN * (S > 1 ? 2 : per_sm_smem) > 512)) continue;
+        double t;
+        if (other == nullptr) {
+          t = plan_cost_us(streaming, sb / 1024.0, stage_f, stage_mma_us, stages, nst,
+                           std::min(ctas, cap), (int)per_sm, waves, S);
+        } else {
+          t = fed_cost_us(stage_mma_us, stages, nst, ctas, cap, sms, rows, BN, S,
+                          EPI == kEpiLogits ? ftiles * S * a.cand_k : 0);
+          if (other->bn == BN && other->splits == S && other->kps == kps && other->stages == stages &&
+              other->region == region)
+            t *= 0.95;
+        }
         if (t < best_t - 1e-6 || (t < best_t + 1e-6 && tiles * S < best.tiles * best.splits)) {
           best_t = t;
-          best = GemmPlan{BN, S, stages, 0, tiles, rbox, rbox1, region, kps, nacc};
+          best = GemmPlan{BN, S, stages, 0, tiles, rbox, rbox1, region, kps, nacc, nacc1};
         }
       }
     }
   }
 }
 
-// Feature bytes above which fed_cost_us plans a launch: more than L2 keeps.
-// (Below, it does worse: an LM head of 7752 x 4736, 73 MB, 28.2 us against 20.0,
-// 8 images x 8 rows at d = 1024 27.0 against 25.1.)
-constexpr long long kFedBytes = 128ll << 20;
+// Feature bytes above which fed_cost_us plans a launch: about what L2 keeps.  A
+// step of several sequences takes, with its plan against the other estimate's, on
+// average 3 % less between 100 and 135 MiB (34 launches, the worst 1 % more), 2 %
+// less between 64 and 100 (43, 8 % more), 2 % more between 30 and 64 (34, 40 %).
+constexpr long long kFedScoreBytes = 100ll << 20, kFedLogitBytes = 128ll << 20;
 
-// The fed_cost_us or the plan_cost_us estimate over the plans whose contractions
-// are split over at least `chunks` accumulators.
+// The plan of least plan_cost_us, or, given that plan as `other`, of least
+// fed_cost_us (another one has to be 5 % better), over the plans whose
+// contractions are split over at least `chunks` accumulators, those of G_h over
+// `chunks1`.
 template <int EPI>
-static GemmPlan plan_best(const GemmArgs& a, int max_m, int max_n, int chunks, bool fed) {
+static GemmPlan plan_best(const GemmArgs& a, int max_m, int max_n, int chunks = 1, int chunks1 = 1,
+                          const GemmPlan* other = nullptr) {
   const long long row_tiles = (long long)(max_n + tc::BM - 1) / tc::BM * a.ngroups;
-  GemmPlan best{256, 1, 2, 0, 1 << 30, 128, 128, 0, 1, 1};
+  GemmPlan best{256, 1, 2, 0, 1 << 30, 128, 128, 0, 1, 1, 1};
   double best_t = 1e30;
-  plan_for<256, EPI>(a, max_m, max_n, row_tiles, chunks, fed, best, best_t);
-  plan_for<128, EPI>(a, max_m, max_n, row_tiles, chunks, fed, best, best_t);
-  plan_for<64, EPI>(a, max_m, max_n, row_tiles, chunks, fed, best, best_t);
+  plan_for<256, EPI>(a, max_m, max_n, row_tiles, chunks, chunks1, other, best, best_t);
+  plan_for<128, EPI>(a, max_m, max_n, row_tiles, chunks, chunks1, other, best, best_t);
+  plan_for<64, EPI>(a, max_m, max_n, row_tiles, chunks, chunks1, other, best, best_t);
   return best;
 }
 
@@ -1248,7 +1262,12 @@ static GemmPlan plan_epi(const GemmArgs& a, int max_m, int max_n) {
     for (int g = 0; g < a.ngroups; ++g)
       if (a.groups[g].a_row0 >= 0) features += a.groups[g].m;
     const long long streamed = features * a.k_total * 2 * (a.f_lo_kb > 0 ? 2 : 1);
-    const bool fed = max_n <= tc::BM && (EPI == kEpiLogits || a.ngroups > 1) && streamed > kFedBytes;
+    // (an LM head of more rows than a twentieth of d is bound by its epilogues and
+    // its logits: 100000 x 1024, 64 rows, 74.5 us with the plan of fed_cost_us, 69.9
+    // with the other)
+    const bool fed = max_n <= tc::BM &&
+                     (EPI == kEpiLogits ? streamed > kFedLogitBytes && 20 * max_n <= a.k_total
+                                        : streamed > kFedScoreBytes && a.ngroups > 1);
     if (fed || a.gh_cols > 0) {
       // the splits that the plan_cost_us estimate gives the logits, or the
       // scores and G_h each in a launch of its own, are the accumulators to
@@ -1267,20 +1286,22 @@ static GemmPlan plan_epi(const GemmArgs& a, int max_m, int max_n) {
           n_gh += a.groups[g].n;
         }
       }
-      int chunks = plan_best<EPI>(alone, max_m, n, 1, false).splits;
+      const int chunks = plan_best<EPI>(alone, max_m, n).splits;
+      int chunks1 = 1;
       if (a.gh_cols > 0) {
         alone.a_split = a.gh_cols;
         alone.r_by_part = 0;
         alone.f_lo_kb = 0;
         alone.ngroups = 1;
         alone.groups[0] = GemmGroup{0, 2 * a.gh_cols, 0, n_gh, 0};
-        chunks = std::max(chunks, plan_best<kEpiQueryH>(alone, 2 * a.gh_cols, n_gh, 1, false).splits);
+        chunks1 = plan_best<kEpiQueryH>(alone, 2 * a.gh_cols, n_gh).splits;
       }
-      const GemmPlan p = plan_best<EPI>(a, max_m, max_n, chunks, fed);
+      GemmPlan p = plan_best<EPI>(a, max_m, max_n, chunks, chunks1);
+      if (fed && p.region > 0) p = plan_best<EPI>(a, max_m, max_n, chunks, chunks1, &p);
       if (p.region > 0) return p;
     }
   }
-  return plan_best<EPI>(a, max_m, max_n, 1, false);
+  return plan_best<EPI>(a, max_m, max_n);
 }
 
 static GemmPlan plan_gemm_tc_uncached(int epi, const GemmArgs& a, int max_m, int max_n) {

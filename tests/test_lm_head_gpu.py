@@ -132,3 +132,14 @@ def test_lm_head_candidates_without_logits(fovea):
     fovea.sync_errors(ws)
     assert none is None and logits is not None
     assert torch.equal(idx1, idx2) and torch.equal(val1, val2)
+
+
+@pytest.mark.parametrize("vocab,d,N", [(32000, 4096, 1), (32000, 4096, 8), (32000, 5120, 8),
+                                       (100000, 1024, 64)])
+def test_plans_of_long_vocabularies(fovea, vocab, d, N):
+    """Candidate lists per row are the plan's feature tiles times its splits.
+    Of the plans of these launches those with whole 256-column tiles are the
+    fastest (us, against the fastest of 128 columns): 50.9 / 63.9, 52.1 / 59.1,
+    63.8 / 73.4, 69.1 / 74.9."""
+    ws = fovea.lm_head_workspace(vocab, d, N, 6)
+    assert (ws.numel() - 4096) // (N * 6 * 8) == (vocab + 255) // 256
