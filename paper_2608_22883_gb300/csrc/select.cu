@@ -46,12 +46,12 @@ __global__ void __launch_bounds__(kSelThreads, 4) select_kernel(const __grid_con
   const int key_off = tab.key_off[b];
   BlockSyncT<kLargeCaps> sync;
   if constexpr (PT > 0) {
-    select_row<PT>(a, n, M, key_off, src, sm, tid, sync);
+    select_row<PT, true>(a, n, M, key_off, src, sm, tid, sync);
   } else {
     for (int i = tid; i < M; i += kSelThreads) s_sc[i] = norm_score(src[i]);
     __syncthreads();
     if (!select_wide(a, n, M, key_off, s_sc, sm, tid, sync))
-      select_radix(a, n, M, key_off, s_sc, sm, tid, sync);
+      select_radix_call(a, n, M, key_off, s_sc, sm, tid, sync);
   }
 }
 
@@ -361,9 +361,9 @@ __global__ void __launch_bounds__(NT) select_gather_kernel(
     } else {
       const float* src = a.scores + tab.score_off[b] + (long long)(n - tab.row_start[b]) * M;
       if constexpr (NT == kSelThreads)
-        select_row<kFastMaxM / kSelThreads>(a, n, M, tab.key_off[b], src, sm, tid, BlockSync{});
+        select_row<kFastMaxM / kSelThreads, false>(a, n, M, tab.key_off[b], src, sm, tid, BlockSync{});
       else
-        select_row<kFastMaxM / kSelThreads>(a, n, M, tab.key_off[b], src, sm, tid, SelGroupSync{});
+        select_row<kFastMaxM / kSelThreads, false>(a, n, M, tab.key_off[b], src, sm, tid, SelGroupSync{});
     }
   }
   // rank 0's selection visible to the cluster (one CTA: a CTA barrier, which
