@@ -369,18 +369,21 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
   m->M_max = M_max;
   m->d = d;
   m->dtype = p->dtype;
-  // temporaries: error word, valid counts | source rows | LN(v) | marks of the
-  // key elements | W_Q^T
+  // temporaries: error word, valid counts, norms of W_K's rows | source rows |
+  // LN(v) | marks of the key elements, RMS of the token rows | W_Q^T
   void* scratch = nullptr;
   void* src_row = nullptr;
   void* xv = nullptr;
   void* fix = nullptr;
   void* wqt = nullptr;
   auto run = [&]() -> fovea_status {
-    fovea_status rs = alloc_dev(&scratch, 256 + align_up(B * sizeof(int32_t), 256), "build scratch", pool, s);
+    const bool bf = p->dtype == FOVEA_BF16;
+    const size_t count_bytes = align_up(B * sizeof(int32_t), 256);
+    fovea_status rs = alloc_dev(&scratch, 256 + count_bytes + d * sizeof(float), "build scratch", pool, s);
     if (rs != FOVEA_OK) return rs;
     int* errw = static_cast<int*>(scratch);           // error word
     int32_t* d_counts = reinterpret_cast<int32_t*>(static_cast<uint8_t*>(scratch) + 256);
+    float* feat_norm = reinterpret_cast<float*>(static_cast<uint8_t*>(scratch) + 256 + count_bytes);
     FOVEA_CUDA(cudaMemsetAsync(scratch, 0, 256, s), "cudaMemsetAsync");
     m->counts.assign(B, M_max);
     cudaError_t err = cudaSuccess;
@@ -407,7 +410,6 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
     m->total = (int)m->offsets[B];
     const int total = m->total;
     if (total == 0) return FOVEA_OK;
-    const bool bf = p->dtype == FOVEA_BF16;
     const int H = p->mlp_hidden;
     // bf16 with W_Q given: the folded keys; with the fusion weights given: the
     // projected values and their transpose per image
@@ -415,13 +417,15 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
     const bool proj = bf && p->W_f1 != nullptr && p->W_g1 != nullptr && H > 0 && H % 128 == 0 &&
                       H <= FOVEA_MAX_H && aligned16(p->W_f1) && aligned16(p->W_g1);
     const int ld = (m_max + 63) / 64 * 64;
+    // bf16: the marks, the RMS of the token rows
+    const size_t mark_bytes = align_up((size_t)total * d / 8, 256);
     if ((rs = alloc_dev(&m->keys, (size_t)total * d * es, "keys", pool, s)) != FOVEA_OK ||
         (rs = alloc_dev(&m->values, (size_t)total * d * es, "values", pool, s)) != FOVEA_OK ||
         (rs = alloc_dev(reinterpret_cast<void**>(&m->orig_index), total * sizeof(int32_t), "index",
                         pool, s)) != FOVEA_OK ||
         (rs = alloc_dev(&src_row, total * sizeof(int32_t), "source rows", pool, s)) != FOVEA_OK ||
         (rs = alloc_dev(&xv, (size_t)total * d * es, "LN(v)", pool, s)) != FOVEA_OK ||
-        (bf && (rs = alloc_dev(&fix, (size_t)total * d / 8, "key marks", pool, s)) != FOVEA_OK) ||
+        (bf && (rs = alloc_dev(&fix, mark_bytes + (size_t)total * 4, "key marks", pool, s)) != FOVEA_OK) ||
         (fold && (rs = alloc_dev(&m->folded, (size_t)total * 2 * d * 2, "folded keys", pool, s)) != FOVEA_OK) ||
         (fold && total > kFoldByRowTokens &&
          (rs = alloc_dev(&wqt, (size_t)d * d * 2, "transposed W_Q", pool, s)) != FOVEA_OK) ||
@@ -429,12 +433,14 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
         (proj && (rs = alloc_dev(&m->projT, (size_t)B * 2 * H * ld * 2, "transposed projected values",
                                  pool, s)) != FOVEA_OK))
       return rs;
+    float* row_rms = bf ? reinterpret_cast<float*>(static_cast<uint8_t*>(fix) + mark_bytes) : nullptr;
     { KernelTimer t("compact", s);
-      err = launch_compact(mask, B, M_max, itab, m->orig_index, (int32_t*)src_row, s); }
+      err = launch_compact(mask, B, M_max, itab, m->orig_index, (int32_t*)src_row,
+                           RowNorms{p->W_K, d, bf ? feat_norm : nullptr}, s); }
     if (err != cudaSuccess) return cuda_fail(err, "compact");
     { KernelTimer t("ln_v", s);
       err = launch_ln_rows(p->dtype, v, (const int32_t*)src_row, total, d, p->ln_v_gamma,
-                           p->ln_v_beta, p->ln_eps, xv, s); }
+                           p->ln_v_beta, p->ln_eps, xv, row_rms, s); }
     if (err != cudaSuccess) return cuda_fail(err, "ln_v");
     if (!bf) {
       static thread_local GemmArgs a;
@@ -458,6 +464,8 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
       pg.out[0] = m->keys; pg.out[1] = m->values;
       pg.ldc[0] = pg.ldc[1] = d;
       pg.fix_bits = static_cast<uint32_t*>(fix);
+      pg.row_rms = row_rms;
+      pg.feat_norm = feat_norm;
       const TmaOperand none{nullptr, 0, 0, 0}, tokens{xv, total, d, d};
       const TmaOperand kv[3] = {TmaOperand{p->W_K, d, d, d}, TmaOperand{p->W_U, d, d, d}, none};
       { KernelTimer t("memory_proj", s);

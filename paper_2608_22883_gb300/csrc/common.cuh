@@ -253,9 +253,10 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t sme
 // Sets the message fovea_last_error() returns on this thread (api.cu).
 fovea_status report_error(fovea_status st, const char* msg);
 
-// LN of the gathered token rows (rowops.cu): out[r] = LN(x[src_row[r]]).
+// LN of the gathered token rows (rowops.cu): out[r] = LN(x[src_row[r]]); bf16:
+// the root mean square of out[r] to rms[r].
 cudaError_t launch_ln_rows(int dtype, const void* x, const int32_t* src_row, int rows, int d,
-                           const void* gamma, const void* beta, float eps, void* out,
+                           const void* gamma, const void* beta, float eps, void* out, float* rms,
                            cudaStream_t s);
 // LN of the draft hidden states plus the depth embedding (rowops.cu), fp32.
 cudaError_t launch_ln_query(int dtype, const void* h, int rows, int d, const void* gamma,
@@ -269,8 +270,15 @@ struct ImageTable {
   int off[FOVEA_MAX_SEQ];
   int m[FOVEA_MAX_SEQ];
 };
+// The norms of the rows of W (bf16 [d, d]; norms null: none), which the
+// compaction's launch takes along.
+struct RowNorms {
+  const void* W;
+  int d;
+  float* norms;
+};
 cudaError_t launch_compact(const uint8_t* mask, int B, int M_max, const ImageTable& tab,
-                           int32_t* orig_index, int32_t* src_row, cudaStream_t s);
+                           int32_t* orig_index, int32_t* src_row, const RowNorms& nw, cudaStream_t s);
 // Selection alone (select.cu): counts, indices, and per row the selected
 // compacted memory rows and weights (sel_pos, sel_w, sel_cnt; any may be
 // null), and / or the weights as dense bf16 hi / lo rows over the row's
@@ -371,6 +379,8 @@ struct PairGemm {
   void* out[3]; long long ldc[3]; void* out_lo;
   bool f0_by_row;
   uint32_t* fix_bits;                            // keys: bit c % 32 of [row * ldc[0] / 32 + c / 32]
+  const float* row_rms;                          // keys: root mean square of each token row,
+  const float* feat_norm;                        // norm of each row of F[0]
   int* err;
   // filled by the launch
   int k_blocks, cols[3], tile_end[3], feat_tiles, row_tiles;

@@ -88,14 +88,24 @@ constexpr uint64_t kMnBlock = (uint64_t)(KPS * 64 * 128 >> 4);
 static_assert(BNH == KPS * 64, "one box for both orders of the features");
 
 // Key window: an element is marked when its sum lies within
-// kKeyWindow * max(|sum|, scale) of a bf16 rounding midpoint, scale being the
-// RMS of the token's sums over its half of the tile.  With chunked sums the
-// farthest mis-rounded key from its midpoint, over 3.7e8 keys at d = 256 ..
-// 8192 (none refined, compared with float64), lay 2^-20.4 of that magnitude
-// away, with no trend in d (0.017 % of the keys were mis-rounded); 2^-19
-// keeps a margin of 2.6x and marks 0.47 % of the keys.  One accumulator over
-// the whole contraction needs 2^-15 and marks 5 %: at 32768 tokens, d = 4096
-// their recomputation took 11.0 ms of a 17.5 ms build, now 0.85 ms.
+// kKeyWindow * max(|sum|, scale) of a bf16 rounding midpoint.  The error of a sum
+// follows its partial sums, so scale is the largest of three sizes of theirs: the
+// RMS of the token's sums over its half of the tile, the same of the chunks that
+// they are made of (a component that every token shares and the row cancels), and
+// |x| |w| / sqrt(d) of the element's own token and feature (rows of unequal size).
+// With chunked sums the farthest mis-rounded key from its midpoint, over 3.7e8
+// keys of independent normal data at d = 256 .. 8192 (none refined, compared with
+// float64), lay 2^-20.4 of the first size away, with no trend in d (0.017 % of the
+// keys were mis-rounded); 2^-19 keeps a margin of 2.6x.  Of 2.1e6 keys at d = 4096
+// with a shared component 10 and 33 times the rest, the first size alone left 176
+// and 3820 wrong, and with rows 64 times their neighbours that the tokens cancel
+// 261; with all three none is.  (Products whose signs are arranged along the
+// contraction within a chunk, so that every chunk cancels by itself, can err by
+// more: no bound short of |x| |w| holds for them, and that marks a third of the
+// keys.)  The two further sizes cost a build of 32768 tokens about 45 us here, 22 in
+// the recomputation and 6 for the norms, of 3410.  One accumulator over the whole
+// contraction needs 2^-15 and marks 5 % instead of 0.5: at 32768 tokens, d = 4096
+// their recomputation took 11.0 ms of a 17.5 ms build, now 0.87 ms.
 constexpr float kKeyWindow = 1.0f / 524288.0f;   // 2^-19
 
 __device__ __forceinline__ uint32_t cta_rank() {
@@ -366,6 +376,7 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
       float acc[BNH];
 #pragma unroll
       for (int j = 0; j < BNH; ++j) acc[j] = 0.0f;
+      float cs[2] = {};                          // keys: squares of every fourth column's chunk sums
       const int chunk = a.chunk[ti.part];
       int su0 = 0;
       for (int len = a.chunk0[ti.part]; su0 < su_total; su0 += len, len = chunk, ++c) {
@@ -384,6 +395,10 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
           tmem_ld16(src + (uint32_t)(16 * q), v);
 #pragma unroll
           for (int j = 0; j < 16; ++j) acc[16 * q + j] += v[j];
+          if (KEYS) {
+#pragma unroll
+            for (int j = 0; j < 16; j += 4) cs[(j >> 2) & 1] = fmaf(v[j], v[j], cs[(j >> 2) & 1]);
+          }
         }
         tc_fence_before();
         __syncwarp();
@@ -399,14 +414,20 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
         float ss = 0.0f;                       // columns past the matrix are zeros
 #pragma unroll
         for (int j = 0; j < BNH; ++j) ss = fmaf(acc[j], acc[j], ss);
-        const float scale = sqrtf(ss / (float)cols);
+        const float scale = sqrtf(fmaxf(ss, 4.0f * (cs[0] + cs[1])) / (float)cols);
+        const float rms = row + lane < a.rows ? a.row_rms[row + lane] : 0.0f;
 #pragma unroll
         for (int q = 0; q < BNH / 32; ++q) {
           uint32_t bits = 0u;
           if (row + lane < a.rows && 32 * q < cols) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j)
-              if (near_midpoint(acc[32 * q + j], scale)) bits |= 1u << j;
+            for (int j = 0; j < 32; j += 4) {
+              const float4 w = __ldg(reinterpret_cast<const float4*>(a.feat_norm + col0 + 32 * q + j));
+              if (near_midpoint(acc[32 * q + j], fmaxf(scale, rms * w.x))) bits |= 1u << j;
+              if (near_midpoint(acc[32 * q + j + 1], fmaxf(scale, rms * w.y))) bits |= 2u << j;
+              if (near_midpoint(acc[32 * q + j + 2], fmaxf(scale, rms * w.z))) bits |= 4u << j;
+              if (near_midpoint(acc[32 * q + j + 3], fmaxf(scale, rms * w.w))) bits |= 8u << j;
+            }
           }
           need[q] = bits;
         }

@@ -173,7 +173,7 @@ template <int kRowWarps>
 __global__ void __launch_bounds__(32 * kLnTokWarps) ln_tokens_kernel(
     const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ src_row, int rows, int d,
     const __nv_bfloat16* __restrict__ gamma, const __nv_bfloat16* __restrict__ beta, float eps,
-    __nv_bfloat16* __restrict__ out) {
+    __nv_bfloat16* __restrict__ out, float* __restrict__ rms) {
   extern __shared__ __align__(16) uint4 ln_sm[];     // gamma [d], beta [d], the rows in work
   __shared__ float4 parts[kLnTokWarps];
   constexpr int kRows = kLnTokWarps / kRowWarps;     // rows a CTA works on at a time
@@ -243,6 +243,7 @@ __global__ void __launch_bounds__(32 * kLnTokWarps) ln_tokens_kernel(
     // 2^-22 (|product| + |y|) + 2^-23 |mean| rstd |gamma|
     const float mr = fabsf(mean.hi) * rstd.hi * 1.1920929e-7f;
     __nv_bfloat16* o = out + (long long)row * d;
+    f32x2 sq = x2_pack(0.0f, 0.0f);                        // of the results, for their RMS
 #pragma unroll 1                                       // a lane reads the vectors it stored above
     for (int vi = lane; vi < nvec; vi += kLanes) {
       const uint4 xv = x_s[vi], gr = g_s[vi], br = b_s[vi];
@@ -269,6 +270,8 @@ __global__ void __launch_bounds__(32 * kLnTokWarps) ln_tokens_kernel(
         }
         const __nv_bfloat162 p = __floats2bfloat162_rn(y[0], y[1]);
         ow[q] = *reinterpret_cast<const uint32_t*>(&p);
+        const f32x2 yy = x2_pack(y[0], y[1]);
+        sq = x2_add(sq, x2_mul(yy, yy));
       }
       reinterpret_cast<uint4*>(o)[vi] = make_uint4(ow[0], ow[1], ow[2], ow[3]);
       while (slow != 0u) {                             // the exact value, after the vector store
@@ -281,6 +284,16 @@ __global__ void __launch_bounds__(32 * kLnTokWarps) ln_tokens_kernel(
         o[e] = df_to_bf16(df_add_f(df_mul_f(t, gf), bf));
       }
     }
+    float ssq = warp_sum(x2_unpack(sq).x + x2_unpack(sq).y);
+    if constexpr (kRowWarps > 1) {
+      if ((threadIdx.x & 31) == 0) parts[threadIdx.x >> 5].x = ssq;
+      __syncthreads();
+      ssq = 0.0f;
+#pragma unroll
+      for (int w = 0; w < kRowWarps; ++w) ssq += parts[w].x;
+      __syncthreads();                               // before the next row's parts
+    }
+    if (lane == 0) rms[row] = sqrtf(ssq / (float)d);
   }
 }
 
@@ -443,7 +456,7 @@ cudaError_t launch_ln_query(int dtype, const void* h, int rows, int d, const voi
 }
 
 cudaError_t launch_ln_rows(int dtype, const void* x, const int32_t* src_row, int rows, int d,
-                           const void* gamma, const void* beta, float eps, void* out,
+                           const void* gamma, const void* beta, float eps, void* out, float* rms,
                            cudaStream_t s) {
   if (rows == 0) return cudaSuccess;
   if (dtype != FOVEA_BF16)
@@ -466,7 +479,7 @@ cudaError_t launch_ln_rows(int dtype, const void* x, const int32_t* src_row, int
   const int most = sms * (per_sm > 0 ? per_sm : 1);
   return launch_pdl(kern, dim3(ctas < most ? ctas : most), dim3(32 * kLnTokWarps),
                     smem, s, (const __nv_bfloat16*)x, src_row, rows, d, (const __nv_bfloat16*)gamma,
-                    (const __nv_bfloat16*)beta, eps, (__nv_bfloat16*)out);
+                    (const __nv_bfloat16*)beta, eps, (__nv_bfloat16*)out, rms);
 }
 
 // ---------------------------------------------------------------------------
@@ -474,6 +487,22 @@ cudaError_t launch_ln_rows(int dtype, const void* x, const int32_t* src_row, int
 // counts, then an ordered compaction of valid positions.
 // ---------------------------------------------------------------------------
 constexpr int kScanThreads = 256;
+
+// Norms of the rows of W, a warp each: CTA `cta` of the extra ones of a launch.
+__device__ __forceinline__ void row_norms(const RowNorms& nw, int cta) {
+  const int r = cta * (kScanThreads / 32) + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (r >= nw.d) return;
+  const uint4* w = static_cast<const uint4*>(nw.W) + (long long)r * (nw.d / 8);
+  float ss = 0.0f;
+  for (int v = lane; v < nw.d / 8; v += 32) {
+    float x[8];
+    ln_unpack<__nv_bfloat16>(__ldg(w + v), x);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) ss = fmaf(x[i], x[i], ss);
+  }
+  ss = warp_sum(ss);
+  if (lane == 0) nw.norms[r] = sqrtf(ss);
+}
 
 __global__ void __launch_bounds__(kScanThreads) count_valid_kernel(const uint8_t* __restrict__ mask,
                                                                   int M_max,
@@ -491,9 +520,11 @@ __global__ void __launch_bounds__(kScanThreads) compact_kernel(const uint8_t* __
                                                               int M_max,
                                                               const __grid_constant__ ImageTable tab,
                                                               int32_t* __restrict__ orig_index,
-                                                              int32_t* __restrict__ src_row) {
+                                                              int32_t* __restrict__ src_row,
+                                                              const RowNorms nw) {
   __shared__ int warp_tot[kScanThreads / 32];
   const int b = blockIdx.x;
+  if (b >= tab.B) return row_norms(nw, b - tab.B);
   const int chunk = (M_max + kScanThreads - 1) / kScanThreads;
   const int beg = min(M_max, threadIdx.x * chunk), end = min(M_max, beg + chunk);
   const uint8_t* mb = mask ? mask + (long long)b * M_max : nullptr;
@@ -529,8 +560,9 @@ cudaError_t launch_count_valid(const uint8_t* mask, int B, int M_max, int32_t* c
 }
 
 cudaError_t launch_compact(const uint8_t* mask, int B, int M_max, const ImageTable& tab,
-                           int32_t* orig_index, int32_t* src_row, cudaStream_t s) {
-  compact_kernel<<<B, kScanThreads, 0, s>>>(mask, M_max, tab, orig_index, src_row);
+                           int32_t* orig_index, int32_t* src_row, const RowNorms& nw, cudaStream_t s) {
+  const int norm_ctas = nw.norms != nullptr ? (nw.d + kScanThreads / 32 - 1) / (kScanThreads / 32) : 0;
+  compact_kernel<<<B + norm_ctas, kScanThreads, 0, s>>>(mask, M_max, tab, orig_index, src_row, nw);
   return cudaGetLastError();
 }
 

@@ -203,6 +203,48 @@ def test_keys_beside_a_rounding_midpoint(fovea, d, m):
     mem.destroy()
 
 
+def round_bf16(x):
+    """float64 values rounded once to bf16 (.to() rounds to float32 on the way)."""
+    b = x.contiguous().view(torch.int64)
+    b = (b + (1 << 44) - 1 + ((b >> 45) & 1)) >> 45 << 45
+    return b.view(torch.float64)
+
+
+# partial sums far above the keys: a component that every token shares (the bias
+# of the token norm) and that the rows of W_K nearly cancel; rows of W_K far
+# larger than their neighbours whose sums cancel; both, below one chunk of 256
+# elements, of a few and of many chunks
+@pytest.mark.parametrize("d", [128, 1024, 4096])
+@pytest.mark.parametrize("shared,tall", [(0.0, 1.0), (10.0, 1.0), (33.0, 1.0), (0.0, 64.0), (10.0, 64.0)])
+def test_keys_whose_partial_sums_cancel(fovea, d, shared, tall):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d)
+    m = 1 << 21 >> (d.bit_length() - 1)
+    weights, normal = device_weights(g, d)
+    weights["ln_v_gamma"].fill_(1.0)
+    weights["ln_v_beta"] = normal(d, scale=shared)
+    W = torch.randn((d, d), generator=g, device="cuda", dtype=torch.float64) / d ** 0.5
+    if shared:
+        b = weights["ln_v_beta"].double()
+        W -= torch.outer(W @ b, b) / (b @ b)
+    W[::64] *= tall
+    weights["W_K"] = W.to(torch.bfloat16)
+    params = fovea.Params(weights, d_model=d)
+    v = normal(1, m, d)
+    if tall > 1:                            # the tall rows' sums cancel for these tokens, roughly
+        t = W[::64]
+        v = (v.double()[0] - v.double()[0] @ torch.linalg.pinv(t) @ t).to(torch.bfloat16)[None]
+    mem = fovea.build_memory(params, v)
+    x = v[0].double()
+    c = x - x.mean(1, keepdim=True)
+    x = c / torch.sqrt((c * c).mean(1, keepdim=True) + LN_EPS) + weights["ln_v_beta"].double()
+    ref = round_bf16(round_bf16(x) @ weights["W_K"].double().T)
+    wrong = int((mem.views()[0].double() != ref).sum())
+    print(f"d {d} shared {shared} tall {tall}: {wrong} of {ref.numel()}")
+    assert wrong <= 1e-6 * ref.numel()
+    mem.destroy()
+
+
 # row lengths below, at and past a warp's pass of 256 elements and its batch of
 # eight vectors per lane, four warps per row (few rows) and one; means up to 1000
 # standard deviations away, where the fp32 map is seldom sure of its rounding
