@@ -63,12 +63,13 @@ __device__ __forceinline__ float sigmoidf_(float z) { return __frcp_rn(1.0f + __
 // -z log2 e, its rounding error put back to first order, and one approximate
 // division.  Measured against float64 for z in [-86, 30]: mean error 0.73 x
 // 2^-24, largest 5.2 (z * sigmoidf_(z): 12.0 and 65; for |z| < 4 0.73 and 0.81).
-// The exponential's argument is held to [-88, 87]: below z = -87 SiLU is below
-// 1e-35 in size and stays there.
+// Below z = -87.3, where SiLU is under 1e-36 in size, the divisor lies between 2^126
+// and 2^128 (the exponential's argument is held to [-88, 88]), and __fdividef gives
+// 0 there.
 __device__ __forceinline__ float siluf_(float z) {
   constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
   constexpr float kLog2eLo = (float)(1.4426950408889634 - (double)kLog2e);
-  const float zc = fminf(fmaxf(z, -87.0f), 88.0f);
+  const float zc = fminf(fmaxf(z, -88.0f), 88.0f);
   const float t = -zc * kLog2e;
   const float lo = fmaf(-zc, kLog2eLo, fmaf(-zc, kLog2e, -t));
   const float e = exp2f(t);

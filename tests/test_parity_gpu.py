@@ -368,6 +368,66 @@ def test_gather_after_the_selection(fovea, d, m_sizes, rows, k, H):
     compare(gpu, orc, s, mem=mem, max_exempt=0.2)
 
 
+def test_silu_against_float64(fovea):
+    """fp32, W_f1 = W_g1 = 0: the activations left in the workspace are
+    SiLU(b), 8192 of them a step.  The exponential errs by a unit in its last
+    place and the division by two, and the sum 1 + exp(-z) rounds once: 6 x
+    2^-24 in all, half a unit on average for each.  Below -87 the value is
+    subnormal or zero; it never grows again."""
+    d, H = 64, 4096
+    w = workloads.generate_custom("silu", d, [3], [1], dtype="fp32", k_max=2, H=H)
+    for n in ("W_f1", "W_g1"):
+        w.params[n] = np.zeros_like(w.params[n])
+    sweeps = [np.linspace(-86, 30, 2 * H), np.linspace(-4, 4, 2 * H)]
+    sweeps.append(np.concatenate([np.linspace(-120, -87, H), -np.logspace(2, 38.5, H)]))
+    for k, z in enumerate(sweeps):
+        z = z.astype(np.float32)
+        w.params["b_f1"], w.params["b_g1"] = z[:H], z[H:]
+        s = store(w)
+        params = params_for(s, fovea)
+        mem = fovea.build_memory(params, s.dev["v"], s.dev.get("mask"))
+        out = fovea.step(params, mem, s.dev["h"], s.dev["depth"], w.row_offsets, None, w.rho, 1, 2)
+        fovea.sync_errors(out["workspace"])
+        off = 4096
+        for n in (4 * d, 4 * d, 12, 8, 8, 4, 4 * d):      # x, q, scores, positions, weights, count, r
+            off += (n + 255) // 256 * 256
+        act = out["workspace"][off:off + 8 * H].view(torch.float32).double().cpu().numpy()
+        z = z.astype(np.float64)
+        with np.errstate(over="ignore"):
+            ref = z / (1.0 + np.exp(-z))
+        if k < 2:
+            err = np.abs(act - ref)[ref != 0] / np.abs(ref[ref != 0]) * 2.0 ** 24
+            assert err.max() <= 6.0 and err.mean() <= 1.0, (err.max(), err.mean())
+        else:
+            assert np.all(np.abs(act - ref) <= 2.0 ** -118), np.abs(act - ref).max()
+        mem.destroy()
+
+
+# the activation epilogues of the selection + gather, the gather and the
+# weighted-sum kernels, the first fusion layer's GEMM (other weights than the
+# memory was built with) and fp32
+@pytest.mark.parametrize("d,m,rows,k,dtype,plain", [(256, 90, 5, 16, "bf16", False), (256, 200, 5, 100, "bf16", False),
+                                                    (256, 600, 5, 400, "bf16", False), (256, 90, 5, 16, "bf16", True),
+                                                    (64, 90, 5, 16, "fp32", False)])
+def test_very_negative_pre_activations_vanish(fovea, d, m, rows, k, dtype, plain):
+    """b_f1 near the type's lowest value: SiLU gives 0 and the correction is
+    b_f2 alone."""
+    w = workloads.generate_custom("silu-tail", d, [m], [rows], dtype=dtype, k_max=k, seed=k, H=128)
+    w.params["b_f1"] = np.full_like(w.params["b_f1"], -3e38)
+    s = store(w)
+    params = params_for(s, fovea)
+    mem = fovea.build_memory(params, s.dev["v"], s.dev.get("mask"))
+    if plain:
+        weights = {n: s.dev[n] for n in workloads.PARAM_NAMES}
+        weights["W_f1"], weights["W_g1"] = weights["W_f1"].clone(), weights["W_g1"].clone()
+        params = fovea.Params(weights, d_model=d, mlp_hidden=128, max_depth=w.params["E_dep"].shape[0] - 1)
+    gpu = run_gpu(s, fovea, params=params, memory=mem)
+    y = s.f64["h"] + gpu["gate"].astype(np.float64)[:, None] * s.f64["b_f2"]
+    want = oracle.rms_norm(y, s.f64["rms_gamma"], RMS_EPS)
+    assert rel_err_rows(gpu["h_out"].astype(np.float64), want).max() <= (5e-3 if dtype == "bf16" else 1e-5)
+    mem.destroy()
+
+
 def test_plain_fusion_when_weights_differ(fovea):
     """The memory keeps the values projected through the r-half of the first
     fusion layer for the W_f1 / W_g1 it was built with.  A bf16 call given
