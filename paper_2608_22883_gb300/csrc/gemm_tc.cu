@@ -751,7 +751,6 @@ __global__ void __launch_bounds__(kThreads, 2)
           }
         }
       }
-      __syncwarp();
       cluster_sync();
       const int qlo = (int)rank * (BN / 4) / S, qhi = ((int)rank + 1) * (BN / 4) / S;
       const int q4 = qhi - qlo;
@@ -799,10 +798,7 @@ __global__ void __launch_bounds__(kThreads, 2)
               acc[k].w += t[k][sidx].w;
             }
         }
-        if (rd == rounds - 1) {
-          __syncwarp();
-          cluster_arrive();   // this CTA's remote reads are done
-        }
+        if (rd == rounds - 1) cluster_arrive();   // this CTA's remote reads are done
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
           if (rr[k] < 0) continue;
@@ -825,10 +821,7 @@ __global__ void __launch_bounds__(kThreads, 2)
           }
         }
       }
-      if (rounds == 0) {
-        __syncwarp();
-        cluster_arrive();
-      }
+      if (rounds == 0) cluster_arrive();
       if constexpr (EPI == kEpiLogits) {
         __syncthreads();
         tile_topk<BN>(args, (long long)g.b_row0 + n0, rows_real, sums, q4 * 4, m0 + qlo * 4,

@@ -107,7 +107,9 @@ constexpr int kRoUnroll = 8;
 constexpr int kStageRows = 64;                 // staged gather: rows per round
 constexpr int kGatherSmemMax = 200 * 1024;     // dynamic shared memory of the gather kernel
 static inline size_t align_up_sz(size_t x, size_t a) { return (x + a - 1) / a * a; }
+using tc::cluster_arrive;
 using tc::cluster_sync;
+using tc::cluster_wait;
 using tc::ld_dsmem_f4;
 using tc::map_dsmem;
 using tc::smem_u32;
@@ -116,12 +118,6 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
-}
-__device__ __forceinline__ void cluster_arrive() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() {
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ int ld_dsmem_s32(uint32_t caddr) {
   int v;

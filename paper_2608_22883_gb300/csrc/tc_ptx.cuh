@@ -93,17 +93,21 @@ static __device__ __noinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, vo
 // Thread-block cluster: a full barrier over every thread of the cluster
 // (shared-memory writes before it are visible to the cluster after it), the
 // address of a shared-memory location in CTA `rank` of the cluster, and a
-// 16-byte load through that address (distributed shared memory).
+// 16-byte load through that address (distributed shared memory).  The barriers
+// are .aligned: each makes its warp converge first, whatever loops it left.
 __device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
                "barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // The two halves of cluster_sync, for work placed between them (every thread
 // of the cluster arrives once and then waits once).
 __device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ uint32_t map_dsmem(uint32_t saddr, uint32_t rank) {

@@ -277,6 +277,8 @@ def test_token_layer_norm_is_correctly_rounded(fovea, d, mean, std, m):
 # split) up to a full split, more tiles than the GPU holds
 @pytest.mark.parametrize("d,m_sizes,rows", [(64, [1, 65], [1, 63]), (64, [64], [65]),
                                             (192, [127, 0, 3], [2, 5, 64]), (1024, [130], [64]),
+                                            # a warp's two rows of the split sum: one past the last
+                                            (1024, [130], [33]),
                                             (512, [700] * 6, [100] * 6)])
 def test_fp32_tile_edges(fovea, d, m_sizes, rows):
     w = workloads.generate_custom("fp32-edges", d, m_sizes, rows, dtype="fp32", k_max=16, seed=d,
