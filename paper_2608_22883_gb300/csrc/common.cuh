@@ -104,13 +104,7 @@ __device__ __forceinline__ float warp_sum(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-__device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-
-// Block-wide sum / max; `scratch` holds >= 32 floats.  Every thread returns
+// Block-wide sum; `scratch` holds >= 32 floats.  Every thread returns
 // the result.  Contains __syncthreads().
 __device__ __forceinline__ float block_sum(float v, float* scratch) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
@@ -120,15 +114,6 @@ __device__ __forceinline__ float block_sum(float v, float* scratch) {
   __syncthreads();
   float t = lane < nw ? scratch[lane] : 0.0f;
   return warp_sum(t);
-}
-__device__ __forceinline__ float block_max(float v, float* scratch) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  v = warp_max(v);
-  __syncthreads();
-  if (lane == 0) scratch[warp] = v;
-  __syncthreads();
-  float t = lane < nw ? scratch[lane] : -INFINITY;
-  return warp_max(t);
 }
 
 // ---------------------------------------------------------------------------
@@ -351,7 +336,6 @@ struct TmaOperand {     // a row-major [rows, cols] bf16 matrix with a row strid
 // the fp32 scratch (partial tiles) that split needs.
 struct GemmPlan {
   int bn, splits, stages;
-  long long partial_floats;   // global fp32 scratch the launch needs (0: none)
   long long tiles;            // output tiles
   int rbox, rbox1;            // rows of a row-operand load of B0 and of B1 (64 .. 128)
   int region;                 // bytes of the ring / partial-tile staging region

@@ -1219,7 +1219,7 @@ static void plan_for(const GemmArgs& a, int max_m, int max_n, long long row_tile
         }
         if (t < best_t - 1e-6 || (t < best_t + 1e-6 && tiles * S < best.tiles * best.splits)) {
           best_t = t;
-          best = GemmPlan{BN, S, stages, 0, tiles, rbox, rbox1, region, kps, nacc, nacc1};
+          best = GemmPlan{BN, S, stages, tiles, rbox, rbox1, region, kps, nacc, nacc1};
         }
       }
     }
@@ -1240,7 +1240,7 @@ template <int EPI>
 static GemmPlan plan_best(const GemmArgs& a, int max_m, int max_n, int chunks = 1, int chunks1 = 1,
                           const GemmPlan* other = nullptr) {
   const long long row_tiles = (long long)(max_n + tc::BM - 1) / tc::BM * a.ngroups;
-  GemmPlan best{256, 1, 2, 0, 1 << 30, 128, 128, 0, 1, 1, 1};
+  GemmPlan best{256, 1, 2, 1 << 30, 128, 128, 0, 1, 1, 1};
   double best_t = 1e30;
   plan_for<256, EPI>(a, max_m, max_n, row_tiles, chunks, chunks1, other, best, best_t);
   plan_for<128, EPI>(a, max_m, max_n, row_tiles, chunks, chunks1, other, best, best_t);

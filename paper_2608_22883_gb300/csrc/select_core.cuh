@@ -94,7 +94,7 @@ struct SelectSmem {
   int warp_first[kSelWarps];
   unsigned int red_u[kSelWarps];
   unsigned int sh_digit, sh_above;
-  int sh_cnt_gt, sh_first;
+  int sh_cnt_gt;
   float sh_max, sh_sum;
 };
 
