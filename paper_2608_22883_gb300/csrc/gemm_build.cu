@@ -152,13 +152,25 @@ __device__ __forceinline__ uint32_t try_wait_cluster(uint64_t* bar, uint32_t par
       : "memory");
   return ok;
 }
+// The same without suspending the thread while the phase is incomplete.
+__device__ __forceinline__ uint32_t test_wait_cluster(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok;
+}
 // mbar_wait with cluster-scope acquire: the barrier is signalled by the peer.
 static __device__ __noinline__ bool wait_cluster(uint64_t* bar, uint32_t parity,
                                                  volatile int* abort_flag, uint64_t limit_ns) {
-  if (try_wait_cluster(bar, parity)) return true;
+  if (test_wait_cluster(bar, parity)) return true;
   const uint64_t t0 = globaltimer_ns();
-  while (true) {                            // (a try suspends the thread for a while by itself)
-    if (try_wait_cluster(bar, parity)) return true;
+  while (true) {
+    if (limit_ns < kSuspendNs ? test_wait_cluster(bar, parity) : try_wait_cluster(bar, parity)) return true;
     if (abort_flag != nullptr && *abort_flag) return false;
     if (globaltimer_ns() - t0 > limit_ns) return false;
   }

@@ -809,6 +809,32 @@ def test_bounded_wait_that_gives_up_reports_timeout(fovea):
     compare(gpu, orc, s, mem=omem, max_exempt=SMALL_MAX_EXEMPT["bf16-temperature"])
 
 
+@pytest.mark.parametrize("d,m", [(256, 700), (1024, 3000)])
+def test_bounded_waits_of_a_build_report_timeout(fovea, d, m):
+    """The same for the memory build's CTA pairs: the build fails with TIMEOUT
+    and frees what it had allocated, and the next one is not affected."""
+    w = workloads.generate_custom("build-timeout", d, [m], [1], seed=d, H=128)
+    s = store(w)
+    params = params_for(s, fovea)
+
+    def result():
+        mem = fovea.build_memory(params, s.dev["v"], s.dev.get("mask"))
+        out = [t.clone() for t in (*mem.views()[:2], mem.folded_keys(params))]
+        mem.destroy()
+        return out
+
+    want = result()
+    fovea.debug_wait_limit(1)
+    try:
+        for _ in range(2):
+            with pytest.raises(fovea.FoveaError, match="TIMEOUT"):
+                fovea.build_memory(params, s.dev["v"], s.dev.get("mask"))
+    finally:
+        fovea.debug_wait_limit(0)
+    for a, b in zip(want, result()):
+        assert torch.equal(a, b)
+
+
 def test_bad_row_offsets_and_workspace(fovea):
     w = small_workload("bf16-ragged")
     s = store(w)
