@@ -141,8 +141,11 @@ typedef struct fovea_params {
  * precision the unfolded scores give q = W_Q x_n), so both score forms
  * follow the paper's q . k to within fp32 accumulation.  Pass W_Q = NULL here
  * to keep the unfolded scores.
- * This call allocates the handle's device buffers and synchronises `stream`
- * once (to size them).  B in [1, FOVEA_MAX_SEQ], M_max in [0, ...],
+ * This call allocates the handle's device buffers (cudaMalloc memory, kept for
+ * later handles when this one goes: at most 2 GiB per device with the memory of
+ * the build's temporaries, all given back with the device's last handle) and
+ * synchronises `stream`, at the end and, with a mask, once more for the valid
+ * counts.  B in [1, FOVEA_MAX_SEQ], M_max in [0, ...],
  * per-image valid count <= FOVEA_MAX_ENTRIES.
  * Errors: INVALID_ARG, UNSUPPORTED, OOM, CUDA; *out is untouched on error.
  */
@@ -151,7 +154,9 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
                                           void* stream, fovea_memory** out);
 
 /* Release a memory handle (NULL is ignored).  The caller must make sure no
- * enqueued work still reads it (e.g. synchronise the stream first). */
+ * enqueued work still reads it (e.g. synchronise the stream first).  The call
+ * waits for the device; where that is not allowed (a stream is being captured)
+ * the memory is set aside until a later one has waited. */
 FOVEA_API void fovea_memory_destroy(fovea_memory* mem);
 
 /* Shape of a memory: number of images, total valid entries, and (if

@@ -109,8 +109,15 @@ struct KernelTimer {
 // ---------------------------------------------------------------------------
 // Memory handle
 // ---------------------------------------------------------------------------
+struct MemoryBlock {                 // a cudaMalloc allocation
+  void* ptr = nullptr;
+  size_t bytes = 0;
+};
+constexpr size_t kBlockGrain = 64 << 10;
+
 struct fovea_memory {
   int device = 0;
+  std::vector<MemoryBlock> blocks;   // what the buffers below lie in
   int B = 0, M_max = 0, d = 0, dtype = 0;
   int total = 0;
   std::vector<int32_t> counts;       // valid entries per image (host)
@@ -198,18 +205,22 @@ static fovea_status check_step_params(const fovea_params* p) {
 }
 
 // ---------------------------------------------------------------------------
-// Device memory of the handles and of a build's temporaries: one stream-ordered
-// pool per device.  cudaMalloc and cudaFree cost 30 - 180 us each, ten to
-// twelve of them 0.8 ms of a one-image build whose kernels take 0.3 ms; an
-// allocation from the pool costs about 1 us (mapping it anew, 0.3 ms for a
-// one-image build's buffers).  After every build and every freed handle the
-// pool keeps at most kPoolKeep bytes that nothing uses (under 1 % of the
-// device), and it gives everything back when the device's last handle goes.
-// (Its own release threshold counts the bytes in use too, so it is off.)  The
-// driver orders the pool's reuse between streams and threads.
+// Device memory.  cudaMalloc and cudaFree cost 30 - 180 us each, ten to twelve of
+// them 0.8 ms of a one-image build whose kernels take 0.2 ms, so both kinds of
+// memory are kept for the next build, per device:
+//   * a handle's buffers are cudaMalloc blocks (their views can be exported to
+//     other processes and read by peers), rounded up by an eighth at most; a freed handle's blocks serve later handles, any stream, because
+//     free_memory waits for the device first;
+//   * a build's temporaries come from a stream-ordered pool, whose reuse the
+//     driver orders between streams and threads.  (The pool's own release
+//     threshold counts the bytes in use too, so it is off; pool_trim keeps the
+//     bound.)
+// At most kBlocksKeep + kPoolKeep bytes (2 GiB, under 1 % of the device) are kept
+// that nothing uses, and all of it is given back when the device's last handle
+// goes: a program that frees each memory before it builds the next allocates anew.
 // ---------------------------------------------------------------------------
 namespace {
-constexpr unsigned long long kPoolKeep = 2ull << 30;
+constexpr unsigned long long kBlocksKeep = 1536ull << 20, kPoolKeep = 512ull << 20;
 // Tokens up to which the folding GEMM reads W_Q along its rows (an MN-major
 // operand) instead of a transposed copy.  The GEMM takes the same time either
 // way (787 us at 32768 tokens of d = 4096); the copy costs its 13 us and the
@@ -219,18 +230,21 @@ constexpr unsigned long long kPoolKeep = 2ull << 30;
 // build, 3495 and 3374, so the copy stays there.
 constexpr int kFoldByRowTokens = 16384;
 constexpr int kMaxDevices = 64;
-struct DevicePool {
+struct DeviceMemory {
   cudaMemPool_t pool = nullptr;
   int users = 0;                     // live handles and builds under way
+  std::vector<MemoryBlock> unused;   // oldest first
+  size_t unused_bytes = 0;
+  std::vector<MemoryBlock> parked;   // freed without a wait for the device: not to be used yet
 };
-std::mutex g_pool_mu;
-DevicePool g_pools[kMaxDevices];
+std::mutex g_mem_mu;
+DeviceMemory g_mem[kMaxDevices];
 
-// The pool of device `dev`, created at its first use; one more user of it.
-cudaError_t pool_enter(int dev, cudaMemPool_t* out) {
+// One more user of device `dev` and its pool, created at its first use.
+cudaError_t mem_enter(int dev, cudaMemPool_t* out) {
   if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-  std::lock_guard<std::mutex> lk(g_pool_mu);
-  DevicePool& p = g_pools[dev];
+  std::lock_guard<std::mutex> lk(g_mem_mu);
+  DeviceMemory& p = g_mem[dev];
   if (p.pool == nullptr) {
     cudaMemPoolProps props = {};
     props.allocType = cudaMemAllocationTypePinned;
@@ -259,46 +273,120 @@ void pool_trim(cudaMemPool_t pool) {
       held > used + kPoolKeep)
     cudaMemPoolTrimTo(pool, used + kPoolKeep);
 }
-// One user less; the last one returns all unused memory.
-void pool_leave(int dev) {
-  std::lock_guard<std::mutex> lk(g_pool_mu);
-  DevicePool& p = g_pools[dev];
-  if (--p.users == 0) cudaMemPoolTrimTo(p.pool, 0);
+// Gives back unused blocks, the oldest first, down to `keep` bytes.  (Nothing on
+// the device uses them, so cudaFree's wait is none.)
+void blocks_trim(DeviceMemory& p, size_t keep) {
+  size_t n = 0;
+  while (n < p.unused.size() && p.unused_bytes > keep) {
+    if (cudaFree(p.unused[n].ptr) != cudaSuccess) {      // not now (a capture): stays
+      cudaGetLastError();
+      break;
+    }
+    p.unused_bytes -= p.unused[n++].bytes;
+  }
+  p.unused.erase(p.unused.begin(), p.unused.begin() + n);
+}
+// The blocks of a handle that goes.  waited: the device has finished all work that
+// was enqueued when they were let go (and so with the parked ones); otherwise they
+// are kept aside until a wait has succeeded.  One user less; the last one returns
+// everything.
+void mem_leave(int dev, const std::vector<MemoryBlock>& blocks, bool waited) {
+  std::lock_guard<std::mutex> lk(g_mem_mu);
+  DeviceMemory& p = g_mem[dev];
+  p.parked.insert(p.parked.end(), blocks.begin(), blocks.end());
+  if (waited) {
+    for (const MemoryBlock& b : p.parked) {
+      p.unused.push_back(b);
+      p.unused_bytes += b.bytes;
+    }
+    p.parked.clear();
+  }
+  const bool last = --p.users == 0;
+  blocks_trim(p, last ? 0 : kBlocksKeep);
+  if (last) cudaMemPoolTrimTo(p.pool, 0);
   else pool_trim(p.pool);
 }
 }  // namespace
 
-static fovea_status alloc_dev(void** ptr, size_t bytes, const char* what, cudaMemPool_t pool,
-                              cudaStream_t s) {
+static fovea_status alloc_failed(const char* what, size_t bytes, cudaError_t e) {
+  cudaGetLastError();
+  return fail(FOVEA_ERR_OOM, "allocation of %s (%zu bytes): %s", what, bytes, cudaGetErrorString(e));
+}
+static bool alloc_fault() {
+  const char* fault = getenv("FOVEA_FAULT_ALLOC");
+  return fault != nullptr && fault[0] == '1';
+}
+
+// A temporary of a build of handle m, from the pool.
+static fovea_status alloc_temp(void** ptr, size_t bytes, const char* what, const fovea_memory* m,
+                               cudaMemPool_t pool, cudaStream_t s) {
   *ptr = nullptr;
   if (bytes == 0) return FOVEA_OK;
-  const char* fault = getenv("FOVEA_FAULT_ALLOC");
-  if (fault != nullptr && fault[0] == '1')
-    return fail(FOVEA_ERR_OOM, "allocation of %s (%zu bytes) failed (FOVEA_FAULT_ALLOC=1)", what,
-                bytes);
   cudaError_t e = cudaMallocFromPoolAsync(ptr, bytes, pool, s);
-  if (e != cudaSuccess) {
+  if (e == cudaErrorMemoryAllocation) {                  // make room, once
     cudaGetLastError();
-    *ptr = nullptr;
-    return fail(FOVEA_ERR_OOM, "allocation of %s (%zu bytes): %s", what, bytes,
-                cudaGetErrorString(e));
+    std::lock_guard<std::mutex> lk(g_mem_mu);
+    blocks_trim(g_mem[m->device], 0);
+    e = cudaMallocFromPoolAsync(ptr, bytes, pool, s);
   }
+  if (e == cudaSuccess) return FOVEA_OK;
+  *ptr = nullptr;
+  return alloc_failed(what, bytes, e);
+}
+
+// A buffer of handle m: an unused block that it fills to four fifths at least, or
+// a new one.
+static fovea_status alloc_block(void** ptr, size_t bytes, const char* what, fovea_memory* m) {
+  *ptr = nullptr;
+  if (bytes == 0) return FOVEA_OK;
+  std::lock_guard<std::mutex> lk(g_mem_mu);
+  DeviceMemory& p = g_mem[m->device];
+  size_t best = p.unused.size();
+  for (size_t i = 0; i < p.unused.size(); ++i)
+    if (p.unused[i].bytes >= bytes && p.unused[i].bytes / 5 * 4 <= align_up(bytes, kBlockGrain) &&
+        (best == p.unused.size() || p.unused[i].bytes < p.unused[best].bytes))
+      best = i;
+  MemoryBlock b;
+  if (best < p.unused.size()) {
+    b = p.unused[best];
+    p.unused.erase(p.unused.begin() + best);
+    p.unused_bytes -= b.bytes;
+  } else {
+    size_t grain = kBlockGrain;
+    while (grain * 16 < bytes) grain *= 2;
+    b.bytes = align_up(bytes, grain);
+    cudaError_t e = cudaMalloc(&b.ptr, b.bytes);
+    if (e == cudaErrorMemoryAllocation && p.unused_bytes > 0) {   // make room, once
+      cudaGetLastError();
+      blocks_trim(p, 0);
+      cudaMemPoolTrimTo(p.pool, 0);
+      e = cudaMalloc(&b.ptr, b.bytes);
+    }
+    if (e == cudaErrorMemoryAllocation && b.bytes > bytes) {
+      cudaGetLastError();
+      b.bytes = bytes;
+      e = cudaMalloc(&b.ptr, b.bytes);
+    }
+    if (e != cudaSuccess) return alloc_failed(what, bytes, e);
+  }
+  m->blocks.push_back(b);
+  *ptr = b.ptr;
   return FOVEA_OK;
 }
 
 // Frees a handle.  Like cudaFree, it waits for the device first, so work still
-// enqueued when the caller lets go of the handle finishes on its memory.
+// enqueued when the caller lets go of the handle finishes on its memory.  Where
+// the wait is not allowed (a stream of the device is being captured), the memory
+// is set aside until a later wait.
 static void free_memory(fovea_memory* m) {
   if (m == nullptr) return;
   int cur = -1;
   cudaGetDevice(&cur);
   if (cur != m->device) cudaSetDevice(m->device);
-  cudaDeviceSynchronize();
-  for (void* p : {m->keys, m->values, m->proj, m->projT, m->folded,
-                  static_cast<void*>(m->orig_index)})
-    if (p != nullptr) cudaFreeAsync(p, nullptr);
-  cudaStreamSynchronize(nullptr);
-  pool_leave(m->device);
+  const char* fault = getenv("FOVEA_FAULT_WAIT");
+  const bool waited = !(fault != nullptr && fault[0] == '1') && cudaDeviceSynchronize() == cudaSuccess;
+  if (!waited) cudaGetLastError();
+  mem_leave(m->device, m->blocks, waited);
   if (cur >= 0 && cur != m->device) cudaSetDevice(cur);
   delete m;
 }
@@ -351,13 +439,12 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
 
   if (capturing(s))
     return fail(FOVEA_ERR_CUDA, "fovea_build_memory synchronises: the stream is being captured");
-  const char* fault = getenv("FOVEA_FAULT_ALLOC");
-  if (fault != nullptr && fault[0] == '1')
+  if (alloc_fault())
     return fail(FOVEA_ERR_OOM, "allocation of build scratch failed (FOVEA_FAULT_ALLOC=1)");
   int dev = 0;
   cudaMemPool_t pool = nullptr;
   cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = pool_enter(dev, &pool);
+  if (e == cudaSuccess) e = mem_enter(dev, &pool);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(FOVEA_ERR_OOM, "device memory pool: %s", cudaGetErrorString(e));
@@ -379,7 +466,7 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
   auto run = [&]() -> fovea_status {
     const bool bf = p->dtype == FOVEA_BF16;
     const size_t count_bytes = align_up(B * sizeof(int32_t), 256);
-    fovea_status rs = alloc_dev(&scratch, 256 + count_bytes + d * sizeof(float), "build scratch", pool, s);
+    fovea_status rs = alloc_temp(&scratch, 256 + count_bytes + d * sizeof(float), "build scratch", m, pool, s);
     if (rs != FOVEA_OK) return rs;
     int* errw = static_cast<int*>(scratch);           // error word
     int32_t* d_counts = reinterpret_cast<int32_t*>(static_cast<uint8_t*>(scratch) + 256);
@@ -419,20 +506,23 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
     const int ld = (m_max + 63) / 64 * 64;
     // bf16: the marks, the RMS of the token rows
     const size_t mark_bytes = align_up((size_t)total * d / 8, 256);
-    if ((rs = alloc_dev(&m->keys, (size_t)total * d * es, "keys", pool, s)) != FOVEA_OK ||
-        (rs = alloc_dev(&m->values, (size_t)total * d * es, "values", pool, s)) != FOVEA_OK ||
-        (rs = alloc_dev(reinterpret_cast<void**>(&m->orig_index), total * sizeof(int32_t), "index",
-                        pool, s)) != FOVEA_OK ||
-        (rs = alloc_dev(&src_row, total * sizeof(int32_t), "source rows", pool, s)) != FOVEA_OK ||
-        (rs = alloc_dev(&xv, (size_t)total * d * es, "LN(v)", pool, s)) != FOVEA_OK ||
-        (bf && (rs = alloc_dev(&fix, mark_bytes + (size_t)total * 4, "key marks", pool, s)) != FOVEA_OK) ||
-        (fold && (rs = alloc_dev(&m->folded, (size_t)total * 2 * d * 2, "folded keys", pool, s)) != FOVEA_OK) ||
+    // (few allocations: a new one costs 30 us and more.  The index lies behind the
+    // values, the transposed projected values behind the projected ones.)
+    const size_t value_bytes = align_up((size_t)total * d * es, 256);
+    const size_t proj_bytes = align_up((size_t)total * 2 * H * 2, 256);
+    if ((rs = alloc_block(&m->keys, (size_t)total * d * es, "keys", m)) != FOVEA_OK ||
+        (rs = alloc_block(&m->values, value_bytes + total * sizeof(int32_t), "values", m)) != FOVEA_OK ||
+        (fold && (rs = alloc_block(&m->folded, (size_t)total * 2 * d * 2, "folded keys", m)) != FOVEA_OK) ||
+        (proj && (rs = alloc_block(&m->proj, proj_bytes + (size_t)B * 2 * H * ld * 2, "projected values",
+                                   m)) != FOVEA_OK) ||
+        (rs = alloc_temp(&src_row, total * sizeof(int32_t), "source rows", m, pool, s)) != FOVEA_OK ||
+        (rs = alloc_temp(&xv, (size_t)total * d * es, "LN(v)", m, pool, s)) != FOVEA_OK ||
+        (bf && (rs = alloc_temp(&fix, mark_bytes + (size_t)total * 4, "key marks", m, pool, s)) != FOVEA_OK) ||
         (fold && total > kFoldByRowTokens &&
-         (rs = alloc_dev(&wqt, (size_t)d * d * 2, "transposed W_Q", pool, s)) != FOVEA_OK) ||
-        (proj && (rs = alloc_dev(&m->proj, (size_t)total * 2 * H * 2, "projected values", pool, s)) != FOVEA_OK) ||
-        (proj && (rs = alloc_dev(&m->projT, (size_t)B * 2 * H * ld * 2, "transposed projected values",
-                                 pool, s)) != FOVEA_OK))
+         (rs = alloc_temp(&wqt, (size_t)d * d * 2, "transposed W_Q", m, pool, s)) != FOVEA_OK))
       return rs;
+    m->orig_index = reinterpret_cast<int32_t*>(static_cast<uint8_t*>(m->values) + value_bytes);
+    if (proj) m->projT = static_cast<uint8_t*>(m->proj) + proj_bytes;
     float* row_rms = bf ? reinterpret_cast<float*>(static_cast<uint8_t*>(fix) + mark_bytes) : nullptr;
     { KernelTimer t("compact", s);
       err = launch_compact(mask, B, M_max, itab, m->orig_index, (int32_t*)src_row,

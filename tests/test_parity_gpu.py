@@ -835,6 +835,76 @@ def test_bounded_waits_of_a_build_report_timeout(fovea, d, m):
         assert torch.equal(a, b)
 
 
+def test_memory_views_can_be_exported(fovea):
+    """The tensors of a handle lie in memory that other processes can open and
+    peers can read (a stream-ordered pool's could not)."""
+    import ctypes
+    w = small_workload("bf16-ragged")
+    s = store(w)
+    params = params_for(s, fovea)
+    mem = fovea.build_memory(params, s.dev["v"], s.dev.get("mask"))
+    cu = ctypes.CDLL("libcuda.so.1")
+    handle = ctypes.create_string_buffer(64)
+    for t in (*mem.views()[:3], mem.folded_keys(params)):
+        assert cu.cuIpcGetMemHandle(handle, ctypes.c_uint64(t.data_ptr())) == 0
+    mem.destroy()
+
+
+def test_memory_freed_without_a_wait_is_not_reused(fovea, monkeypatch):
+    """When the wait for the device fails (FOVEA_FAULT_WAIT=1 stands for a
+    stream under capture), later handles get other memory until a wait has
+    succeeded, and then the memory that was set aside."""
+    w = small_workload("bf16-ragged")
+    s = store(w)
+    params = params_for(s, fovea)
+
+    def build():
+        return fovea.build_memory(params, s.dev["v"], s.dev.get("mask"))
+
+    def spans(m):
+        ts = (*m.views()[:3], m.folded_keys(params))
+        return {(t.data_ptr(), t.data_ptr() + t.numel() * t.element_size()) for t in ts}
+
+    def overlap(a, b):
+        return any(x0 < y1 and y0 < x1 for x0, x1 in a for y0, y1 in b)
+
+    held, first = build(), build()          # (the last handle gives everything back)
+    old = spans(first)
+    monkeypatch.setenv("FOVEA_FAULT_WAIT", "1")
+    first.destroy()
+    monkeypatch.delenv("FOVEA_FAULT_WAIT")
+    later = [build() for _ in range(3)]
+    for m in later:
+        assert not overlap(old, spans(m))
+    later.pop().destroy()                   # waits
+    again = [build(), build()]
+    assert any(overlap(old, spans(m)) for m in again)
+    for m in (held, *later, *again):
+        m.destroy()
+
+
+def test_memory_of_freed_handles_is_given_back(fovea):
+    """What is kept for later handles is bounded, and the last handle gives all
+    of it back."""
+    import gc
+    gc.collect()
+    d = 1024
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    weights, normal = device_weights(g, d)
+    params = fovea.Params(weights, d_model=d)
+    v = [normal(1, m, d) for m in (600, 5000, 20000, 60000, 131, 60000)]
+    held = fovea.build_memory(params, v[0])
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    for x in v[1:] * 2:
+        fovea.build_memory(params, x[:, :32768] if x.shape[1] > 32768 else x).destroy()
+    assert before - torch.cuda.mem_get_info()[0] <= (2 << 30) + (64 << 20)
+    held.destroy()
+    # (other handles of this process, if any, keep at most the same)
+    assert torch.cuda.mem_get_info()[0] >= before - (64 << 20)
+
+
 def test_bad_row_offsets_and_workspace(fovea):
     w = small_workload("bf16-ragged")
     s = store(w)
