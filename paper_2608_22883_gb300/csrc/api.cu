@@ -221,14 +221,6 @@ static fovea_status check_step_params(const fovea_params* p) {
 // ---------------------------------------------------------------------------
 namespace {
 constexpr unsigned long long kBlocksKeep = 1536ull << 20, kPoolKeep = 512ull << 20;
-// Tokens up to which the folding GEMM reads W_Q along its rows (an MN-major
-// operand) instead of a transposed copy.  The GEMM takes the same time either
-// way (787 us at 32768 tokens of d = 4096); the copy costs its 13 us and the
-// temporary.  Builds one at a time, without and with the copy: 303 and 384 us
-// (576 tokens, d = 4096), 1476 and 1533 (9216), 2412 and 2474 (16384), 4560
-// and 4621 (32768); back to back at 32768, where the copy is 0.4 % of the
-// build, 3495 and 3374, so the copy stays there.
-constexpr int kFoldByRowTokens = 16384;
 constexpr int kMaxDevices = 64;
 struct DeviceMemory {
   cudaMemPool_t pool = nullptr;
@@ -457,12 +449,11 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
   m->d = d;
   m->dtype = p->dtype;
   // temporaries: error word, valid counts, norms of W_K's rows | source rows |
-  // LN(v) | marks of the key elements, RMS of the token rows | W_Q^T
+  // LN(v) | marks of the key elements, RMS of the token rows
   void* scratch = nullptr;
   void* src_row = nullptr;
   void* xv = nullptr;
   void* fix = nullptr;
-  void* wqt = nullptr;
   auto run = [&]() -> fovea_status {
     const bool bf = p->dtype == FOVEA_BF16;
     const size_t count_bytes = align_up(B * sizeof(int32_t), 256);
@@ -517,9 +508,7 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
                                    m)) != FOVEA_OK) ||
         (rs = alloc_temp(&src_row, total * sizeof(int32_t), "source rows", m, pool, s)) != FOVEA_OK ||
         (rs = alloc_temp(&xv, (size_t)total * d * es, "LN(v)", m, pool, s)) != FOVEA_OK ||
-        (bf && (rs = alloc_temp(&fix, mark_bytes + (size_t)total * 4, "key marks", m, pool, s)) != FOVEA_OK) ||
-        (fold && total > kFoldByRowTokens &&
-         (rs = alloc_temp(&wqt, (size_t)d * d * 2, "transposed W_Q", m, pool, s)) != FOVEA_OK))
+        (bf && (rs = alloc_temp(&fix, mark_bytes + (size_t)total * 4, "key marks", m, pool, s)) != FOVEA_OK))
       return rs;
     m->orig_index = reinterpret_cast<int32_t*>(static_cast<uint8_t*>(m->values) + value_bytes);
     if (proj) m->projT = static_cast<uint8_t*>(m->proj) + proj_bytes;
@@ -567,20 +556,10 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
       if (err != cudaSuccess) return cuda_fail(err, "refine_keys");
       TmaOperand F[3] = {none, none, none};
       if (fold) {
-        // kappa_i = W_Q^T k_i, a GEMM of W_Q^T (read along W_Q's rows, or
-        // transposed once here) with the stored keys, kept as the hi / lo pair of its fp32 accumulator (no
-        // bf16 rounding of the query map)
-        if (wqt != nullptr) {
-          static thread_local ImageTable one;
-          one.B = 1;
-          one.off[0] = 0;
-          one.m[0] = d;
-          { KernelTimer t("transpose_wq", s);
-            err = launch_transpose_images(p->W_Q, d, d, one, wqt, s); }
-          if (err != cudaSuccess) return cuda_fail(err, "transpose W_Q");
-        }
-        pg.f0_by_row = wqt == nullptr;
-        F[0] = TmaOperand{wqt != nullptr ? wqt : p->W_Q, d, d, d};
+        // kappa_i = W_Q^T k_i, a GEMM of W_Q^T (read along W_Q's rows) with the
+        // stored keys, kept as the hi / lo pair of its fp32 accumulator (no bf16
+        // rounding of the query map)
+        F[0] = TmaOperand{p->W_Q, d, d, d};
         pg.out[0] = m->folded;
         pg.out_lo = static_cast<__nv_bfloat16*>(m->folded) + d;
         pg.ldc[0] = 2 * d;
@@ -620,7 +599,7 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
     return FOVEA_OK;
   };
   st = run();
-  for (void* t : {scratch, src_row, xv, fix, wqt})
+  for (void* t : {scratch, src_row, xv, fix})
     if (t != nullptr) cudaFreeAsync(t, s);
   cudaStreamSynchronize(s);
   pool_trim(pool);

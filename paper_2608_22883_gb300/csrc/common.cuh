@@ -357,12 +357,11 @@ cudaError_t launch_gemm_tc(int epi, const GemmArgs& a, const TmaOperand& A0, con
 // three feature matrices F[i] [cols, K] (bf16; a null base: no such part),
 // fp32 sums stored as bf16 with row stride ldc[i].  keys: part 0's elements
 // near a rounding midpoint are marked; else part 0 is stored as a pair, hi =
-// bf16(sum) to out[0] and bf16(sum - hi) to out_lo, and with f0_by_row its
-// (square) matrix is F[0]^T, read along F[0]'s rows.
+// bf16(sum) to out[0] and bf16(sum - hi) to out_lo, and its (square) matrix is
+// F[0]^T, read along F[0]'s rows.
 struct PairGemm {
   int rows;                                      // token rows
   void* out[3]; long long ldc[3]; void* out_lo;
-  bool f0_by_row;
   uint32_t* fix_bits;                            // keys: bit c % 32 of [row * ldc[0] / 32 + c / 32]
   const float* row_rms;                          // keys: root mean square of each token row,
   const float* feat_norm;                        // norm of each row of F[0]

@@ -79,8 +79,8 @@ constexpr uint32_t kTmemCols = 512;
 // kind::f16: D fp32, A and B bf16, both K-major, N = 256, M = 256
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
                             ((uint32_t)(2 * BM >> 4) << 24);
-// f0_by_row: the folded part's features are W_Q read as it lies, the contraction
-// along its rows: B MN-major (bit 16).  A stage holds two blocks of 64 features, each
+// The folded part's features are W_Q read as it lies, the contraction along its
+// rows: B MN-major (bit 16).  A stage holds two blocks of 64 features, each
 // KPS * 64 contraction rows of 128 bytes (128-byte swizzle): 16 KB from one
 // block of features to the next, 1 KB from 8 contraction rows to the next.
 constexpr uint32_t kIdescMn = kIdesc | (1u << 16);
@@ -231,7 +231,7 @@ __device__ __forceinline__ Tile tile_at(const PairGemm& a, int t) {
 
 // KEYS: part 0 is the keys (rounded, near-midpoint elements marked); HILO: part
 // 0's sums are stored as hi = bf16(sum) to out[0] and bf16(sum - hi) to out_lo,
-// and its feature matrix may lie as [K, cols] (f0_by_row).  The
+// and its feature matrix lies as [K, cols].  The
 // other parts are rounded sums.  Part 0 reads the tokens of tmR0, the others
 // those of tmR1.
 template <bool KEYS, bool HILO>
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
         }
         if (lane == 0 && rank == 0) mbar_expect_tx(&full[st], 2u * kStageBytes);
         const uint32_t dst = smem_u32(smem + st * kStageBytes) + (lane == 1 ? 0u : (uint32_t)(KPS * kSmemRows));
-        if (HILO && lane == 0 && ti.part == 0 && a.f0_by_row)
+        if (HILO && lane == 0 && ti.part == 0)
           tma_load_pair(dst, map, map_dsmem(smem_u32(&full[st]), 0), 0, su * KPS * 64, y / 64);
         else
           tma_load_pair(dst, map, map_dsmem(smem_u32(&full[st]), 0), 0, y, su * KPS);
@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
     for (int t = pid; go && t < tiles; t += pairs) {
       const int part = tile_at(a, t).part;
       const int chunk = a.chunk[part];
-      const bool mn = HILO && part == 0 && a.f0_by_row;
+      const bool mn = HILO && part == 0;
       int su0 = 0;
       for (int len = a.chunk0[part]; go && su0 < su_total; su0 += len, len = chunk, ++c) {
         const int buf = c & 1;

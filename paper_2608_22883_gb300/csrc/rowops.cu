@@ -755,12 +755,11 @@ __global__ void __launch_bounds__(kRefineThreads) refine_keys_kernel(
 
 // Per image b: out[(b C + c) * ld + j] = in[(off_b + j) * C + c] for entries
 // j < m_b and columns c < C, zero for m_b <= j < ld: the transposed projected
-// values the weighted-sum GEMM reads, K-major over the image's entries, and
-// (as one image of d rows) W_Q^T for the query folding.  Bound by HBM: each
-// CTA moves a 64 x 64 tile with 16-byte accesses on both sides (a row of the
+// values the weighted-sum GEMM reads, K-major over the image's entries.  Bound
+// by HBM: each CTA moves a 64 x 64 tile with 16-byte accesses on both sides (a row of the
 // tile is a full 128-byte line), and its pitch of 33 words keeps the 4-byte
-// stores free of bank conflicts and the 2-byte reads at two ways.  W_Q at d =
-// 4096 (67 MB moved): 21 us against 42 us with 2-byte global accesses.
+// stores free of bank conflicts and the 2-byte reads at two ways.  A 4096 x 4096
+// matrix (67 MB moved): 21 us against 42 us with 2-byte global accesses.
 __global__ void __launch_bounds__(256) transpose_images_kernel(const __nv_bfloat16* __restrict__ in,
                                                                int C, int ld,
                                                                const __grid_constant__ ImageTable tab,

@@ -148,7 +148,7 @@ def test_memory_build_matches_oracle(fovea, name):
 # two and chunks of four: token counts at the edges of a CTA's and a pair's
 # rows and past a band of 8 row tiles; d with partial feature tiles, an odd
 # number of k-blocks, fewer k-blocks than a stage, a chunk, the ring; and more
-# tokens than the folding GEMM reads W_Q along its rows for
+# tokens than the folded keys keep several accumulators for
 @pytest.mark.parametrize("d,m_sizes", [(64, [1]), (192, [128]), (256, [129, 3]), (320, [255]),
                                        (448, [257]), (576, [385, 0, 130]), (128, [2100]),
                                        (64, [8192, 8193])])
