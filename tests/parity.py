@@ -223,13 +223,14 @@ def _check_order(orc, w, mem, n, idx_g):
         assert a >= c - BAND * max(1.0, abs(a)) * 4, f"row {n}: selected list not in descending order"
 
 
-def run_gpu(s: Stored, fovea, params=None, memory=None, l_max=None):
+def run_gpu(s: Stored, fovea, params=None, memory=None, l_max=None, want_readout=True):
     """Build the memory and run one step through the C ABI; returns numpy outputs."""
     w = s.w
     params = params or params_for(s, fovea)
     mem = memory or fovea.build_memory(params, s.dev["v"], s.dev.get("mask"))
     out = fovea.step(params, mem, s.dev["h"], s.dev["depth"], w.row_offsets,
-                     s.dev.get("row_scale"), w.rho, w.k_min, w.k_max, l_max=l_max)
+                     s.dev.get("row_scale"), w.rho, w.k_min, w.k_max, l_max=l_max,
+                     want_readout=want_readout)
     fovea.sync_errors(out["workspace"])
     res = {k: (v.float().cpu().numpy() if v.is_floating_point() else v.cpu().numpy())
            for k, v in out.items() if v is not None and k != "workspace"}

@@ -339,7 +339,9 @@ def test_selection_row_lengths(fovea, M, k, ties):
                                             ([256, 320, 63], [130, 7, 64], 512),
                                             ([700], [2], 128)])
 def test_dense_weights_entry_edges(fovea, m_sizes, rows, H):
-    w = workloads.generate_custom("act", 128, m_sizes, rows, k_max=300, rho=0.97, seed=len(rows), H=H)
+    """K fixed (k_min = k_max): only cuts between near-equal scores are boundary
+    rows."""
+    w = workloads.generate_custom("act", 128, m_sizes, rows, k_max=300, k_min=300, seed=len(rows), H=H)
     s = store(w)
     fovea.timing_enable(True)
     gpu = run_gpu(s, fovea)
@@ -347,14 +349,12 @@ def test_dense_weights_entry_edges(fovea, m_sizes, rows, H):
     fovea.timing_enable(False)
     assert "act_gemm" in names
     orc, mem = run_oracle(s, mirror=True)
-    # flat rows with K in the hundreds: one entry moves the mass by ~1e-3, so
-    # the 1e-4 band catches up to a quarter of them
-    compare(gpu, orc, s, mem=mem, max_exempt=0.35)
+    compare(gpu, orc, s, mem=mem)
 
 
-# caps above 64, or more rows than SMs without a readout, gather in a kernel of
-# their own: fewer and more entries than its 8 warps x 8 loads, a partial
-# column chunk (2H = 256, d = 320), gated rows, empty images, K = 0
+# caps above 64 gather in a kernel of their own: fewer and more entries than its
+# 8 warps x 8 loads, a partial column chunk (2H = 256, d = 320), gated rows, empty
+# images, K = 0
 @pytest.mark.parametrize("d,m_sizes,rows,k,H", [(320, [300, 0, 70], [9, 2, 3], 65, 128),
                                                 (256, [600], [7], 256, 512),
                                                 (256, [5, 130], [1, 8], 128, 256)])
@@ -427,6 +427,52 @@ def test_very_negative_pre_activations_vanish(fovea, d, m, rows, k, dtype, plain
     y = s.f64["h"] + gpu["gate"].astype(np.float64)[:, None] * s.f64["b_f2"]
     want = oracle.rms_norm(y, s.f64["rms_gamma"], RMS_EPS)
     assert rel_err_rows(gpu["h_out"].astype(np.float64), want).max() <= (5e-3 if dtype == "bf16" else 1e-5)
+    mem.destroy()
+
+
+# without a readout (what a decoding loop asks for): the selection + gather kernel,
+# the selection and a gather of the projected values alone, the dense weights
+# without a list of the selection, the unfolded and the plain path, fp32; None rows:
+# one more than the SMs, for which caps of up to 64 too gather in a kernel of their own
+@pytest.mark.parametrize("kw,kernel", [
+    (dict(d=256, m_sizes=[200, 0, 129], rows=[37, 5, 20], k_max=16), "select_fuse"),
+    (dict(d=320, m_sizes=[300, 0, 70], rows=[9, 2, 3], k_max=100), "gather_fuse"),
+    (dict(d=256, m_sizes=[600, 90], rows=None, k_max=64), "gather_fuse"),
+    (dict(d=256, m_sizes=[2500, 300], rows=[12, 5], k_max=64), "act_gemm"),
+    (dict(d=256, m_sizes=[600], rows=[20], k_max=500, k_min=500), "act_gemm"),
+    (dict(d=256, m_sizes=[200, 37], rows=[17, 5], k_max=16, plain=True), "fuse_hidden"),
+    (dict(d=256, m_sizes=[2500], rows=[6], k_max=300, plain=True), "fuse_hidden"),
+    (dict(d=192, m_sizes=[300, 20], rows=[17, 3], k_max=64, dtype="fp32"), "fuse_hidden")])
+def test_steps_without_a_readout(fovea, kw, kernel):
+    kw = dict(kw)
+    plain = kw.pop("plain", False)
+    if kw["rows"] is None:
+        n = torch.cuda.get_device_properties(0).multi_processor_count + 1
+        kw["rows"] = [n // 2, n - n // 2]
+    w = workloads.generate_custom("no-readout", kw.pop("d"), kw.pop("m_sizes"), kw.pop("rows"),
+                                  temperature=(0.5, 2.0), H=128, **kw)
+    s = store(w)
+    params = params_for(s, fovea)
+    mem = fovea.build_memory(params, s.dev["v"], s.dev.get("mask"))
+    if plain:
+        weights = {n: s.dev[n] for n in workloads.PARAM_NAMES}
+        for n in ("W_Q", "W_f1", "W_g1"):
+            weights[n] = weights[n].clone()
+        params = fovea.Params(weights, d_model=w.d, mlp_hidden=128,
+                              max_depth=w.params["E_dep"].shape[0] - 1)
+    fovea.timing_enable(True)
+    gpu = run_gpu(s, fovea, params=params, memory=mem, l_max=3, want_readout=False)
+    names = set(fovea.timing_read())
+    fovea.timing_enable(True)               # clears the records
+    full = run_gpu(s, fovea, params=params, memory=mem, l_max=3)
+    fovea.timing_enable(False)
+    assert kernel in names and gpu.get("readout") is None, names
+    orc, omem = run_oracle(s, mirror=(w.dtype == "bf16"), l_max=3)
+    # (one entry moves the mass of a flat row with K in the hundreds by about 1e-3)
+    compare(gpu, orc, s, mem=omem, mirror=(w.dtype == "bf16"), max_exempt=0.35)
+    for k in ("counts", "indices"):
+        np.testing.assert_array_equal(gpu[k], full[k])
+    assert rel_err_rows(gpu["h_out"].astype(np.float64), full["h_out"].astype(np.float64)).max() <= 2e-2
     mem.destroy()
 
 
@@ -510,10 +556,11 @@ def test_folded_and_unfolded_steps_select_the_same_entries(fovea, name):
 
 
 def test_paths_are_taken(fovea):
-    """bf16 rows of up to 2048 entries, caps of up to 256 and batches of up
-    to twice the SMs run the selection, the projected readout and the first
-    fusion layer's activation in one kernel; otherwise the selection writes
-    dense weights and one GEMM against the transposed projected values forms
+    """bf16 rows of up to 2048 entries, caps of up to 64 and batches of up to
+    the SMs (twice the SMs with a readout) run the selection, the projected
+    readout and the first fusion layer's activation in one kernel; caps of up
+    to 256 and batches of up to twice the SMs select first and gather in a
+    second kernel; otherwise the selection writes dense weights and one GEMM against the transposed projected values forms
     the activation (the readout, when asked for, has its own kernel); fp32
     takes the unfolded SIMT path with the first fusion layer as a GEMM."""
     try:
