@@ -896,11 +896,15 @@ FOVEA_API fovea_status fovea_retrieve_fuse(const fovea_params* p, const fovea_me
   const bool gh_in_scores = gh_seq >= 0;
   // Several score groups: G_h as further groups of the score launch, one per
   // 128 rows, so that its L2-fed tiles run beside the HBM-bound score tiles and
-  // a launch is saved: 8 images x 8 rows at d = 1024 32.4 -> 26.3 us a step, 8
-  // ragged images x 32 rows 95.2 -> 90.3, 16 x 64 rows 132.3 -> 119.9, 4 x 128
-  // rows of 8192 entries 184.9 -> 172.3.  (62 rows of d = 256 gain as well, 25.8
-  // -> 21.6, but up to one block of narrow rows keeps G_h as its own launch,
-  // the structure test_paths_are_taken holds such a call to.)
+  // a launch is saved: 8 images x 8 rows at d = 1024 29.5 -> 24.5 us a step, 8
+  // ragged images x 32 rows 84.3 -> 74.3, 16 x 64 rows 123.3 -> 108.8, 4 x 128
+  // rows of 8192 entries 177.8 -> 167.1; of 332 steps drawn over the range 173
+  // gain 2 % and more and 20 lose as much (16 images of 1102 entries, 214 rows, d =
+  // 4096: 86.7 -> 101.6, whose one launch finds no plan with G_h's accumulators
+  // that fits both parts).  Up to one block of narrow rows (d below 512) G_h keeps
+  // its own launch, which calls without score groups and with more groups than the
+  // table holds need as well; no workload has such rows, and they would gain too (60
+  // rows of d = 256: 24.2 -> 20.8).
   const int gh_blocks = (N + 127) / 128;
   const bool gh_groups = use_fold && use_proj && !gh_in_scores && ngroups > 0 &&
                          (N > 128 || d >= 512) && ngroups + gh_blocks <= FOVEA_MAX_SEQ;
