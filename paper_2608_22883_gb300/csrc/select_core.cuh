@@ -340,7 +340,6 @@ __device__ void select_finish(const SelectArgs& a, int n, int M, int key_off, co
     const int chunk = (M + kSelThreads - 1) / kSelThreads;
     const int beg = min(M, tid * chunk), end = min(M, beg + chunk);
     int c = 0;
-#pragma unroll U
     for (int i = beg; i < end; ++i) c += ord_key(norm_score(s_sc[i])) == T;
     int incl = c;
 #pragma unroll
