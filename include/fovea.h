@@ -141,9 +141,10 @@ typedef struct fovea_params {
  * precision the unfolded scores give q = W_Q x_n), so both score forms
  * follow the paper's q . k to within fp32 accumulation.  Pass W_Q = NULL here
  * to keep the unfolded scores.
- * This call allocates the handle's device buffers (cudaMalloc memory, kept for
- * later handles when this one goes: at most 2 GiB per device with the memory of
- * the build's temporaries, all given back with the device's last handle) and
+ * This call allocates the handle's device buffers (in one cudaMalloc block: an
+ * IPC handle of a view opens the block, at whose start the keys lie; a freed
+ * handle's block is kept for later ones, at most 2 GiB per device with the memory
+ * of the builds' temporaries, all given back with the device's last handle) and
  * synchronises `stream`, at the end and, with a mask, once more for the valid
  * counts.  B in [1, FOVEA_MAX_SEQ], M_max in [0, ...],
  * per-image valid count <= FOVEA_MAX_ENTRIES.

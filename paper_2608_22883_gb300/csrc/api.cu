@@ -117,7 +117,7 @@ constexpr size_t kBlockGrain = 64 << 10;
 
 struct fovea_memory {
   int device = 0;
-  std::vector<MemoryBlock> blocks;   // what the buffers below lie in
+  MemoryBlock block;                 // what the buffers below lie in
   int B = 0, M_max = 0, d = 0, dtype = 0;
   int total = 0;
   std::vector<int32_t> counts;       // valid entries per image (host)
@@ -208,9 +208,10 @@ static fovea_status check_step_params(const fovea_params* p) {
 // Device memory.  cudaMalloc and cudaFree cost 30 - 180 us each, ten to twelve of
 // them 0.8 ms of a one-image build whose kernels take 0.2 ms, so both kinds of
 // memory are kept for the next build, per device:
-//   * a handle's buffers are cudaMalloc blocks (their views can be exported to
-//     other processes and read by peers), rounded up by an eighth at most; a freed handle's blocks serve later handles, any stream, because
-//     free_memory waits for the device first;
+//   * a handle's buffers lie in one cudaMalloc block (so that they can be exported
+//     to other processes and read by peers), rounded up by an eighth at most; a
+//     freed handle's block serves later handles on any stream, because free_memory
+//     waits for the device first;
 //   * a build's temporaries come from a stream-ordered pool, whose reuse the
 //     driver orders between streams and threads.  (The pool's own release
 //     threshold counts the bytes in use too, so it is off; pool_trim keeps the
@@ -278,14 +279,14 @@ void blocks_trim(DeviceMemory& p, size_t keep) {
   }
   p.unused.erase(p.unused.begin(), p.unused.begin() + n);
 }
-// The blocks of a handle that goes.  waited: the device has finished all work that
-// was enqueued when they were let go (and so with the parked ones); otherwise they
-// are kept aside until a wait has succeeded.  One user less; the last one returns
+// The block of a handle that goes.  waited: the device has finished all work that
+// was enqueued when it was let go (and so with the parked ones); otherwise it is
+// kept aside until a wait has succeeded.  One user less; the last one returns
 // everything.
-void mem_leave(int dev, const std::vector<MemoryBlock>& blocks, bool waited) {
+void mem_leave(int dev, const MemoryBlock& block, bool waited) {
   std::lock_guard<std::mutex> lk(g_mem_mu);
   DeviceMemory& p = g_mem[dev];
-  p.parked.insert(p.parked.end(), blocks.begin(), blocks.end());
+  if (block.ptr != nullptr) p.parked.push_back(block);
   if (waited) {
     for (const MemoryBlock& b : p.parked) {
       p.unused.push_back(b);
@@ -326,11 +327,9 @@ static fovea_status alloc_temp(void** ptr, size_t bytes, const char* what, const
   return alloc_failed(what, bytes, e);
 }
 
-// A buffer of handle m: an unused block that it fills to four fifths at least, or
-// a new one.
-static fovea_status alloc_block(void** ptr, size_t bytes, const char* what, fovea_memory* m) {
-  *ptr = nullptr;
-  if (bytes == 0) return FOVEA_OK;
+// The block of handle m: an unused one that it fills to four fifths at least, or a
+// new one.
+static fovea_status alloc_block(size_t bytes, fovea_memory* m) {
   std::lock_guard<std::mutex> lk(g_mem_mu);
   DeviceMemory& p = g_mem[m->device];
   size_t best = p.unused.size();
@@ -359,10 +358,9 @@ static fovea_status alloc_block(void** ptr, size_t bytes, const char* what, fove
       b.bytes = bytes;
       e = cudaMalloc(&b.ptr, b.bytes);
     }
-    if (e != cudaSuccess) return alloc_failed(what, bytes, e);
+    if (e != cudaSuccess) return alloc_failed("the handle's buffers", bytes, e);
   }
-  m->blocks.push_back(b);
-  *ptr = b.ptr;
+  m->block = b;
   return FOVEA_OK;
 }
 
@@ -378,7 +376,7 @@ static void free_memory(fovea_memory* m) {
   const char* fault = getenv("FOVEA_FAULT_WAIT");
   const bool waited = !(fault != nullptr && fault[0] == '1') && cudaDeviceSynchronize() == cudaSuccess;
   if (!waited) cudaGetLastError();
-  mem_leave(m->device, m->blocks, waited);
+  mem_leave(m->device, m->block, waited);
   if (cur >= 0 && cur != m->device) cudaSetDevice(cur);
   delete m;
 }
@@ -448,12 +446,10 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
   m->M_max = M_max;
   m->d = d;
   m->dtype = p->dtype;
-  // temporaries: error word, valid counts, norms of W_K's rows | source rows |
-  // LN(v) | marks of the key elements, RMS of the token rows
+  // temporaries: error word, valid counts, norms of W_K's rows | LN(v), source
+  // rows, marks of the key elements, RMS of the token rows
   void* scratch = nullptr;
-  void* src_row = nullptr;
-  void* xv = nullptr;
-  void* fix = nullptr;
+  void* temps = nullptr;
   auto run = [&]() -> fovea_status {
     const bool bf = p->dtype == FOVEA_BF16;
     const size_t count_bytes = align_up(B * sizeof(int32_t), 256);
@@ -497,28 +493,41 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
     const int ld = (m_max + 63) / 64 * 64;
     // bf16: the marks, the RMS of the token rows
     const size_t mark_bytes = align_up((size_t)total * d / 8, 256);
-    // (few allocations: a new one costs 30 us and more.  The index lies behind the
-    // values, the transposed projected values behind the projected ones.)
-    const size_t value_bytes = align_up((size_t)total * d * es, 256);
-    const size_t proj_bytes = align_up((size_t)total * 2 * H * 2, 256);
-    if ((rs = alloc_block(&m->keys, (size_t)total * d * es, "keys", m)) != FOVEA_OK ||
-        (rs = alloc_block(&m->values, value_bytes + total * sizeof(int32_t), "values", m)) != FOVEA_OK ||
-        (fold && (rs = alloc_block(&m->folded, (size_t)total * 2 * d * 2, "folded keys", m)) != FOVEA_OK) ||
-        (proj && (rs = alloc_block(&m->proj, proj_bytes + (size_t)B * 2 * H * ld * 2, "projected values",
-                                   m)) != FOVEA_OK) ||
-        (rs = alloc_temp(&src_row, total * sizeof(int32_t), "source rows", m, pool, s)) != FOVEA_OK ||
-        (rs = alloc_temp(&xv, (size_t)total * d * es, "LN(v)", m, pool, s)) != FOVEA_OK ||
-        (bf && (rs = alloc_temp(&fix, mark_bytes + (size_t)total * 4, "key marks", m, pool, s)) != FOVEA_OK))
+    // the handle's buffers, back to back in one block
+    const size_t kv_bytes = align_up((size_t)total * d * es, 256);
+    const size_t index_bytes = align_up(total * sizeof(int32_t), 256);
+    const size_t fold_bytes = fold ? (size_t)total * 2 * d * 2 : 0;
+    const size_t proj_bytes = proj ? align_up((size_t)total * 2 * H * 2, 256) : 0;
+    const size_t projT_bytes = proj ? (size_t)B * 2 * H * ld * 2 : 0;
+    if ((rs = alloc_block(2 * kv_bytes + index_bytes + fold_bytes + proj_bytes + projT_bytes, m)) != FOVEA_OK ||
+        (rs = alloc_temp(&temps, kv_bytes + index_bytes + (bf ? mark_bytes + (size_t)total * 4 : 0),
+                         "build temporaries", m, pool, s)) != FOVEA_OK)
       return rs;
-    m->orig_index = reinterpret_cast<int32_t*>(static_cast<uint8_t*>(m->values) + value_bytes);
-    if (proj) m->projT = static_cast<uint8_t*>(m->proj) + proj_bytes;
-    float* row_rms = bf ? reinterpret_cast<float*>(static_cast<uint8_t*>(fix) + mark_bytes) : nullptr;
+    uint8_t* at = static_cast<uint8_t*>(temps);
+    auto take = [&](size_t bytes) {
+      uint8_t* here = at;
+      at += bytes;
+      return static_cast<void*>(here);
+    };
+    void* xv = take(kv_bytes);                      // LN(v)
+    int32_t* src_row = static_cast<int32_t*>(take(index_bytes));
+    uint32_t* fix = bf ? static_cast<uint32_t*>(take(mark_bytes)) : nullptr;
+    float* row_rms = reinterpret_cast<float*>(at);  // bf16
+    at = static_cast<uint8_t*>(m->block.ptr);
+    m->keys = take(kv_bytes);
+    m->values = take(kv_bytes);
+    m->orig_index = static_cast<int32_t*>(take(index_bytes));
+    if (fold) m->folded = take(fold_bytes);
+    if (proj) {
+      m->proj = take(proj_bytes);
+      m->projT = take(projT_bytes);
+    }
     { KernelTimer t("compact", s);
-      err = launch_compact(mask, B, M_max, itab, m->orig_index, (int32_t*)src_row,
+      err = launch_compact(mask, B, M_max, itab, m->orig_index, src_row,
                            RowNorms{p->W_K, d, bf ? feat_norm : nullptr}, s); }
     if (err != cudaSuccess) return cuda_fail(err, "compact");
     { KernelTimer t("ln_v", s);
-      err = launch_ln_rows(p->dtype, v, (const int32_t*)src_row, total, d, p->ln_v_gamma,
+      err = launch_ln_rows(p->dtype, v, src_row, total, d, p->ln_v_gamma,
                            p->ln_v_beta, p->ln_eps, xv, row_rms, s); }
     if (err != cudaSuccess) return cuda_fail(err, "ln_v");
     if (!bf) {
@@ -542,7 +551,7 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
       pg.err = errw;
       pg.out[0] = m->keys; pg.out[1] = m->values;
       pg.ldc[0] = pg.ldc[1] = d;
-      pg.fix_bits = static_cast<uint32_t*>(fix);
+      pg.fix_bits = fix;
       pg.row_rms = row_rms;
       pg.feat_norm = feat_norm;
       const TmaOperand none{nullptr, 0, 0, 0}, tokens{xv, total, d, d};
@@ -599,7 +608,7 @@ FOVEA_API fovea_status fovea_build_memory(const fovea_params* p, const void* v,
     return FOVEA_OK;
   };
   st = run();
-  for (void* t : {scratch, src_row, xv, fix})
+  for (void* t : {scratch, temps})
     if (t != nullptr) cudaFreeAsync(t, s);
   cudaStreamSynchronize(s);
   pool_trim(pool);
