@@ -160,7 +160,7 @@ __device__ __forceinline__ void sum2_join(float& s, float& c, float s2, float c2
 // and about 15 of the map and its midpoint test.  A row per warp needs no CTA
 // barrier and one reduction, where a CTA per row took two barriers and
 // double-float arithmetic on every element: 32768 rows of 4096 took 932 us, now
-// 219 us (2.4 TB/s).
+// 225 us (2.4 TB/s; 6 of them for the RMS of the results).
 constexpr int kLnTokWarps = 4;
 constexpr int kLnTokLoads = 8;          // 16-byte loads in flight per lane
 // Rows per SM up to which the four warps of a CTA share a row: with a row per
@@ -682,7 +682,8 @@ cudaError_t launch_readout(int dtype, const RowGather& a, int N, cudaStream_t s)
 // = 4096, 8 KB each) and by the summation's instructions, two products side by
 // side in packed fp32 arithmetic.  A warp per element of a list in no order
 // read both rows from L2 and summed one product at a time: 1025 us at 32768
-// tokens of d = 4096, now 846, and 291 us at 10368 tokens of d = 3584, now 227.
+// tokens of d = 4096, now 864 (846 before the window of the marks was widened),
+// and 291 us at 10368 tokens of d = 3584, now 231.
 // ---------------------------------------------------------------------------
 constexpr int kRefineThreads = 256;
 // Tokens per SM up to which two CTAs share a token: five CTAs fit an SM, so

@@ -930,6 +930,47 @@ def test_memory_freed_without_a_wait_is_not_reused(fovea, monkeypatch):
         m.destroy()
 
 
+def test_builds_on_two_streams(fovea):
+    """Two threads build and free memories of changing sizes at the same time:
+    blocks pass between them, and every result is that of a build by itself."""
+    import threading
+    d = 512
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    weights, normal = device_weights(g, d)
+    params = fovea.Params(weights, d_model=d)
+    sizes = (700, 90, 2500, 640, 1300)
+    v = {m: normal(1, m, d) for m in sizes}
+
+    def result(m):
+        mem = fovea.build_memory(params, v[m])
+        out = [t.clone() for t in (*mem.views()[:3], mem.folded_keys(params))]
+        torch.cuda.current_stream().synchronize()
+        mem.destroy()
+        return out
+
+    want = {m: result(m) for m in sizes}
+    torch.cuda.synchronize()
+    wrong = []
+
+    def loop(first):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for k in range(25):
+                    m = sizes[(first + k) % len(sizes)]
+                    if not all(torch.equal(a, b) for a, b in zip(want[m], result(m))):
+                        wrong.append(m)
+        except Exception as e:              # reported by the main thread
+            wrong.append(e)
+
+    threads = [threading.Thread(target=loop, args=(i,)) for i in (0, 2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong, wrong
+
+
 def test_memory_of_freed_handles_is_given_back(fovea):
     """What is kept for later handles is bounded, and the last handle gives all
     of it back."""
